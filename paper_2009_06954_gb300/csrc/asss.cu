@@ -1949,8 +1949,7 @@ static asss_status do_setup(asss_handle* h, const asss_csr* Ain, asss_stats* st)
         ASSS_TRY(h->Q64.alloc((int64_t)n * h->kp));
         ASSS_TRY(to_rowmajor(h->Qcm.p, n, h->k, n, h->kp, h->Q64.p, s));
         if (o.precision == ASSS_PREC_MIXED && !qb) {
-            ASSS_TRY(h->Q32.alloc((int64_t)n * h->kp));
-            ASSS_TRY(to_rowmajor_f(h->Qcm.p, n, h->k, n, h->kp, h->Q32.p, s));
+            ASSS_TRY(q_to_f32(h->Qcm.p, n, h->k, n, h->kp, h->use_dia || h->factored, h->Q32, s));
         }
     }
     // work buffers and the mrs workspace
@@ -2437,8 +2436,7 @@ asss_status asss_mrs_multi(const asss_csr* J, int k, const double* q, const doub
     if (k) {
         ASSS_TRY(to_device(Qcm, q, (int64_t)n * k, s));
         if (fp32) {
-            ASSS_TRY(Q32.alloc((int64_t)n * kp));
-            ASSS_TRY(to_rowmajor_f(Qcm.p, n, k, n, kp, Q32.p, s));
+            ASSS_TRY(q_to_f32(Qcm.p, n, k, n, kp, dia != 0, Q32, s));
         } else {
             ASSS_TRY(Q64.alloc((int64_t)n * kp));
             ASSS_TRY(to_rowmajor(Qcm.p, n, k, n, kp, Q64.p, s));
@@ -2515,8 +2513,7 @@ asss_status asss_mrs(const asss_csr* J, int k, const double* q, const double* al
     if (k) {
         ASSS_TRY(to_device(Qcm, q, (int64_t)n * k, s));
         if (fp32) {
-            ASSS_TRY(Q32.alloc((int64_t)n * kp));
-            ASSS_TRY(to_rowmajor_f(Qcm.p, n, k, n, kp, Q32.p, s));
+            ASSS_TRY(q_to_f32(Qcm.p, n, k, n, kp, dia != 0, Q32, s));
         } else {
             ASSS_TRY(Q64.alloc((int64_t)n * kp));
             ASSS_TRY(to_rowmajor(Qcm.p, n, k, n, kp, Q64.p, s));

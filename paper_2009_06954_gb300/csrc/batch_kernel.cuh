@@ -163,10 +163,14 @@ __device__ __forceinline__ void bq_row(const BatchMat& M, int i, float (&q)[KP >
                 }
             }
         } else {
-            const float4* row = reinterpret_cast<const float4*>(M.Q32 + (size_t)i * KP);
+            // skew diagonals visit the rows in order: Q in slices of 32 rows (see q_blocked)
+            const bool blk = M.ndiag > 0;
+            const float4* row = reinterpret_cast<const float4*>(M.Q32 + (size_t)(blk ? i & ~31 : i) * KP) +
+                                (blk ? i & 31 : 0);
+            const int st = blk ? 32 : 1;
 #pragma unroll
             for (int t = 0; t < KP / 4; ++t) {
-                float4 v = __ldg(row + t);
+                float4 v = __ldg(row + t * st);
                 q[4 * t] = v.x;
                 q[4 * t + 1] = v.y;
                 q[4 * t + 2] = v.z;

@@ -265,9 +265,22 @@ asss_status to_rowmajor(const double* A, int lda, int p, int n, int kp, double* 
     ASSS_CHECK_LAUNCH();
     return ASSS_OK;
 }
-asss_status to_rowmajor_f(const double* A, int lda, int p, int n, int kp, float* out, cudaStream_t s) {
+// FP32 copy for the mrs kernels: row by row, or (blocked) in slices of 32 rows with the
+// values m..m+3 of a slice's rows side by side (rows past n hold zeros)
+__global__ void k_q_blocked(const double* A, int lda, int p, int n, int kp, int64_t total, float* out) {
+    const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (t >= total) return;
+    const int64_t per = (int64_t)32 * kp;
+    const int64_t i = t / per * 32 + t % 128 / 4;
+    const int a = (int)(t % per / 128 * 4 + t % 4);
+    out[t] = (i < n && a < p) ? (float)A[(size_t)a * lda + i] : 0.f;
+}
+asss_status q_to_f32(const double* A, int lda, int p, int n, int kp, bool blocked, DBuf<float>& out, cudaStream_t s) {
     if (kp == 0) return ASSS_OK;
-    k_to_rowmajor<float><<<cdiv((int64_t)n * kp, 256), 256, 0, s>>>(A, lda, p, n, kp, out);
+    const int64_t total = blocked ? ((int64_t)n + 31) / 32 * 32 * kp : (int64_t)n * kp;
+    ASSS_TRY(out.alloc(total));
+    if (blocked) k_q_blocked<<<cdiv(total, 256), 256, 0, s>>>(A, lda, p, n, kp, total, out.p);
+    else k_to_rowmajor<float><<<cdiv(total, 256), 256, 0, s>>>(A, lda, p, n, kp, out.p);
     ASSS_CHECK_LAUNCH();
     return ASSS_OK;
 }

@@ -41,7 +41,9 @@ asss_status colmajor_gemv(const double* A, int lda, int p, const double* c, int 
 asss_status small_inverse(double* K, int m, int* singular, cudaStream_t s);
 // col-major n x p -> row-major n x kp (zero padded), in double or float
 asss_status to_rowmajor(const double* A, int lda, int p, int n, int kp, double* out, cudaStream_t s);
-asss_status to_rowmajor_f(const double* A, int lda, int p, int n, int kp, float* out, cudaStream_t s);
+// FP32 copy of Q_k for the mrs kernels, allocated here: blocked in slices of 32 rows for the
+// operators that visit the rows in natural order (skew diagonals, factored), else row-major
+asss_status q_to_f32(const double* A, int lda, int p, int n, int kp, bool blocked, DBuf<float>& out, cudaStream_t s);
 
 // vector helpers (device scalars where noted)
 asss_status vscale(double* y, const double* x, double a, int n, cudaStream_t s);                 // y = a x
@@ -63,7 +65,7 @@ struct MrsOperator {
     const DSkewDia<float>* D32 = nullptr;
     int k = 0, kp = 0;           // Lanczos vectors and padded row stride
     const double* Q64 = nullptr; // n x kp row-major
-    const float* Q32 = nullptr;
+    const float* Q32 = nullptr;  // FP32 copy (q_to_f32; blocked with D32 or F, row-major with J32)
     const void* Q16 = nullptr;   // BF16 n x kp16 row-major (FP32 solve only); used instead of Q32 when set
     int kp16 = 0;
     const double* alpha = nullptr;  // device, k-1 values (S_k superdiagonal)
@@ -202,7 +204,7 @@ struct BatchMat {
     const int* scol;
     const float* sval;
     const int* rowmap;    // slot -> row (n for padding), or null for the identity
-    const float* Q32;               // n x kp row-major (or null)
+    const float* Q32;               // n x kp, blocked with ndiag > 0, else row-major (or null)
     const void* Q16;                // BF16 n x kp row-major (or null)
     const double* alpha;            // k-1
     const float* Y32;               // SMW data, n x m row-major

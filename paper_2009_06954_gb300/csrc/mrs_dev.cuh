@@ -31,33 +31,41 @@ __device__ __forceinline__ void load_qrow16(const __nv_bfloat16* __restrict__ Q,
     }
 }
 
+// Whether Q_k is stored in slices of 32 rows (FP32, operators that visit the rows in their
+// natural order: natural = true) or row by row.  In a slice the four values m..m+3 of
+// its 32 rows stand side by side, so a warp's load is 512 contiguous bytes; the same load
+// of 80-byte rows touched 20 lines, five times over (row pass at n = 100^3, k = 20: 26 -> 22 us).
+template <class T>
+__host__ __device__ constexpr bool q_blocked(bool natural) { return sizeof(T) == 4 && natural; }
+// floats of n rows of kp values in that layout
+__host__ __device__ inline int64_t q_blocked_size(int n, int kp) { return ((int64_t)n + 31) / 32 * 32 * kp; }
+
 // cs: Q is streamed once per step and the step's data exceed L2, so its rows are
 // loaded evict-first to keep the reused vectors in L2 (see stream_evict_first)
-template <class T, int KP>
+template <class T, int KP, bool BLK>
 __device__ __forceinline__ void load_qrow(const T* __restrict__ Q, int i, T (&q)[KP > 0 ? KP : 1],
                                           bool cs = false) {
     if constexpr (KP > 0) {
-        const T* row = Q + (size_t)i * KP;
-        if constexpr (sizeof(T) == 4 && (KP % 4) == 0) {
+        if constexpr (sizeof(T) == 4) {
+            // every padded width is a multiple of 4
+            const float4* a = BLK ? reinterpret_cast<const float4*>(Q + (size_t)(i & ~31) * KP) + (i & 31)
+                                  : reinterpret_cast<const float4*>(Q + (size_t)i * KP);
 #pragma unroll
-            for (int m = 0; m < KP; m += 4) {
-                const float4* a = reinterpret_cast<const float4*>(row + m);
+            for (int m = 0; m < KP; m += 4, a += BLK ? 32 : 1) {
                 float4 v = cs ? __ldcs(a) : __ldg(a);
                 q[m] = v.x;
                 q[m + 1] = v.y;
                 q[m + 2] = v.z;
                 q[m + 3] = v.w;
             }
-        } else if constexpr (sizeof(T) == 8 && (KP % 2) == 0) {
+        } else {
+            const T* row = Q + (size_t)i * KP;
 #pragma unroll
             for (int m = 0; m < KP; m += 2) {
                 double2 v = *reinterpret_cast<const double2*>(row + m);
                 q[m] = v.x;
                 q[m + 1] = v.y;
             }
-        } else {
-#pragma unroll
-            for (int m = 0; m < KP; ++m) q[m] = row[m];
         }
     }
 }

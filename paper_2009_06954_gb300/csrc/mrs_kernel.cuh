@@ -185,6 +185,7 @@ __device__ __forceinline__ T row_dot8(const int* __restrict__ ci, const T* __res
 template <class T, int KP, int FMT, bool QB = false>
 __global__ void __launch_bounds__((mrs_threads<T, FMT>()), 1) k_mrs(MrsParams<T> p) {
     constexpr int NV = KP + 1;
+    constexpr bool QBLK = q_blocked<T>(FMT != 0 && FMT != 2);
     constexpr int NT = mrs_threads<T, FMT>(), NW = NT / 32;
     if (p.skip && *p.skip) {  // enqueued ahead of a decision that went the other way
         if (blockIdx.x == 0 && threadIdx.x == 0) {
@@ -396,7 +397,7 @@ __global__ void __launch_bounds__((mrs_threads<T, FMT>()), 1) k_mrs(MrsParams<T>
             tacc[0] += b * b;
             T q[KP > 0 ? KP : 1];
             if constexpr (QB) load_qrow16<T, KP>(p.Q16, i, q);
-            else load_qrow<T, KP>(p.Q, i, q, p.qcs != 0);
+            else load_qrow<T, KP, QBLK>(p.Q, i, q, p.qcs != 0);
 #pragma unroll
             for (int m = 0; m < KP; ++m) tacc[1 + m] += q[m] * b;
         }
@@ -627,7 +628,7 @@ __global__ void __launch_bounds__((mrs_threads<T, FMT>()), 1) k_mrs(MrsParams<T>
                         }
                     }
                 } else {
-                    load_qrow<T, KP>(Qr, i, q, p.qcs != 0);
+                    load_qrow<T, KP, QBLK>(Qr, i, q, p.qcs != 0);
                 }
                 T dq = (T)0;
 #pragma unroll

@@ -185,7 +185,7 @@ __global__ void __launch_bounds__(MRS_THREADS, 1) k_mrs_multi(MultiParams<T> p) 
             if (colok) p.x[c][i] = (T)0;
             tacc[0] += b * b;
             T q[KQ];
-            load_qrow<T, KP>(p.Q, i, q, p.qcs != 0);
+            load_qrow<T, KP, q_blocked<T>(FMT == 1)>(p.Q, i, q, p.qcs != 0);
 #pragma unroll
             for (int m = 0; m < KP; ++m) tacc[1 + m] += q[m] * b;
         }
@@ -274,7 +274,7 @@ __global__ void __launch_bounds__(MRS_THREADS, 1) k_mrs_multi(MultiParams<T> p) 
                     }
                 }
                 T q[KQ];
-                load_qrow<T, KP>(p.Q, i, q, p.qcs != 0);
+                load_qrow<T, KP, q_blocked<T>(FMT == 1)>(p.Q, i, q, p.qcs != 0);
                 T dq = (T)0;
 #pragma unroll
                 for (int m = 0; m < KP; ++m) dq += q[m] * s_u[c][m];
