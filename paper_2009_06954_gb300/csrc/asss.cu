@@ -590,6 +590,8 @@ struct asss_handle {
     DSell<float> J32;
     DSkewDia<double> D64;
     DSkewDia<float> D32;
+    DStream<double> R64;   // long rows: what the single-column solve reads instead of SELL
+    DStream<float> R32;
     bool use_dia = false;
     // incomplete L D L^T (options.factor = ASSS_FACTOR_ILDL0): J~ in factored form, W = 1
     // in the operators above and L~ applied by triangular solves instead
@@ -851,6 +853,8 @@ static asss_status apply_prec(asss_handle* h, int tr, const double* u, double* o
     op.J32 = (!h->use_dia && h->J32.n) ? &h->J32 : nullptr;
     op.D64 = h->use_dia ? &h->D64 : nullptr;
     op.D32 = (h->use_dia && h->D32.n) ? &h->D32 : nullptr;
+    op.R64 = h->R64.n ? &h->R64 : nullptr;
+    op.R32 = h->R32.n ? &h->R32 : nullptr;
     op.F = h->factored ? &h->fac : nullptr;
     op.k = h->k;
     op.kp = h->kp;
@@ -1904,6 +1908,13 @@ static asss_status do_setup(asss_handle* h, const asss_csr* Ain, asss_stats* st)
             ASSS_TRY(tune_sell(h, &sigma, &split));
         ASSS_TRY(build_sell<double>(h->Jt, true, h->J64, s, sigma, split));
         if (o.precision == ASSS_PREC_MIXED) ASSS_TRY(build_sell<float>(h->Jt, true, h->J32, s, sigma, split));
+        // long rows, no layout asked for: the single-column solve of this precision takes the row
+        // stream (the SELL copies stay for the multi-column and batched kernels and the set-up)
+        const bool rows = o.inner_format == ASSS_FORMAT_AUTO && o.sell_sigma == 0 && o.sell_split == 0;
+        if (rows && o.precision == ASSS_PREC_MIXED && stream_fits<float>(n, h->J32.nnz))
+            ASSS_TRY(build_stream<float>(h->Jt, h->R32, s));
+        if (rows && o.precision == ASSS_PREC_FP64 && stream_fits<double>(n, h->J64.nnz))
+            ASSS_TRY(build_stream<double>(h->Jt, h->R64, s));
         st->sell_sigma = h->J64.sigma;
         st->sell_split = h->J64.split;
     }

@@ -139,6 +139,20 @@ struct DSell {
 };
 constexpr int SELL_SPLIT = 1024;
 
+// Row-stream storage for long rows whose vector fits shared memory: the rows one after
+// the other, each padded to a multiple of 4 entries (value 0 on its own column), columns in
+// 16 bits.  The row kernel reads 4 entries a lane and gathers from a copy of the vector
+// in shared memory (see stream_fits).
+template <class T>
+struct DStream {
+    int n = 0;
+    int64_t nnz = 0;
+    int64_t nstored = 0;      // with the padding
+    DBuf<int> rp;             // n + 1 offsets, multiples of 4
+    DBuf<unsigned short> col;
+    DBuf<T> val;
+};
+
 // Skew half-diagonal storage of an exactly skew matrix J whose entries lie on a
 // few diagonals (stencil-like patterns): only the diagonals with positive offset
 // are stored, U[d*n + i] = J[i, i + off[d]] (0 where absent), and the lower

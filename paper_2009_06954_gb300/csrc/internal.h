@@ -19,6 +19,12 @@ asss_status build_pattern(const DCsr& Abar, const DCsr& AbarT, const DCsr& S, co
                           DBuf<int>& mirror, DBuf<int>& diagpos, cudaStream_t s);
 template <class T>
 asss_status build_sell(const DCsr& A, bool skip_diag, DSell<T>& out, cudaStream_t s, int sigma = 0, int split = 0);
+// Row-stream storage of A without its diagonal (see DStream); stream_fits: whether the
+// vector fits shared memory (in T) and the rows are long enough for a warp each
+template <class T>
+bool stream_fits(int n, int64_t nnz);
+template <class T>
+asss_status build_stream(const DCsr& A, DStream<T>& out, cudaStream_t s);
 // Skew half-diagonal storage of J when J is exactly skew, has at most max_diag
 // positive offsets and fills at least min_fill of the stored diagonals; *ok = 0
 // (and nothing allocated) otherwise.
@@ -60,6 +66,9 @@ struct MrsOperator {
     // J~ (exactly skew) in SELL-C, FP64 and/or FP32 copies
     const DSell<double>* J64 = nullptr;
     const DSell<float>* J32 = nullptr;
+    // row-stream copies (used instead of SELL by the single-column solve when present)
+    const DStream<double>* R64 = nullptr;
+    const DStream<float>* R32 = nullptr;
     // skew half-diagonal copies (used instead of SELL when present)
     const DSkewDia<double>* D64 = nullptr;
     const DSkewDia<float>* D32 = nullptr;

@@ -46,7 +46,7 @@ void mrs_work_destroy(MrsWork* w) { delete w; }
 // the layout changes; the kernel never writes the halos)
 template <class T>
 static asss_status y_layout(MrsWork* w, DBuf<T>& Ybuf, int& cur, int H, cudaStream_t s, T** Y, long long* ystride) {
-    long long st = (long long)w->n + 2LL * H;
+    long long st = ((long long)w->n + 2LL * H + 31) / 32 * 32;   // every slot starts on 128 bytes (H = 0)
     if (cur != H || Ybuf.n < 3 * st) {
         if (Ybuf.n < 3 * st) ASSS_TRY(Ybuf.alloc(3 * st));
         ASSS_CUDA(cudaMemsetAsync(Ybuf.p, 0, sizeof(T) * (size_t)Ybuf.n, s));
@@ -62,7 +62,7 @@ static asss_status dispatch_mrs(const Ctx& c, MrsWork* w, const DSell<T>* sell, 
                                 const double* alpha, int k, int kp, double shift, double sign, const double* rhs,
                                 T* x, DBuf<T>& Ybuf, int& ylay, T* P, double tol, int maxit, long long* nnz_read,
                                 LaunchOut lo, const __nv_bfloat16* Q16 = nullptr, int kp16 = 0,
-                                const IldlFactor* fac = nullptr) {
+                                const IldlFactor* fac = nullptr, const DStream<T>* rows = nullptr) {
     OpView<T> v;
     if (dia && dia->ndiag > MRS_MAXDIAG) dia = nullptr;
     T* Y = nullptr;
@@ -99,6 +99,23 @@ static asss_status dispatch_mrs(const Ctx& c, MrsWork* w, const DSell<T>* sell, 
                                              maxit, lo);
         }
         return dispatch_kp<T, 1>(c, w, v, Q, alpha, k, kp, shift, sign, rhs, x, Y, ystride, P, tol, maxit, lo);
+    }
+    if (rows) {
+        v.n = rows->n;
+        v.fmt = 4;
+        v.nslices = cdiv(rows->n, 32);
+        v.rrp = rows->rp.p;
+        v.rcol = rows->col.p;
+        v.rval = rows->val.p;
+        v.rstored = rows->nstored;
+        v.key = rows;
+        v.nnz = rows->nnz;
+        *nnz_read = v.nnz;
+        if constexpr (sizeof(T) == 4) {
+            if (Q16) return dispatch_kp16<4>(c, w, v, Q16, alpha, k, kp16, shift, sign, rhs, x, Y, ystride, P, tol,
+                                             maxit, lo);
+        }
+        return dispatch_kp<T, 4>(c, w, v, Q, alpha, k, kp, shift, sign, rhs, x, Y, ystride, P, tol, maxit, lo);
     }
     if (!sell) {
         set_error("mrs: no operator storage");
@@ -141,22 +158,23 @@ asss_status mrs_solve(const Ctx& c, MrsWork* w, const MrsOperator& op, bool fp32
     }
     long long nnz_read = 0;
     if (fp32) {
-        if ((!op.J32 && !op.D32 && !op.F) || !x32) {
+        if ((!op.J32 && !op.D32 && !op.F && !op.R32) || !x32) {
             set_error("FP32 mrs needs the FP32 operator and an FP32 output");
             return ASSS_ERR_ARG;
         }
         if (!w->P32.p) ASSS_TRY(w->P32.alloc((int64_t)2 * n));
         ASSS_TRY(dispatch_mrs<float>(c, w, op.J32, op.D32, op.Q32, op.alpha, op.k, op.kp, shift, sign, rhs, x32,
                                      w->Y32, w->halo32, w->P32.p, tol, maxit, &nnz_read, lo,
-                                     (const __nv_bfloat16*)op.Q16, op.kp16, op.F));
+                                     (const __nv_bfloat16*)op.Q16, op.kp16, op.F, op.R32));
     } else {
-        if ((!op.J64 && !op.D64 && !op.F) || !x64) {
+        if ((!op.J64 && !op.D64 && !op.F && !op.R64) || !x64) {
             set_error("FP64 mrs needs the FP64 operator and an FP64 output");
             return ASSS_ERR_ARG;
         }
         if (!w->P64.p) ASSS_TRY(w->P64.alloc((int64_t)2 * n));
         ASSS_TRY(dispatch_mrs<double>(c, w, op.J64, op.D64, op.Q64, op.alpha, op.k, op.kp, shift, sign, rhs, x64,
-                                      w->Y64, w->halo64, w->P64.p, tol, maxit, &nnz_read, lo, nullptr, 0, op.F));
+                                      w->Y64, w->halo64, w->P64.p, tol, maxit, &nnz_read, lo, nullptr, 0, op.F,
+                                      op.R64));
     }
     // algorithmic bytes: set-up pass (rhs in FP64, Y/x/P written, Q row), per step
     // (matrix entries - SELL ones with a 4-byte index -, Q row, gathered/own y,
@@ -164,7 +182,9 @@ asss_status mrs_solve(const Ctx& c, MrsWork* w, const MrsOperator& op, bool fp32
     long long T = fp32 ? 4 : 8;
     long long nn = n, kp = op.kp;
     long long qrow = (fp32 && op.Q16) ? 2LL * op.kp16 : kp * T;  // bytes of one Q row as read
-    long long per_entry = (!op.F && (fp32 ? (op.D32 != nullptr) : (op.D64 != nullptr))) ? T : T + 4;
+    const bool dia = !op.F && (fp32 ? op.D32 != nullptr : op.D64 != nullptr);
+    const bool rows = !op.F && !dia && (fp32 ? op.R32 != nullptr : op.R64 != nullptr);
+    const long long per_entry = dia ? T : rows ? T + 2 : T + 4;   // SELL: 32-bit columns; row stream: 16-bit
     if ((int)w->log_nnz.size() <= lo.slot) {
         w->log_nnz.resize(lo.slot + 1);
         w->log_per_row.resize(lo.slot + 1);

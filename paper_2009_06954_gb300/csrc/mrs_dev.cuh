@@ -193,4 +193,24 @@ static __global__ void k_partition(const int* sptr, int nslices, int nblk, int* 
     blk[b] = lo;
 }
 
+// row-stream storage: block b owns rows [blk[b], blk[b+1]), balanced by stored entries plus
+// rowcost a row
+static __global__ void k_partition_rows(const int* rp, int n, int rowcost, int nblk, int* blk) {
+    const int b = blockIdx.x * blockDim.x + threadIdx.x;
+    if (b > nblk) return;
+    if (b == nblk) {
+        blk[b] = n;
+        return;
+    }
+    const long long total = (long long)rp[n] + (long long)n * rowcost;
+    const long long target = total * b / nblk;
+    int lo = 0, hi = n;
+    while (lo < hi) {
+        const int mid = lo + ((hi - lo) >> 1);
+        if ((long long)rp[mid] + (long long)mid * rowcost < target) lo = mid + 1;
+        else hi = mid;
+    }
+    blk[b] = lo;
+}
+
 }  // namespace asss

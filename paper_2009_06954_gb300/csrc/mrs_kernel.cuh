@@ -111,6 +111,11 @@ struct MrsParams {
     T* hacc;             // partial sums of the parts of long slices (32 per long slice, left at 0)
     unsigned* hcnt;      // parts finished per long slice (left at 0)
     int split;           // entries per lane of one work unit
+    // row-stream operator
+    const int* rrp;
+    const unsigned short* rcol;
+    const T* rval;
+    int racc;            // row sums held in shared memory (the most rows a block owns)
     // skew half-diagonal operator: U points at U_0[0]; diagonal d starts ustride later
     int ndiag;
     const int* off;
@@ -180,12 +185,96 @@ __device__ __forceinline__ T row_dot8(const int* __restrict__ ci, const T* __res
     return a;
 }
 
+// the products of one warp of the row-stream pass: entries [e, e1), which start in row r
+// (rp: the block's row offsets, in shared memory).  Sums of rows that start here go to
+// acc[row], the sum of a row that began in an earlier warp to carry / crow.
+template <class T>
+__device__ __forceinline__ void stream_rows(const T* __restrict__ val, const unsigned short* __restrict__ col,
+                                            const T* __restrict__ y, const int* rp, int r, int e, int e1, bool cs,
+                                            T* acc, T& carry, int& crow) {
+    constexpr int U = sizeof(T) == 4 ? 4 : 2;   // groups of 4 entries in flight per lane and batch
+    constexpr int V = sizeof(T) / 4;            // 16-byte loads of the 4 values
+    struct Batch {
+        int4 v[U][V];
+        uint2 c[U];
+    };
+    const int lane = threadIdx.x & 31;
+    if (e >= e1) return;
+    const int first = e;
+    auto load = [&](int from, int end, Batch& B) {
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            const int q = from + u * 128 + lane * 4;
+            if (q < end) {
+                const int4* vp = reinterpret_cast<const int4*>(val + q);
+                const uint2* cp = reinterpret_cast<const uint2*>(col + q);
+#pragma unroll
+                for (int t = 0; t < V; ++t) B.v[u][t] = cs ? __ldcs(vp + t) : __ldg(vp + t);
+                B.c[u] = cs ? __ldcs(cp) : __ldg(cp);
+            }
+        }
+    };
+    int end = min(rp[r + 1], e1);
+    Batch cur, nxt;
+    load(e, end, cur);
+    T sum = (T)0;
+    while (true) {
+        // the batch after this one, possibly in a later row
+        int ne = e + U * 128, nr = r, nend = end;
+        const bool rowdone = ne >= end;
+        if (rowdone) {
+            ne = end;
+            nr = r + 1;
+            if (ne < e1) {
+                while (rp[nr + 1] == ne) ++nr;   // rows without entries
+                nend = min(rp[nr + 1], e1);
+            }
+        }
+        if (ne < e1) load(ne, nend, nxt);
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            if (e + u * 128 + lane * 4 < end) {
+                const unsigned c01 = cur.c[u].x, c23 = cur.c[u].y;
+                const T* v = reinterpret_cast<const T*>(cur.v[u]);
+                sum += v[0] * y[c01 & 0xffffu];
+                sum += v[1] * y[c01 >> 16];
+                sum += v[2] * y[c23 & 0xffffu];
+                sum += v[3] * y[c23 >> 16];
+            }
+        }
+        if (rowdone) {
+            const T t = warp_sum(sum);
+            if (lane == 0) {
+                if (rp[r] >= first) {
+                    acc[r] = t;
+                } else {
+                    carry = t;
+                    crow = r;
+                }
+            }
+            sum = (T)0;
+            if (ne >= e1) break;
+        }
+        cur = nxt;
+        e = ne;
+        r = nr;
+        end = nend;
+    }
+}
+
 // FMT 0: SELL-C storage of J~; FMT 1: skew half-diagonal storage; FMT 2: plain CSR;
 // FMT 3: factored J~ = L~^-1 J^ L~^-T (incomplete L D L^T in a multicolour order)
+// FMT 4: row-stream storage.  Long rows (hundreds of entries, some thousands): with a lane
+// per row (SELL) a system of 2 10^4 rows has fewer work units than the GPU has warps and each
+// is one lane's serial chain of gathers.  Here a block's entries are cut evenly over its 16
+// warps, a warp reads a row 128 entries at a time (512 + 256 contiguous bytes) with the next
+// batch already in flight, and gathers from a copy of y in shared memory; the sums of the
+// rows that a cut splits are added in warp order.  Bound: L2 bandwidth of the stream (6 bytes
+// an entry in FP32) and the bank conflicts of the gathers.
 template <class T, int KP, int FMT, bool QB = false>
 __global__ void __launch_bounds__((mrs_threads<T, FMT>()), 1) k_mrs(MrsParams<T> p) {
     constexpr int NV = KP + 1;
-    constexpr bool QBLK = q_blocked<T>(FMT != 0 && FMT != 2);
+    constexpr bool QBLK = q_blocked<T>(FMT == 1 || FMT == 3);
     constexpr int NT = mrs_threads<T, FMT>(), NW = NT / 32;
     if (p.skip && *p.skip) {  // enqueued ahead of a decision that went the other way
         if (blockIdx.x == 0 && threadIdx.x == 0) {
@@ -244,8 +333,11 @@ __global__ void __launch_bounds__((mrs_threads<T, FMT>()), 1) k_mrs(MrsParams<T>
     };
     const int nblk = gridDim.x;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int s0 = p.blk_slice[blockIdx.x], s1 = p.blk_slice[blockIdx.x + 1];
-    const int n = p.n;
+    // FMT 4: the block's rows [rb, re); its slices are cut from there
+    const int rb = FMT == 4 ? p.blk_slice[blockIdx.x] : 0, re = FMT == 4 ? p.blk_slice[blockIdx.x + 1] : 0;
+    const int s0 = FMT == 4 ? 0 : p.blk_slice[blockIdx.x];
+    const int s1 = FMT == 4 ? (re - rb + 31) >> 5 : p.blk_slice[blockIdx.x + 1];
+    const int n = FMT == 4 ? re : p.n;   // the end of this block's rows
     const size_t ys = p.ystride;
     volatile int* err = p.gb.err;
     // timeline slots: 0 start, 1 phase-0 pass, 2 phase-0 barrier, 3 set-up scalars; then per
@@ -361,6 +453,30 @@ __global__ void __launch_bounds__((mrs_threads<T, FMT>()), 1) k_mrs(MrsParams<T>
     };
     const bool want_qtx = KP > 0 && p.qtz != nullptr;
     unsigned phase = 0;  // grid barriers passed in this launch
+    // row-stream storage: this warp's entries [e0, e1) of the block's, from row wr on, and in
+    // dynamic shared memory y, the block's row sums and row offsets
+    extern __shared__ __align__(16) unsigned char s_dyn[];
+    __shared__ T s_carry[FMT == 4 ? NW : 1];
+    __shared__ int s_crow[FMT == 4 ? NW : 1];
+    T* s_y = reinterpret_cast<T*>(s_dyn);
+    T* s_acc = s_y + ((p.n + 3) & ~3);
+    int* s_rp = reinterpret_cast<int*>(s_acc + p.racc);
+    int e0 = 0, e1 = 0, wr = 0;
+    if constexpr (FMT == 4) {
+        const int nr = re - rb;
+        for (int t = threadIdx.x; t <= nr; t += NT) s_rp[t] = __ldg(&p.rrp[rb + t]);
+        __syncthreads();
+        const int chunk = ((s_rp[nr] - s_rp[0] + NW - 1) / NW + 127) & ~127;
+        e0 = min(s_rp[0] + warp * chunk, s_rp[nr]);
+        e1 = min(e0 + chunk, s_rp[nr]);
+        int lo = 0, hi = nr;   // the last row that starts at or before e0
+        while (lo < hi) {
+            const int mid = lo + ((hi - lo + 1) >> 1);
+            if (s_rp[mid] <= e0) lo = mid;
+            else hi = mid - 1;
+        }
+        wr = lo;
+    }
     // ---- phase 0: y_1 = b, x = 0, p = 0, ||b||^2 and Q^T b ----
     T tacc[NV];
 #pragma unroll
@@ -384,7 +500,7 @@ __global__ void __launch_bounds__((mrs_threads<T, FMT>()), 1) k_mrs(MrsParams<T>
         if constexpr (FMT == 0) {
             if (p.rowmap) return __ldg(&p.rowmap[sl * 32 + lane]);
         }
-        return sl * 32 + lane;
+        return rb + sl * 32 + lane;
     };
     for (int sl = s0 + warp; sl < s1; sl += NW) {
         int i = row_of(sl);
@@ -393,7 +509,7 @@ __global__ void __launch_bounds__((mrs_threads<T, FMT>()), 1) k_mrs(MrsParams<T>
             p.Y[i] = b;
             p.x[i] = (T)0;
             p.P[i] = (T)0;
-            p.P[n + i] = (T)0;
+            p.P[p.n + i] = (T)0;
             tacc[0] += b * b;
             T q[KP > 0 ? KP : 1];
             if constexpr (QB) load_qrow16<T, KP>(p.Q16, i, q);
@@ -462,7 +578,7 @@ __global__ void __launch_bounds__((mrs_threads<T, FMT>()), 1) k_mrs(MrsParams<T>
         const T* __restrict__ Ycur = p.Y + (size_t)((j - 1) % 3) * ys;
         const T* __restrict__ Yold = p.Y + (size_t)((j + 1) % 3) * ys;
         T* __restrict__ Ynew = p.Y + (size_t)(j % 3) * ys;
-        T* __restrict__ Pj1 = p.P + (size_t)((j - 1) & 1) * n;
+        T* __restrict__ Pj1 = p.P + (size_t)((j - 1) & 1) * p.n;
         T* __restrict__ xv = p.x;
         const T* __restrict__ Ub = p.U;
         const T* __restrict__ Qr = p.Q;
@@ -501,6 +617,64 @@ __global__ void __launch_bounds__((mrs_threads<T, FMT>()), 1) k_mrs(MrsParams<T>
         }
 #pragma unroll
         for (int v = 0; v < NV; ++v) tacc[v] = (T)0;
+        // a row once its product with J~ is there: y_{j+1}, its sums, the p/x update of step j-1
+        auto finish = [&](int i, T acc, T yold, T pold, T(&q)[KP > 0 ? KP : 1]) {
+            T dq = (T)0;
+#pragma unroll
+            for (int m = 0; m < KP; ++m) dq += q[m] * s_u[m];
+            T ynew = tnu * acc - tsg * dq + tco * yold;
+            Ynew[i] = ynew;
+            tacc[0] += ynew * ynew;
+#pragma unroll
+            for (int m = 0; m < KP; ++m) tacc[1 + m] += q[m] * ynew;
+            if (j >= 2) {
+                T pv = (tnp * yold - tdpp * pold) * tthp;
+                Pj1[i] = pv;
+                xv[i] += txp * pv;
+            }
+        };
+        if constexpr (FMT == 4) {
+            auto qrow = [&](int i, T(&q)[KP > 0 ? KP : 1]) {
+                if constexpr (QB) load_qrow16<T, KP>(p.Q16, i, q);
+                else load_qrow<T, KP, QBLK>(Qr, i, q, p.qcs != 0);
+            };
+            // the first row's own data, in flight during the products
+            int i = rb + threadIdx.x;
+            T q[KP > 0 ? KP : 1], yold = (T)0, pold = (T)0;
+            if (i < re) {
+                if (j >= 2) {
+                    yold = Yold[i];
+                    pold = Pj1[i];
+                }
+                qrow(i, q);
+            }
+            // y into shared memory (every slot starts on 16 bytes and is padded to 16)
+            constexpr int VW = 16 / sizeof(T);
+            const int4* yv4 = reinterpret_cast<const int4*>(Ycur);
+            int4* sy4 = reinterpret_cast<int4*>(s_y);
+            const int nv4 = (p.n + VW - 1) / VW;
+#pragma unroll 8
+            for (int t = threadIdx.x; t < nv4; t += NT) sy4[t] = yv4[t];
+            for (int t = threadIdx.x; t < re - rb; t += NT) s_acc[t] = (T)0;
+            if (threadIdx.x < NW) s_crow[threadIdx.x] = -1;
+            __syncthreads();
+            stream_rows<T>(p.rval, p.rcol, s_y, s_rp, wr, e0, e1, p.qcs != 0, s_acc, s_carry[warp], s_crow[warp]);
+            __syncthreads();
+            for (; i < re; i += NT) {
+                T acc = s_acc[i - rb];
+#pragma unroll
+                for (int w = 0; w < NW; ++w)
+                    if (s_crow[w] == i - rb) acc += s_carry[w];
+                finish(i, acc, yold, pold, q);
+                if (i + NT < re) {
+                    if (j >= 2) {
+                        yold = Yold[i + NT];
+                        pold = Pj1[i + NT];
+                    }
+                    qrow(i + NT, q);
+                }
+            }
+        } else {
         for (int uu = u0 + warp; uu < u1; uu = next_slice(uu)) {
             int sl = uu, part = 0, nparts = 1, hix = -1;
             if constexpr (FMT == 0) {
@@ -630,20 +804,9 @@ __global__ void __launch_bounds__((mrs_threads<T, FMT>()), 1) k_mrs(MrsParams<T>
                 } else {
                     load_qrow<T, KP, QBLK>(Qr, i, q, p.qcs != 0);
                 }
-                T dq = (T)0;
-#pragma unroll
-                for (int m = 0; m < KP; ++m) dq += q[m] * s_u[m];
-                T ynew = tnu * acc - tsg * dq + tco * yold;
-                Ynew[i] = ynew;
-                tacc[0] += ynew * ynew;
-#pragma unroll
-                for (int m = 0; m < KP; ++m) tacc[1 + m] += q[m] * ynew;
-                if (j >= 2) {
-                    T pv = (tnp * yold - tdpp * pold) * tthp;
-                    Pj1[i] = pv;
-                    xv[i] += txp * pv;
-                }
+                finish(i, acc, yold, pold, q);
             }
+        }
         }
         double* buf = p.part + (size_t)(j & 1) * NV * nblk;
         stamp(tb);
@@ -697,7 +860,7 @@ __global__ void __launch_bounds__((mrs_threads<T, FMT>()), 1) k_mrs(MrsParams<T>
         }
         __syncthreads();
         if (sc.stop) {
-            T* Pj = p.P + (size_t)(j & 1) * n;
+            T* Pj = p.P + (size_t)(j & 1) * p.n;
             const T tn = s_cf[7], td = s_cf[8], tth = s_cf[9], tx = s_cf[10];
 #pragma unroll
             for (int v = 0; v < NV; ++v) tacc[v] = (T)0;
@@ -746,6 +909,10 @@ struct OpView {
     const void* key = nullptr;
     long long nnz = 0;  // matrix entries one application reads
     const IldlFactor* fac = nullptr;  // FMT 3
+    const int* rrp = nullptr;         // FMT 4
+    const unsigned short* rcol = nullptr;
+    const T* rval = nullptr;
+    long long rstored = 0;
 };
 
 struct LaunchOut {
@@ -757,16 +924,31 @@ template <class T, int KP, int FMT, bool QB = false>
 static asss_status launch_mrs(const Ctx& c, MrsWork* w, const OpView<T>& J, const T* Q, const double* alpha,
                               int k, double shift, double sign, const double* rhs, T* x, T* Y, long long ystride,
                               T* P, double tol, int maxit, LaunchOut lo, const __nv_bfloat16* Q16 = nullptr) {
+    // row-stream storage: a row weighs its entries plus what its own data cost, so that a
+    // block owns at most (total weight / blocks) / that cost + 2 rows, whose sums and offsets
+    // stand in shared memory behind y
+    int rowcost = 0, racc = 0, smem = 0;
+    if constexpr (FMT == 4) {
+        rowcost = (int)std::max<long long>(48, J.rstored / J.n / 8);
+        racc = (int)((J.rstored + (long long)rowcost * J.n) / ((long long)rowcost * std::min(c.sms, J.n))) + 4;
+        racc = (racc + 3) & ~3;
+        smem = (int)(sizeof(T) * (((long long)J.n + 3) / 4 * 4 + racc) + sizeof(int) * (racc + 1));
+        ASSS_TRY(raise_dynamic_smem((const void*)k_mrs<T, KP, FMT, QB>, smem));
+    }
     int occ = 0;
-    ASSS_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_mrs<T, KP, FMT, QB>, (mrs_threads<T, FMT>()), 0));
+    ASSS_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_mrs<T, KP, FMT, QB>, (mrs_threads<T, FMT>()),
+                                                            smem));
     if (occ < 1) {
         set_error("mrs kernel cannot be resident");
         return ASSS_ERR_CUDA;
     }
-    const int nblk = mrs_blocks<T, FMT>(c.sms, occ, J.nslices);
+    const int nblk = FMT == 4 ? std::min(c.sms, J.n) : mrs_blocks<T, FMT>(c.sms, occ, J.nslices);
     if (w->part_key != J.key || w->part_nblk != nblk) {
-        k_partition<<<cdiv(nblk + 1, 128), 128, 0, c.stream>>>(FMT == 0 ? J.sptr : nullptr, J.nslices, nblk,
-                                                               w->blk_slice.p);
+        if (FMT == 4)
+            k_partition_rows<<<cdiv(nblk + 1, 128), 128, 0, c.stream>>>(J.rrp, J.n, rowcost, nblk, w->blk_slice.p);
+        else
+            k_partition<<<cdiv(nblk + 1, 128), 128, 0, c.stream>>>(FMT == 0 ? J.sptr : nullptr, J.nslices, nblk,
+                                                                   w->blk_slice.p);
         ASSS_CHECK_LAUNCH();
         w->part_key = J.key;
         w->part_nblk = nblk;
@@ -793,6 +975,10 @@ static asss_status launch_mrs(const Ctx& c, MrsWork* w, const OpView<T>& J, cons
     prm.off = J.off;
     prm.U = J.U;
     prm.ustride = J.ustride;
+    prm.rrp = J.rrp;
+    prm.rcol = J.rcol;
+    prm.rval = J.rval;
+    prm.racc = racc;
     prm.crp = nullptr;
     prm.cci = nullptr;
     prm.cval = nullptr;
@@ -863,7 +1049,7 @@ static asss_status launch_mrs(const Ctx& c, MrsWork* w, const OpView<T>& J, cons
     void* args[] = {&prm};
     ASSS_CUDA(cudaEventRecord(w->evs[2 * lo.slot], c.stream));
     ASSS_CUDA(cudaLaunchCooperativeKernel((const void*)k_mrs<T, KP, FMT, QB>, dim3(nblk), dim3(mrs_threads<T, FMT>()),
-                                          args, 0, c.stream));
+                                          args, smem, c.stream));
     count_launch();
     ASSS_CUDA(cudaEventRecord(w->evs[2 * lo.slot + 1], c.stream));
     return ASSS_OK;
@@ -924,14 +1110,17 @@ asss_status dispatch_kp16(const Ctx& c, MrsWork* w, const OpView<float>& J, cons
 #define ASSS_MRS_DISPATCH16_ARGS                                                                                     \
     const Ctx&, MrsWork*, const OpView<float>&, const __nv_bfloat16*, const double*, int, int, double, double,       \
         const double*, float*, float*, long long, float*, double, int, LaunchOut
-// instantiated in mrs_dia32.cu, mrs_dia64.cu, mrs_sell.cu and mrs_fac.cu, which build in
-// parallel
+// instantiated in mrs_dia32.cu, mrs_dia64.cu, mrs_sell.cu, mrs_stream.cu and mrs_fac.cu, which
+// build in parallel
 extern template asss_status dispatch_kp<float, 0>(ASSS_MRS_DISPATCH_ARGS(float));
 extern template asss_status dispatch_kp<float, 1>(ASSS_MRS_DISPATCH_ARGS(float));
 extern template asss_status dispatch_kp<float, 3>(ASSS_MRS_DISPATCH_ARGS(float));
 extern template asss_status dispatch_kp<double, 0>(ASSS_MRS_DISPATCH_ARGS(double));
 extern template asss_status dispatch_kp<double, 1>(ASSS_MRS_DISPATCH_ARGS(double));
 extern template asss_status dispatch_kp<double, 3>(ASSS_MRS_DISPATCH_ARGS(double));
+extern template asss_status dispatch_kp<float, 4>(ASSS_MRS_DISPATCH_ARGS(float));
+extern template asss_status dispatch_kp<double, 4>(ASSS_MRS_DISPATCH_ARGS(double));
+extern template asss_status dispatch_kp16<4>(ASSS_MRS_DISPATCH16_ARGS);
 extern template asss_status dispatch_kp16<0>(ASSS_MRS_DISPATCH16_ARGS);
 extern template asss_status dispatch_kp16<1>(ASSS_MRS_DISPATCH16_ARGS);
 

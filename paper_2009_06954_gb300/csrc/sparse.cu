@@ -1060,6 +1060,80 @@ asss_status build_sell(const DCsr& A, bool skip_diag, DSell<T>& out, cudaStream_
 template asss_status build_sell<double>(const DCsr&, bool, DSell<double>&, cudaStream_t, int, int);
 template asss_status build_sell<float>(const DCsr&, bool, DSell<float>&, cudaStream_t, int, int);
 
+// ---------------------------------------------------------------------------
+// row-stream storage (DStream) of A without its diagonal
+// ---------------------------------------------------------------------------
+// The vector stays below 192 KB, which leaves the block its partial sums and row sums, and
+// its indices below 16 bits.  From 64 entries a row on, half of a warp's lanes or more
+// have an entry in the row's first load; below that SELL's lane per row wastes less.
+template <class T>
+bool stream_fits(int n, int64_t nnz) {
+    return (int64_t)n * (int64_t)sizeof(T) <= 192000 && nnz >= (int64_t)64 * n;
+}
+template bool stream_fits<double>(int, int64_t);
+template bool stream_fits<float>(int, int64_t);
+
+__global__ void k_stream_len(int n, const int* len, int* padded) {
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i < n) padded[i] = (len[i] + 3) & ~3;
+}
+
+// one warp per row; the entries behind the diagonal move up by one place
+template <class T>
+__global__ void k_stream_fill(int n, const int* rp, const int* ci, const double* v, const int* len, const int* orp,
+                              unsigned short* oc, T* ov) {
+    const int i = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
+    if (i >= n) return;
+    const int b = rp[i], l = rp[i + 1] - b, o = orp[i];
+    const int shift = l - len[i];   // 1 when the diagonal is stored
+    for (int e = lane; e < l; e += 32) {
+        const int c = ci[b + e];
+        if (c == i) continue;
+        const int q = o + e - (c > i ? shift : 0);
+        oc[q] = (unsigned short)c;
+        ov[q] = (T)v[b + e];
+    }
+    for (int q = o + len[i] + lane; q < orp[i + 1]; q += 32) {
+        oc[q] = (unsigned short)i;
+        ov[q] = (T)0;
+    }
+}
+
+template <class T>
+asss_status build_stream(const DCsr& A, DStream<T>& out, cudaStream_t s) {
+    const int n = A.n;
+    DBuf<int> len, padded;
+    ASSS_TRY(len.alloc(n));
+    ASSS_TRY(padded.alloc(n));
+    k_sell_rowlen<<<cdiv(n, 256), 256, 0, s>>>(n, A.rp.p, A.ci.p, 1, len.p);
+    ASSS_CHECK_LAUNCH();
+    k_stream_len<<<cdiv(n, 256), 256, 0, s>>>(n, len.p, padded.p);
+    ASSS_CHECK_LAUNCH();
+    ASSS_TRY(out.rp.alloc(n + 1));
+    // every offset is below n^2 <= 48000^2 < 2^32; one that reaches 2^31 is refused here
+    long long tot = 0;
+    DBuf<long long> off64;
+    ASSS_TRY(off64.alloc(n + 1));
+    ASSS_TRY(exclusive_scan64(padded.p, off64.p, n, &tot, s));
+    if (tot >= (1LL << 31) - 1024) {
+        set_error("row-stream storage of %lld entries exceeds 32-bit offsets", tot);
+        return ASSS_ERR_UNSUPPORTED;
+    }
+    ASSS_TRY(exclusive_scan(padded.p, out.rp.p, n, nullptr, s));
+    ASSS_TRY(out.col.alloc(tot > 0 ? tot : 1));
+    ASSS_TRY(out.val.alloc(tot > 0 ? tot : 1));
+    k_stream_fill<T><<<cdiv((int64_t)n * 32, 256), 256, 0, s>>>(n, A.rp.p, A.ci.p, A.v.p, len.p, out.rp.p, out.col.p,
+                                                                out.val.p);
+    ASSS_CHECK_LAUNCH();
+    out.n = n;
+    out.nnz = A.nnz;
+    out.nstored = tot;
+    ASSS_CUDA(cudaStreamSynchronize(s));   // len and padded are freed here
+    return ASSS_OK;
+}
+template asss_status build_stream<double>(const DCsr&, DStream<double>&, cudaStream_t);
+template asss_status build_stream<float>(const DCsr&, DStream<float>&, cudaStream_t);
+
 }  // namespace asss
 
 namespace asss {

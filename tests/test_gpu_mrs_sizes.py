@@ -29,3 +29,39 @@ def test_mrs_iterate_at_split_edges(pkg, n, k, precision, fmt):  # noqa: F811
     rtol = 1e-12 if precision == "fp64" else 2e-5
     assert abs(ratio - ratio_o) <= rtol * max(ratio_o, 1.0)
     np.testing.assert_allclose(x, xo, rtol=0, atol=rtol * np.abs(xo).max())
+
+
+@pytest.mark.parametrize("precision", ["fp64", "mixed"])
+@pytest.mark.parametrize("n,q_bf16", [(150, False), (1001, False), (5003, False), (5003, True)])
+def test_long_rows_match_sell(pkg, n, q_bf16, precision, monkeypatch):  # noqa: F811
+    """J~ with long rows (one of them full, one empty but for its diagonal) through the
+    row-stream pass against the SELL pass of the same set-up: the same products in another
+    order.  Fewer rows than SMs, a row longer than a warp's share, evict-first loads."""
+    from workloads import random_powerlaw
+    if q_bf16 and precision == "fp64":
+        pytest.skip("BF16 Q belongs to the FP32 solve")
+    A = random_powerlaw(n=n, lmin=4, lmean=16.0, lmax=min(512, n // 2), band=n // 4, dom_frac=1.0, seed=n)[0].tolil()
+    A[7, :] = 0.01
+    A[7, 7] = 0.02 * n
+    A[n - 3, :] = 0.0
+    A[:, n - 3] = 0.0
+    A[n - 3, n - 3] = 1.0
+    A = A.tocsr()
+    if q_bf16:
+        monkeypatch.setenv("ASSS_FORCE_EVICT_FIRST", "1")
+    rng = np.random.default_rng(n)
+    u = rng.standard_normal(n)
+    opts = dict(precision=precision, outer="fgmres", inner_tol=1e-11 if precision == "fp64" else 1e-5, setup_tol=1e-11,
+                lls_maxit=40, q_bf16=q_bf16)
+    s = pkg.Solver(A, **opts)
+    assert s.setup_stats["nnz_pattern"] >= 65 * n
+    z, its = s.apply_preconditioner(u)
+    zt, _ = s.apply_preconditioner(u, transpose=True)
+    s2 = pkg.Solver(A, inner_format="sell", **opts)
+    z2, its2 = s2.apply_preconditioner(u)
+    z2t, _ = s2.apply_preconditioner(u, transpose=True)
+    # both stop at the same tolerance, so they may differ by it
+    tol = 1e-9 if precision == "fp64" else 1e-4
+    assert abs(its - its2) <= 1
+    np.testing.assert_allclose(z, z2, rtol=0, atol=tol * np.abs(z2).max())
+    np.testing.assert_allclose(zt, z2t, rtol=0, atol=tol * np.abs(z2t).max())
