@@ -82,7 +82,6 @@ __global__ void __launch_bounds__(AO_THREADS, 1) k_arnoldi_orth(AoParams p) {
     const int nv = p.nv;
     const double* __restrict__ V = p.V;  // v_0..v_j (read) and v_{j+1} (written) do not overlap w
     double* __restrict__ w = p.w;
-    volatile int* err = p.gb.err;
     // a block may still be adding the previous pass's partials while a faster one
     // writes the next pass's, so consecutive passes use the two halves of p.part
     double* part = p.part;
@@ -166,8 +165,7 @@ __global__ void __launch_bounds__(AO_THREADS, 1) k_arnoldi_orth(AoParams p) {
 
     // ---- pass 1: h1 = V^T w ----
     dots();
-    grid_sync_phase(p.gb, nblk, p.phase0 + 0, p.budget);
-    if (*err) return;
+    if (!grid_sync_phase(p.gb, nblk, p.phase0 + 0, p.budget)) return;
     reduce(nv, s_h1);
     if (blockIdx.x == 0)
         for (int a = threadIdx.x; a < nv; a += AO_THREADS) p.hv[a] = s_h1[a];
@@ -219,8 +217,7 @@ __global__ void __launch_bounds__(AO_THREADS, 1) k_arnoldi_orth(AoParams p) {
         put_partials_n(accn, 0);
         dots();
     }
-    grid_sync_phase(p.gb, nblk, p.phase0 + 1, p.budget);
-    if (*err) return;
+    if (!grid_sync_phase(p.gb, nblk, p.phase0 + 1, p.budget)) return;
     reduce(nv, s_h2);
     {
         // ||w1||^2 from its slot
@@ -325,7 +322,6 @@ asss_status arnoldi_orth(const Ctx& c, ArnoldiWork& aw, const double* V, double*
     p.thr = thr;
     p.stop = stop;
     p.gb.count = aw.bar.p;
-    p.gb.gen = aw.bar.p + 1;
     p.gb.err = aw.err.p;
     p.phase0 = aw.phase;
     p.budget = c.wait_cycles;

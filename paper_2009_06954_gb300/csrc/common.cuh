@@ -187,68 +187,94 @@ __device__ __forceinline__ int warp_sum(int v) {
     return v;
 }
 
+// Sums of NV per-lane values over the warp into out[0..NV) (each written by one lane).
+// Every exchange halves the values that a lane still carries, so NV = 21 costs 23 adds where
+// one shuffle tree per value costs 105; on the FP64 pipe (16 cycles a warp instruction)
+// those adds are what a block's partial sums cost.  v is overwritten.
+template <int NV, class T>
+__device__ __forceinline__ void warp_fold_to(T (&v)[NV], T* out) {
+    const int lane = threadIdx.x & 31;
+    if constexpr (NV <= 32) {
+        int idx = 0, have = NV;   // the values idx .. idx + have - 1 are this lane's
+        int cnt = NV;
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+            const bool up = (lane & o) != 0;
+            if (cnt > 1) {
+                const int h = (cnt + 1) / 2;   // the upper lanes go on with values h..cnt-1
+#pragma unroll
+                for (int i = 0; i < (NV + 1) / 2; ++i) {
+                    if (i < h) {
+                        const T lo = v[i], hi = h + i < cnt ? v[h + i < NV ? h + i : 0] : (T)0;
+                        const T keep = up ? hi : lo, send = up ? lo : hi;
+                        v[i] = keep + __shfl_xor_sync(0xffffffffu, send, o);
+                    }
+                }
+                idx += up ? h : 0;
+                have = up ? have - h : min(have, h);
+                cnt = h;
+            } else {
+                v[0] += __shfl_xor_sync(0xffffffffu, v[0], o);
+                if (up) have = 0;   // the lower lane writes it
+            }
+        }
+        if (have > 0) out[idx] = v[0];
+    } else {
+        T head[32], tail[NV - 32];
+#pragma unroll
+        for (int i = 0; i < 32; ++i) head[i] = v[i];
+#pragma unroll
+        for (int i = 0; i < NV - 32; ++i) tail[i] = v[32 + i];
+        warp_fold_to<32>(head, out);
+        warp_fold_to<NV - 32>(tail, out + 32);
+    }
+}
+
+// Grid-wide barrier for a cooperative (co-resident) launch, on a counter that only grows
+// during a launch: barrier number `phase` (0-based) is complete once the counter reaches
+// (phase + 1) * nblocks.  One atomic per block between acquire-release fences (the
+// sequentially consistent ones of __threadfence cost 0.2-0.4 us a step more at n = 10^3 ..
+// 47^3, where a step takes 4.5-7.2 us); the last block to arrive does not wait.  The wait is
+// bounded: after `budget` clock cycles the block records ASSS_ERR_TIMEOUT in *err, and a
+// block that waits gives up too when another one has.  Returns false (to the whole block)
+// when it gave up, so that no thread has to read *err.
+struct GridBarrier {
+    unsigned* count;  // arrivals
+    int* err;         // device status word
+};
+
 __device__ __forceinline__ unsigned ld_acquire(const unsigned* p) {
     unsigned v;
     asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
     return v;
 }
-
-// Grid-wide barrier for a cooperative (co-resident) launch.  Every block calls
-// it the same number of times.  The wait is bounded: after `budget` clock cycles
-// the block records ASSS_ERR_TIMEOUT in *err and returns.
-struct GridBarrier {
-    unsigned* count;  // arrivals in the current phase
-    unsigned* gen;    // phase counter
-    int* err;         // device status word
-};
-
-__device__ __forceinline__ void grid_sync(const GridBarrier& gb, unsigned nblocks, long long budget) {
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        unsigned g = ld_acquire(gb.gen);
-        __threadfence();
-        unsigned ticket = atomicAdd(gb.count, 1u);
-        if (ticket == nblocks - 1) {
-            atomicExch(gb.count, 0u);
-            __threadfence();
-            atomicAdd(gb.gen, 1u);
-        } else {
-            long long t0 = clock64();
-            while (ld_acquire(gb.gen) == g) {
-                if (clock64() - t0 > budget) {
-                    atomicExch(gb.err, (int)ASSS_ERR_TIMEOUT);
-                    break;
-                }
-            }
-        }
-        __threadfence();
-    }
-    __syncthreads();
-}
-
-// Grid barrier on a counter that only grows during a launch (set to 0 before it):
-// barrier number `phase` (0-based) is complete once the counter reaches
-// (phase + 1) * nblocks.  One atomic per block and no reset on the critical path;
-// the last block to arrive does not wait.  Waits are bounded like grid_sync.
-__device__ __forceinline__ void grid_sync_phase(const GridBarrier& gb, unsigned nblocks, unsigned phase,
+__device__ __forceinline__ bool grid_sync_phase(const GridBarrier& gb, unsigned nblocks, unsigned phase,
                                                 long long budget) {
     __syncthreads();
+    int gave_up = 0;
     if (threadIdx.x == 0) {
         const unsigned target = (phase + 1u) * nblocks;
-        __threadfence();
-        const unsigned arrived = atomicAdd(gb.count, 1u) + 1u;
-        if (arrived != target) {
-            long long t0 = clock64();
+        unsigned got, polls = 0;
+        asm volatile("fence.acq_rel.gpu;" ::: "memory");
+        asm volatile("atom.add.relaxed.gpu.global.u32 %0, [%1], 1;" : "=r"(got) : "l"(gb.count) : "memory");
+        if (got + 1u != target) {
+            const long long t0 = clock64();
             while ((int)(ld_acquire(gb.count) - target) < 0) {
                 if (clock64() - t0 > budget) {
                     atomicExch(gb.err, (int)ASSS_ERR_TIMEOUT);
+                    gave_up = 1;
+                    break;
+                }
+                if ((++polls & 63u) == 0 && *(volatile int*)gb.err) {
+                    gave_up = 1;
                     break;
                 }
             }
+        } else {
+            asm volatile("fence.acq_rel.gpu;" ::: "memory");
         }
-        __threadfence();
     }
-    __syncthreads();
+    return __syncthreads_or(gave_up) == 0;
 }
 
 // ---------------------------------------------------------------------------

@@ -484,7 +484,6 @@ extern "C" asss_status asss_mrs_noalloc(int64_t n, int64_t nnz, const int64_t* r
     prm.P = P;
     prm.part = part;
     prm.gb.count = ctrl;
-    prm.gb.gen = ctrl + 1;
     prm.gb.err = reinterpret_cast<int*>(ctrl + 2);
     prm.blk_slice = blk;
     prm.tol = tol;

@@ -89,57 +89,6 @@ __device__ __forceinline__ float2 df_add(float2 a, float2 b) {
     return make_float2(hi, lo);
 }
 
-// Sums of CNT (<= 32) per-lane values over the warp: lane l < CNT returns the total of
-// v[l].  Each exchange halves the values a lane still carries, so CNT = 21 costs 31 adds
-// where one shuffle tree per value costs 105; on the FP64 pipe (16 cycles a warp
-// instruction) those adds are what a block's partial sums cost.  v is overwritten.
-template <int CNT, class T>
-__device__ __forceinline__ T warp_fold(T (&v)[CNT]) {
-    static_assert(CNT >= 1 && CNT <= 32, "one value a lane");
-    const int lane = threadIdx.x & 31;
-    int cnt = CNT;
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        if (cnt > o) {
-            const bool up = (lane & o) != 0;   // these lanes go on with values o..cnt-1
-#pragma unroll
-            for (int i = 0; i < o; ++i) {
-                if (i + o < cnt) {
-                    const T keep = up ? v[i + o < CNT ? i + o : 0] : v[i];
-                    const T send = up ? v[i] : v[i + o < CNT ? i + o : 0];
-                    v[i] = keep + __shfl_xor_sync(0xffffffffu, send, o);
-                } else if (i < cnt) {
-                    v[i] += __shfl_xor_sync(0xffffffffu, v[i], o);
-                }
-            }
-            cnt = o;
-        } else {
-#pragma unroll
-            for (int i = 0; i < CNT; ++i)
-                if (i < cnt) v[i] += __shfl_xor_sync(0xffffffffu, v[i], o);
-        }
-    }
-    return v[0];
-}
-
-// the same for any count: out[0..NV) receives the totals (lane l writes l, l + 32, ...)
-template <int NV, class T>
-__device__ __forceinline__ void warp_fold_to(T (&v)[NV], T* out) {
-    const int lane = threadIdx.x & 31;
-    if constexpr (NV <= 32) {
-        const T r = warp_fold<NV>(v);
-        if (lane < NV) out[lane] = r;
-    } else {
-        T head[32], tail[NV - 32];
-#pragma unroll
-        for (int i = 0; i < 32; ++i) head[i] = v[i];
-#pragma unroll
-        for (int i = 0; i < NV - 32; ++i) tail[i] = v[32 + i];
-        out[lane] = warp_fold<32>(head);
-        warp_fold_to<NV - 32>(tail, out + 32);
-    }
-}
-
 // sum of N values by a balanced tree in a fixed order (log2 N dependent additions)
 template <class P, int N, class Add>
 __device__ __forceinline__ P pair_tree(P (&a)[N], Add add) {

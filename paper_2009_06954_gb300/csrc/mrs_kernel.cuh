@@ -339,7 +339,6 @@ __global__ void __launch_bounds__((mrs_threads<T, FMT>()), 1) k_mrs(MrsParams<T>
     const int s1 = FMT == 4 ? (re - rb + 31) >> 5 : p.blk_slice[blockIdx.x + 1];
     const int n = FMT == 4 ? re : p.n;   // the end of this block's rows
     const size_t ys = p.ystride;
-    volatile int* err = p.gb.err;
     // timeline slots: 0 start, 1 phase-0 pass, 2 phase-0 barrier, 3 set-up scalars; then per
     // step j (1-based, first MRS_TRACE_STEPS): 4+5(j-1)+{0 pass, 1 partials, 2 barrier, 3 reduce, 4 scalars+u}
     const bool tr = p.trace && blockIdx.x == 0 && threadIdx.x == 0;
@@ -520,9 +519,9 @@ __global__ void __launch_bounds__((mrs_threads<T, FMT>()), 1) k_mrs(MrsParams<T>
     }
     stamp(1);
     block_partials(tacc, p.part);
-    grid_sync_phase(p.gb, nblk, phase++, p.budget);
+    const bool met = grid_sync_phase(p.gb, nblk, phase++, p.budget);
     stamp(2);
-    if (*err) return;
+    if (!met) return;
     reduce_all(p.part);
 
     if (warp == 0) {
@@ -601,8 +600,7 @@ __global__ void __launch_bounds__((mrs_threads<T, FMT>()), 1) k_mrs(MrsParams<T>
                     }
                     p.ft[i] = a - row_dot8<T>(p.fuci, p.fuv, p.ft, __ldg(&p.furp[i]), __ldg(&p.furp[i + 1]));
                 }
-                grid_sync_phase(p.gb, nblk, phase++, p.budget);
-                if (*err) ok = false;
+                ok = grid_sync_phase(p.gb, nblk, phase++, p.budget);
             }
             for (int cc = 0; cc < p.ncol && ok; ++cc) {
                 for (int e = s_ls[cc] + gt; e < s_ls[cc + 1]; e += gs) {
@@ -610,8 +608,7 @@ __global__ void __launch_bounds__((mrs_threads<T, FMT>()), 1) k_mrs(MrsParams<T>
                     const T a = row_dot8<T>(p.fjci, p.fjv, p.ft, __ldg(&p.fjrp[i]), __ldg(&p.fjrp[i + 1]));
                     p.fw[i] = a - row_dot8<T>(p.flci, p.flv, p.fw, __ldg(&p.flrp[i]), __ldg(&p.flrp[i + 1]));
                 }
-                grid_sync_phase(p.gb, nblk, phase++, p.budget);
-                if (*err) ok = false;
+                ok = grid_sync_phase(p.gb, nblk, phase++, p.budget);
             }
             if (!ok) break;
         }
@@ -812,9 +809,9 @@ __global__ void __launch_bounds__((mrs_threads<T, FMT>()), 1) k_mrs(MrsParams<T>
         stamp(tb);
         block_partials(tacc, buf);
         stamp(tb + 1);
-        grid_sync_phase(p.gb, nblk, phase++, p.budget);
+        const bool met = grid_sync_phase(p.gb, nblk, phase++, p.budget);
         stamp(tb + 2);
-        if (*err) break;
+        if (!met) break;
         reduce_all(buf);
         stamp(tb + 3);
 
@@ -1031,7 +1028,6 @@ static asss_status launch_mrs(const Ctx& c, MrsWork* w, const OpView<T>& J, cons
     prm.P = P;
     prm.part = w->part.p;
     prm.gb.count = w->bar.p;
-    prm.gb.gen = w->bar.p + 1;
     prm.gb.err = w->err.p;
     prm.blk_slice = w->blk_slice.p;
     prm.tol = tol;

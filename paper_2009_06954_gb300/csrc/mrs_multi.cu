@@ -86,7 +86,6 @@ __global__ void __launch_bounds__(MRS_THREADS, 1) k_mrs_multi(MultiParams<T> p) 
     const int n = p.n;
     const int r0 = p.blk_slice[blockIdx.x] * 32;
     const int r1 = min(p.blk_slice[blockIdx.x + 1] * 32, n);
-    volatile int* err = p.gb.err;
     if constexpr (FMT == 1) {
         for (int d = threadIdx.x; d < p.ndiag; d += MRS_THREADS) s_off[d] = p.off[d];
     }
@@ -192,8 +191,7 @@ __global__ void __launch_bounds__(MRS_THREADS, 1) k_mrs_multi(MultiParams<T> p) 
     }
     if (threadIdx.x < MM_R) s_live[threadIdx.x] = 1;   // reduce_all reads every column once
     block_partials(tacc, p.part);
-    grid_sync_phase(p.gb, nblk, phase++, p.budget);
-    if (*err) return;
+    if (!grid_sync_phase(p.gb, nblk, phase++, p.budget)) return;
     reduce_all(p.part);
     if (warp == 0) {
         if (lane < MM_R) {
@@ -293,8 +291,7 @@ __global__ void __launch_bounds__(MRS_THREADS, 1) k_mrs_multi(MultiParams<T> p) 
         if (finalpass) break;
         double* buf = p.part + (size_t)(j & 1) * MM_R * NV * nblk;
         block_partials(tacc, buf);
-        grid_sync_phase(p.gb, nblk, phase++, p.budget);
-        if (*err) break;
+        if (!grid_sync_phase(p.gb, nblk, phase++, p.budget)) break;
         reduce_all(buf);
         if (warp == 0) {
             if (lane < MM_R) {
@@ -458,7 +455,6 @@ static asss_status multi_typed(const Ctx& c, const DSell<T>* sell, const DSkewDi
     prm.Y = Y.p + (size_t)H * MM_R;
     prm.P = P.p;
     prm.gb.count = bar.p;
-    prm.gb.gen = bar.p + 1;
     prm.gb.err = errw.p;
     prm.tol = tol;
     prm.maxit = maxit;
