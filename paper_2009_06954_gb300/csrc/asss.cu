@@ -18,6 +18,7 @@
 
 #include "common.cuh"
 #include "internal.h"
+#include "solve_cluster.cuh"
 
 using namespace asss;
 
@@ -637,6 +638,11 @@ struct asss_handle {
     std::unique_ptr<KrylovWork> kwb[BLK];
     DBuf<double> blk_r, blk_rh, blk_dy, blk_z64, blk_G, blk_T, blk_b, blk_x;
     DBuf<float> blk_z32;
+    // cluster-scope solves: resident clusters of each size (-1: not asked yet), the workspace of
+    // the clusters, staging of the columns and statistics
+    int cl_counts[CL_NSIZES] = {-1, -1, -1, -1};
+    DBuf<double> cl_work, cl_b, cl_x;
+    DBuf<ClStat> cl_st;
     ~asss_handle() {
         if (mw) mrs_work_destroy(mw);
     }
@@ -1980,6 +1986,198 @@ static asss_status do_setup(asss_handle* h, const asss_csr* Ain, asss_stats* st)
     return ASSS_OK;
 }
 
+// ---------------------------------------------------------------------------
+// cluster-scope solves (solve_cluster.cuh)
+// ---------------------------------------------------------------------------
+// Cluster size for nrhs columns (0: the launch-by-launch path, also where no cluster fits).
+// One cluster has its SMs' share of the bandwidth and the FP64 pipe, the launch-by-launch path
+// the whole GPU but 30 to 100 launches and two to three microseconds a grid-wide step, and
+// several clusters run side by side.  Both grow linearly with n; in microseconds for 4 outer
+// and 20 inner steps, measured at n = 8^3 .. 64^3 (dissipative Hamiltonian, k = 20; both scale
+// with the steps alike):
+//   FP32 inner: cluster 100 + 0.0082 n x 16 / size a wave of columns, launches 470 + 0.0012 n a column
+//   FP64 inner: cluster 200 + 0.034 n x 16 / size,                  launches 560 + 0.0033 n
+// (10^3: 144 against 394; 32^3: 392 against 508; 40^3: 598 against 522; FP64 20^3: 502 against
+// 614, 24^3: 665 against 618; eight columns at 16^3: 199 against 3193 in lockstep blocks, at 48^3
+// 1266 against 4963).
+static int cluster_size(const asss_handle* h, int nrhs) {
+    const bool fp32 = h->opt.precision == ASSS_PREC_MIXED;
+    const double n = h->n;
+    double best = nrhs * (fp32 ? 470.0 + 0.0012 * n : 560.0 + 0.0033 * n) * 0.95;
+    int size = 0;
+    for (int t = 0; t < CL_NSIZES; ++t) {
+        if (h->cl_counts[t] < 1) continue;
+        const int waves = cdiv(nrhs, h->cl_counts[t]);
+        const double us = waves * (fp32 ? 100.0 + 0.0082 * n * 16 / CL_SIZES[t] : 200.0 + 0.034 * n * 16 / CL_SIZES[t]);
+        if (us < best) {
+            best = us;
+            size = CL_SIZES[t];
+        }
+    }
+    return size;
+}
+
+// the cluster size of a call (0: launch by launch); CL_MOST: above it the vectors of the
+// columns side by side leave L2 (not measured)
+static asss_status cluster_plan(asss_handle* h, int nrhs, int* size) {
+    constexpr int CL_MOST = 300000;
+    const asss_options& o = h->opt;
+    *size = 0;
+    if (nrhs < 1 || h->n > CL_MOST || o.outer != ASSS_OUTER_FGMRES || o.restart > CL_RESTART || !h->use_dia ||
+        h->factored || h->Q16.p || h->kp > 32 || h->k + h->r > CL_MMAX ||
+        getenv("ASSS_TRACE"))   // which asks for the phases of the launch-by-launch path
+        return ASSS_OK;
+    if (h->cl_counts[0] < 0) {
+        if (o.precision == ASSS_PREC_MIXED) {
+            ClArgs<float> a = {};
+            a.restart = o.restart;
+            ASSS_TRY(cl_dispatch<float>(h->ctx, a, h->kp, 0, 0, h->cl_counts));
+        } else {
+            ClArgs<double> a = {};
+            a.restart = o.restart;
+            ASSS_TRY(cl_dispatch<double>(h->ctx, a, h->kp, 0, 0, h->cl_counts));
+        }
+    }
+    *size = cluster_size(h, nrhs);
+    return ASSS_OK;
+}
+
+static ClMat cl_mat(const DCsr& A) {
+    ClMat m;
+    m.ndiag = A.dia.ndiag;
+    m.off = A.dia.off.p;
+    m.val = A.dia.val.p;
+    m.rp = A.rp.p;
+    m.ci = A.ci.p;
+    m.v = A.v.p;
+    return m;
+}
+
+// nc columns of a solve by clusters of `size` CTAs, x on the device; out: one entry per column
+template <class T>
+static asss_status solve_cluster(asss_handle* h, int tr, int size, int nc, const double* b, int64_t ldb, double* x, int64_t ldx,
+                                 ClStat* out) {
+    NvtxRange nv_(tr ? "asss:adjoint-solve" : "asss:solve");
+    const Ctx& c = h->ctx;
+    cudaStream_t s = c.stream;
+    const asss_options& o = h->opt;
+    ASSS_TRY(ensure_smw(h, tr));
+    if (tr) ASSS_TRY(ensure_adjoint_ops(h));
+    const SmwData& S = h->smw[tr];
+    ClArgs<T> a;
+    memset(&a, 0, sizeof(a));
+    a.n = h->n;
+    a.restart = o.restart;
+    a.k = h->k;
+    a.m = S.m;
+    a.r = h->r;
+    if constexpr (sizeof(T) == 4) {
+        a.ndiag = h->D32.ndiag;
+        a.halo = h->D32.halo;
+        a.off = h->D32.off.p;
+        a.U = h->D32.U.p + h->D32.halo;
+        a.ustride = h->D32.ustride;
+        a.Q = h->Q32.p;
+        a.Ys = S.Y32.p;
+    } else {
+        a.ndiag = h->D64.ndiag;
+        a.halo = h->D64.halo;
+        a.off = h->D64.off.p;
+        a.U = h->D64.U.p + h->D64.halo;
+        a.ustride = h->D64.ustride;
+        a.Q = h->Q64.p;
+        a.Ys = S.Y.p;
+    }
+    a.alpha = h->alpha_d.p;
+    const UrCols U = ur_cols(h);
+    a.neg = U.neg;
+    a.neg2 = U.neg2;
+    a.negc1 = U.c1;
+    a.negc2 = U.c2;
+    a.op1 = cl_mat(tr ? h->AwT : h->Sw);
+    a.op2 = cl_mat(tr ? h->SwT : h->Aw);
+    a.Sm = cl_mat(tr ? h->ST : h->S);
+    a.Am = cl_mat(tr ? h->AT : h->A);
+    a.dr = h->dr.p;
+    a.dc = h->dc.p;
+    a.w = h->w.p;
+    a.perm = h->has_perm ? h->perm.p : nullptr;
+    a.tr = tr;
+    a.sign = tr ? -1.0 : 1.0;
+    a.outer_tol = o.outer_tol;
+    a.inner_tol = o.inner_tol;
+    a.outer_maxit = o.outer_maxit;
+    a.inner_maxit = o.inner_maxit;
+    int count = 0;
+    for (int t = 0; t < CL_NSIZES; ++t)
+        if (CL_SIZES[t] == size) count = nc < h->cl_counts[t] ? nc : h->cl_counts[t];
+    a.ncol = nc;
+    a.b = b;
+    a.ldb = ldb;
+    a.x = x;
+    a.ldx = ldx;
+    a.work_stride = cl_work_doubles(h->n, a.halo, o.restart, (int)sizeof(T));
+    if (h->cl_work.n < a.work_stride * count) ASSS_TRY(h->cl_work.alloc(a.work_stride * count));
+    if (h->cl_st.n < nc) ASSS_TRY(h->cl_st.alloc(nc));
+    a.work = h->cl_work.p;
+    a.stats = h->cl_st.p;
+    ASSS_TRY(cl_dispatch<T>(c, a, h->kp, size, count, nullptr));
+    ASSS_CUDA(cudaMemcpyAsync(out, h->cl_st.p, sizeof(ClStat) * nc, cudaMemcpyDeviceToHost, s));
+    return ASSS_OK;
+}
+
+// statistics of one column, as refine fills them
+static void cluster_stats(const asss_handle* h, int tr, const ClStat& c, asss_stats* st) {
+    const bool fp32 = h->opt.precision == ASSS_PREC_MIXED;
+    const long long T = fp32 ? 4 : 8, n = h->n, qrow = h->kp * T, nnz = fp32 ? h->D32.nnz : h->D64.nnz;
+    const DCsr& a = tr ? h->AwT : h->Aw;
+    const DCsr& b = tr ? h->SwT : h->Sw;
+    st->status = c.status;
+    st->outer_its = c.outer_its;
+    st->cycles = c.cycles;
+    st->relres = c.relres;
+    st->inner_its_total = c.inner_its;
+    st->inner_solves = st->inner_launches = c.solves;
+    st->inner_its_avg = c.solves ? (double)c.inner_its / c.solves : 0.0;
+    st->t_inner_ms = 1e-6 * (double)c.ns_inner;
+    st->inner_bytes = c.solves * n * (8 + 8 * T + qrow) + c.inner_its * (nnz * T + n * (7 * T + qrow));
+    st->t_op_ms = 1e-6 * (double)c.ns_op;
+    st->op_calls = c.op_calls;
+    st->op_bytes = c.op_calls * (spmv_bytes(a) + spmv_bytes(b));
+    st->op_flops = c.op_calls * (spmv_flops(a) + spmv_flops(b));
+    st->t_orth_ms = 1e-6 * (double)c.ns_orth;
+    st->orth_calls = c.orth_calls;
+    st->orth_bytes = 8 * n * (2 * c.orth_vecs + 5 * c.orth_calls);
+    st->orth_flops = 8 * n * c.orth_vecs;
+}
+
+// dA = -lambda_i x_j on A's nonzeros for right-hand side j (lam on the device; x and dA may be
+// the host's, staged in buffers that the handle keeps)
+static asss_status grad_A(asss_handle* h, int j, const double* lam, const double* xfwd, int64_t ldxf, double* dA) {
+    cudaStream_t s = h->ctx.stream;
+    const int n = h->n;
+    DBuf<double>& xf = h->xf_stage;
+    DBuf<double>& dAd = h->dA_stage;
+    const bool fdev = is_device_ptr(xfwd), adev = is_device_ptr(dA);
+    const double* xf_p = xfwd + (size_t)j * ldxf;
+    if (!fdev) {
+        if (xf.n < n) ASSS_TRY(xf.alloc(n));
+        ASSS_CUDA(cudaMemcpyAsync(xf.p, xf_p, sizeof(double) * n, cudaMemcpyHostToDevice, s));
+        xf_p = xf.p;
+    }
+    double* dA_p = dA + (size_t)j * h->A.nnz;
+    if (!adev) {
+        if (dAd.n < h->A.nnz) ASSS_TRY(dAd.alloc(h->A.nnz));
+        dA_p = dAd.p;
+    }
+    k_grad_A<<<cdiv(n, 256), 256, 0, s>>>(h->A.rp.p, h->A.ci.p, lam, xf_p, n, dA_p);
+    ASSS_CHECK_LAUNCH();
+    if (!adev)
+        ASSS_CUDA(cudaMemcpyAsync(dA + (size_t)j * h->A.nnz, dA_p, sizeof(double) * h->A.nnz, cudaMemcpyDeviceToHost,
+                                  s));
+    return ASSS_OK;
+}
+
 // ===========================================================================
 // exported functions
 // ===========================================================================
@@ -2058,21 +2256,63 @@ static asss_status solve_common(asss_handle* h, int tr, int nrhs, const double* 
     int n = h->n;
     auto t0 = std::chrono::steady_clock::now();
     bool bdev = is_device_ptr(b), xdev = is_device_ptr(x);
-    DBuf<double>& xf = h->xf_stage;    // staging of host x / dA for the gradient, kept by the handle
-    DBuf<double>& dAd = h->dA_stage;
-    if (!h->bb.p) {
-        ASSS_TRY(h->bb.alloc(n));
-        ASSS_TRY(h->xx.alloc(n));
-    }
-    DBuf<double>& bb = h->bb;
-    DBuf<double>& xx = h->xx;
     asss_stats lst = h->setup_stats;
     asss_status worst = ASSS_OK;
     // several right-hand sides of a forward FGMRES solve: lockstep blocks of up to 8
     // columns whose preconditioner applications share each pass over J~ and Q_k
-    const bool block = h->opt.rhs_block && !tr && nrhs >= 2 && h->opt.outer == ASSS_OUTER_FGMRES &&
-                       h->kp <= MRS_MULTI_KPMAX && !h->Q16.p && !h->factored;
-    if (block) {
+    const bool as_block = h->opt.rhs_block && !tr && nrhs >= 2 && h->opt.outer == ASSS_OUTER_FGMRES &&
+                          h->kp <= MRS_MULTI_KPMAX && !h->Q16.p && !h->factored;
+    int cl = 0;
+    ASSS_TRY(cluster_plan(h, nrhs, &cl));
+    // small and middling systems: whole solves in one launch, a cluster per column
+    for (int j0 = 0; cl > 0 && j0 < nrhs;) {
+        constexpr int CHUNK = 16;   // columns staged at a time
+        const int nc = nrhs - j0 < CHUNK ? nrhs - j0 : CHUNK;
+        // b is copied (x may be the same memory), x staged when it is the host's
+        if (h->cl_b.n < (int64_t)nc * n) ASSS_TRY(h->cl_b.alloc((int64_t)nc * n));
+        if (!xdev && h->cl_x.n < (int64_t)nc * n) ASSS_TRY(h->cl_x.alloc((int64_t)nc * n));
+        if (nc == 1)
+            ASSS_CUDA(cudaMemcpyAsync(h->cl_b.p, b + (size_t)j0 * ldb, sizeof(double) * n,
+                                      bdev ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice, s));
+        else
+            ASSS_CUDA(cudaMemcpy2DAsync(h->cl_b.p, sizeof(double) * n, b + (size_t)j0 * ldb, sizeof(double) * ldb,
+                                        sizeof(double) * n, nc,
+                                        bdev ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice, s));
+        double* xt = xdev ? x + (size_t)j0 * ldx : h->cl_x.p;
+        const int64_t ldt = xdev ? ldx : n;
+        ClStat cs[CHUNK];
+        if (h->opt.precision == ASSS_PREC_MIXED)
+            ASSS_TRY(solve_cluster<float>(h, tr, cl, nc, h->cl_b.p, n, xt, ldt, cs));
+        else
+            ASSS_TRY(solve_cluster<double>(h, tr, cl, nc, h->cl_b.p, n, xt, ldt, cs));
+        if (!xdev && nc == 1)
+            ASSS_CUDA(cudaMemcpyAsync(x + (size_t)j0 * ldx, xt, sizeof(double) * n, cudaMemcpyDeviceToHost, s));
+        else if (!xdev)
+            ASSS_CUDA(cudaMemcpy2DAsync(x + (size_t)j0 * ldx, sizeof(double) * ldx, xt, sizeof(double) * n,
+                                        sizeof(double) * n, nc, cudaMemcpyDeviceToHost, s));
+        if (tr && xfwd && dA)
+            for (int t = 0; t < nc; ++t) ASSS_TRY(grad_A(h, j0 + t, xt + (size_t)t * ldt, xfwd, ldxf, dA));
+        ASSS_CUDA(cudaStreamSynchronize(s));
+        for (int t = 0; t < nc; ++t) {
+            const asss_stats prev = lst;
+            cluster_stats(h, tr, cs[t], &lst);
+            if (as_block && j0 + t > 0) {   // a block's statistics cover all columns
+                lst.outer_its = std::max(lst.outer_its, prev.outer_its);
+                lst.cycles += prev.cycles;
+                lst.relres = std::max(lst.relres, prev.relres);
+                lst.inner_its_total += prev.inner_its_total;
+                lst.inner_solves += prev.inner_solves;
+                lst.inner_launches += prev.inner_launches;
+                lst.inner_its_avg = lst.inner_solves ? (double)lst.inner_its_total / lst.inner_solves : 0.0;
+                lst.t_inner_ms += prev.t_inner_ms;
+                lst.inner_bytes += prev.inner_bytes;
+            }
+            if (cs[t].status != ASSS_OK && worst == ASSS_OK) worst = (asss_status)cs[t].status;
+        }
+        j0 += nc;
+        if (j0 == nrhs) nrhs = 0;   // every column is done
+    }
+    if (as_block && nrhs > 0) {
         const int B = asss_handle::BLK;
         if (!h->blk_b.p) {
             ASSS_TRY(h->blk_b.alloc((int64_t)B * n));
@@ -2125,6 +2365,12 @@ static asss_status solve_common(asss_handle* h, int tr, int nrhs, const double* 
         lst.inner_launches = mlaunch;
         nrhs = 0;   // every column is done
     }
+    if (nrhs > 0 && !h->bb.p) {
+        ASSS_TRY(h->bb.alloc(n));
+        ASSS_TRY(h->xx.alloc(n));
+    }
+    DBuf<double>& bb = h->bb;
+    DBuf<double>& xx = h->xx;
     for (int j = 0; j < nrhs; ++j) {
         ASSS_CUDA(cudaMemcpyAsync(bb.p, b + (size_t)j * ldb, sizeof(double) * n,
                                   bdev ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice, s));
@@ -2133,26 +2379,7 @@ static asss_status solve_common(asss_handle* h, int tr, int nrhs, const double* 
         if (!xdev) {
             ASSS_CUDA(cudaMemcpyAsync(x + (size_t)j * ldx, xt, sizeof(double) * n, cudaMemcpyDeviceToHost, s));
         }
-        if (tr && xfwd && dA) {
-            bool fdev = is_device_ptr(xfwd), adev = is_device_ptr(dA);
-            const double* xf_p = xfwd + (size_t)j * ldxf;
-            if (!fdev) {
-                if (xf.n < n) ASSS_TRY(xf.alloc(n));
-                ASSS_CUDA(cudaMemcpyAsync(xf.p, xf_p, sizeof(double) * n, cudaMemcpyHostToDevice, s));
-                xf_p = xf.p;
-            }
-            double* dA_p = dA + (size_t)j * h->A.nnz;
-            if (!adev) {
-                if (dAd.n < h->A.nnz) ASSS_TRY(dAd.alloc(h->A.nnz));
-                dA_p = dAd.p;
-            }
-            k_grad_A<<<cdiv(n, 256), 256, 0, s>>>(h->A.rp.p, h->A.ci.p, xt, xf_p, n, dA_p);
-            ASSS_CHECK_LAUNCH();
-            if (!adev) {
-                ASSS_CUDA(cudaMemcpyAsync(dA + (size_t)j * h->A.nnz, dA_p, sizeof(double) * h->A.nnz,
-                                          cudaMemcpyDeviceToHost, s));
-            }
-        }
+        if (tr && xfwd && dA) ASSS_TRY(grad_A(h, j, xt, xfwd, ldxf, dA));
         ASSS_CUDA(cudaStreamSynchronize(s));
         if (lst.status != ASSS_OK && worst == ASSS_OK) worst = (asss_status)lst.status;
     }

@@ -1,0 +1,850 @@
+// Whole solves in one launch, a thread-block cluster per right-hand side: the refinement loop
+// on the true FP64 residual, flexible GMRES (FP64) and P^-1 by Eq. smw around the mrs
+// iteration of App. B in T, the algorithms of refine / fgmres_cycle / apply_prec (asss.cu) and of
+// k_mrs in cluster scope.
+//
+// What bounds a solve of a small or middling system in the launch-by-launch path is not its
+// data but its 30 to 100 launches, the host's decisions between them and the grid-wide
+// barriers inside them.  Here the 16 CTAs of a cluster own contiguous rows; sums over the system
+// are exchanged through distributed shared memory, every CTA adds them in the same order and
+// takes the same decisions, and vectors that other CTAs read go through L2 around a cluster
+// barrier.  Several right-hand sides are as many clusters side by side (nine fit on the GPU).
+// Bound: the latency of a row's loads and of a synchronisation; above solve_cluster_limit's sizes
+// 16 SMs' share of the bandwidth and of the FP64 pipe (the rule there has both sides measured).
+#pragma once
+
+#include "cluster_dev.cuh"
+#include "internal.h"
+#include "mrs_dev.cuh"
+
+namespace asss {
+
+constexpr int CL_RESTART = 60;           // longest restart (the Hessenberg matrix stands in shared memory)
+constexpr int CL_XV = CL_RESTART + 6;    // values of one exchange
+constexpr int CL_MMAX = 320;             // largest SMW rank k + r
+// CTAs of a cluster to choose from.  A cluster lives in one GPC, of which this GPU has seven
+// with 16 SMs to spare, eight with 12: 7, 8, 13 and 15 clusters of these sizes are resident.
+constexpr int CL_NSIZES = 4;
+constexpr int CL_SIZES[CL_NSIZES] = {16, 12, 10, 8};
+constexpr int CL_REGV = 6;               // vectors whose dot products run together in registers
+
+// y_i = sum_j M_ij x_j: a diagonal copy (at most 16 diagonals) or CSR
+struct ClMat {
+    int ndiag;
+    const int* off;
+    const double* val;
+    const int *rp, *ci;
+    const double* v;
+};
+
+struct ClStat {
+    int outer_its, cycles, status, solves, op_calls, orth_calls;
+    long long inner_its, orth_vecs;
+    unsigned long long ns_inner, ns_op, ns_orth;
+    double relres;
+};
+
+template <class T>
+struct ClArgs {
+    int n, ncol, restart;
+    // J~ by skew diagonals (as k_mrs FMT 1), Q_k (q_blocked), S_k, SMW data
+    int ndiag, halo, k, m, r;
+    const int* off;
+    const T* U;
+    long long ustride;
+    const T* Q;
+    const double* alpha;
+    const T* Ys;              // n x m row-major
+    const int *neg, *neg2;    // U_r (UrCols of asss.cu)
+    const double *negc1, *negc2;
+    // op1 then op2: the outer operator; Sm and Am: update and residual (their transposes with tr)
+    ClMat op1, op2, Sm, Am;
+    const double *dr, *dc, *w;
+    const int* perm;
+    int tr;
+    double sign;
+    const double* b;          // column c at b + c * ldb
+    long long ldb;
+    double* x;
+    long long ldx;
+    double* work;             // per resident cluster
+    long long work_stride;
+    double outer_tol, inner_tol;
+    int outer_maxit, inner_maxit;
+    ClStat* stats;
+};
+
+// doubles of workspace per cluster
+inline long long cl_work_doubles(int n, int halo, int restart, int tbytes) {
+    const long long nd = (long long)(5 + 2 * restart + 1) * n;
+    const long long nt = 3LL * ((long long)n + 2LL * halo + 32) + 3LL * n;
+    return nd + (nt * tbytes + 7) / 8 + 64;
+}
+
+template <class T, int KP>
+struct ClShared {
+    using P2 = typename std::conditional<sizeof(T) == 4, float2, double>::type;
+    unsigned long long x[2][CL_MAX][CL_XV];   // exchanged block sums, written by the other CTAs
+    T wsum[CL_WARPS][KP + 1];
+    double wd[CL_WARPS][CL_REGV + 2];
+    double bp[CL_XV], tot[CL_XV];
+    T red[KP + 1], u[KP > 0 ? KP : 1], alpha[KP > 0 ? KP : 1], cf[12];
+    T qty[KP > 0 ? KP : 1], qtp[2][KP > 0 ? KP : 1], qtx[KP > 0 ? KP : 1], pq[4];
+    T wv[CL_MMAX];
+    int off[64], moff[4][16];
+    double h1[CL_RESTART + 1], cs[CL_RESTART + 1], sn[CL_RESTART + 1], g[CL_RESTART + 2], yv[CL_RESTART + 1];
+    double fin[3];
+    MrsScalars<T> sc;
+    int stop;
+};
+
+template <class T, int KP>
+__global__ void __launch_bounds__(CL_THREADS, 1) k_solve_cl(const ClArgs<T> p) {
+    constexpr int NT = CL_THREADS, NW = CL_WARPS, NV = KP + 1, KQ = KP > 0 ? KP : 1;
+    using Sh = ClShared<T, KP>;
+    using P2 = typename Sh::P2;
+    extern __shared__ __align__(16) unsigned char s_dyn[];
+    Sh& sh = *reinterpret_cast<Sh*>(s_dyn);
+    double* H = reinterpret_cast<double*>(s_dyn + ((sizeof(Sh) + 15) & ~15));   // (restart + 1) x restart, column-major
+    const int R = p.restart, n = p.n;
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int rank = (int)cl_rank(), C = (int)cl_size();
+    const int nsl = (n + 31) >> 5;
+    const int rb = (int)((long long)nsl * rank / C) * 32;
+    const int re = min(n, (int)((long long)nsl * (rank + 1) / C) * 32);
+    const int nact = min(NW, max(re - rb + 31, 0) >> 5);   // warps that hold rows; the others' sums stay zero
+    double* base = p.work + (size_t)cl_id() * (size_t)p.work_stride;
+    const long long nn = n;
+    double *r = base, *rh = r + nn, *t1 = rh + nn, *t2 = t1 + nn, *wv = t2 + nn;
+    double* V = wv + nn;
+    double* Z = V + (R + 1) * nn;
+    T* fb = reinterpret_cast<T*>(Z + R * nn);
+    const long long ys = nn + 2LL * p.halo + 32;
+    T* Y = fb + p.halo;
+    T* P = fb + 3 * ys;
+    T* z = P + 2 * nn;
+
+    for (int t = tid; t < p.ndiag && t < 64; t += NT) sh.off[t] = p.off[t];
+    if (tid < 64) {
+        const ClMat& M = tid < 16 ? p.op1 : tid < 32 ? p.op2 : tid < 48 ? p.Sm : p.Am;
+        const int d = tid & 15;
+        sh.moff[tid >> 4][d] = d < M.ndiag ? M.off[d] : 0;
+    }
+    for (int t = tid; t < NW * NV; t += NT) (&sh.wsum[0][0])[t] = (T)0;
+    for (int t = tid; t < NW * (CL_REGV + 2); t += NT) (&sh.wd[0][0])[t] = 0.0;
+    for (int t = tid; t + 1 < p.k && t < KP; t += NT) sh.alpha[t] = (T)p.alpha[t];
+    // the halos of the three Lanczos slots (nothing else writes them)
+    for (int t = rank * NT + tid; t < 6 * p.halo; t += C * NT) {
+        const int slot = t / (2 * p.halo), e = t % (2 * p.halo);
+        Y[slot * ys + (e < p.halo ? e - p.halo : nn + (e - p.halo))] = (T)0;
+    }
+    cl_sync();   // every CTA of the cluster runs: its shared memory may be written
+
+    auto add_t = [](P2 a, P2 b) {
+        if constexpr (sizeof(T) == 4) return df_add(a, b);
+        else return a + b;
+    };
+    auto add_d = [](double a, double b) { return a + b; };
+    auto now = [&]() -> unsigned long long { return (rank == 0 && tid == 0) ? gtimer() : 0ull; };
+    unsigned xphase = 0;
+    // out[v] = sum over `rows` rows of a[row * ld + v]: four threads a value
+    auto sum_rows = [&](const double* a, int ld, int rows, int cnt, double* out) {
+        for (int t0 = 0; t0 < cnt * 4; t0 += NT) {
+            const int t = t0 + tid, v = t >> 2;
+            double s = 0.0;
+            if (v < cnt)
+                for (int row = t & 3; row < rows; row += 4) s += a[(size_t)row * ld + v];
+            s += __shfl_xor_sync(0xffffffffu, s, 1);
+            s += __shfl_xor_sync(0xffffffffu, s, 2);
+            if (v < cnt && (t & 3) == 0) out[v] = s;
+        }
+    };
+    // cluster totals of the block sums bp[0..cnt) into tot[0..cnt) (a cluster barrier)
+    auto exchange = [&](int cnt) {
+        __syncthreads();
+        const int buf = xphase++ & 1;
+        for (int t = tid; t < cnt * C; t += NT) {
+            const int q = t / cnt, v = t % cnt;
+            cl_store8(&sh.x[buf][rank][v], q, cl_bits(sh.bp[v]));
+        }
+        cl_sync();
+        sum_rows(reinterpret_cast<const double*>(&sh.x[buf][0][0]), CL_XV, C, cnt, sh.tot);
+        __syncthreads();
+    };
+    // block sums of CNT accumulators into bp[slot..)
+    auto block_sums = [&](auto& acc, int slot) {
+        constexpr int CNT = sizeof(acc) / sizeof(double);
+        __syncthreads();
+        if (warp < nact) warp_fold_to<CNT>(acc, sh.wd[warp]);
+        __syncthreads();
+        sum_rows(&sh.wd[0][0], CL_REGV + 2, NW, CNT, sh.bp + slot);
+    };
+    auto norm2 = [&](const double* a) -> double {
+        double acc[1] = {0.0};
+        for (int i = rb + tid; i < re; i += NT) acc[0] += a[i] * a[i];
+        block_sums(acc, 0);
+        exchange(1);
+        return sh.tot[0];
+    };
+    // row i of M x (x complete in L2)
+    auto mat_row = [&](const ClMat& M, const int* off, const double* x, int i) -> double {
+        double s = 0.0;
+        if (M.ndiag > 0) {
+            for (int d0 = 0; d0 < M.ndiag; d0 += 8) {
+                double v[8], xv[8];
+#pragma unroll
+                for (int u = 0; u < 8; ++u) {
+                    const int d = d0 + u, j = i + off[d & 15];
+                    const bool in = d < M.ndiag && j >= 0 && j < n;
+                    v[u] = in ? __ldg(&M.val[(size_t)d * n + i]) : 0.0;
+                    xv[u] = in ? x[j] : 0.0;
+                }
+#pragma unroll
+                for (int u = 0; u < 8; ++u)
+                    if (d0 + u < M.ndiag) s += v[u] * xv[u];
+            }
+        } else {
+            const int e1 = __ldg(&M.rp[i + 1]);
+            for (int e = __ldg(&M.rp[i]); e < e1; e += 8) {
+                int cc[8];
+                double v[8], xv[8];
+#pragma unroll
+                for (int u = 0; u < 8; ++u) {
+                    cc[u] = e + u < e1 ? __ldg(&M.ci[e + u]) : 0;
+                    v[u] = e + u < e1 ? __ldg(&M.v[e + u]) : 0.0;
+                }
+#pragma unroll
+                for (int u = 0; u < 8; ++u) xv[u] = e + u < e1 ? x[cc[u]] : 0.0;
+#pragma unroll
+                for (int u = 0; u < 8; ++u) s += v[u] * xv[u];
+            }
+        }
+        return s;
+    };
+
+    // ---------------------------------------------------------------------------
+    // mrs (App. B) on (I + sign (J~ - Q S_k Q^T)) z = u; Q^T z into sh.wv[0..k)
+    // ---------------------------------------------------------------------------
+    auto mrs_sums = [&](T(&tacc)[NV]) {   // cluster totals into sh.red, for warp 0
+        if (warp < nact) warp_fold_to<NV>(tacc, sh.wsum[warp]);
+        __syncthreads();
+        const int buf = xphase++ & 1;
+        if (warp == 0) {
+            for (int v = lane; v < NV; v += 32) {
+                P2 a[NW];
+#pragma unroll
+                for (int q = 0; q < NW; ++q) {
+                    if constexpr (sizeof(T) == 4) a[q] = make_float2(sh.wsum[q][v], 0.f);
+                    else a[q] = sh.wsum[q][v];
+                }
+                const unsigned long long bits = cl_bits(pair_tree(a, add_t));
+                for (int q = 0; q < C; ++q) cl_store8(&sh.x[buf][rank][v], q, bits);
+            }
+        }
+        cl_sync();
+        if (warp == 0) {
+            for (int v = lane; v < NV; v += 32) {
+                P2 a[CL_MAX];
+#pragma unroll
+                for (int q = 0; q < CL_MAX; ++q) {
+                    a[q] = P2{};
+                    if (q < C) a[q] = *reinterpret_cast<const P2*>(&sh.x[buf][q][v]);
+                }
+                const P2 t = pair_tree(a, add_t);
+                if constexpr (sizeof(T) == 4) sh.red[v] = t.x + t.y;
+                else sh.red[v] = t;
+            }
+            __syncwarp();
+        }
+    };
+    auto make_u = [&]() {   // u = S_k (nu Q^T y), warp 0
+        for (int a = lane; a < KP; a += 32) {
+            T u = (T)0;
+            if (a < p.k) {
+                if (a + 1 < p.k) u += sh.alpha[a] * sh.red[2 + a] * sh.sc.nu;
+                if (a > 0) u -= sh.alpha[a - 1] * sh.red[a] * sh.sc.nu;
+            }
+            sh.u[a] = u;
+        }
+    };
+    auto set_coefs = [&]() {
+        const MrsScalars<T>& c = sh.sc;
+        sh.cf[0] = (T)p.sign * c.nu;
+        sh.cf[1] = (T)p.sign;
+        sh.cf[2] = c.coef_old;
+        sh.cf[3] = c.nu_p;
+        sh.cf[4] = c.delta_pp;
+        sh.cf[5] = c.rtheta_p;
+        sh.cf[6] = c.xcoef_p;
+        if (c.stop) {
+            sh.cf[7] = c.fin_nu;
+            sh.cf[8] = c.fin_delta;
+            sh.cf[9] = c.fin_rtheta;
+            sh.cf[10] = c.fin_xcoef;
+        }
+    };
+    auto qtx_fold = [&](int jj) {   // warp 1: direction p_jj into Q^T z
+        for (int a = lane; a < p.k; a += 32) {
+            T* pp = sh.qtp[jj & 1];
+            const T v = (sh.pq[0] * sh.qty[a] - sh.pq[1] * pp[a]) * sh.pq[2];
+            pp[a] = v;
+            sh.qtx[a] += sh.pq[3] * v;
+        }
+    };
+    auto mrs = [&](const double* rhs) -> int {
+        for (int a = tid; a < KP; a += NT) {
+            sh.qtp[0][a] = (T)0;
+            sh.qtp[1][a] = (T)0;
+            sh.qtx[a] = (T)0;
+        }
+        T tacc[NV];
+#pragma unroll
+        for (int v = 0; v < NV; ++v) tacc[v] = (T)0;
+        for (int i = rb + tid; i < re; i += NT) {
+            const T b = (T)rhs[i];
+            Y[i] = b;
+            z[i] = (T)0;
+            P[i] = (T)0;
+            P[nn + i] = (T)0;
+            tacc[0] += b * b;
+            T q[KQ];
+            load_qrow<T, KP, q_blocked<T>(true)>(p.Q, i, q);
+#pragma unroll
+            for (int a = 0; a < KP; ++a) tacc[1 + a] += q[a] * b;
+        }
+        mrs_sums(tacc);
+        if (warp == 0) {
+            if (lane == 0) {
+                MrsScalars<T>& c = sh.sc;
+                const T r0 = sqrt(sh.red[0]);
+                c.r0 = r0;
+                c.rr0 = r0 > (T)0 ? (T)1 / r0 : (T)0;
+                c.nu = c.rr0;
+                c.coef_old = (T)0;
+                c.theta_t = (T)1;
+                c.c_prev = (T)1;
+                c.s_prev = (T)0;
+                c.delta_prev = (T)0;
+                c.G = r0;
+                c.nu_p = (T)0;
+                c.delta_pp = (T)0;
+                c.rtheta_p = (T)1;
+                c.xcoef_p = (T)0;
+                c.its = 0;
+                c.stop = r0 > (T)0 ? 0 : 1;
+                set_coefs();
+            }
+            __syncwarp();
+            if (!sh.sc.stop) make_u();
+        }
+        __syncthreads();
+        if (sh.sc.stop) {
+            for (int a = tid; a < p.k; a += NT) sh.wv[a] = (T)0;
+            return 0;
+        }
+        for (int j = 1; j <= p.inner_maxit; ++j) {
+            if (KP > 0 && warp == 1) {
+                if (j >= 2) qtx_fold(j - 1);
+                for (int a = lane; a < p.k; a += 32) sh.qty[a] = sh.red[1 + a];
+            }
+            const T* Ycur = Y + (size_t)((j - 1) % 3) * ys;
+            const T* __restrict__ Yold = Y + (size_t)((j + 1) % 3) * ys;   // own rows
+            T* __restrict__ Ynew = Y + (size_t)(j % 3) * ys;
+            T* __restrict__ Pj1 = P + (size_t)((j - 1) & 1) * nn;
+            T* __restrict__ zz = z;
+            const T tnu = sh.cf[0], tsg = sh.cf[1], tco = sh.cf[2], tnp = sh.cf[3], tdpp = sh.cf[4], tthp = sh.cf[5],
+                    txp = sh.cf[6];
+#pragma unroll
+            for (int v = 0; v < NV; ++v) tacc[v] = (T)0;
+            for (int i = rb + tid; i < re; i += NT) {
+                const T yold = j >= 2 ? Yold[i] : (T)0;
+                const T pold = j >= 2 ? Pj1[i] : (T)0;
+                T acc = (T)0;
+                const T* Ud = p.U + i;
+                const T* yi = Ycur + i;
+#pragma unroll 12
+                for (int d = 0; d < p.ndiag; ++d, Ud += p.ustride) {
+                    const int mo = sh.off[d];
+                    if constexpr (sizeof(T) == 8) {
+                        acc = fma(__ldg(Ud), yi[mo], acc);
+                        acc = fma(-__ldg(Ud - mo), yi[-mo], acc);
+                    } else {
+                        acc += __ldg(Ud) * yi[mo] - __ldg(Ud - mo) * yi[-mo];
+                    }
+                }
+                T q[KQ];
+                load_qrow<T, KP, q_blocked<T>(true)>(p.Q, i, q);
+                T dq = (T)0;
+#pragma unroll
+                for (int a = 0; a < KP; ++a) dq += q[a] * sh.u[a];
+                const T ynew = tnu * acc - tsg * dq + tco * yold;
+                Ynew[i] = ynew;
+                tacc[0] += ynew * ynew;
+#pragma unroll
+                for (int a = 0; a < KP; ++a) tacc[1 + a] += q[a] * ynew;
+                if (j >= 2) {
+                    const T pv = (tnp * yold - tdpp * pold) * tthp;
+                    Pj1[i] = pv;
+                    zz[i] += txp * pv;
+                }
+            }
+            mrs_sums(tacc);
+            if (warp == 0) {
+                MrsScalars<T>& c = sh.sc;
+                // beta and 1 / beta in lane 0, theta and 1 / theta in lane 1
+                const T rad = lane == 0 ? sh.red[0] : c.theta_t * c.theta_t + sh.red[0];
+                T root, inv;
+                if constexpr (sizeof(T) == 4) {
+                    root = sqrt(rad);
+                    inv = (T)1 / root;
+                } else {
+                    inv = rsqrt(rad);
+                    root = rad != (T)0 ? rad * inv : (T)0;
+                }
+                const T beta = __shfl_sync(0xffffffffu, root, 0), rbeta = __shfl_sync(0xffffffffu, inv, 0);
+                const T theta = __shfl_sync(0xffffffffu, root, 1), rth = __shfl_sync(0xffffffffu, inv, 1);
+                if (lane == 0) {
+                    const T cc = c.theta_t * rth, s = beta * rth;
+                    const T delta = -c.s_prev * beta;
+                    const T theta_t_next = c.c_prev * theta;
+                    const T xcoef = c.G * cc;
+                    const T Gn = -c.G * s;
+                    sh.pq[0] = c.nu;
+                    sh.pq[1] = c.delta_prev;
+                    sh.pq[2] = rth;
+                    sh.pq[3] = xcoef;
+                    c.ratio = fabs(Gn) * c.rr0;
+                    c.its = j;
+                    if (c.ratio < (T)p.inner_tol || j == p.inner_maxit) {
+                        c.stop = 1;
+                        c.fin_nu = c.nu;
+                        c.fin_delta = c.delta_prev;
+                        c.fin_rtheta = rth;
+                        c.fin_xcoef = xcoef;
+                    } else {
+                        c.nu_p = c.nu;
+                        c.delta_pp = c.delta_prev;
+                        c.rtheta_p = rth;
+                        c.xcoef_p = xcoef;
+                        c.coef_old = beta * c.nu;
+                        c.nu = (beta != (T)0) ? rbeta : (T)0;
+                        c.s_prev = s;
+                        c.c_prev = cc;
+                        c.delta_prev = delta;
+                        c.theta_t = theta_t_next;
+                        c.G = Gn;
+                    }
+                    set_coefs();
+                }
+                __syncwarp();
+                if (!sh.sc.stop) make_u();
+            }
+            __syncthreads();
+            if (sh.sc.stop) {
+                const T* Pj = P + (size_t)(j & 1) * nn;
+                const T tn = sh.cf[7], td = sh.cf[8], tth = sh.cf[9], tx = sh.cf[10];
+                for (int i = rb + tid; i < re; i += NT) {
+                    const T pv = (tn * Ycur[i] - td * Pj[i]) * tth;
+                    z[i] = z[i] + tx * pv;
+                }
+                if (KP > 0 && warp == 1) {
+                    qtx_fold(j);
+                    __syncwarp();
+                    for (int a = lane; a < p.k; a += 32) sh.wv[a] = sh.qtx[a];
+                }
+                break;
+            }
+        }
+        return sh.sc.its;
+    };
+
+    // f(count as a constant) for the vector counts whose dot products run together
+    auto by_count = [&](int nv, auto f) {
+        switch (nv) {
+            case 1: f(std::integral_constant<int, 1>{}); break;
+            case 2: f(std::integral_constant<int, 2>{}); break;
+            case 3: f(std::integral_constant<int, 3>{}); break;
+            case 4: f(std::integral_constant<int, 4>{}); break;
+            case 5: f(std::integral_constant<int, 5>{}); break;
+            default: f(std::integral_constant<int, 6>{}); break;
+        }
+    };
+    // block sums of V_a^T w, a < nv, one warp per vector, into bp[0..nv)
+    auto dots_by_warp = [&](int nv) {
+        __syncthreads();
+        for (int a = warp; a < nv; a += NW) {
+            const double* va = V + (size_t)a * nn;
+            double acc[4] = {0.0, 0.0, 0.0, 0.0};
+            int i = rb + lane;
+            for (; i + 96 < re; i += 128)
+#pragma unroll
+                for (int u = 0; u < 4; ++u) acc[u] += va[i + u * 32] * wv[i + u * 32];
+            for (; i < re; i += 32) acc[0] += va[i] * wv[i];
+            const double t = warp_sum((acc[0] + acc[1]) + (acc[2] + acc[3]));
+            if (lane == 0) sh.bp[a] = t;
+        }
+    };
+    auto project = [&](int i, int nv, const double* h) -> double {
+        double s = 0.0;
+        for (int a = 0; a < nv; a += 8) {
+            double ld[8];
+#pragma unroll
+            for (int u = 0; u < 8; ++u) ld[u] = a + u < nv ? V[(size_t)(a + u) * nn + i] : 0.0;
+#pragma unroll
+            for (int u = 0; u < 8; ++u)
+                if (a + u < nv) s += ld[u] * h[a + u];
+        }
+        return wv[i] - s;
+    };
+
+    for (int col = (int)cl_id(); col < p.ncol; col += (int)cl_count()) {
+        const double* b = p.b + (size_t)col * p.ldb;
+        double* x = p.x + (size_t)col * p.ldx;
+        unsigned long long ns_inner = 0, ns_op = 0, ns_orth = 0;
+        int outer = 0, cycles = 0, status = ASSS_OK, stall = 0, solves = 0, ops = 0, orths = 0;
+        long long inner = 0, vecs = 0;
+        double relres = 0.0, best = INFINITY;
+        for (int i = rb + tid; i < re; i += NT) {
+            x[i] = 0.0;
+            r[i] = b[i];
+        }
+        const double bn = sqrt(norm2(r));
+        double rn = bn;
+        if (!(bn < INFINITY)) {   // a NaN or an infinity in b
+            status = ASSS_ERR_BREAKDOWN;
+            relres = 1.0;
+        }
+        // a right-hand side of norm 0, infinity or NaN counts the one inner solve of zero steps
+        // that the launch-by-launch path has enqueued by the time it knows
+        if (!(bn > 0.0 && bn < INFINITY) && p.outer_tol < 1.0 && p.outer_maxit > 0) solves = 1;
+        while (bn > 0.0 && status == ASSS_OK) {
+            relres = rn / bn;
+            if (relres <= p.outer_tol) break;
+            if (!(rn == rn)) {
+                status = ASSS_ERR_BREAKDOWN;
+                break;
+            }
+            if (outer >= p.outer_maxit) {
+                status = ASSS_ERR_NOT_CONVERGED;
+                break;
+            }
+            if (rn < 0.999 * best) {
+                best = rn;
+                stall = 0;
+            } else if (++stall >= 5) {
+                status = ASSS_ERR_STAGNATION;
+                break;
+            }
+            // r^ = W P D_r r, or W S^T D_c r (the barrier of the last norm published r)
+            if (!p.tr) {
+                for (int i = rb + tid; i < re; i += NT) {
+                    const int q = p.perm ? p.perm[i] : i;
+                    rh[i] = p.w[i] * p.dr[q] * r[q];
+                }
+            } else {
+                for (int i = rb + tid; i < re; i += NT) t1[i] = p.dc[i] * r[i];
+                cl_sync();
+                for (int i = rb + tid; i < re; i += NT) rh[i] = p.w[i] * mat_row(p.Sm, sh.moff[2], t1, i);
+            }
+            const double eta = fmin(0.5, 0.5 * p.outer_tol * bn / rn);
+            const int mcyc = min(R, p.outer_maxit - outer);
+            // ---- one flexible GMRES cycle ----
+            const double rr = norm2(rh);
+            int steps = 0;
+            if (rr > 0.0 && rr < INFINITY) {
+                const double beta0 = sqrt(rr), inv0 = 1.0 / beta0, thr = eta * beta0;
+                for (int i = rb + tid; i < re; i += NT) V[i] = inv0 * rh[i];
+                if (tid == 0) sh.g[0] = beta0;
+                for (int j = 0; j < mcyc; ++j) {
+                    double* zj = Z + (size_t)j * nn;
+                    const unsigned long long tm0 = now();
+                    inner += mrs(V + (size_t)j * nn);
+                    const unsigned long long tm1 = now();
+                    ++solves;
+                    // z_j = z - Y (U^T z)
+                    if (p.r > 0 && p.m > 0) {
+                        cl_sync();   // z complete: U_r^T z gathers from every CTA's rows
+                        for (int a = tid; a < p.r; a += NT) {
+                            double v;
+                            if (!p.neg2) {
+                                v = (double)z[p.neg[a]];
+                            } else {
+                                v = p.negc1[a] * (double)z[p.neg[a]];
+                                const int q = p.neg2[a];
+                                if (q >= 0) v += p.negc2[a] * (double)z[q];
+                            }
+                            sh.wv[p.k + a] = (T)v;
+                        }
+                    }
+                    __syncthreads();
+                    for (int i = rb + tid; i < re; i += NT) {
+                        T acc = (T)0;
+                        const T* yr = p.Ys + (size_t)i * p.m;
+                        if (sizeof(T) == 4 && (p.m & 3) == 0) {
+                            const float4* y4 = reinterpret_cast<const float4*>(yr);
+#pragma unroll 5
+                            for (int c = 0; c < (p.m >> 2); ++c) {
+                                const float4 v = __ldg(y4 + c);
+                                acc += (T)v.x * sh.wv[4 * c] + (T)v.y * sh.wv[4 * c + 1] + (T)v.z * sh.wv[4 * c + 2] +
+                                       (T)v.w * sh.wv[4 * c + 3];
+                            }
+                        } else {
+                            for (int c = 0; c < p.m; ++c) acc += yr[c] * sh.wv[c];
+                        }
+                        zj[i] = (double)(z[i] - acc);
+                    }
+                    // w = A_cal z_j
+                    cl_sync();
+                    const unsigned long long tm2 = now();
+                    for (int i = rb + tid; i < re; i += NT) t1[i] = mat_row(p.op1, sh.moff[0], zj, i);
+                    cl_sync();
+                    for (int i = rb + tid; i < re; i += NT) wv[i] = mat_row(p.op2, sh.moff[1], t1, i);
+                    const unsigned long long tm3 = now();
+                    ++ops;
+                    // two classical Gram-Schmidt passes; ||w2||^2 = ||w1||^2 - ||h2||^2
+                    const int nv = j + 1;
+                    vecs += nv;
+                    if (nv <= CL_REGV) {
+                        by_count(nv, [&](auto nvc) {
+                            constexpr int NVC = decltype(nvc)::value;
+                            double acc[NVC];
+#pragma unroll
+                            for (int t = 0; t < NVC; ++t) acc[t] = 0.0;
+                            for (int i = rb + tid; i < re; i += NT) {
+                                const double wi = wv[i];
+#pragma unroll
+                                for (int t = 0; t < NVC; ++t) acc[t] += V[(size_t)t * nn + i] * wi;
+                            }
+                            block_sums(acc, 0);
+                        });
+                    } else {
+                        dots_by_warp(nv);
+                    }
+                    exchange(nv);
+                    for (int a = tid; a < nv; a += NT) sh.h1[a] = sh.tot[a];
+                    if (nv <= CL_REGV) {
+                        by_count(nv, [&](auto nvc) {
+                            constexpr int NVC = decltype(nvc)::value;
+                            double acc[NVC + 1], h[NVC];
+#pragma unroll
+                            for (int t = 0; t <= NVC; ++t) acc[t] = 0.0;
+#pragma unroll
+                            for (int t = 0; t < NVC; ++t) h[t] = sh.tot[t];
+                            for (int i = rb + tid; i < re; i += NT) {
+                                double vi[NVC], s = 0.0;
+#pragma unroll
+                                for (int t = 0; t < NVC; ++t) {
+                                    vi[t] = V[(size_t)t * nn + i];
+                                    s += vi[t] * h[t];
+                                }
+                                const double wn = wv[i] - s;
+                                wv[i] = wn;
+#pragma unroll
+                                for (int t = 0; t < NVC; ++t) acc[t] += vi[t] * wn;
+                                acc[NVC] += wn * wn;
+                            }
+                            block_sums(acc, 0);
+                        });
+                    } else {
+                        double acc[1] = {0.0};
+                        for (int i = rb + tid; i < re; i += NT) {
+                            const double wn = project(i, nv, sh.tot);
+                            wv[i] = wn;
+                            acc[0] += wn * wn;
+                        }
+                        block_sums(acc, nv);
+                        dots_by_warp(nv);
+                    }
+                    exchange(nv + 1);
+                    if (warp == 0) {   // the norm, then the Givens update (every CTA the same)
+                        double h2n = 0.0;
+                        for (int a = 0; a < nv; ++a) h2n += sh.tot[a] * sh.tot[a];
+                        const double hn2 = fmax(sh.tot[nv] - h2n, 0.0);
+                        const double inv = hn2 > 0.0 ? rsqrt(hn2) : 0.0, hn = hn2 * inv;
+                        if (lane == 0) {
+                            sh.fin[0] = hn2;
+                            sh.fin[1] = hn;
+                            sh.fin[2] = inv;
+                        }
+                    }
+                    __syncthreads();
+                    const double inv = sh.fin[2];
+                    double* vn = V + (size_t)nv * nn;
+                    for (int i = rb + tid; i < re; i += NT) vn[i] = project(i, nv, sh.tot) * inv;
+                    if (tid == NT - 1) {
+                        const double hn2 = sh.fin[0], hn = sh.fin[1];
+                        double* hc = H + (size_t)j * (R + 1);
+                        double cur = sh.h1[0] + sh.tot[0];
+                        for (int a = 0; a < j; ++a) {
+                            const double next = sh.h1[a + 1] + sh.tot[a + 1];
+                            hc[a] = sh.cs[a] * cur + sh.sn[a] * next;
+                            cur = sh.cs[a] * next - sh.sn[a] * cur;
+                        }
+                        const double big = fmax(fabs(cur), hn);
+                        double rot, c, s;
+                        if (big > 1e-140 && big < 1e140) {
+                            const double q2 = cur * cur + hn * hn, ir = rsqrt(q2);
+                            rot = q2 * ir;
+                            c = cur * ir;
+                            s = hn * ir;
+                        } else {
+                            rot = hypot(cur, hn);
+                            c = (rot != 0.0) ? cur / rot : 1.0;
+                            s = (rot != 0.0) ? hn / rot : 0.0;
+                        }
+                        hc[j] = rot;
+                        sh.cs[j] = c;
+                        sh.sn[j] = s;
+                        const double gj = sh.g[j];
+                        sh.g[j + 1] = -s * gj;
+                        sh.g[j] = c * gj;
+                        sh.stop = (hn2 == 0.0 || fabs(s * gj) <= thr) ? 1 : 0;
+                    }
+                    __syncthreads();
+                    const unsigned long long tm4 = now();
+                    ns_inner += tm1 - tm0;
+                    ns_op += tm3 - tm2;
+                    ns_orth += tm4 - tm3;
+                    ++orths;
+                    steps = j + 1;
+                    if (sh.stop) break;
+                }
+                // y from the triangular system, column by column
+                if (warp == 0) {
+                    for (int a = lane; a < steps; a += 32) sh.yv[a] = sh.g[a];
+                    __syncwarp();
+                    for (int a = steps - 1; a >= 0; --a) {
+                        const double ya = sh.yv[a] / H[(size_t)a * (R + 1) + a];
+                        __syncwarp();
+                        for (int q = lane; q < a; q += 32) sh.yv[q] -= H[(size_t)a * (R + 1) + q] * ya;
+                        if (lane == 0) sh.yv[a] = ya;
+                        __syncwarp();
+                    }
+                }
+                __syncthreads();
+            }
+            // x += D_c S W dy, or lambda += D_r P^T W dy, with dy = Z y
+            for (int i = rb + tid; i < re; i += NT) {
+                double dy = 0.0;
+                for (int a = 0; a < steps; a += 8) {
+                    double ld[8];
+#pragma unroll
+                    for (int u = 0; u < 8; ++u) ld[u] = a + u < steps ? Z[(size_t)(a + u) * nn + i] : 0.0;
+#pragma unroll
+                    for (int u = 0; u < 8; ++u)
+                        if (a + u < steps) dy += ld[u] * sh.yv[a + u];
+                }
+                if (!p.tr) {
+                    t1[i] = p.w[i] * dy;
+                } else {
+                    const int q = p.perm ? p.perm[i] : i;
+                    x[q] += p.dr[q] * p.w[i] * dy;
+                }
+            }
+            cl_sync();
+            if (!p.tr) {
+                for (int i = rb + tid; i < re; i += NT) x[i] += p.dc[i] * mat_row(p.Sm, sh.moff[2], t1, i);
+                cl_sync();
+            }
+            for (int i = rb + tid; i < re; i += NT) r[i] = b[i] - mat_row(p.Am, sh.moff[3], x, i);
+            outer += steps;
+            ++cycles;
+            rn = sqrt(norm2(r));
+        }
+        if (rank == 0 && tid == 0) {
+            ClStat st;
+            st.outer_its = outer;
+            st.cycles = cycles;
+            st.status = status;
+            st.solves = solves;
+            st.op_calls = ops;
+            st.orth_calls = orths;
+            st.inner_its = inner;
+            st.orth_vecs = vecs;
+            st.ns_inner = ns_inner;
+            st.ns_op = ns_op;
+            st.ns_orth = ns_orth;
+            st.relres = relres;
+            p.stats[col] = st;
+        }
+        cl_sync();   // the column is done before the cluster's buffers are reused
+    }
+}
+
+// ---------------------------------------------------------------------------
+// host side
+// ---------------------------------------------------------------------------
+// clusters of `size` CTAs that can be resident at once (0: none fits)
+template <class T, int KP>
+static asss_status cl_clusters(int size, size_t smem, int* count) {
+    const void* fn = (const void*)k_solve_cl<T, KP>;
+    ASSS_TRY(raise_dynamic_smem(fn, (int)smem));
+    if (size > 8) ASSS_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(size);
+    cfg.blockDim = dim3(CL_THREADS);
+    cfg.dynamicSmemBytes = smem;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = size;
+    at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    if (cudaOccupancyMaxActiveClusters(count, fn, &cfg) != cudaSuccess) {
+        cudaGetLastError();   // a size this device does not take
+        *count = 0;
+    }
+    return ASSS_OK;
+}
+
+// launches `count` clusters of `size` CTAs, or (size == 0) asks how many clusters of each of
+// CL_SIZES can be resident, into counts
+template <class T, int KP>
+static asss_status cl_run(const Ctx& c, const ClArgs<T>& a, int size, int count, int* counts) {
+    const size_t smem = ((sizeof(ClShared<T, KP>) + 15) & ~(size_t)15) +
+                        sizeof(double) * (size_t)(a.restart + 1) * (size_t)a.restart;
+    if (size == 0) {
+        for (int t = 0; t < CL_NSIZES; ++t) ASSS_TRY((cl_clusters<T, KP>(CL_SIZES[t], smem, &counts[t])));
+        return ASSS_OK;
+    }
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(size * count);
+    cfg.blockDim = dim3(CL_THREADS);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = c.stream;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = size;
+    at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    ASSS_CUDA(cudaLaunchKernelEx(&cfg, k_solve_cl<T, KP>, a));
+    count_launch();
+    return ASSS_OK;
+}
+
+template <class T>
+asss_status cl_dispatch(const Ctx& c, const ClArgs<T>& a, int kp, int size, int count, int* counts) {
+    switch (kp) {
+#define ASSS_CL_CASE(KPV) \
+    case KPV:             \
+        return cl_run<T, KPV>(c, a, size, count, counts);
+        ASSS_CL_CASE(0)
+        ASSS_CL_CASE(4)
+        ASSS_CL_CASE(8)
+        ASSS_CL_CASE(12)
+        ASSS_CL_CASE(16)
+        ASSS_CL_CASE(20)
+        ASSS_CL_CASE(24)
+        ASSS_CL_CASE(32)
+#undef ASSS_CL_CASE
+        default:
+            set_error("cluster solve: unsupported padded Lanczos width %d", kp);
+            return ASSS_ERR_UNSUPPORTED;
+    }
+}
+
+extern template asss_status cl_dispatch<float>(const Ctx&, const ClArgs<float>&, int, int, int, int*);
+extern template asss_status cl_dispatch<double>(const Ctx&, const ClArgs<double>&, int, int, int, int*);
+
+}  // namespace asss
