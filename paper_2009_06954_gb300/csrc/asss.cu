@@ -2004,6 +2004,7 @@ static int cluster_size(const asss_handle* h, int nrhs) {
     const bool fp32 = h->opt.precision == ASSS_PREC_MIXED;
     const double n = h->n;
     double best = nrhs * (fp32 ? 470.0 + 0.0012 * n : 560.0 + 0.0033 * n) * 0.95;
+    if (h->factored) best = nrhs * 3000.0;   // a grid barrier or a launch per colour: 24^3 4295 us against 1133
     int size = 0;
     for (int t = 0; t < CL_NSIZES; ++t) {
         if (h->cl_counts[t] < 1) continue;
@@ -2017,31 +2018,6 @@ static int cluster_size(const asss_handle* h, int nrhs) {
     return size;
 }
 
-// the cluster size of a call (0: launch by launch); CL_MOST: above it the vectors of the
-// columns side by side leave L2 (not measured)
-static asss_status cluster_plan(asss_handle* h, int nrhs, int* size) {
-    constexpr int CL_MOST = 300000;
-    const asss_options& o = h->opt;
-    *size = 0;
-    if (nrhs < 1 || h->n > CL_MOST || o.outer != ASSS_OUTER_FGMRES || o.restart > CL_RESTART || !h->use_dia ||
-        h->factored || h->Q16.p || h->kp > 32 || h->k + h->r > CL_MMAX ||
-        getenv("ASSS_TRACE"))   // which asks for the phases of the launch-by-launch path
-        return ASSS_OK;
-    if (h->cl_counts[0] < 0) {
-        if (o.precision == ASSS_PREC_MIXED) {
-            ClArgs<float> a = {};
-            a.restart = o.restart;
-            ASSS_TRY(cl_dispatch<float>(h->ctx, a, h->kp, 0, 0, h->cl_counts));
-        } else {
-            ClArgs<double> a = {};
-            a.restart = o.restart;
-            ASSS_TRY(cl_dispatch<double>(h->ctx, a, h->kp, 0, 0, h->cl_counts));
-        }
-    }
-    *size = cluster_size(h, nrhs);
-    return ASSS_OK;
-}
-
 static ClMat cl_mat(const DCsr& A) {
     ClMat m;
     m.ndiag = A.dia.ndiag;
@@ -2053,25 +2029,49 @@ static ClMat cl_mat(const DCsr& A) {
     return m;
 }
 
-// nc columns of a solve by clusters of `size` CTAs, x on the device; out: one entry per column
+// the kernel's view of the handle (everything but the columns)
 template <class T>
-static asss_status solve_cluster(asss_handle* h, int tr, int size, int nc, const double* b, int64_t ldb, double* x, int64_t ldx,
-                                 ClStat* out) {
-    NvtxRange nv_(tr ? "asss:adjoint-solve" : "asss:solve");
-    const Ctx& c = h->ctx;
-    cudaStream_t s = c.stream;
-    const asss_options& o = h->opt;
+static asss_status cluster_args(asss_handle* h, int tr, ClArgs<T>& a) {
     ASSS_TRY(ensure_smw(h, tr));
     if (tr) ASSS_TRY(ensure_adjoint_ops(h));
     const SmwData& S = h->smw[tr];
-    ClArgs<T> a;
-    memset(&a, 0, sizeof(a));
+    const asss_options& o = h->opt;
     a.n = h->n;
     a.restart = o.restart;
     a.k = h->k;
     a.m = S.m;
     a.r = h->r;
-    if constexpr (sizeof(T) == 4) {
+    if (h->factored) {
+        const IldlFactor& F = h->fac;
+        ClFactor<T>& f = a.fac;
+        f.ncol = F.ncol;
+        f.ls = F.ls.p;
+        f.lvl = F.lvl.p;
+        f.pos = F.pos.p;
+        f.wd = F.wd.p;
+        f.wo = F.wo.p;
+        f.part = F.npairs > 0 ? F.part.p : nullptr;
+        const IldlFactor::Ordered* M[3] = {&F.oL, &F.oU, &F.oJ};
+        ClRows<T>* R[3] = {&f.L, &f.U, &f.J};
+        for (int t = 0; t < 3; ++t) {
+            R[t]->rp = M[t]->rp.p;
+            R[t]->ci = M[t]->ci.p;
+            R[t]->d = M[t]->v.p;
+            if constexpr (sizeof(T) == 4) R[t]->v = M[t]->v32.p;
+            else R[t]->v = M[t]->v.p;
+        }
+        if constexpr (sizeof(T) == 4) {
+            f.wdT = F.wd32.p;
+            f.woT = F.wo32.p;
+            a.Q = h->Q32.p;
+            a.Ys = S.Y32.p;
+        } else {
+            f.wdT = F.wd.p;
+            f.woT = F.wo.p;
+            a.Q = h->Q64.p;
+            a.Ys = S.Y.p;
+        }
+    } else if constexpr (sizeof(T) == 4) {
         a.ndiag = h->D32.ndiag;
         a.halo = h->D32.halo;
         a.off = h->D32.off.p;
@@ -2108,6 +2108,47 @@ static asss_status solve_cluster(asss_handle* h, int tr, int size, int nc, const
     a.inner_tol = o.inner_tol;
     a.outer_maxit = o.outer_maxit;
     a.inner_maxit = o.inner_maxit;
+    return ASSS_OK;
+}
+
+// the cluster size of a call (0: launch by launch); CL_MOST: above it the vectors of the
+// columns side by side leave L2 (not measured)
+static asss_status cluster_plan(asss_handle* h, int nrhs, int* size) {
+    constexpr int CL_MOST = 300000;
+    const asss_options& o = h->opt;
+    *size = 0;
+    if (nrhs < 1 || h->n > CL_MOST || o.outer != ASSS_OUTER_FGMRES || o.restart > CL_RESTART ||
+        !(h->use_dia || (h->factored && h->fac.pos.p)) || h->Q16.p || h->kp > 32 || h->k + h->r > CL_MMAX ||
+        getenv("ASSS_TRACE"))   // which asks for the phases of the launch-by-launch path
+        return ASSS_OK;
+    if (h->cl_counts[0] < 0) {
+        if (o.precision == ASSS_PREC_MIXED) {
+            ClArgs<float> a = {};
+            ASSS_TRY(cluster_args<float>(h, 0, a));
+            if (h->factored) ASSS_TRY((cl_dispatch<float, 3>(h->ctx, a, h->kp, 0, 0, h->cl_counts)));
+            else ASSS_TRY((cl_dispatch<float, 1>(h->ctx, a, h->kp, 0, 0, h->cl_counts)));
+        } else {
+            ClArgs<double> a = {};
+            ASSS_TRY(cluster_args<double>(h, 0, a));
+            if (h->factored) ASSS_TRY((cl_dispatch<double, 3>(h->ctx, a, h->kp, 0, 0, h->cl_counts)));
+            else ASSS_TRY((cl_dispatch<double, 1>(h->ctx, a, h->kp, 0, 0, h->cl_counts)));
+        }
+    }
+    *size = cluster_size(h, nrhs);
+    return ASSS_OK;
+}
+
+// nc columns of a solve by clusters of `size` CTAs, x on the device; out: one entry per column
+template <class T>
+static asss_status solve_cluster(asss_handle* h, int tr, int size, int nc, const double* b, int64_t ldb, double* x, int64_t ldx,
+                                 ClStat* out) {
+    NvtxRange nv_(tr ? "asss:adjoint-solve" : "asss:solve");
+    const Ctx& c = h->ctx;
+    cudaStream_t s = c.stream;
+    const asss_options& o = h->opt;
+    ClArgs<T> a;
+    memset(&a, 0, sizeof(a));
+    ASSS_TRY(cluster_args<T>(h, tr, a));
     int count = 0;
     for (int t = 0; t < CL_NSIZES; ++t)
         if (CL_SIZES[t] == size) count = nc < h->cl_counts[t] ? nc : h->cl_counts[t];
@@ -2121,7 +2162,8 @@ static asss_status solve_cluster(asss_handle* h, int tr, int size, int nc, const
     if (h->cl_st.n < nc) ASSS_TRY(h->cl_st.alloc(nc));
     a.work = h->cl_work.p;
     a.stats = h->cl_st.p;
-    ASSS_TRY(cl_dispatch<T>(c, a, h->kp, size, count, nullptr));
+    if (h->factored) ASSS_TRY((cl_dispatch<T, 3>(c, a, h->kp, size, count, nullptr)));
+    else ASSS_TRY((cl_dispatch<T, 1>(c, a, h->kp, size, count, nullptr)));
     ASSS_CUDA(cudaMemcpyAsync(out, h->cl_st.p, sizeof(ClStat) * nc, cudaMemcpyDeviceToHost, s));
     return ASSS_OK;
 }
@@ -2145,6 +2187,13 @@ static void cluster_stats(const asss_handle* h, int tr, const ClStat& c, asss_st
     st->op_calls = c.op_calls;
     st->op_bytes = c.op_calls * (spmv_bytes(a) + spmv_bytes(b));
     st->op_flops = c.op_calls * (spmv_flops(a) + spmv_flops(b));
+    if (h->factored) {   // two triangular solves a product; t, w and the weights in an inner step
+        const long long tri = h->fac.nl + h->fac.nu;
+        st->inner_bytes = c.solves * n * (8 + 8 * T + qrow) +
+                          c.inner_its * ((tri + h->fac.nj) * (T + 4) + n * (12 * T + qrow));
+        st->op_bytes += c.op_calls * (tri * 12 + 48 * n);
+        st->op_flops += c.op_calls * (2 * tri + 2 * n);
+    }
     st->t_orth_ms = 1e-6 * (double)c.ns_orth;
     st->orth_calls = c.orth_calls;
     st->orth_bytes = 8 * n * (2 * c.orth_vecs + 5 * c.orth_calls);

@@ -37,6 +37,38 @@ __device__ __forceinline__ unsigned cl_count() {
 __device__ __forceinline__ void cl_sync() {
     asm volatile("barrier.cluster.arrive.release.aligned;\nbarrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
+// the two halves of cl_sync: work between them overlaps the barrier
+__device__ __forceinline__ void cl_arrive() {
+    __syncwarp();
+    asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+}
+__device__ __forceinline__ void cl_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
+// one value into the same shared variable of CTAs first, first + 4, ... (four lanes together
+// reach them all)
+__device__ __forceinline__ void cl_store_every4(float* var, unsigned first, unsigned n, float v) {
+    const unsigned a = (unsigned)__cvta_generic_to_shared(var);
+#pragma unroll
+    for (unsigned u = 0; u < CL_MAX / 4; ++u) {
+        const unsigned q = first + 4 * u;
+        if (q < n) {
+            unsigned ra;
+            asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(ra) : "r"(a), "r"(q));
+            asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(ra), "f"(v) : "memory");
+        }
+    }
+}
+__device__ __forceinline__ void cl_store_every4(double* var, unsigned first, unsigned n, double v) {
+    const unsigned a = (unsigned)__cvta_generic_to_shared(var);
+#pragma unroll
+    for (unsigned u = 0; u < CL_MAX / 4; ++u) {
+        const unsigned q = first + 4 * u;
+        if (q < n) {
+            unsigned ra;
+            asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(ra) : "r"(a), "r"(q));
+            asm volatile("st.shared::cluster.f64 [%0], %1;" ::"r"(ra), "d"(v) : "memory");
+        }
+    }
+}
 // 8 bytes into the same shared variable of CTA `rank`
 __device__ __forceinline__ void cl_store8(void* var, unsigned rank, unsigned long long bits) {
     unsigned a = (unsigned)__cvta_generic_to_shared(var), ra;

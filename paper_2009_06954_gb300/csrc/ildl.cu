@@ -807,6 +807,44 @@ asss_status ildl_build(const Ctx& c, const DCsr& P0, const int* mirror0, const d
     return ASSS_OK;
 }
 
+__global__ void k_level_pos(int n, const int* lvl, int* pos) {
+    const int e = blockIdx.x * blockDim.x + threadIdx.x;
+    if (e < n) pos[lvl[e]] = e;
+}
+__global__ void k_ordered_len(int n, const int* lvl, const int* rp, int* len) {
+    const int e = blockIdx.x * blockDim.x + threadIdx.x;
+    if (e < n) len[e] = rp[lvl[e] + 1] - rp[lvl[e]];
+}
+__global__ void k_ordered_fill(int n, const int* lvl, const int* pos, const int* rp, const int* ci, const double* v,
+                               const int* orp, int* oci, double* ov, float* ov32) {
+    const int e = blockIdx.x * blockDim.x + threadIdx.x;
+    if (e >= n) return;
+    int o = orp[e];
+    for (int q = rp[lvl[e]]; q < rp[lvl[e] + 1]; ++q, ++o) {
+        oci[o] = pos[ci[q]];
+        ov[o] = v[q];
+        if (ov32) ov32[o] = (float)v[q];
+    }
+}
+// rows and columns of a CSR matrix in (colour, index) order
+static asss_status order_rows(const IldlFactor& F, const int* rp, const int* ci, const double* v, int64_t nnz, bool fp32,
+                              IldlFactor::Ordered& out, cudaStream_t s) {
+    const int n = F.n;
+    DBuf<int> len;
+    ASSS_TRY(len.alloc(n));
+    k_ordered_len<<<cdiv(n, 256), 256, 0, s>>>(n, F.lvl.p, rp, len.p);
+    ASSS_CHECK_LAUNCH();
+    ASSS_TRY(out.rp.alloc(n + 1));
+    ASSS_TRY(exclusive_scan(len.p, out.rp.p, n, nullptr, s));
+    ASSS_TRY(out.ci.alloc(nnz > 0 ? nnz : 1));
+    ASSS_TRY(out.v.alloc(nnz > 0 ? nnz : 1));
+    if (fp32) ASSS_TRY(out.v32.alloc(nnz > 0 ? nnz : 1));
+    k_ordered_fill<<<cdiv(n, 256), 256, 0, s>>>(n, F.lvl.p, F.pos.p, rp, ci, v, out.rp.p, out.ci.p, out.v.p, out.v32.p);
+    ASSS_CHECK_LAUNCH();
+    ASSS_CUDA(cudaStreamSynchronize(s));   // len is freed here
+    return ASSS_OK;
+}
+
 asss_status ildl_set_skew(const Ctx& c, IldlFactor& F, const DCsr& Jh, bool fp32) {
     F.jrp = Jh.rp.p;
     F.jci = Jh.ci.p;
@@ -816,6 +854,14 @@ asss_status ildl_set_skew(const Ctx& c, IldlFactor& F, const DCsr& Jh, bool fp32
         ASSS_TRY(F.jv32.alloc(Jh.nnz > 0 ? Jh.nnz : 1));
         if (Jh.nnz) k_d2f_n<<<cdiv(Jh.nnz, 256), 256, 0, c.stream>>>(Jh.v.p, Jh.nnz, F.jv32.p);
         ASSS_CHECK_LAUNCH();
+    }
+    if (F.n > 0 && F.n <= ILDL_CLUSTER_MAX) {
+        ASSS_TRY(F.pos.alloc(F.n));
+        k_level_pos<<<cdiv(F.n, 256), 256, 0, c.stream>>>(F.n, F.lvl.p, F.pos.p);
+        ASSS_CHECK_LAUNCH();
+        ASSS_TRY(order_rows(F, F.lrp.p, F.lci.p, F.lv.p, F.nl, fp32, F.oL, c.stream));
+        ASSS_TRY(order_rows(F, F.urp.p, F.uci.p, F.uv.p, F.nu, fp32, F.oU, c.stream));
+        ASSS_TRY(order_rows(F, F.jrp, F.jci, F.jv, F.nj, fp32, F.oJ, c.stream));
     }
     return ASSS_OK;
 }

@@ -138,6 +138,7 @@ asss_status mrs_multi_solve_cols(const Ctx& c, const MrsOperator& op, bool fp32,
 // ildl.cu: no-fill incomplete L D L^T of M^ in a multicolour order (§3 after Eq.
 // absfac, §4.1 ~ildl(0)); original indexing, "lower" = of a smaller colour.
 constexpr int ILDL_MAXCOL = 256;
+constexpr int ILDL_CLUSTER_MAX = 20000;
 struct IldlFactor {
     int n = 0, ncol = 0, rounds = 0;
     int64_t nl = 0, nu = 0, nj = 0;
@@ -160,6 +161,16 @@ struct IldlFactor {
     DBuf<int> part;
     DBuf<double> doff, wo;
     DBuf<float> wo32;
+    // the same matrices with rows and columns in (colour, index) order, for the solves whose
+    // triangular sweeps run in shared memory (empty above ILDL_CLUSTER_MAX rows): position of
+    // each vertex, and L, U, J^ by position
+    struct Ordered {
+        DBuf<int> rp, ci;
+        DBuf<double> v;
+        DBuf<float> v32;
+    };
+    DBuf<int> pos;
+    Ordered oL, oU, oJ;
     int nur = 0;
     DBuf<int> ur_i1, ur_i2;
     DBuf<double> ur_c1, ur_c2;

@@ -13,6 +13,8 @@
 // 16 SMs' share of the bandwidth and of the FP64 pipe (the rule there has both sides measured).
 #pragma once
 
+#include <algorithm>
+
 #include "cluster_dev.cuh"
 #include "internal.h"
 #include "mrs_dev.cuh"
@@ -37,6 +39,25 @@ struct ClMat {
     const double* v;
 };
 
+// one triangle or J^ in (colour, index) order
+template <class T>
+struct ClRows {
+    const int *rp, *ci;
+    const T* v;         // in the precision of the inner solve
+    const double* d;    // FP64
+};
+// the incomplete factor (FMT 3): colours, their rows, L, U and J^ by position, the weights
+// |D|^-1/2 (wo: off-diagonals of the 2x2 pivots, part null without any)
+template <class T>
+struct ClFactor {
+    int ncol, own_max;   // own_max: the most rows of all colours that a CTA owns (cl_run)
+    const int *ls, *lvl, *pos;
+    ClRows<T> L, U, J;
+    const double *wd, *wo;
+    const T *wdT, *woT;
+    const int* part;
+};
+
 struct ClStat {
     int outer_its, cycles, status, solves, op_calls, orth_calls;
     long long inner_its, orth_vecs;
@@ -59,6 +80,7 @@ struct ClArgs {
     const double *negc1, *negc2;
     // op1 then op2: the outer operator; Sm and Am: update and residual (their transposes with tr)
     ClMat op1, op2, Sm, Am;
+    ClFactor<T> fac;          // FMT 3
     const double *dr, *dc, *w;
     const int* perm;
     int tr;
@@ -98,7 +120,82 @@ struct ClShared {
     int stop;
 };
 
-template <class T, int KP>
+// shared memory behind the Hessenberg matrix with FMT 3: the replicated vectors of the sweeps
+// (two in T, or one in FP64 in the same place), and per own row its value, vertex and the
+// row of L, U and J^; then the colours' first own row and first position
+template <class T>
+inline long long cl_factor_smem(int n, int own_max, int ncol) {
+    return std::max<long long>(2LL * n * (long long)sizeof(T), 8LL * n) + 8 + (long long)own_max * (8 + 4 + 3 * 8) +
+           4LL * (2 * ncol + 2);
+}
+
+// One triangular solve, colour by colour (back: from the last colour down): vec[e] =
+// own[row of e] - sum_q v_q vec[col_q], vec replicated in every CTA; own: this CTA's right-hand
+// side, in the order of its rows.  Four lanes share a row (an FP64 operation of a warp takes 64
+// cycles, however many of its lanes work) and its stores to the other CTAs; the entries
+// of the next two colours are on their way while a colour is solved.  Not inlined: its
+// registers would add to the solve's, at five places.
+template <class E>
+__device__ __noinline__ void cl_tri_sweep(E* vec, const E* own, const int2* rows, const int* __restrict__ ci,
+                                          const E* __restrict__ v, bool back, int ncol, const int* s_off,
+                                          const int* s_beg) {
+    constexpr int PF = 4;   // entries a lane fetches ahead
+    struct Slot {
+        int2 rw;
+        int cc[PF];
+        E vv[PF];
+    };
+    const int tid = threadIdx.x, sub = tid & 3;
+    const unsigned C = cl_size();
+    auto fetch = [&](int o, int end, Slot& S) {
+        S.rw = o < end ? rows[o] : make_int2(0, 0);
+#pragma unroll
+        for (int u = 0; u < PF; ++u) {
+            const int q = sub + 4 * u;
+            S.cc[u] = q < S.rw.y ? __ldg(ci + S.rw.x + q) : 0;
+            S.vv[u] = q < S.rw.y ? __ldg(v + S.rw.x + q) : (E)0;
+        }
+    };
+    auto fetch_phase = [&](int k, Slot& S) {
+        if (k >= ncol) return;
+        const int c = back ? ncol - 1 - k : k;
+        fetch(s_off[c] + (tid >> 2), s_off[c + 1], S);
+    };
+    auto phase = [&](int k, Slot& S) {
+        const int c = back ? ncol - 1 - k : k, o0 = s_off[c], o1 = s_off[c + 1];
+        for (int b0 = o0; b0 < o1; b0 += CL_THREADS / 4) {
+            const int o = b0 + (tid >> 2);
+            if (b0 > o0) fetch(o, o1, S);
+            E a = (E)0;
+#pragma unroll
+            for (int u = 0; u < PF; ++u)
+                if (sub + 4 * u < S.rw.y) a += S.vv[u] * vec[S.cc[u]];
+            for (int q = sub + 4 * PF; q < S.rw.y; q += 4) a += __ldg(v + S.rw.x + q) * vec[__ldg(ci + S.rw.x + q)];
+            a += __shfl_xor_sync(0xffffffffu, a, 1);
+            a += __shfl_xor_sync(0xffffffffu, a, 2);
+            if (o < o1) cl_store_every4(&vec[s_beg[c] + o - o0], sub, C, own[o] - a);
+        }
+        cl_arrive();
+        fetch_phase(k + 2, S);
+        cl_wait();
+    };
+    Slot A, B;
+    fetch_phase(0, A);
+    fetch_phase(1, B);
+    for (int k = 0; k < ncol; k += 2) {
+        phase(k, A);
+        if (k + 1 < ncol) phase(k + 1, B);
+    }
+}
+
+// FMT 1: skew diagonals; FMT 3: the incomplete factor, J~ = L~^-1 J^ L~^-T.  Its triangular
+// solves take one phase per colour (15 to 17 on the 3D stencil, twice per mrs step and twice per
+// outer product).  In the launch-by-launch path a phase is a grid barrier after a chain of
+// four dependent loads (6 us) or a launch; here a vector being solved for is replicated in the
+// shared memory of every CTA, a phase gathers from there, stores its few rows into all CTAs
+// and crosses one cluster barrier, with the next colours' entries already on their way: about
+// 1 us a phase (mrs steps at 10^3 32 us instead of 129, at 24^3 51 instead of 227).
+template <class T, int KP, int FMT>
 __global__ void __launch_bounds__(CL_THREADS, 1) k_solve_cl(const ClArgs<T> p) {
     constexpr int NT = CL_THREADS, NW = CL_WARPS, NV = KP + 1, KQ = KP > 0 ? KP : 1;
     using Sh = ClShared<T, KP>;
@@ -137,6 +234,44 @@ __global__ void __launch_bounds__(CL_THREADS, 1) k_solve_cl(const ClArgs<T> p) {
     for (int t = rank * NT + tid; t < 6 * p.halo; t += C * NT) {
         const int slot = t / (2 * p.halo), e = t % (2 * p.halo);
         Y[slot * ys + (e < p.halo ? e - p.halo : nn + (e - p.halo))] = (T)0;
+    }
+    // FMT 3: replicated vectors, own rows
+    const ClFactor<T>& fa = p.fac;
+    double* s_vecd = H + (size_t)(R + 1) * R;
+    T* s_t = reinterpret_cast<T*>(s_vecd);
+    T* s_f = s_t + n;
+    double* s_own = nullptr;
+    int2 *s_lq = nullptr, *s_uq = nullptr, *s_jq = nullptr;
+    int *s_lvl = nullptr, *s_off = nullptr, *s_beg = nullptr;
+    if constexpr (FMT == 3) {
+        const size_t vb = sizeof(T) == 8 ? 2 * (size_t)n : (size_t)n;   // in doubles
+        s_own = s_vecd + vb + (vb & 1);
+        s_lq = reinterpret_cast<int2*>(s_own + fa.own_max);
+        s_uq = s_lq + fa.own_max;
+        s_jq = s_uq + fa.own_max;
+        s_lvl = reinterpret_cast<int*>(s_jq + fa.own_max);
+        s_off = s_lvl + fa.own_max;
+        s_beg = s_off + fa.ncol + 1;
+        if (tid == 0) {
+            int o = 0;
+            for (int c = 0; c < fa.ncol; ++c) {
+                const int l0 = fa.ls[c], cnt = fa.ls[c + 1] - l0;
+                const int b0 = (int)((long long)cnt * rank / C), b1 = (int)((long long)cnt * (rank + 1) / C);
+                s_off[c] = o;
+                s_beg[c] = l0 + b0;
+                o += b1 - b0;
+            }
+            s_off[fa.ncol] = o;
+        }
+        __syncthreads();
+        for (int c = 0; c < fa.ncol; ++c)
+            for (int o = s_off[c] + tid; o < s_off[c + 1]; o += NT) {
+                const int e = s_beg[c] + o - s_off[c];
+                s_lvl[o] = fa.lvl[e];
+                s_lq[o] = make_int2(fa.L.rp[e], fa.L.rp[e + 1] - fa.L.rp[e]);
+                s_uq[o] = make_int2(fa.U.rp[e], fa.U.rp[e + 1] - fa.U.rp[e]);
+                s_jq[o] = make_int2(fa.J.rp[e], fa.J.rp[e + 1] - fa.J.rp[e]);
+            }
     }
     cl_sync();   // every CTA of the cluster runs: its shared memory may be written
 
@@ -220,6 +355,61 @@ __global__ void __launch_bounds__(CL_THREADS, 1) k_solve_cl(const ClArgs<T> p) {
             }
         }
         return s;
+    };
+
+    // out = |D|^-1/2 (I + L)^-1 a, own rows; a complete in L2
+    auto apply_F = [&](const double* a, double* out) {
+        for (int o = tid; o < s_off[fa.ncol]; o += NT) s_own[o] = a[s_lvl[o]];
+        __syncthreads();
+        cl_tri_sweep<double>(s_vecd, s_own, s_lq, fa.L.ci, fa.L.d, false, fa.ncol, s_off, s_beg);
+        for (int i = rb + tid; i < re; i += NT) {
+            double v = fa.wd[i] * s_vecd[fa.pos[i]];
+            if (fa.part && fa.part[i] >= 0) v += fa.wo[i] * s_vecd[fa.pos[fa.part[i]]];
+            out[i] = v;
+        }
+    };
+    // out = (I + L)^-T |D|^-1/2 a, own rows; a complete in L2
+    auto apply_G = [&](const double* a, double* out) {
+        for (int o = tid; o < s_off[fa.ncol]; o += NT) {
+            const int i = s_lvl[o];
+            double v = fa.wd[i] * a[i];
+            if (fa.part && fa.part[i] >= 0) v += fa.wo[i] * a[fa.part[i]];
+            s_own[o] = v;
+        }
+        __syncthreads();
+        cl_tri_sweep<double>(s_vecd, s_own, s_uq, fa.U.ci, fa.U.d, true, fa.ncol, s_off, s_beg);
+        for (int i = rb + tid; i < re; i += NT) out[i] = s_vecd[fa.pos[i]];
+    };
+    // s_f = (I + L)^-1 J^ (I + L)^-T (wd .* y) by position, y complete in L2
+    auto apply_skew = [&](const T* y) {
+        T* own = reinterpret_cast<T*>(s_own);
+        for (int o = tid; o < s_off[fa.ncol]; o += NT) {
+            const int i = s_lvl[o];
+            T v = __ldg(&fa.wdT[i]) * y[i];
+            if (fa.part && __ldg(&fa.part[i]) >= 0) v += __ldg(&fa.woT[i]) * y[__ldg(&fa.part[i])];
+            own[o] = v;
+        }
+        __syncthreads();
+        cl_tri_sweep<T>(s_t, own, s_uq, fa.U.ci, fa.U.v, true, fa.ncol, s_off, s_beg);
+        for (int o = tid; o < s_off[fa.ncol]; o += NT) {
+            const int2 rw = s_jq[o];
+            T a = (T)0;
+            for (int q = 0; q < rw.y; q += 12) {
+                int cc[12];
+                T vv[12];
+#pragma unroll
+                for (int u = 0; u < 12; ++u) {
+                    cc[u] = q + u < rw.y ? __ldg(fa.J.ci + rw.x + q + u) : 0;
+                    vv[u] = q + u < rw.y ? __ldg(fa.J.v + rw.x + q + u) : (T)0;
+                }
+#pragma unroll
+                for (int u = 0; u < 12; ++u)
+                    if (q + u < rw.y) a += vv[u] * s_t[cc[u]];
+            }
+            own[o] = a;
+        }
+        __syncthreads();
+        cl_tri_sweep<T>(s_f, own, s_lq, fa.L.ci, fa.L.v, false, fa.ncol, s_off, s_beg);
     };
 
     // ---------------------------------------------------------------------------
@@ -356,14 +546,20 @@ __global__ void __launch_bounds__(CL_THREADS, 1) k_solve_cl(const ClArgs<T> p) {
                     txp = sh.cf[6];
 #pragma unroll
             for (int v = 0; v < NV; ++v) tacc[v] = (T)0;
+            if constexpr (FMT == 3) apply_skew(Ycur);
             for (int i = rb + tid; i < re; i += NT) {
                 const T yold = j >= 2 ? Yold[i] : (T)0;
                 const T pold = j >= 2 ? Pj1[i] : (T)0;
                 T acc = (T)0;
+                if constexpr (FMT == 3) {
+                    acc = __ldg(&fa.wdT[i]) * s_f[__ldg(&fa.pos[i])];
+                    if (fa.part && __ldg(&fa.part[i]) >= 0)
+                        acc += __ldg(&fa.woT[i]) * s_f[__ldg(&fa.pos[__ldg(&fa.part[i])])];
+                }
                 const T* Ud = p.U + i;
                 const T* yi = Ycur + i;
 #pragma unroll 12
-                for (int d = 0; d < p.ndiag; ++d, Ud += p.ustride) {
+                for (int d = 0; d < (FMT == 1 ? p.ndiag : 0); ++d, Ud += p.ustride) {
                     const int mo = sh.off[d];
                     if constexpr (sizeof(T) == 8) {
                         acc = fma(__ldg(Ud), yi[mo], acc);
@@ -536,15 +732,21 @@ __global__ void __launch_bounds__(CL_THREADS, 1) k_solve_cl(const ClArgs<T> p) {
                 break;
             }
             // r^ = W P D_r r, or W S^T D_c r (the barrier of the last norm published r)
+            // (FMT 3: F P D_r r or F S^T D_c r, W = 1 there)
+            double* rs = FMT == 3 ? t2 : rh;
             if (!p.tr) {
                 for (int i = rb + tid; i < re; i += NT) {
                     const int q = p.perm ? p.perm[i] : i;
-                    rh[i] = p.w[i] * p.dr[q] * r[q];
+                    rs[i] = p.w[i] * p.dr[q] * r[q];
                 }
             } else {
                 for (int i = rb + tid; i < re; i += NT) t1[i] = p.dc[i] * r[i];
                 cl_sync();
-                for (int i = rb + tid; i < re; i += NT) rh[i] = p.w[i] * mat_row(p.Sm, sh.moff[2], t1, i);
+                for (int i = rb + tid; i < re; i += NT) rs[i] = p.w[i] * mat_row(p.Sm, sh.moff[2], t1, i);
+            }
+            if constexpr (FMT == 3) {
+                cl_sync();
+                apply_F(rs, rh);
             }
             const double eta = fmin(0.5, 0.5 * p.outer_tol * bn / rn);
             const int mcyc = min(R, p.outer_maxit - outer);
@@ -596,9 +798,19 @@ __global__ void __launch_bounds__(CL_THREADS, 1) k_solve_cl(const ClArgs<T> p) {
                     // w = A_cal z_j
                     cl_sync();
                     const unsigned long long tm2 = now();
-                    for (int i = rb + tid; i < re; i += NT) t1[i] = mat_row(p.op1, sh.moff[0], zj, i);
+                    if constexpr (FMT == 3) {   // F A^ G z_j
+                        apply_G(zj, t2);
+                        cl_sync();
+                    }
+                    const double* zin = FMT == 3 ? t2 : zj;
+                    for (int i = rb + tid; i < re; i += NT) t1[i] = mat_row(p.op1, sh.moff[0], zin, i);
                     cl_sync();
-                    for (int i = rb + tid; i < re; i += NT) wv[i] = mat_row(p.op2, sh.moff[1], t1, i);
+                    double* wout = FMT == 3 ? t2 : wv;
+                    for (int i = rb + tid; i < re; i += NT) wout[i] = mat_row(p.op2, sh.moff[1], t1, i);
+                    if constexpr (FMT == 3) {
+                        cl_sync();
+                        apply_F(t2, wv);
+                    }
                     const unsigned long long tm3 = now();
                     ++ops;
                     // two classical Gram-Schmidt passes; ||w2||^2 = ||w1||^2 - ||h2||^2
@@ -734,7 +946,9 @@ __global__ void __launch_bounds__(CL_THREADS, 1) k_solve_cl(const ClArgs<T> p) {
                     for (int u = 0; u < 8; ++u)
                         if (a + u < steps) dy += ld[u] * sh.yv[a + u];
                 }
-                if (!p.tr) {
+                if (FMT == 3) {
+                    t2[i] = dy;
+                } else if (!p.tr) {
                     t1[i] = p.w[i] * dy;
                 } else {
                     const int q = p.perm ? p.perm[i] : i;
@@ -742,6 +956,15 @@ __global__ void __launch_bounds__(CL_THREADS, 1) k_solve_cl(const ClArgs<T> p) {
                 }
             }
             cl_sync();
+            if constexpr (FMT == 3) {   // G dy instead of W dy
+                apply_G(t2, t1);
+                if (p.tr)
+                    for (int i = rb + tid; i < re; i += NT) {
+                        const int q = p.perm ? p.perm[i] : i;
+                        x[q] += p.dr[q] * t1[i];
+                    }
+                cl_sync();
+            }
             if (!p.tr) {
                 for (int i = rb + tid; i < re; i += NT) x[i] += p.dc[i] * mat_row(p.Sm, sh.moff[2], t1, i);
                 cl_sync();
@@ -775,9 +998,9 @@ __global__ void __launch_bounds__(CL_THREADS, 1) k_solve_cl(const ClArgs<T> p) {
 // host side
 // ---------------------------------------------------------------------------
 // clusters of `size` CTAs that can be resident at once (0: none fits)
-template <class T, int KP>
+template <class T, int KP, int FMT>
 static asss_status cl_clusters(int size, size_t smem, int* count) {
-    const void* fn = (const void*)k_solve_cl<T, KP>;
+    const void* fn = (const void*)k_solve_cl<T, KP, FMT>;
     ASSS_TRY(raise_dynamic_smem(fn, (int)smem));
     if (size > 8) ASSS_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
     cudaLaunchConfig_t cfg = {};
@@ -799,14 +1022,27 @@ static asss_status cl_clusters(int size, size_t smem, int* count) {
 
 // launches `count` clusters of `size` CTAs, or (size == 0) asks how many clusters of each of
 // CL_SIZES can be resident, into counts
-template <class T, int KP>
+template <class T, int KP, int FMT>
 static asss_status cl_run(const Ctx& c, const ClArgs<T>& a, int size, int count, int* counts) {
-    const size_t smem = ((sizeof(ClShared<T, KP>) + 15) & ~(size_t)15) +
-                        sizeof(double) * (size_t)(a.restart + 1) * (size_t)a.restart;
+    ClArgs<T> b = a;
+    auto bytes = [&](int sz) -> size_t {
+        size_t smem = ((sizeof(ClShared<T, KP>) + 15) & ~(size_t)15) +
+                      sizeof(double) * (size_t)(a.restart + 1) * (size_t)a.restart;
+        if (FMT == 3) {
+            b.fac.own_max = a.n / sz + a.fac.ncol + 1;
+            smem += (size_t)cl_factor_smem<T>(a.n, b.fac.own_max, a.fac.ncol);
+        }
+        return smem;
+    };
     if (size == 0) {
-        for (int t = 0; t < CL_NSIZES; ++t) ASSS_TRY((cl_clusters<T, KP>(CL_SIZES[t], smem, &counts[t])));
+        for (int t = 0; t < CL_NSIZES; ++t) {
+            const size_t need = bytes(CL_SIZES[t]);
+            counts[t] = 0;
+            if (need <= 227 * 1024) ASSS_TRY((cl_clusters<T, KP, FMT>(CL_SIZES[t], need, &counts[t])));
+        }
         return ASSS_OK;
     }
+    const size_t smem = bytes(size);
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(size * count);
     cfg.blockDim = dim3(CL_THREADS);
@@ -818,17 +1054,17 @@ static asss_status cl_run(const Ctx& c, const ClArgs<T>& a, int size, int count,
     at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
     cfg.attrs = at;
     cfg.numAttrs = 1;
-    ASSS_CUDA(cudaLaunchKernelEx(&cfg, k_solve_cl<T, KP>, a));
+    ASSS_CUDA(cudaLaunchKernelEx(&cfg, k_solve_cl<T, KP, FMT>, b));
     count_launch();
     return ASSS_OK;
 }
 
-template <class T>
+template <class T, int FMT>
 asss_status cl_dispatch(const Ctx& c, const ClArgs<T>& a, int kp, int size, int count, int* counts) {
     switch (kp) {
 #define ASSS_CL_CASE(KPV) \
     case KPV:             \
-        return cl_run<T, KPV>(c, a, size, count, counts);
+        return cl_run<T, KPV, FMT>(c, a, size, count, counts);
         ASSS_CL_CASE(0)
         ASSS_CL_CASE(4)
         ASSS_CL_CASE(8)
@@ -844,7 +1080,10 @@ asss_status cl_dispatch(const Ctx& c, const ClArgs<T>& a, int kp, int size, int 
     }
 }
 
-extern template asss_status cl_dispatch<float>(const Ctx&, const ClArgs<float>&, int, int, int, int*);
-extern template asss_status cl_dispatch<double>(const Ctx&, const ClArgs<double>&, int, int, int, int*);
+// (solve_cluster32.cu, solve_cluster64.cu, solve_cluster_fac32.cu, solve_cluster_fac64.cu)
+extern template asss_status cl_dispatch<float, 1>(const Ctx&, const ClArgs<float>&, int, int, int, int*);
+extern template asss_status cl_dispatch<double, 1>(const Ctx&, const ClArgs<double>&, int, int, int, int*);
+extern template asss_status cl_dispatch<float, 3>(const Ctx&, const ClArgs<float>&, int, int, int, int*);
+extern template asss_status cl_dispatch<double, 3>(const Ctx&, const ClArgs<double>&, int, int, int, int*);
 
 }  // namespace asss

@@ -1,8 +1,8 @@
-// Instantiations of the cluster-scope solve (solve_cluster.cuh): inner solves in FP32.
+// Instantiations of the cluster-scope solve (solve_cluster.cuh): skew diagonals, inner solves in FP32.
 #include "solve_cluster.cuh"
 
 namespace asss {
 
-template asss_status cl_dispatch<float>(const Ctx&, const ClArgs<float>&, int, int, int, int*);
+template asss_status cl_dispatch<float, 1>(const Ctx&, const ClArgs<float>&, int, int, int, int*);
 
 }  // namespace asss

@@ -1,8 +1,8 @@
-// Instantiations of the cluster-scope solve (solve_cluster.cuh): inner solves in FP64.
+// Instantiations of the cluster-scope solve (solve_cluster.cuh): skew diagonals, inner solves in FP64.
 #include "solve_cluster.cuh"
 
 namespace asss {
 
-template asss_status cl_dispatch<double>(const Ctx&, const ClArgs<double>&, int, int, int, int*);
+template asss_status cl_dispatch<double, 1>(const Ctx&, const ClArgs<double>&, int, int, int, int*);
 
 }  // namespace asss

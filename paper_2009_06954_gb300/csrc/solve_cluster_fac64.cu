@@ -1,0 +1,8 @@
+// Instantiations of the cluster-scope solve (solve_cluster.cuh): the incomplete factor, inner solves in FP64.
+#include "solve_cluster.cuh"
+
+namespace asss {
+
+template asss_status cl_dispatch<double, 3>(const Ctx&, const ClArgs<double>&, int, int, int, int*);
+
+}  // namespace asss

@@ -128,3 +128,34 @@ def test_early_ends_match(pkg, monkeypatch, what):  # noqa: F811
         np.testing.assert_array_equal(xa, xb)
     else:
         close(xa, xb)
+
+
+@pytest.mark.parametrize("precision", ["mixed", "fp64"])
+@pytest.mark.parametrize("case", ["dh3", "dh11", "dh20", "pairs", "general"])
+def test_incomplete_factor_matches(pkg, monkeypatch, case, precision):  # noqa: F811
+    """Triangular sweeps in shared memory: fewer rows than CTAs, colours with more rows than a
+    CTA has threads, 2x2 pivots with U_r columns of two entries, rows longer than the
+    entries fetched ahead."""
+    from workloads import random_powerlaw, saddle_pairs
+    opts = dict(OPTS[precision], factor="ildl0")
+    if case.startswith("dh"):
+        A = dissipative_hamiltonian_3d(side=int(case[2:]), seed=4, with_rhs=False)[0]
+    elif case == "pairs":
+        A = saddle_pairs(300, seed=5, singles=40)
+        n = A.shape[0]
+        opts.update(factor="ildl0_bk", s_pattern=sp.identity(n, format="csr"), s_values=np.ones(n), lls_maxit=0,
+                    inner_tol=1e-8, r_max=256)
+    else:
+        A = random_powerlaw(n=400, lmin=4, lmax=60, band=50, dom_frac=1.0, seed=6)[0]
+        opts.update(s_pattern=pattern_diagonal(400), lls_maxit=50)
+    n = A.shape[0]
+    s = pkg.Solver(A, k=min(20, n), **opts)
+    rng = np.random.default_rng(8)
+    X = rng.standard_normal((n, 2))
+    B = np.asfortranarray(A @ X)
+    (xa, sa), (xb, sb) = both(monkeypatch, lambda: s.solve(B))
+    close(xa, xb)
+    assert [sa[k] for k in SAME] == [sb[k] for k in SAME] and sa["status"] == 0
+    g = rng.standard_normal(n)
+    (la, _, _), (lb, _, _) = both(monkeypatch, lambda: s.solve_adjoint(g))
+    close(la, lb)
