@@ -115,23 +115,27 @@ __global__ void k_lls_BT(int nS, const int* __restrict__ srow, const int* __rest
 }
 
 // ---------------------------------------------------------------------------
-// B and B^T stored explicitly (when they fit a memory budget): the entries each merge
-// above would visit, in the same order, so the products are bit for bit those of the
-// merge kernels while each iteration streams two sparse matrices instead of redoing
-// the intersections.  B row k: the C_ij terms (unknown, abar_il) then - off the
-// diagonal - the C_ji terms from position bsplit[k]; B^T row u: (P position, abar_lj),
-// a position stored as ~pos where the diagonal weight sqrt(gamma) applies.
+// B and B^T stored explicitly (when they fit a memory budget) in SELL slices of 32 rows: the
+// entries each merge above would visit, in the same order, so an iteration streams two
+// sparse matrices instead of redoing the intersections.
+//   B: one row per constraint (the upper and diagonal entries of P; the lower ones are left
+//   out), in slots sorted by length within windows; the weight sqrt(gamma) of the diagonal
+//   constraints is in the values.
+//   B^T: one row per unknown, the two unknowns of a preconditioner pair in neighbouring slots
+//   (2t, 2t + 1), so that the lane next door holds the partner's residual.
+// All vectors of the iteration stand in these slot orders.
 // ---------------------------------------------------------------------------
+// entries of the intersection: count (oc == nullptr) or fill with stride 32, columns through map
 __device__ __forceinline__ int merge_list(const int* __restrict__ ac, const double* __restrict__ av, int alen,
                                           const int* __restrict__ bc, const int* __restrict__ bu, int blen,
-                                          int* oc, double* ov) {
+                                          const int* __restrict__ map, double f, int* oc, double* ov) {
     int x = 0, y = 0, k = 0;
     while (x < alen && y < blen) {
         int ca = ac[x], cb = bc[y];
         if (ca == cb) {
             if (oc) {
-                oc[k] = bu[y];
-                ov[k] = av[x];
+                oc[k * 32] = map[bu[y]];
+                ov[k * 32] = f * av[x];
             }
             ++k;
             ++x;
@@ -145,78 +149,99 @@ __device__ __forceinline__ int merge_list(const int* __restrict__ ac, const doub
     return k;
 }
 
-// count (bcol == nullptr) or fill row k of B
-__global__ void k_bx_rows(int nP, const int* __restrict__ prow, const int* __restrict__ pci,
-                          const int* __restrict__ arp, const int* __restrict__ aci, const double* __restrict__ av,
-                          const int* __restrict__ strp, const int* __restrict__ stci, const int* __restrict__ stsrc,
-                          const int* brp, int* bcnt, int* bsplit, int* bcol, double* bval) {
-    int k = blockIdx.x * blockDim.x + threadIdx.x;
-    if (k >= nP) return;
-    int i = prow[k], j = pci[k];
-    if (j < i) {
-        if (!bcol) bcnt[k] = 0;
-        else bsplit[k] = 0;
-        return;
-    }
-    int* oc = bcol ? bcol + brp[k] : nullptr;
-    double* ov = bcol ? bval + brp[k] : nullptr;
-    int a = merge_list(aci + arp[i], av + arp[i], arp[i + 1] - arp[i], stci + strp[j], stsrc + strp[j],
-                       strp[j + 1] - strp[j], oc, ov);
-    int b = 0;
-    if (j != i)
-        b = merge_list(aci + arp[j], av + arp[j], arp[j + 1] - arp[j], stci + strp[i], stsrc + strp[i],
-                       strp[i + 1] - strp[i], oc ? oc + a : nullptr, ov ? ov + a : nullptr);
-    if (!bcol) bcnt[k] = a + b;
-    else bsplit[k] = a;
-}
-
-// q = B s, summed as the merge kernel does: C_ij and C_ji separately, then added
-__global__ void k_bx_apply(int nP, const int* __restrict__ prow, const int* __restrict__ pci,
-                           const int* __restrict__ brp, const int* __restrict__ bsplit,
-                           const int* __restrict__ bcol, const double* __restrict__ bval,
-                           const double* __restrict__ s, double sg, double* q) {
+// entries of each row of B (0 for the lower entries of P) and the constraint flags
+__global__ void k_bx_count(int nP, const int* __restrict__ prow, const int* __restrict__ pci,
+                           const int* __restrict__ arp, const int* __restrict__ aci, const double* __restrict__ av,
+                           const int* __restrict__ strp, const int* __restrict__ stci, const int* __restrict__ stsrc,
+                           int* bcnt, int* flag) {
     int k = blockIdx.x * blockDim.x + threadIdx.x;
     if (k >= nP) return;
     const int i = prow[k], j = pci[k];
-    if (j < i) {
-        q[k] = 0.0;
-        return;
+    int c = 0;
+    if (j >= i) {
+        c = merge_list(aci + arp[i], av + arp[i], arp[i + 1] - arp[i], stci + strp[j], stsrc + strp[j],
+                       strp[j + 1] - strp[j], nullptr, 1.0, nullptr, nullptr);
+        if (j != i)
+            c += merge_list(aci + arp[j], av + arp[j], arp[j + 1] - arp[j], stci + strp[i], stsrc + strp[i],
+                            strp[i + 1] - strp[i], nullptr, 1.0, nullptr, nullptr);
     }
-    const int e0 = brp[k], e1 = brp[k + 1], em = e0 + bsplit[k];
-    double cij = 0.0;
-    for (int e = e0; e < em; ++e) cij += bval[e] * s[bcol[e]];
-    if (j == i) {
-        q[k] = sg * cij;
-        return;
+    bcnt[k] = c;
+    flag[k] = j >= i ? 1 : 0;
+}
+// constraint c is entry klist[c] of P, with len[c] entries
+__global__ void k_bx_list(int nP, const int* flag, const int* cidx, const int* bcnt, int* klist, int* len) {
+    int k = blockIdx.x * blockDim.x + threadIdx.x;
+    if (k >= nP || !flag[k]) return;
+    klist[cidx[k]] = k;
+    len[cidx[k]] = bcnt[k];
+}
+// a slot's row of B and its start value of rho (the right-hand side v)
+__global__ void k_bx_fill(int nslots, int nC, const int* __restrict__ rowmap, const int* __restrict__ klist,
+                          const int* __restrict__ prow, const int* __restrict__ pci, const int* __restrict__ arp,
+                          const int* __restrict__ aci, const double* __restrict__ av, const int* __restrict__ strp,
+                          const int* __restrict__ stci, const int* __restrict__ stsrc, const int* __restrict__ upos,
+                          double sg, const int* __restrict__ sptr, int* col, double* val, double* rho) {
+    const int slot = blockIdx.x * blockDim.x + threadIdx.x;
+    if (slot >= nslots) return;
+    const int c = rowmap ? rowmap[slot] : slot;
+    const int b = sptr[slot >> 5], width = (sptr[(slot >> 5) + 1] - b) >> 5;
+    int* oc = col + b + (slot & 31);
+    double* ov = val + b + (slot & 31);
+    int m = 0;
+    double r = 0.0;
+    if (c < nC) {
+        const int k = klist[c], i = prow[k], j = pci[k];
+        m = merge_list(aci + arp[i], av + arp[i], arp[i + 1] - arp[i], stci + strp[j], stsrc + strp[j],
+                       strp[j + 1] - strp[j], upos, j == i ? sg : 1.0, oc, ov);
+        if (j != i)
+            m += merge_list(aci + arp[j], av + arp[j], arp[j + 1] - arp[j], stci + strp[i], stsrc + strp[i],
+                            strp[i + 1] - strp[i], upos, 1.0, oc + m * 32, ov + m * 32);
+        r = j == i ? sg : 0.0;
     }
-    double cji = 0.0;
-    for (int e = em; e < e1; ++e) cji += bval[e] * s[bcol[e]];
-    q[k] = cij + cji;
+    for (; m < width; ++m) {
+        oc[m * 32] = 0;
+        ov[m * 32] = 0.0;
+    }
+    rho[slot] = r;
 }
 
-// count (tcol == nullptr) or fill row u of B^T (same walk as k_lls_BT)
-__global__ void k_btx_rows(int nS, const int* __restrict__ srow, const int* __restrict__ sci,
-                           const int* __restrict__ atrp, const int* __restrict__ atci, const double* __restrict__ atv,
-                           const int* __restrict__ prp, const int* __restrict__ pci, const int* __restrict__ mirror,
-                           const int* trp, int* tcnt, int* tcol, double* tval) {
+// pairs first (slots 2t, 2t + 1), then the unknowns without a partner
+__global__ void k_pair_flags(int nS, const int* partner, int* lead, int* single) {
     int u = blockIdx.x * blockDim.x + threadIdx.x;
     if (u >= nS) return;
-    int l = srow[u], j = sci[u];
+    const int p = partner[u];
+    lead[u] = p > u ? 1 : 0;
+    single[u] = p < 0 ? 1 : 0;
+}
+__global__ void k_pair_slots(int nS, const int* partner, const int* lpos, const int* spos, int npairs, int* upos,
+                             int* uslot) {
+    int u = blockIdx.x * blockDim.x + threadIdx.x;
+    if (u >= nS) return;
+    const int p = partner[u];
+    const int slot = p < 0 ? 2 * npairs + spos[u] : p > u ? 2 * lpos[u] : 2 * lpos[p] + 1;
+    upos[u] = slot;
+    uslot[slot] = u;
+}
+// walk of row u of B^T (as k_lls_BT): count, or fill with columns in constraint slots
+__device__ __forceinline__ int btx_row(int u, const int* __restrict__ srow, const int* __restrict__ sci,
+                                       const int* __restrict__ atrp, const int* __restrict__ atci,
+                                       const double* __restrict__ atv, const int* __restrict__ prp,
+                                       const int* __restrict__ pci, const int* __restrict__ mirror,
+                                       const int* __restrict__ cidx, const int* __restrict__ cpos, double sg, int* oc,
+                                       double* ov) {
+    const int l = srow[u], j = sci[u];
     int x = atrp[l], xe = atrp[l + 1];
     int y = prp[j], ye = prp[j + 1];
-    int o = tcol ? trp[u] : 0;
     int k = 0;
     while (x < xe && y < ye) {
-        int ia = atci[x], ib = pci[y];
+        const int ia = atci[x], ib = pci[y];
         if (ia == ib) {
-            int pos;
-            if (ia > j) pos = y;
-            else if (ia < j) pos = mirror[y] >= 0 ? mirror[y] : -1;   // none: a zero term, left out
-            else pos = ~y;                                           // the diagonal: weight sqrt(gamma)
-            if (ia == j || pos >= 0) {
-                if (tcol) {
-                    tcol[o + k] = pos;
-                    tval[o + k] = atv[x];
+            const int pos = ia >= j ? y : mirror[y];   // no mirror: a zero term, left out
+            if (pos >= 0) {
+                if (oc) {
+                    const int c = cidx[pos];
+                    oc[k * 32] = cpos ? cpos[c] : c;
+                    ov[k * 32] = ia == j ? sg * atv[x] : atv[x];
                 }
                 ++k;
             }
@@ -228,20 +253,198 @@ __global__ void k_btx_rows(int nS, const int* __restrict__ srow, const int* __re
             ++y;
         }
     }
-    if (!tcol) tcnt[u] = k;
+    return k;
+}
+__global__ void k_btx_count(int nslots, const int* __restrict__ uslot, const int* srow, const int* sci, const int* atrp,
+                            const int* atci, const double* atv, const int* prp, const int* pci, const int* mirror,
+                            int* len) {
+    const int t = blockIdx.x * blockDim.x + threadIdx.x;
+    if (t >= nslots) return;
+    const int u = uslot[t];
+    len[t] = u < 0 ? 0 : btx_row(u, srow, sci, atrp, atci, atv, prp, pci, mirror, nullptr, nullptr, 1.0, nullptr, nullptr);
+}
+// a slot's row of B^T, its start value of s and the two coefficients of its preconditioner
+// block: z = m1 r + m2 r(partner)
+__global__ void k_btx_fill(int nslots, const int* __restrict__ uslot, const int* srow, const int* sci, const int* atrp,
+                           const int* atci, const double* atv, const int* prp, const int* pci, const int* mirror,
+                           const int* cidx, const int* cpos, double sg, const int* sptr, int* col, double* val,
+                           const double* N, const int* partner, const double* cross, const double* s0, double* m1,
+                           double* m2, double* s) {
+    const int t = blockIdx.x * blockDim.x + threadIdx.x;
+    if (t >= nslots) return;
+    const int u = uslot[t];
+    const int b = sptr[t >> 5], width = (sptr[(t >> 5) + 1] - b) >> 5;
+    int* oc = col + b + (t & 31);
+    double* ov = val + b + (t & 31);
+    int m = 0;
+    double c1 = 0.0, c2 = 0.0, sv = 0.0;
+    if (u >= 0) {
+        m = btx_row(u, srow, sci, atrp, atci, atv, prp, pci, mirror, cidx, cpos, sg, oc, ov);
+        const double nu = N[u];
+        const int p = partner[u];
+        if (nu > 0.0) {
+            c1 = 1.0 / nu;
+            if (p >= 0) {
+                const double np = N[p], c = cross[u], det = nu * np - c * c;
+                if (det > 1e-12 * nu * np) {
+                    c1 = np / det;
+                    c2 = -c / det;
+                }
+            }
+        }
+        if (s0) sv = s0[u];
+    }
+    for (; m < width; ++m) {
+        oc[m * 32] = 0;
+        ov[m * 32] = 0.0;
+    }
+    m1[t] = c1;
+    m2[t] = c2;
+    s[t] = sv;
+}
+__global__ void k_unslot(int nS, const int* upos, const double* s, double* s_val) {
+    int u = blockIdx.x * blockDim.x + threadIdx.x;
+    if (u < nS) s_val[u] = s[upos[u]];
 }
 
-__global__ void k_btx_apply(int nS, const int* __restrict__ trp, const int* __restrict__ tcol,
-                            const double* __restrict__ tval, const double* __restrict__ t, double sg, double* g) {
-    int u = blockIdx.x * blockDim.x + threadIdx.x;
-    if (u >= nS) return;
-    double acc = 0.0;
-    for (int e = trp[u]; e < trp[u + 1]; ++e) {
-        const int c = tcol[e];
-        const double G = c >= 0 ? t[c] : sg * t[~c];
-        acc += tval[e] * G;
+// ---------------------------------------------------------------------------
+// the whole PCG in one cooperative launch.  An iteration was eight launches with rows of three
+// to seven entries read one thread a row (85 us at n = 32^3, where its data, all in L2, need
+// about 10); here it is four phases between grid barriers, a warp a slice:
+//   q = B p, ||q||^2 | rho -= a q, s += a p | r = B^T rho, z = M^-1 r, r.z, ||r||^2 | p = z + b p
+// r is not stored (z and the two sums are all that is needed of it).  Bound: the FP64 pipe and
+// L2 / HBM reads of the entries (12 bytes each).  An iteration at 10^3: 38 -> 7 us, at 32^3: 85 ->
+// 25 us, at 64^3: 437 -> 111 us.  Two blocks of 64 registers a thread: one of 117 took 23 us at
+// 32^3 but 165 us at 64^3, where the reads come from HBM and want more warps.
+// ---------------------------------------------------------------------------
+constexpr int PCG_THREADS = 512;
+struct PcgParams {
+    int nb, nt;                       // slices of B and B^T
+    const int *bsp, *bcol, *tsp, *tcol;
+    const double *bval, *tval, *m1, *m2;
+    double *q, *rho, *p, *z, *s;      // 32 nb, 32 nb, 32 nt, 32 nt, 32 nt
+    double* part;                     // 2 x [nblk][2]
+    GridBarrier gb;
+    long long budget;
+    double tol;
+    int maxit, has_s0, cs;
+    int* its;
+    double* rel;
+};
+
+__global__ void __launch_bounds__(PCG_THREADS, 2) k_lls_pcg(PcgParams P) {
+    constexpr int NW = PCG_THREADS / 32;
+    __shared__ double s_w[NW][2];
+    __shared__ double s_sum[2];
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int nblk = gridDim.x;
+    const int b0 = (int)((long long)P.nb * blockIdx.x / nblk), b1 = (int)((long long)P.nb * (blockIdx.x + 1) / nblk);
+    const int t0 = (int)((long long)P.nt * blockIdx.x / nblk), t1 = (int)((long long)P.nt * (blockIdx.x + 1) / nblk);
+    unsigned phase = 0;
+    int sums = 0;
+    // sum of a slice's row over x, eight entries in flight
+    auto row = [&](const int* sp, const int* col, const double* val, int sl, const double* x) -> double {
+        const int b = __ldg(&sp[sl]), width = (__ldg(&sp[sl + 1]) - b) >> 5;
+        const int* c = col + b + lane;
+        const double* v = val + b + lane;
+        double acc = 0.0;
+        for (int k = 0; k < width; k += 8) {
+            int cc[8];
+            double vv[8], g[8];
+#pragma unroll
+            for (int u = 0; u < 8; ++u) {
+                const bool in = k + u < width;
+                cc[u] = in ? (P.cs ? __ldcs(c + (k + u) * 32) : __ldg(c + (k + u) * 32)) : 0;
+                vv[u] = in ? (P.cs ? __ldcs(v + (k + u) * 32) : __ldg(v + (k + u) * 32)) : 0.0;
+            }
+#pragma unroll
+            for (int u = 0; u < 8; ++u) g[u] = k + u < width ? x[cc[u]] : 0.0;
+#pragma unroll
+            for (int u = 0; u < 8; ++u)
+                if (k + u < width) acc += vv[u] * g[u];
+        }
+        return acc;
+    };
+    // grid totals of two values a thread into s_sum (a grid barrier); false: gave up
+    auto grid_sum = [&](double a, double b) -> bool {
+        double v[2] = {a, b};
+        warp_fold_to<2>(v, s_w[warp]);
+        __syncthreads();
+        double* part = P.part + (size_t)(sums++ & 1) * 2 * nblk;
+        if (threadIdx.x < 2) {
+            double t = 0.0;
+            for (int w = 0; w < NW; ++w) t += s_w[w][threadIdx.x];
+            part[2 * blockIdx.x + threadIdx.x] = t;
+        }
+        if (!grid_sync_phase(P.gb, nblk, phase++, P.budget)) return false;
+        if (warp < 2) {
+            double t = 0.0;
+            for (int q = lane; q < nblk; q += 32) t += __ldcg(&part[2 * q + warp]);
+            t = warp_sum(t);
+            if (lane == 0) s_sum[warp] = t;
+        }
+        __syncthreads();
+        return true;
+    };
+    auto residual = [&]() -> bool {   // z = M^-1 B^T rho; s_sum = r.z, ||r||^2
+        double rz = 0.0, rr = 0.0;
+        for (int sl = t0 + warp; sl < t1; sl += NW) {
+            const int t = sl * 32 + lane;
+            const double r = row(P.tsp, P.tcol, P.tval, sl, P.rho);
+            const double ro = __shfl_xor_sync(0xffffffffu, r, 1);
+            const double zv = P.m1[t] * r + P.m2[t] * ro;
+            P.z[t] = zv;
+            rz += r * zv;
+            rr += r * r;
+        }
+        return grid_sum(rz, rr);
+    };
+    // the tolerance is relative to ||B^T v||, the gradient at s = 0, also from given values s0
+    if (!residual()) return;
+    const double rr0 = s_sum[1];
+    double rz = s_sum[0], rel = rr0 > 0.0 ? 1.0 : 0.0;
+    if (P.has_s0 && rr0 > 0.0) {   // rho = v - B s0 (the slots of a warp are its own)
+        for (int sl = b0 + warp; sl < b1; sl += NW) P.rho[sl * 32 + lane] -= row(P.bsp, P.bcol, P.bval, sl, P.s);
+        if (!grid_sync_phase(P.gb, nblk, phase++, P.budget)) return;
+        if (!residual()) return;
+        rz = s_sum[0];
+        rel = sqrt(s_sum[1] / rr0);
     }
-    g[u] = acc;
+    for (int sl = t0 + warp; sl < t1; sl += NW) P.p[sl * 32 + lane] = P.z[sl * 32 + lane];
+    if (!grid_sync_phase(P.gb, nblk, phase++, P.budget)) return;
+    int its = 0;
+    while (rr0 > 0.0 && rel > P.tol && its < P.maxit) {
+        double qq = 0.0;
+        for (int sl = b0 + warp; sl < b1; sl += NW) {
+            const double v = row(P.bsp, P.bcol, P.bval, sl, P.p);
+            P.q[sl * 32 + lane] = v;
+            qq += v * v;
+        }
+        if (!grid_sum(qq, 0.0)) return;
+        const double a = s_sum[0] > 0.0 ? rz / s_sum[0] : 0.0;
+#pragma unroll 4
+        for (int sl = b0 + warp; sl < b1; sl += NW) P.rho[sl * 32 + lane] -= a * P.q[sl * 32 + lane];
+#pragma unroll 4
+        for (int sl = t0 + warp; sl < t1; sl += NW) P.s[sl * 32 + lane] += a * P.p[sl * 32 + lane];
+        if (!grid_sync_phase(P.gb, nblk, phase++, P.budget)) return;
+        if (!residual()) return;
+        const double b = rz != 0.0 ? s_sum[0] / rz : 0.0;
+        rz = s_sum[0];
+#pragma unroll 4
+        for (int sl = t0 + warp; sl < t1; sl += NW) P.p[sl * 32 + lane] = P.z[sl * 32 + lane] + b * P.p[sl * 32 + lane];
+        ++its;
+        if (its % 8 == 0 || its == P.maxit) {
+            rel = sqrt(s_sum[1] / rr0);
+            if (rel <= P.tol) break;
+        }
+        if (!grid_sync_phase(P.gb, nblk, phase++, P.budget)) return;
+    }
+    if (!(rr0 > 0.0))   // no gradient at s = 0: S = 0, whatever was given
+        for (int sl = t0 + warp; sl < t1; sl += NW) P.s[sl * 32 + lane] = 0.0;
+    if (blockIdx.x == 0 && threadIdx.x == 0) {
+        *P.its = its;
+        *P.rel = rel;
+    }
 }
 
 __global__ void k_diag_values(const int* rp, const int* ci, const double* v, int n, double* dv) {
@@ -356,6 +559,35 @@ asss_status lls_product_on_pattern(const Ctx& c, const DCsr& Abar, const DCsr& S
     return ASSS_OK;
 }
 
+// slice offsets of rows in the given order (no sorting)
+__global__ void k_slice_width(const int* len, int ns, int* w) {
+    const int sl = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
+    if (sl >= ns) return;
+    int m = len[sl * 32 + lane];
+    for (int o = 16; o > 0; o >>= 1) m = max(m, __shfl_xor_sync(0xffffffffu, m, o));
+    if (lane == 0) w[sl] = m * 32;
+}
+static asss_status pair_layout(const int* len, int nslots, DBuf<int>& sptr, int64_t* total, cudaStream_t s) {
+    const int ns = nslots / 32;
+    DBuf<int> w;
+    DBuf<long long> off64;
+    ASSS_TRY(w.alloc(ns > 0 ? ns : 1));
+    ASSS_TRY(off64.alloc(ns + 1));
+    ASSS_TRY(sptr.alloc(ns + 1));
+    k_slice_width<<<cdiv(32LL * ns, 256), 256, 0, s>>>(len, ns, w.p);
+    ASSS_CHECK_LAUNCH();
+    long long tot = 0;
+    ASSS_TRY(exclusive_scan64(w.p, off64.p, ns, &tot, s));
+    if (tot >= (1LL << 31) - 1) {
+        set_error("least-squares storage of %lld entries exceeds 32-bit slice offsets", tot);
+        return ASSS_ERR_UNSUPPORTED;
+    }
+    ASSS_TRY(exclusive_scan(w.p, sptr.p, ns, nullptr, s));
+    ASSS_CUDA(cudaStreamSynchronize(s));   // w is freed here
+    *total = tot;
+    return ASSS_OK;
+}
+
 asss_status lls_fit(const Ctx& c, const DCsr& Abar, const DCsr& AbarT, const DCsr& Spat, double gamma, double tol,
                     int maxit, DBuf<double>& s_val, DCsr& P, DBuf<int>& mirror, DBuf<int>& diagpos,
                     DBuf<double>& Cval, LlsResult* res, const double* s0) {
@@ -390,6 +622,140 @@ asss_status lls_fit(const Ctx& c, const DCsr& Abar, const DCsr& AbarT, const DCs
     ASSS_CHECK_LAUNCH();
 
     const double sg = sqrt(gamma);
+    // B and B^T stored explicitly when they fit min(8 GiB, a quarter of the free device
+    // memory), and the whole iteration in one launch; otherwise the merge kernels apply them
+    // matrix-free
+    {
+        DBuf<int> bcnt, cflag, cidx, uslot, upos, lead, single, lpos, spos, tlen;
+        ASSS_TRY(bcnt.alloc(nP > 0 ? nP : 1));
+        ASSS_TRY(cflag.alloc(nP > 0 ? nP : 1));
+        ASSS_TRY(cidx.alloc(nP + 1));
+        k_bx_count<<<cdiv(nP, 256), 256, 0, s>>>(nP, prow.p, P.ci.p, Abar.rp.p, Abar.ci.p, Abar.v.p, ST.rp.p, ST.ci.p,
+                                                  st_src.p, bcnt.p, cflag.p);
+        ASSS_CHECK_LAUNCH();
+        int64_t nC = 0, npairs = 0, nsingle = 0, nb = 0, nt = 0;
+        ASSS_TRY(exclusive_scan(cflag.p, cidx.p, nP, &nC, s));
+        ASSS_TRY(lead.alloc(nS));
+        ASSS_TRY(single.alloc(nS));
+        ASSS_TRY(lpos.alloc(nS + 1));
+        ASSS_TRY(spos.alloc(nS + 1));
+        k_pair_flags<<<cdiv(nS, 256), 256, 0, s>>>(nS, partner.p, lead.p, single.p);
+        ASSS_CHECK_LAUNCH();
+        ASSS_TRY(exclusive_scan(lead.p, lpos.p, nS, &npairs, s));
+        ASSS_TRY(exclusive_scan(single.p, spos.p, nS, &nsingle, s));
+        const int nuslots = cdiv(2 * npairs + nsingle, 32) * 32;
+        ASSS_TRY(upos.alloc(nS));
+        ASSS_TRY(uslot.alloc(nuslots));
+        ASSS_TRY(tlen.alloc(nuslots));
+        ASSS_CUDA(cudaMemsetAsync(uslot.p, 0xff, sizeof(int) * (size_t)nuslots, s));
+        k_pair_slots<<<cdiv(nS, 256), 256, 0, s>>>(nS, partner.p, lpos.p, spos.p, (int)npairs, upos.p, uslot.p);
+        ASSS_CHECK_LAUNCH();
+        k_btx_count<<<cdiv(nuslots, 256), 256, 0, s>>>(nuslots, uslot.p, srow.p, Spat.ci.p, AbarT.rp.p, AbarT.ci.p,
+                                                        AbarT.v.p, P.rp.p, P.ci.p, mirror.p, tlen.p);
+        ASSS_CHECK_LAUNCH();
+        ASSS_TRY(sum_counts(bcnt.p, nP, &nb, s));
+        ASSS_TRY(sum_counts(tlen.p, nuslots, &nt, s));
+        size_t fr = 0, tot = 0;
+        ASSS_CUDA(cudaMemGetInfo(&fr, &tot));
+        const double need = 12.0 * (double)(nb + nt) + 8.0 * (double)(nP + nS);
+        const double budget = fmin(8.0 * 1024 * 1024 * 1024, 0.25 * (double)fr);
+        if (nb < 0x3fffffffLL && nt < 0x3fffffffLL && need <= budget) {
+            DBuf<int> klist, blen, bmap, bpos, bsp, tmap, tpos, tsp, bcol, tcol, its_d;
+            DBuf<double> bval, tval, m1, m2, sv, zz, pp, qq, rr, part, rel_d;
+            DBuf<unsigned> bar;
+            DBuf<int> err;
+            ASSS_TRY(klist.alloc(nC));
+            ASSS_TRY(blen.alloc(nC));
+            k_bx_list<<<cdiv(nP, 256), 256, 0, s>>>(nP, cflag.p, cidx.p, bcnt.p, klist.p, blen.p);
+            ASSS_CHECK_LAUNCH();
+            int64_t bn = 0, bt = 0, tt = 0;
+            ASSS_TRY(sell_layout(blen.p, (int)nC, SELL_SIGMA, bmap, bpos, bsp, &bn, &bt, s));
+            // pairs stay together: the unknowns keep their slots whatever the padding
+            ASSS_TRY(pair_layout(tlen.p, nuslots, tsp, &tt, s));
+            const int nbs = cdiv(nC, 32), nts = nuslots / 32;
+            ASSS_TRY(bcol.alloc(bt > 0 ? bt : 1));
+            ASSS_TRY(bval.alloc(bt > 0 ? bt : 1));
+            ASSS_TRY(tcol.alloc(tt > 0 ? tt : 1));
+            ASSS_TRY(tval.alloc(tt > 0 ? tt : 1));
+            for (DBuf<double>* v : {&m1, &m2, &sv, &zz, &pp}) ASSS_TRY(v->alloc(nuslots));
+            ASSS_TRY(qq.alloc(32LL * nbs));
+            ASSS_TRY(rr.alloc(32LL * nbs));
+            k_bx_fill<<<cdiv(32LL * nbs, 256), 256, 0, s>>>(32 * nbs, (int)nC, bmap.p, klist.p, prow.p, P.ci.p, Abar.rp.p,
+                                                             Abar.ci.p, Abar.v.p, ST.rp.p, ST.ci.p, st_src.p, upos.p, sg,
+                                                             bsp.p, bcol.p, bval.p, rr.p);
+            ASSS_CHECK_LAUNCH();
+            k_btx_fill<<<cdiv(nuslots, 256), 256, 0, s>>>(nuslots, uslot.p, srow.p, Spat.ci.p, AbarT.rp.p, AbarT.ci.p,
+                                                           AbarT.v.p, P.rp.p, P.ci.p, mirror.p, cidx.p, bpos.p, sg, tsp.p,
+                                                           tcol.p, tval.p, Nn.p, partner.p, cross.p, s0, m1.p, m2.p, sv.p);
+            ASSS_CHECK_LAUNCH();
+            int occ = 0;
+            ASSS_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_lls_pcg, PCG_THREADS, 0));
+            if (occ < 1) {
+                set_error("least-squares kernel cannot be resident");
+                return ASSS_ERR_CUDA;
+            }
+            int nblk = c.sms * (occ > 2 ? 2 : occ);
+            const int want = cdiv(nbs > nts ? nbs : nts, PCG_THREADS / 32);
+            if (nblk > want) nblk = want > 0 ? want : 1;
+            ASSS_TRY(part.alloc(4LL * nblk));
+            ASSS_TRY(bar.alloc(1));
+            ASSS_TRY(err.alloc(1));
+            ASSS_TRY(its_d.alloc(1));
+            ASSS_TRY(rel_d.alloc(1));
+            ASSS_CUDA(cudaMemsetAsync(bar.p, 0, sizeof(unsigned), s));
+            ASSS_CUDA(cudaMemsetAsync(err.p, 0, sizeof(int), s));
+            PcgParams a;
+            a.nb = nbs;
+            a.nt = nts;
+            a.bsp = bsp.p;
+            a.bcol = bcol.p;
+            a.tsp = tsp.p;
+            a.tcol = tcol.p;
+            a.bval = bval.p;
+            a.tval = tval.p;
+            a.m1 = m1.p;
+            a.m2 = m2.p;
+            a.q = qq.p;
+            a.rho = rr.p;
+            a.p = pp.p;
+            a.z = zz.p;
+            a.s = sv.p;
+            a.part = part.p;
+            a.gb.count = bar.p;
+            a.gb.err = err.p;
+            a.budget = c.wait_cycles;
+            a.tol = tol;
+            a.maxit = maxit;
+            a.has_s0 = s0 != nullptr;
+            a.cs = stream_evict_first(c, 12 * (bt + tt)) ? 1 : 0;
+            a.its = its_d.p;
+            a.rel = rel_d.p;
+            void* args[] = {&a};
+            ASSS_CUDA(cudaLaunchCooperativeKernel((const void*)k_lls_pcg, dim3(nblk), dim3(PCG_THREADS), args, 0, s));
+            count_launch();
+            ASSS_TRY(s_val.alloc(nS));
+            k_unslot<<<cdiv(nS, 256), 256, 0, s>>>(nS, upos.p, sv.p, s_val.p);
+            ASSS_CHECK_LAUNCH();
+            ASSS_TRY(Cval.alloc(nP));
+            ASSS_TRY(lls_product_on_pattern(c, Abar, ST, st_src.p, s_val.p, P, prow.p, Cval.p));
+            int hi = 0, he = 0;
+            double hr = 0.0;
+            ASSS_CUDA(cudaMemcpyAsync(&he, err.p, sizeof(int), cudaMemcpyDeviceToHost, s));
+            ASSS_CUDA(cudaMemcpyAsync(&hi, its_d.p, sizeof(int), cudaMemcpyDeviceToHost, s));
+            ASSS_CUDA(cudaMemcpyAsync(&hr, rel_d.p, sizeof(double), cudaMemcpyDeviceToHost, s));
+            ASSS_CUDA(cudaStreamSynchronize(s));
+            if (he) {
+                set_error("least-squares fit: a grid barrier wait exceeded its budget");
+                return (asss_status)he;
+            }
+            if (res) {
+                res->its = hi;
+                res->relgrad = hr;
+            }
+            return ASSS_OK;
+        }
+    }
+    // ---- matrix-free ----
     DBuf<double> rho, q, r, z, p, sc;
     ASSS_TRY(s_val.alloc(nS));
     ASSS_TRY(rho.alloc(nP));
@@ -405,63 +771,15 @@ asss_status lls_fit(const Ctx& c, const DCsr& Abar, const DCsr& AbarT, const DCs
     ASSS_CUDA(cudaMemsetAsync(s_val.p, 0, sizeof(double) * nS, s));
     k_lls_init_rho<<<cdiv(nP, 256), 256, 0, s>>>(nP, prow.p, P.ci.p, sg, rho.p);
     ASSS_CHECK_LAUNCH();
-    // B and B^T stored explicitly when they fit min(8 GiB, a quarter of the free device
-    // memory): the same products, bit for bit, streamed instead of re-intersected each
-    // iteration; otherwise the merge kernels apply them matrix-free
-    DBuf<int> bcnt, brp, bsplit, bcol, tcnt, trp, tcol;
-    DBuf<double> bval, tval;
-    bool explicit_b = false;
-    {
-        ASSS_TRY(bcnt.alloc(nP > 0 ? nP : 1));
-        ASSS_TRY(tcnt.alloc(nS > 0 ? nS : 1));
-        k_bx_rows<<<cdiv(nP, 256), 256, 0, s>>>(nP, prow.p, P.ci.p, Abar.rp.p, Abar.ci.p, Abar.v.p, ST.rp.p, ST.ci.p,
-                                                 st_src.p, nullptr, bcnt.p, nullptr, nullptr, nullptr);
-        ASSS_CHECK_LAUNCH();
-        k_btx_rows<<<cdiv(nS, 256), 256, 0, s>>>(nS, srow.p, Spat.ci.p, AbarT.rp.p, AbarT.ci.p, AbarT.v.p, P.rp.p,
-                                                  P.ci.p, mirror.p, nullptr, tcnt.p, nullptr, nullptr);
-        ASSS_CHECK_LAUNCH();
-        int64_t nb = 0, nt = 0;
-        ASSS_TRY(sum_counts(bcnt.p, nP, &nb, s));
-        ASSS_TRY(sum_counts(tcnt.p, nS, &nt, s));
-        size_t fr = 0, tot = 0;
-        ASSS_CUDA(cudaMemGetInfo(&fr, &tot));
-        const double need = 12.0 * (double)(nb + nt) + 8.0 * (double)(nP + nS);
-        const double budget = fmin(8.0 * 1024 * 1024 * 1024, 0.25 * (double)fr);
-        explicit_b = nb < 0x7fffffffLL && nt < 0x7fffffffLL && need <= budget;
-        if (explicit_b) {
-            ASSS_TRY(brp.alloc(nP + 1));
-            ASSS_TRY(trp.alloc(nS + 1));
-            ASSS_TRY(exclusive_scan(bcnt.p, brp.p, nP, nullptr, s));
-            ASSS_TRY(exclusive_scan(tcnt.p, trp.p, nS, nullptr, s));
-            ASSS_TRY(bsplit.alloc(nP > 0 ? nP : 1));
-            ASSS_TRY(bcol.alloc(nb > 0 ? nb : 1));
-            ASSS_TRY(bval.alloc(nb > 0 ? nb : 1));
-            ASSS_TRY(tcol.alloc(nt > 0 ? nt : 1));
-            ASSS_TRY(tval.alloc(nt > 0 ? nt : 1));
-            k_bx_rows<<<cdiv(nP, 256), 256, 0, s>>>(nP, prow.p, P.ci.p, Abar.rp.p, Abar.ci.p, Abar.v.p, ST.rp.p,
-                                                     ST.ci.p, st_src.p, brp.p, nullptr, bsplit.p, bcol.p, bval.p);
-            ASSS_CHECK_LAUNCH();
-            k_btx_rows<<<cdiv(nS, 256), 256, 0, s>>>(nS, srow.p, Spat.ci.p, AbarT.rp.p, AbarT.ci.p, AbarT.v.p,
-                                                      P.rp.p, P.ci.p, mirror.p, trp.p, nullptr, tcol.p, tval.p);
-            ASSS_CHECK_LAUNCH();
-        }
-    }
     auto applyBT = [&](const double* t, double* g) -> asss_status {
-        if (explicit_b)
-            k_btx_apply<<<cdiv(nS, 256), 256, 0, s>>>(nS, trp.p, tcol.p, tval.p, t, sg, g);
-        else
-            k_lls_BT<<<cdiv(nS, 256), 256, 0, s>>>(nS, srow.p, Spat.ci.p, AbarT.rp.p, AbarT.ci.p, AbarT.v.p, P.rp.p,
-                                                    P.ci.p, mirror.p, t, sg, g);
+        k_lls_BT<<<cdiv(nS, 256), 256, 0, s>>>(nS, srow.p, Spat.ci.p, AbarT.rp.p, AbarT.ci.p, AbarT.v.p, P.rp.p, P.ci.p,
+                                                mirror.p, t, sg, g);
         ASSS_CHECK_LAUNCH();
         return ASSS_OK;
     };
     auto applyB = [&](const double* sv, double* out) -> asss_status {
-        if (explicit_b)
-            k_bx_apply<<<cdiv(nP, 256), 256, 0, s>>>(nP, prow.p, P.ci.p, brp.p, bsplit.p, bcol.p, bval.p, sv, sg,
-                                                      out);
-        else
-            k_lls_B<<<cdiv(nP, 256), 256, 0, s>>>(nP, prow.p, P.ci.p, Abar.rp.p, Abar.ci.p, Abar.v.p, ST.rp.p,
-                                                   ST.ci.p, st_src.p, sv, sg, out);
+        k_lls_B<<<cdiv(nP, 256), 256, 0, s>>>(nP, prow.p, P.ci.p, Abar.rp.p, Abar.ci.p, Abar.v.p, ST.rp.p, ST.ci.p,
+                                               st_src.p, sv, sg, out);
         ASSS_CHECK_LAUNCH();
         return ASSS_OK;
     };

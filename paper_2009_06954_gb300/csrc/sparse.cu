@@ -958,6 +958,52 @@ __global__ void k_sell_fill(int n, int nslices, const int* rp, const int* ci, co
     }
 }
 
+// The slices of rows of the given lengths: natural order, or (sorted windows of sigma rows) when
+// that pads the stored entries by more than a fifth.  rowmap / rowpos stay empty in natural
+// order; *total counts the padding.
+asss_status sell_layout(const int* len, int n, int sigma, DBuf<int>& rowmap, DBuf<int>& rowpos, DBuf<int>& sptr,
+                        int64_t* nnz, int64_t* total, cudaStream_t s) {
+    const int ns = cdiv(n, 32);
+    DBuf<int> w;
+    DBuf<unsigned long long> cnt;
+    DBuf<long long> off64;
+    ASSS_TRY(w.alloc(ns > 0 ? ns : 1));
+    ASSS_TRY(cnt.alloc(1));
+    ASSS_TRY(off64.alloc(ns + 1));
+    rowmap.free();
+    rowpos.free();
+    long long tot = 0;
+    unsigned long long hn = 0;
+    for (int pass = 0; pass < 2; ++pass) {
+        const int* rmap = pass ? rowmap.p : nullptr;
+        ASSS_CUDA(cudaMemsetAsync(cnt.p, 0, sizeof(unsigned long long), s));
+        k_sell_width<<<cdiv(ns, 128), 128, 0, s>>>(n, len, rmap, ns, w.p, cnt.p);
+        ASSS_CHECK_LAUNCH();
+        ASSS_CUDA(cudaMemcpyAsync(&hn, cnt.p, sizeof(hn), cudaMemcpyDeviceToHost, s));
+        ASSS_TRY(exclusive_scan64(w.p, off64.p, ns, &tot, s));   // 64-bit total (synchronises)
+        if (pass == 1 || (double)tot <= 1.2 * (double)hn) break;
+        // heavy-tailed rows: sort each window of sigma rows by length
+        const int nslots = ns * 32;
+        ASSS_TRY(rowmap.alloc(nslots));
+        ASSS_TRY(rowpos.alloc(n));
+        const size_t smem = sizeof(long long) * (size_t)sigma;
+        ASSS_TRY(raise_dynamic_smem((const void*)k_sell_sort_window, (int)smem));
+        k_sell_sort_window<<<cdiv(nslots, sigma), SELL_SORT_THREADS, smem, s>>>(n, nslots, sigma, len, rowmap.p,
+                                                                                rowpos.p);
+        ASSS_CHECK_LAUNCH();
+    }
+    *nnz = (int64_t)hn;
+    *total = tot;
+    if (tot >= (1LL << 31) - 1) {
+        set_error("SELL-C storage of %lld entries exceeds 32-bit slice offsets", tot);
+        return ASSS_ERR_UNSUPPORTED;
+    }
+    ASSS_TRY(sptr.alloc(ns + 1));
+    ASSS_TRY(exclusive_scan(w.p, sptr.p, ns, nullptr, s));
+    ASSS_CUDA(cudaStreamSynchronize(s));   // w is freed here
+    return ASSS_OK;
+}
+
 // Slices of 32 rows in natural order; when that pads the stored entries by more than
 // a fifth over the matrix's own (heavy-tailed row lengths), SELL-C-sigma instead (sigma:
 // the window in rows, a power of two from 1024 to SELL_SIGMA_MAX; 0: SELL_SIGMA).  Slices
@@ -976,50 +1022,18 @@ asss_status build_sell(const DCsr& A, bool skip_diag, DSell<T>& out, cudaStream_
     }
     out.sigma = 0;
     out.split = split;
-    out.rowmap.free();
-    out.rowpos.free();
     int n = A.n;
     int ns = cdiv(n, 32);
     out.n = n;
     out.nslices = ns;
-    DBuf<int> w, len;
-    DBuf<unsigned long long> cnt;
-    ASSS_TRY(w.alloc(ns));
+    DBuf<int> len;
     ASSS_TRY(len.alloc(n > 0 ? n : 1));
-    ASSS_TRY(cnt.alloc(1));
     k_sell_rowlen<<<cdiv(n, 256), 256, 0, s>>>(n, A.rp.p, A.ci.p, skip_diag ? 1 : 0, len.p);
     ASSS_CHECK_LAUNCH();
-    long long tot = 0;
-    unsigned long long hn = 0;
-    DBuf<long long> off64;
-    ASSS_TRY(off64.alloc(ns + 1));
-    for (int pass = 0; pass < 2; ++pass) {
-        const int* rmap = pass ? out.rowmap.p : nullptr;
-        ASSS_CUDA(cudaMemsetAsync(cnt.p, 0, sizeof(unsigned long long), s));
-        k_sell_width<<<cdiv(ns, 128), 128, 0, s>>>(n, len.p, rmap, ns, w.p, cnt.p);
-        ASSS_CHECK_LAUNCH();
-        ASSS_CUDA(cudaMemcpyAsync(&hn, cnt.p, sizeof(hn), cudaMemcpyDeviceToHost, s));
-        ASSS_TRY(exclusive_scan64(w.p, off64.p, ns, &tot, s));   // 64-bit total (synchronises)
-        if (pass == 1 || (double)tot <= 1.2 * (double)hn) break;
-        // heavy-tailed rows: sort each window of sigma rows by length
-        const int nslots = ns * 32;
-        ASSS_TRY(out.rowmap.alloc(nslots));
-        ASSS_TRY(out.rowpos.alloc(n));
-        const size_t smem = sizeof(long long) * (size_t)sigma;
-        ASSS_TRY(raise_dynamic_smem((const void*)k_sell_sort_window, (int)smem));
-        k_sell_sort_window<<<cdiv(nslots, sigma), SELL_SORT_THREADS, smem, s>>>(n, nslots, sigma, len.p,
-                                                                                out.rowmap.p, out.rowpos.p);
-        ASSS_CHECK_LAUNCH();
-        out.sigma = sigma;
-    }
-    out.nnz = (int64_t)hn;
+    int64_t tot = 0;
+    ASSS_TRY(sell_layout(len.p, n, sigma, out.rowmap, out.rowpos, out.sptr, &out.nnz, &tot, s));
+    if (out.rowmap.p) out.sigma = sigma;
     out.nstored = tot;
-    if (tot >= (1LL << 31) - 1) {
-        set_error("SELL-C storage of %lld entries exceeds 32-bit slice offsets", tot);
-        return ASSS_ERR_UNSUPPORTED;
-    }
-    ASSS_TRY(out.sptr.alloc(ns + 1));
-    ASSS_TRY(exclusive_scan(w.p, out.sptr.p, ns, nullptr, s));
     ASSS_TRY(out.col.alloc(tot > 0 ? tot : 1));
     ASSS_TRY(out.val.alloc(tot > 0 ? tot : 1));
     k_sell_fill<T><<<cdiv((int64_t)ns * 32, 256), 256, 0, s>>>(n, ns, A.rp.p, A.ci.p, A.v.p, skip_diag ? 1 : 0,
