@@ -36,6 +36,7 @@ struct AoParams {
     double* inv_hn;   // 1 / ||w|| (0 when w = 0)
     double* part;     // 2 x [AO_MAXV][nblk] block partials (consecutive passes alternate halves)
     double thr;       // the cycle stops when |g[j+1]| <= thr
+    double sign;      // v_{j+1} = sign * w / ||w||
     int* stop;
     GridBarrier gb;
     unsigned phase0;  // barriers completed on gb.count before this launch
@@ -127,7 +128,7 @@ __device__ __forceinline__ void ao_close(const AoParams& p, const double* s_h1, 
     }
     rows();
     __syncthreads();
-    out(s_fin[2]);
+    out(p.sign * s_fin[2]);
     if (blockIdx.x == 0) {
         for (int a = threadIdx.x; a < p.nv; a += blockDim.x) {
             p.hv[a] = s_h1[a];
@@ -459,7 +460,7 @@ static const void* ao_tight(int rows) {
 
 asss_status arnoldi_orth(const Ctx& c, ArnoldiWork& aw, const double* V, double* w, int n, int j, int m, double* H,
                          double* cs, double* sn, double* g, double* hv, double* hv2, double* hn2, double* inv_hn,
-                         double thr, int* stop) {
+                         double thr, int* stop, double sign) {
     if (j + 1 > AO_MAXV - 1) {   // one partial slot is kept for the norm
         set_error("Arnoldi step %d exceeds the fused kernel's %d vectors", j, AO_MAXV - 1);
         return ASSS_ERR_UNSUPPORTED;
@@ -502,6 +503,7 @@ asss_status arnoldi_orth(const Ctx& c, ArnoldiWork& aw, const double* V, double*
     p.inv_hn = inv_hn;
     p.part = aw.part.p;
     p.thr = thr;
+    p.sign = sign;
     p.stop = stop;
     p.gb.count = aw.bar.p;
     p.gb.err = aw.err.p;

@@ -91,7 +91,9 @@ __global__ void k_diag_w(const double* C, const int* diagpos, int n, double* d, 
 __global__ void k_absmax(const double* a, int n, unsigned long long* out) {
     double m = 0.0;
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) m = fmax(m, fabs(a[i]));
-    atomicMax(out, (unsigned long long)__double_as_longlong(m));
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) m = fmax(m, __shfl_xor_sync(0xffffffffu, m, o));
+    if ((threadIdx.x & 31) == 0) atomicMax(out, (unsigned long long)__double_as_longlong(m));
 }
 __global__ void k_zero_pivots(const double* d, int n, double thr, int* cnt) {
     int i = blockIdx.x * blockDim.x + threadIdx.x;
@@ -728,6 +730,49 @@ static asss_status lanczos(const Ctx& c, const DCsr& J, const double* q1, int n,
         return ASSS_ERR_ARG;
     }
     ASSS_TRY(vscale(Qcm.p, q1, 1.0 / sqrt(nn), n, s));
+    if (reorth && k <= AO_MAXV) {
+        // Two passes of classical Gram-Schmidt against q_1..q_i, the norm and q_{i+1} = -z / alpha_i
+        // are the fused Arnoldi step (its first pass also takes out Fig. 2's alpha_{i-1} q_{i-1}
+        // term); no step waits for the host, which finds a breakdown in the alphas afterwards.
+        // A step was eleven launches and a read-back (10^3: set-up with 8 fit steps 7.8 -> 4.0 ms).
+        DBuf<double> H, w1, an;
+        DBuf<int> stop;
+        ArnoldiWork aw;
+        ASSS_TRY(H.alloc((int64_t)(k + 1) * k));
+        ASSS_TRY(w1.alloc(5 * (k + 2)));   // cs, sn, g and the coefficients of both passes
+        ASSS_TRY(an.alloc(2 * k));
+        ASSS_TRY(stop.alloc(1));
+        ASSS_CUDA(cudaMemsetAsync(w1.p, 0, sizeof(double) * 5 * (k + 2), s));
+        const int ld = k + 2;
+        for (int i = 1; i < k; ++i) {
+            const double* q = Qcm.p + (size_t)(i - 1) * n;
+            if (F) ASSS_TRY(apply_jt_factored(c, *F, J, q, z.p, ta, tb));
+            else ASSS_TRY(spmv(J, q, z.p, nullptr, s));
+            ASSS_TRY(arnoldi_orth(c, aw, Qcm.p, z.p, n, i - 1, k, H.p, w1.p, w1.p + ld, w1.p + 2 * ld, w1.p + 3 * ld,
+                                  w1.p + 4 * ld, an.p + i - 1, an.p + k + i - 1, 0.0, stop.p, -1.0));
+        }
+        std::vector<double> hn2(k, 0.0);
+        int he = 0;
+        if (k > 1) {
+            ASSS_CUDA(cudaMemcpyAsync(hn2.data(), an.p, sizeof(double) * (k - 1), cudaMemcpyDeviceToHost, s));
+            ASSS_CUDA(cudaMemcpyAsync(&he, aw.err.p, sizeof(int), cudaMemcpyDeviceToHost, s));
+        }
+        ASSS_CUDA(cudaStreamSynchronize(s));
+        if (he) {
+            set_error("a device wait in the Lanczos step ran out (status %d)", he);
+            return (asss_status)he;
+        }
+        int kk = 1;
+        for (int i = 1; i < k; ++i) {
+            const double a = sqrt(hn2[i - 1]);
+            if (a == 0.0 || (i >= 2 && a <= 1e-12 * alpha[0])) break;
+            alpha[i - 1] = a;
+            kk = i + 1;
+        }
+        alpha.resize(kk - 1);
+        *k_eff = kk;
+        return ASSS_OK;
+    }
     int kk = 1;
     for (int i = 1; i < k; ++i) {
         if (F) ASSS_TRY(apply_jt_factored(c, *F, J, Qcm.p + (size_t)(i - 1) * n, z.p, ta, tb));
@@ -782,9 +827,12 @@ static asss_status ensure_smw(asss_handle* h, int tr) {
     double tol = h->opt.setup_tol > 0 ? h->opt.setup_tol : h->opt.inner_tol;
     double sign = tr ? -1.0 : 1.0;
     const UrCols U = ur_cols(h);
-    if (h->kp <= MRS_MULTI_KPMAX && !h->factored) {
+    if (h->kp <= MRS_MULTI_KPMAX && !h->factored && !h->use_dia) {
         // S_bar X = U_bar as App. B's simultaneous iterations: the k + r columns share
-        // every pass over J~ and Q_k (groups of up to 8 per launch)
+        // every pass over J~ and Q_k (groups of up to 8 per launch).  On diagonals one column
+        // after another is faster: both forms are bound by the FP64 pipe, and the
+        // single-column kernel spends less of it on sums (Lanczos
+        // and these solves together, k = 20: 7.6 -> 2.4 ms at 32^3, 26 -> 7 ms at 64^3)
         DBuf<double> Ub;
         ASSS_TRY(Ub.alloc((int64_t)n * m));
         if (k) ASSS_CUDA(cudaMemcpyAsync(Ub.p, h->Qcm.p, sizeof(double) * (size_t)n * k, cudaMemcpyDeviceToDevice, s));

@@ -294,7 +294,7 @@ struct ArnoldiWork {
 // *stop receives 1 when the cycle ends at this step (||w|| = 0 or |g[j+1]| <= thr)
 asss_status arnoldi_orth(const Ctx& c, ArnoldiWork& aw, const double* V, double* w, int n, int j, int m, double* H,
                          double* cs, double* sn, double* g, double* hv, double* hv2, double* hn2, double* inv_hn,
-                         double thr, int* stop);    // restart length bound of the batched FGMRES
+                         double thr, int* stop, double sign = 1.0);
 long long batch_work_doubles(int n_max, int halo_max, int restart);
 
 }  // namespace asss

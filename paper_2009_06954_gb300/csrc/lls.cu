@@ -314,8 +314,9 @@ __global__ void k_unslot(int nS, const int* upos, const double* s, double* s_val
 //   q = B p, ||q||^2 | rho -= a q, s += a p | r = B^T rho, z = M^-1 r, r.z, ||r||^2 | p = z + b p
 // r is not stored (z and the two sums are all that is needed of it).  Bound: the FP64 pipe and
 // L2 / HBM reads of the entries (12 bytes each).  An iteration at 10^3: 38 -> 7 us, at 32^3: 85 ->
-// 25 us, at 64^3: 437 -> 111 us.  Two blocks of 64 registers a thread: one of 117 took 23 us at
-// 32^3 but 165 us at 64^3, where the reads come from HBM and want more warps.
+// 25 us, at 64^3: 437 -> 111 us.  Two blocks an SM at 64 registers and four entries in flight:
+// eight spill (set-up at 32^3 19.7 ms against 18.5, at 64^3 105 against 95), one block of 117
+// registers is as fast at 32^3 and slower from HBM (140 at 64^3).
 // ---------------------------------------------------------------------------
 constexpr int PCG_THREADS = 512;
 struct PcgParams {
@@ -342,25 +343,25 @@ __global__ void __launch_bounds__(PCG_THREADS, 2) k_lls_pcg(PcgParams P) {
     const int t0 = (int)((long long)P.nt * blockIdx.x / nblk), t1 = (int)((long long)P.nt * (blockIdx.x + 1) / nblk);
     unsigned phase = 0;
     int sums = 0;
-    // sum of a slice's row over x, eight entries in flight
+    // sum of a slice's row over x, four entries in flight
     auto row = [&](const int* sp, const int* col, const double* val, int sl, const double* x) -> double {
         const int b = __ldg(&sp[sl]), width = (__ldg(&sp[sl + 1]) - b) >> 5;
         const int* c = col + b + lane;
         const double* v = val + b + lane;
         double acc = 0.0;
-        for (int k = 0; k < width; k += 8) {
-            int cc[8];
-            double vv[8], g[8];
+        for (int k = 0; k < width; k += 4) {
+            int cc[4];
+            double vv[4], g[4];
 #pragma unroll
-            for (int u = 0; u < 8; ++u) {
+            for (int u = 0; u < 4; ++u) {
                 const bool in = k + u < width;
                 cc[u] = in ? (P.cs ? __ldcs(c + (k + u) * 32) : __ldg(c + (k + u) * 32)) : 0;
                 vv[u] = in ? (P.cs ? __ldcs(v + (k + u) * 32) : __ldg(v + (k + u) * 32)) : 0.0;
             }
 #pragma unroll
-            for (int u = 0; u < 8; ++u) g[u] = k + u < width ? x[cc[u]] : 0.0;
+            for (int u = 0; u < 4; ++u) g[u] = k + u < width ? x[cc[u]] : 0.0;
 #pragma unroll
-            for (int u = 0; u < 8; ++u)
+            for (int u = 0; u < 4; ++u)
                 if (k + u < width) acc += vv[u] * g[u];
         }
         return acc;
