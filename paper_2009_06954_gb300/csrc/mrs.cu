@@ -98,6 +98,13 @@ static asss_status dispatch_mrs(const Ctx& c, MrsWork* w, const DSell<T>* sell, 
             if (Q16) return dispatch_kp16<1>(c, w, v, Q16, alpha, k, kp16, shift, sign, rhs, x, Y, ystride, P, tol,
                                              maxit, lo);
         }
+        if constexpr (sizeof(T) == 8) {
+            // at most a slice per SM: four lanes a row
+            if (v.nslices <= c.sms) {
+                v.fmt = 5;
+                return dispatch_kp<T, 5>(c, w, v, Q, alpha, k, kp, shift, sign, rhs, x, Y, ystride, P, tol, maxit, lo);
+            }
+        }
         return dispatch_kp<T, 1>(c, w, v, Q, alpha, k, kp, shift, sign, rhs, x, Y, ystride, P, tol, maxit, lo);
     }
     if (rows) {

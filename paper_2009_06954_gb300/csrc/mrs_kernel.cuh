@@ -48,7 +48,7 @@ constexpr int MRS_TRACE_SLOTS = 4 + 5 * MRS_TRACE_STEPS;
 // warp instruction holds it for 16 cycles): 8 warps keep it busy, and every warp that
 // takes part costs its share of FP64 adds in the block's partial sums.
 template <class T, int FMT>
-constexpr int mrs_threads() { return sizeof(T) == 8 && (FMT == 1 || FMT == 2) ? 256 : MRS_THREADS; }
+constexpr int mrs_threads() { return sizeof(T) == 8 && (FMT == 1 || FMT == 2 || FMT == 5) ? 256 : MRS_THREADS; }
 
 // Blocks of a launch.  FP32 (and the SELL / factored FP64 passes): one slice per warp before
 // another block is opened.  The FP64-pipe-bound passes instead open a block per slice up
@@ -264,6 +264,11 @@ __device__ __forceinline__ void stream_rows(const T* __restrict__ val, const uns
 
 // FMT 0: SELL-C storage of J~; FMT 1: skew half-diagonal storage; FMT 2: plain CSR;
 // FMT 3: factored J~ = L~^-1 J^ L~^-T (incomplete L D L^T in a multicolour order)
+// FMT 5: as FMT 1, four lanes a row (FP64 systems of at most a slice per SM).  A warp's FP64
+// operation holds its SM quarter's pipe for 64 cycles whatever its lanes do, so a row a lane
+// costs a warp 71 + 23 of them in a chain on one quarter of one SM; four lanes a row put a
+// slice on all four quarters, at 29 + 6 each (a step at n = 2209, k = 20: 9.1 -> 6.2 us with the
+// sums below).
 // FMT 4: row-stream storage.  Long rows (hundreds of entries, some thousands): with a lane
 // per row (SELL) a system of 2 10^4 rows has fewer work units than the GPU has warps and each
 // is one lane's serial chain of gathers.  Here a block's entries are cut evenly over its 16
@@ -284,10 +289,13 @@ __global__ void __launch_bounds__((mrs_threads<T, FMT>()), 1) k_mrs(MrsParams<T>
         return;
     }
     __shared__ T s_wsum[NW][NV];
-    __shared__ typename std::conditional<sizeof(T) == 4, float2, double>::type s_bsum[NW][NV];
+    // cross-block sums: rows of partials summed by a warp each (FP32) or by groups of NV threads
+    constexpr int NG = sizeof(T) == 4 ? NW : (NT / NV > 0 ? NT / NV : 1);
+    __shared__ typename std::conditional<sizeof(T) == 4, float2, double>::type s_bsum[NG][NV];
     __shared__ T s_red[NV];
     __shared__ T s_u[KP > 0 ? KP : 1];
-    __shared__ int s_off[FMT == 1 ? MRS_MAXDIAG : 1];
+    constexpr bool DIA = FMT == 1 || FMT == 5;
+    __shared__ int s_off[DIA ? MRS_MAXDIAG : 1];
     __shared__ int s_ls[FMT == 3 ? ILDL_MAXCOL + 1 : 1];
     __shared__ MrsScalars<T> sc;
     __shared__ T s_alpha[MRS_KPMAX];
@@ -303,7 +311,7 @@ __global__ void __launch_bounds__((mrs_threads<T, FMT>()), 1) k_mrs(MrsParams<T>
     __shared__ T s_qtp[2][KP > 0 ? KP : 1];  // Q^T p of the last two directions (slot j & 1)
     __shared__ T s_qtx[KP > 0 ? KP : 1];     // Q^T x
     __shared__ T s_pq[4];                    // step j: nu_j, delta, 1/theta_j, xcoef_j
-    if constexpr (FMT == 1) {
+    if constexpr (DIA) {
         for (int d = threadIdx.x; d < p.ndiag; d += NT) s_off[d] = p.off[d];
     }
     for (int m = threadIdx.x; m < KP; m += NT) {
@@ -354,9 +362,45 @@ __global__ void __launch_bounds__((mrs_threads<T, FMT>()), 1) k_mrs(MrsParams<T>
         if constexpr (sizeof(T) == 4) return df_add(a, b);
         else return a + b;
     };
-    const int nact = FMT == 0 ? NW : min(NW, max(s1 - s0, 1));
-    auto block_partials = [&](T(&tacc)[NV], double* buf) {
-        if (warp < nact) warp_fold_to<NV>(tacc, s_wsum[warp]);
+    const int nact0 = FMT == 0 ? NW : min(NW, max(s1 - s0, 1));
+    const int nact5 = min(NW, max(4 * (s1 - s0), 1));   // FMT 5: a warp takes a quarter of a slice
+    auto block_partials = [&](T(&tacc)[NV], double* buf, bool quarters) {
+        const int nact = quarters ? nact5 : nact0;
+        if (warp < nact) {
+            if (FMT == 5 && quarters) {
+                // lane (row r, part q): tacc[0] the norm's share, tacc[1 + t] the sum of
+                // column q + 4 t; summed over the eight rows, three exchanges
+                constexpr int TV = KP / 4 + 1;
+                T v[TV];
+#pragma unroll
+                for (int t = 0; t < TV; ++t) v[t] = tacc[t];
+                int idx = 0, have = TV, cnt = TV;
+#pragma unroll
+                for (int o = 16; o >= 4; o >>= 1) {
+                    const bool up = (lane & o) != 0;
+                    const int h = (cnt + 1) / 2;
+#pragma unroll
+                    for (int i = 0; i < (TV + 1) / 2; ++i)
+                        if (i < h) {
+                            const T lo = v[i], hi = h + i < cnt ? v[h + i < TV ? h + i : 0] : (T)0;
+                            v[i] = (up ? hi : lo) + __shfl_xor_sync(0xffffffffu, up ? lo : hi, o);
+                        }
+                    idx += up ? h : 0;
+                    have = up ? have - h : min(have, h);
+                    cnt = h;
+                }
+                // up to TV / 8 rounded up values are left a lane (one for k <= 28)
+#pragma unroll
+                for (int i = 0; i < (TV + 7) / 8; ++i)
+                    if (i < have) {
+                        const int t = idx + i, q = lane & 3;
+                        if (t > 0) s_wsum[warp][1 + q + 4 * (t - 1)] = v[i];
+                        else if (q == 0) s_wsum[warp][0] = v[i];
+                    }
+            } else {
+                warp_fold_to<NV>(tacc, s_wsum[warp]);
+            }
+        }
         __syncthreads();
         for (int v = threadIdx.x; v < NV; v += NT) {
             if constexpr (sizeof(T) == 4) {
@@ -376,9 +420,42 @@ __global__ void __launch_bounds__((mrs_threads<T, FMT>()), 1) k_mrs(MrsParams<T>
     // every block adds the block partials in the same fixed order: warp w takes blocks
     // w, w + NW, ..., a lane one value (a block's values are contiguous; the loads of
     // RCHUNK blocks are in flight together), then warp 0 adds the warps' sums into s_red.
-    // Only warp 0 holds s_red afterwards: it goes on with the scalars.
+    // Only warp 0 holds s_red afterwards: it goes on with the scalars (FP64: every warp).
     constexpr int RCHUNK = 10;
     auto reduce_all = [&](const double* buf) {
+        if constexpr (sizeof(T) == 8) {
+            // FP64: the adds are what this costs (64 cycles a warp and SM quarter), so every
+            // lane takes one: thread g NV + v the value v of blocks g, g + NG, ...; then four
+            // lanes a value
+            for (int t = threadIdx.x; t < NG * NV; t += NT) {
+                const int v = t % NV, g = t / NV;
+                double acc = 0.0;
+                for (int b0 = g; b0 < nblk; b0 += NG * RCHUNK) {
+                    double ld[RCHUNK];
+#pragma unroll
+                    for (int q = 0; q < RCHUNK; ++q) {
+                        const int b = b0 + q * NG;
+                        ld[q] = b < nblk ? __ldcg(&buf[(size_t)b * NV + v]) : 0.0;
+                    }
+#pragma unroll
+                    for (int q = 0; q < RCHUNK; ++q)
+                        if (b0 + q * NG < nblk) acc += ld[q];
+                }
+                s_bsum[g][v] = acc;
+            }
+            __syncthreads();
+            for (int t0 = 0; t0 < 4 * NV; t0 += NT) {
+                const int t = t0 + threadIdx.x, v = t >> 2;
+                double a = 0.0;
+                if (v < NV)
+                    for (int g = t & 3; g < NG && g < nblk; g += 4) a += s_bsum[g][v];
+                a += __shfl_xor_sync(0xffffffffu, a, 1);
+                a += __shfl_xor_sync(0xffffffffu, a, 2);
+                if (v < NV && (t & 3) == 0) s_red[v] = a;
+            }
+            __syncthreads();
+            return;
+        }
         const P2* b2 = reinterpret_cast<const P2*>(buf);
         for (int v = lane; v < NV; v += 32) {
             P2 acc{};
@@ -518,7 +595,7 @@ __global__ void __launch_bounds__((mrs_threads<T, FMT>()), 1) k_mrs(MrsParams<T>
         }
     }
     stamp(1);
-    block_partials(tacc, p.part);
+    block_partials(tacc, p.part, false);
     const bool met = grid_sync_phase(p.gb, nblk, phase++, p.budget);
     stamp(2);
     if (!met) return;
@@ -671,6 +748,51 @@ __global__ void __launch_bounds__((mrs_threads<T, FMT>()), 1) k_mrs(MrsParams<T>
                     qrow(i + NT, q);
                 }
             }
+        } else if constexpr (FMT == 5) {
+            const int sub = lane & 3;
+            for (int qq = 4 * s0 + warp; qq < 4 * s1; qq += NW) {
+                const int i = qq * 8 + (lane >> 2);
+                const bool live = i < n;
+                T part = (T)0, q[KP > 0 ? KP / 4 : 1], yold = (T)0, pold = (T)0;
+                if (live) {
+                    if (j >= 2) {
+                        yold = Yold[i];
+                        if (sub == 0) pold = Pj1[i];
+                    }
+                    const T* qr = Qr + (size_t)i * KP + sub;
+#pragma unroll
+                    for (int t = 0; t < KP / 4; ++t) q[t] = __ldg(qr + 4 * t);
+                    const T* Ud = Ub + i;
+                    const T* yi = Ycur + i;
+                    T acc = (T)0, dq = (T)0;
+#pragma unroll 3
+                    for (int d = sub; d < p.ndiag; d += 4) {
+                        const int m = s_off[d];
+                        const T* Um = Ud + d * p.ustride;
+                        acc = fma(__ldg(Um), yi[m], acc);
+                        acc = fma(-__ldg(Um - m), yi[-m], acc);
+                    }
+#pragma unroll
+                    for (int t = 0; t < KP / 4; ++t) dq += q[t] * s_u[sub + 4 * t];
+                    part = tnu * acc - tsg * dq;
+                }
+                part += __shfl_xor_sync(0xffffffffu, part, 1);
+                part += __shfl_xor_sync(0xffffffffu, part, 2);
+                if (live) {
+                    const T ynew = part + tco * yold;
+#pragma unroll
+                    for (int t = 0; t < KP / 4; ++t) tacc[1 + t] += q[t] * ynew;
+                    if (sub == 0) {
+                        Ynew[i] = ynew;
+                        tacc[0] += ynew * ynew;
+                        if (j >= 2) {
+                            const T pv = (tnp * yold - tdpp * pold) * tthp;
+                            Pj1[i] = pv;
+                            xv[i] += txp * pv;
+                        }
+                    }
+                }
+            }
         } else {
         for (int uu = u0 + warp; uu < u1; uu = next_slice(uu)) {
             int sl = uu, part = 0, nparts = 1, hix = -1;
@@ -807,7 +929,7 @@ __global__ void __launch_bounds__((mrs_threads<T, FMT>()), 1) k_mrs(MrsParams<T>
         }
         double* buf = p.part + (size_t)(j & 1) * NV * nblk;
         stamp(tb);
-        block_partials(tacc, buf);
+        block_partials(tacc, buf, FMT == 5);
         stamp(tb + 1);
         const bool met = grid_sync_phase(p.gb, nblk, phase++, p.budget);
         stamp(tb + 2);
@@ -852,8 +974,13 @@ __global__ void __launch_bounds__((mrs_threads<T, FMT>()), 1) k_mrs(MrsParams<T>
                 set_coefs();
                 s_next = u0 + NW;
             }
-            __syncwarp();
-            if (!sc.stop) make_u_warp0(sc.nu);
+            if constexpr (sizeof(T) == 4) {
+                __syncwarp();
+                if (!sc.stop) make_u_warp0(sc.nu);
+            }
+        } else if (sizeof(T) == 8 && warp == 2) {
+            // FP64: u on another quarter of the SM, beside the scalars (unused after a stop)
+            make_u_warp0(s_red[0] != (T)0 ? (T)rsqrt((double)s_red[0]) : (T)0);
         }
         __syncthreads();
         if (sc.stop) {
@@ -939,6 +1066,7 @@ static asss_status launch_mrs(const Ctx& c, MrsWork* w, const OpView<T>& J, cons
         set_error("mrs kernel cannot be resident");
         return ASSS_ERR_CUDA;
     }
+    // (FMT 5: a slice a block, by the rule that chose it)
     const int nblk = FMT == 4 ? std::min(c.sms, J.n) : mrs_blocks<T, FMT>(c.sms, occ, J.nslices);
     if (w->part_key != J.key || w->part_nblk != nblk) {
         if (FMT == 4)
@@ -1113,6 +1241,7 @@ extern template asss_status dispatch_kp<float, 1>(ASSS_MRS_DISPATCH_ARGS(float))
 extern template asss_status dispatch_kp<float, 3>(ASSS_MRS_DISPATCH_ARGS(float));
 extern template asss_status dispatch_kp<double, 0>(ASSS_MRS_DISPATCH_ARGS(double));
 extern template asss_status dispatch_kp<double, 1>(ASSS_MRS_DISPATCH_ARGS(double));
+extern template asss_status dispatch_kp<double, 5>(ASSS_MRS_DISPATCH_ARGS(double));
 extern template asss_status dispatch_kp<double, 3>(ASSS_MRS_DISPATCH_ARGS(double));
 extern template asss_status dispatch_kp<float, 4>(ASSS_MRS_DISPATCH_ARGS(float));
 extern template asss_status dispatch_kp<double, 4>(ASSS_MRS_DISPATCH_ARGS(double));
