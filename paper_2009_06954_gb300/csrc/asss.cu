@@ -645,6 +645,8 @@ struct asss_handle {
     int cl_counts[CL_NSIZES] = {-1, -1, -1, -1};
     DBuf<double> cl_work, cl_b, cl_x;
     DBuf<ClStat> cl_st;
+    DBuf<double> cl_part;      // grid scope: block partials, barrier and status
+    DBuf<unsigned> cl_bar;
     ~asss_handle() {
         if (mw) mrs_work_destroy(mw);
     }
@@ -2037,23 +2039,26 @@ static asss_status do_setup(asss_handle* h, const asss_csr* Ain, asss_stats* st)
 // ---------------------------------------------------------------------------
 // cluster-scope solves (solve_cluster.cuh)
 // ---------------------------------------------------------------------------
-// Cluster size for nrhs columns (0: the launch-by-launch path, also where no cluster fits).
-// One cluster has its SMs' share of the bandwidth and the FP64 pipe, the launch-by-launch path
-// the whole GPU but 30 to 100 launches and two to three microseconds a grid-wide step, and
-// several clusters run side by side.  Both grow linearly with n; in microseconds for 4 outer
-// and 20 inner steps, measured at n = 8^3 .. 64^3 (dissipative Hamiltonian, k = 20; both scale
-// with the steps alike):
-//   FP32 inner: cluster 100 + 0.0082 n x 16 / size a wave of columns, launches 470 + 0.0012 n a column
-//   FP64 inner: cluster 200 + 0.034 n x 16 / size,                  launches 560 + 0.0033 n
-// (10^3: 144 against 394; 32^3: 392 against 508; 40^3: 598 against 522; FP64 20^3: 502 against
-// 614, 24^3: 665 against 618; eight columns at 16^3: 199 against 3193 in lockstep blocks, at 48^3
-// 1266 against 4963).
+// How nrhs columns are solved: by clusters of that many CTAs side by side, one after another in
+// grid scope (-1), or launch by launch (0: the incomplete factor where no cluster fits).
+// One cluster has its SMs' share of the bandwidth and the FP64 pipe, but cheap synchronisations and
+// company; grid scope has the whole GPU and pays two to three microseconds a synchronisation.
+// Both grow linearly with n; in microseconds for 4 outer and 20 inner steps, measured at n = 8^3 ..
+// 100^3 (dissipative Hamiltonian, k = 20; all scale with the steps alike):
+//   FP32 inner: cluster 100 + 0.0082 n x 16 / size a wave of columns, grid 215 + 0.00124 n a column
+//   FP64 inner: cluster 200 + 0.034 n x 16 / size,                    grid 330 + 0.00365 n
+// (one column, cluster / grid / launch by launch: 10^3 144 / 184 / 394, 24^3 257 / 254 / 504, 47^3
+// 924 / 346 / 604, 64^3 - / 540 / 765, 100^3 - / 1459 / 1687; FP64 10^3 219 / 272 / 431, 24^3 665 /
+// 381 / 604, 64^3 - / 1286 / 1450; eight columns at 16^3 199 against 3193 in lockstep blocks, at
+// 48^3 1266 against 4963).
 static int cluster_size(const asss_handle* h, int nrhs) {
+    constexpr int CL_MOST = 300000;   // above it the columns' vectors leave L2 (not measured)
     const bool fp32 = h->opt.precision == ASSS_PREC_MIXED;
     const double n = h->n;
-    double best = nrhs * (fp32 ? 470.0 + 0.0012 * n : 560.0 + 0.0033 * n) * 0.95;
+    double best = nrhs * (fp32 ? 215.0 + 0.00124 * n : 330.0 + 0.00365 * n);
     if (h->factored) best = nrhs * 3000.0;   // a grid barrier or a launch per colour: 24^3 4295 us against 1133
-    int size = 0;
+    int size = h->factored ? 0 : -1;
+    if (h->n > CL_MOST) return size;
     for (int t = 0; t < CL_NSIZES; ++t) {
         if (h->cl_counts[t] < 1) continue;
         const int waves = cdiv(nrhs, h->cl_counts[t]);
@@ -2159,13 +2164,11 @@ static asss_status cluster_args(asss_handle* h, int tr, ClArgs<T>& a) {
     return ASSS_OK;
 }
 
-// the cluster size of a call (0: launch by launch); CL_MOST: above it the vectors of the
-// columns side by side leave L2 (not measured)
+// what a call takes: see cluster_size
 static asss_status cluster_plan(asss_handle* h, int nrhs, int* size) {
-    constexpr int CL_MOST = 300000;
     const asss_options& o = h->opt;
     *size = 0;
-    if (nrhs < 1 || h->n > CL_MOST || o.outer != ASSS_OUTER_FGMRES || o.restart > CL_RESTART ||
+    if (nrhs < 1 || o.outer != ASSS_OUTER_FGMRES || o.restart > CL_RESTART ||
         !(h->use_dia || (h->factored && h->fac.pos.p)) || h->Q16.p || h->kp > 32 || h->k + h->r > CL_MMAX ||
         getenv("ASSS_TRACE"))   // which asks for the phases of the launch-by-launch path
         return ASSS_OK;
@@ -2197,9 +2200,21 @@ static asss_status solve_cluster(asss_handle* h, int tr, int size, int nc, const
     ClArgs<T> a;
     memset(&a, 0, sizeof(a));
     ASSS_TRY(cluster_args<T>(h, tr, a));
-    int count = 0;
+    int count = 1;
     for (int t = 0; t < CL_NSIZES; ++t)
         if (CL_SIZES[t] == size) count = nc < h->cl_counts[t] ? nc : h->cl_counts[t];
+    if (size < 0) {   // grid scope
+        const int64_t np = 2LL * CL_XV * c.sms;
+        if (h->cl_part.n < np) ASSS_TRY(h->cl_part.alloc(np));
+        if (!h->cl_bar.p) ASSS_TRY(h->cl_bar.alloc(2));
+        ASSS_CUDA(cudaMemsetAsync(h->cl_bar.p, 0, 2 * sizeof(unsigned), s));   // arrivals and status
+        a.part = h->cl_part.p;
+        a.gb.count = h->cl_bar.p;
+        a.gb.err = reinterpret_cast<int*>(h->cl_bar.p + 1);
+        a.budget = c.wait_cycles;
+        const long long tb = (long long)sizeof(T), nnz = tb == 4 ? h->D32.nnz : h->D64.nnz;
+        a.cs = stream_evict_first(c, nnz * tb + (long long)h->n * (7 * tb + tb * h->kp)) ? 1 : 0;
+    }
     a.ncol = nc;
     a.b = b;
     a.ldb = ldb;
@@ -2212,7 +2227,14 @@ static asss_status solve_cluster(asss_handle* h, int tr, int size, int nc, const
     a.stats = h->cl_st.p;
     if (h->factored) ASSS_TRY((cl_dispatch<T, 3>(c, a, h->kp, size, count, nullptr)));
     else ASSS_TRY((cl_dispatch<T, 1>(c, a, h->kp, size, count, nullptr)));
+    int herr = 0;
+    if (size < 0) ASSS_CUDA(cudaMemcpyAsync(&herr, a.gb.err, sizeof(int), cudaMemcpyDeviceToHost, s));
     ASSS_CUDA(cudaMemcpyAsync(out, h->cl_st.p, sizeof(ClStat) * nc, cudaMemcpyDeviceToHost, s));
+    ASSS_CUDA(cudaStreamSynchronize(s));
+    if (herr) {
+        set_error("solve: a grid barrier wait exceeded its budget");
+        return (asss_status)herr;
+    }
     return ASSS_OK;
 }
 
@@ -2361,8 +2383,8 @@ static asss_status solve_common(asss_handle* h, int tr, int nrhs, const double* 
                           h->kp <= MRS_MULTI_KPMAX && !h->Q16.p && !h->factored;
     int cl = 0;
     ASSS_TRY(cluster_plan(h, nrhs, &cl));
-    // small and middling systems: whole solves in one launch, a cluster per column
-    for (int j0 = 0; cl > 0 && j0 < nrhs;) {
+    // whole solves in one launch: a cluster per column, or the whole grid column by column
+    for (int j0 = 0; cl != 0 && j0 < nrhs;) {
         constexpr int CHUNK = 16;   // columns staged at a time
         const int nc = nrhs - j0 < CHUNK ? nrhs - j0 : CHUNK;
         // b is copied (x may be the same memory), x staged when it is the host's

@@ -9,8 +9,9 @@
 // are exchanged through distributed shared memory, every CTA adds them in the same order and
 // takes the same decisions, and vectors that other CTAs read go through L2 around a cluster
 // barrier.  Several right-hand sides are as many clusters side by side (nine fit on the GPU).
-// Bound: the latency of a row's loads and of a synchronisation; above solve_cluster_limit's sizes
-// 16 SMs' share of the bandwidth and of the FP64 pipe (the rule there has both sides measured).
+// Bound: the latency of a row's loads and of a synchronisation; for larger systems 16 SMs' share
+// of the bandwidth and of the FP64 pipe, so those run the same code in grid scope (cluster_size
+// in asss.cu has both sides measured).
 #pragma once
 
 #include <algorithm>
@@ -94,6 +95,12 @@ struct ClArgs {
     double outer_tol, inner_tol;
     int outer_maxit, inner_maxit;
     ClStat* stats;
+    // grid scope: block partials (2 x [blocks][CL_XV]), barrier and its budget, evict-first loads of
+    // what is read once (the data of a step exceed L2)
+    double* part;
+    GridBarrier gb;
+    long long budget;
+    int cs;
 };
 
 // doubles of workspace per cluster
@@ -103,10 +110,11 @@ inline long long cl_work_doubles(int n, int halo, int restart, int tbytes) {
     return nd + (nt * tbytes + 7) / 8 + 64;
 }
 
-template <class T, int KP>
+template <class T, int KP, bool GRID>
 struct ClShared {
     using P2 = typename std::conditional<sizeof(T) == 4, float2, double>::type;
-    unsigned long long x[2][CL_MAX][CL_XV];   // exchanged block sums, written by the other CTAs
+    unsigned long long x[2][GRID ? 1 : CL_MAX][CL_XV];   // exchanged block sums, written by the other CTAs
+    double bsum[GRID ? CL_THREADS / (KP + 1) + 1 : 1][KP + 1];   // grid scope: parts of the cross-block sums
     T wsum[CL_WARPS][KP + 1];
     double wd[CL_WARPS][CL_REGV + 2];
     double bp[CL_XV], tot[CL_XV];
@@ -195,22 +203,26 @@ __device__ __noinline__ void cl_tri_sweep(E* vec, const E* own, const int2* rows
 // shared memory of every CTA, a phase gathers from there, stores its few rows into all CTAs
 // and crosses one cluster barrier, with the next colours' entries already on their way: about
 // 1 us a phase (mrs steps at 10^3 32 us instead of 129, at 24^3 51 instead of 227).
-template <class T, int KP, int FMT>
+// GRID: the same solve by one block per SM in a cooperative launch, for systems that a cluster's
+// share of the GPU would slow down: a synchronisation is the grid barrier, block sums go through L2
+// and every block adds them; what it saves against the launch-by-launch path is the launches and
+// the host's part.  A barrier that gives up ends the solve (dead).
+template <class T, int KP, int FMT, bool GRID>
 __global__ void __launch_bounds__(CL_THREADS, 1) k_solve_cl(const ClArgs<T> p) {
     constexpr int NT = CL_THREADS, NW = CL_WARPS, NV = KP + 1, KQ = KP > 0 ? KP : 1;
-    using Sh = ClShared<T, KP>;
+    using Sh = ClShared<T, KP, GRID>;
     using P2 = typename Sh::P2;
     extern __shared__ __align__(16) unsigned char s_dyn[];
     Sh& sh = *reinterpret_cast<Sh*>(s_dyn);
     double* H = reinterpret_cast<double*>(s_dyn + ((sizeof(Sh) + 15) & ~15));   // (restart + 1) x restart, column-major
     const int R = p.restart, n = p.n;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const int rank = (int)cl_rank(), C = (int)cl_size();
+    const int rank = GRID ? (int)blockIdx.x : (int)cl_rank(), C = GRID ? (int)gridDim.x : (int)cl_size();
     const int nsl = (n + 31) >> 5;
     const int rb = (int)((long long)nsl * rank / C) * 32;
     const int re = min(n, (int)((long long)nsl * (rank + 1) / C) * 32);
     const int nact = min(NW, max(re - rb + 31, 0) >> 5);   // warps that hold rows; the others' sums stay zero
-    double* base = p.work + (size_t)cl_id() * (size_t)p.work_stride;
+    double* base = p.work + (GRID ? (size_t)0 : (size_t)cl_id() * (size_t)p.work_stride);
     const long long nn = n;
     double *r = base, *rh = r + nn, *t1 = rh + nn, *t2 = t1 + nn, *wv = t2 + nn;
     double* V = wv + nn;
@@ -221,6 +233,15 @@ __global__ void __launch_bounds__(CL_THREADS, 1) k_solve_cl(const ClArgs<T> p) {
     T* P = fb + 3 * ys;
     T* z = P + 2 * nn;
 
+    bool dead = false;      // grid scope: a barrier gave up
+    unsigned gphase = 0;
+    auto sync_all = [&]() {
+        if constexpr (GRID) {
+            if (!dead) dead = !grid_sync_phase(p.gb, C, gphase++, p.budget);
+        } else {
+            cl_sync();
+        }
+    };
     for (int t = tid; t < p.ndiag && t < 64; t += NT) sh.off[t] = p.off[t];
     if (tid < 64) {
         const ClMat& M = tid < 16 ? p.op1 : tid < 32 ? p.op2 : tid < 48 ? p.Sm : p.Am;
@@ -273,7 +294,7 @@ __global__ void __launch_bounds__(CL_THREADS, 1) k_solve_cl(const ClArgs<T> p) {
                 s_jq[o] = make_int2(fa.J.rp[e], fa.J.rp[e + 1] - fa.J.rp[e]);
             }
     }
-    cl_sync();   // every CTA of the cluster runs: its shared memory may be written
+    sync_all();   // every CTA of the cluster runs: its shared memory may be written
 
     auto add_t = [](P2 a, P2 b) {
         if constexpr (sizeof(T) == 4) return df_add(a, b);
@@ -298,12 +319,32 @@ __global__ void __launch_bounds__(CL_THREADS, 1) k_solve_cl(const ClArgs<T> p) {
     auto exchange = [&](int cnt) {
         __syncthreads();
         const int buf = xphase++ & 1;
-        for (int t = tid; t < cnt * C; t += NT) {
-            const int q = t / cnt, v = t % cnt;
-            cl_store8(&sh.x[buf][rank][v], q, cl_bits(sh.bp[v]));
+        if constexpr (GRID) {
+            double* gp = p.part + (size_t)buf * CL_XV * C;
+            for (int v = tid; v < cnt; v += NT) gp[(size_t)rank * CL_XV + v] = sh.bp[v];
+            sync_all();
+            for (int v = warp; v < cnt; v += NW) {   // a warp a value
+                double t = 0.0;
+                for (int b0 = 0; b0 < C; b0 += 160) {
+                    double ld[5];
+#pragma unroll
+                    for (int u = 0; u < 5; ++u) {
+                        const int b = b0 + lane + 32 * u;
+                        ld[u] = b < C ? __ldcg(&gp[(size_t)b * CL_XV + v]) : 0.0;
+                    }
+                    t += (ld[0] + ld[1]) + (ld[2] + ld[3]) + ld[4];
+                }
+                t = warp_sum(t);
+                if (lane == 0) sh.tot[v] = t;
+            }
+        } else {
+            for (int t = tid; t < cnt * C; t += NT) {
+                const int q = t / cnt, v = t % cnt;
+                cl_store8(&sh.x[buf][rank][v], q, cl_bits(sh.bp[v]));
+            }
+            sync_all();
+            sum_rows(reinterpret_cast<const double*>(&sh.x[buf][0][0]), CL_XV, C, cnt, sh.tot);
         }
-        cl_sync();
-        sum_rows(reinterpret_cast<const double*>(&sh.x[buf][0][0]), CL_XV, C, cnt, sh.tot);
         __syncthreads();
     };
     // block sums of CNT accumulators into bp[slot..)
@@ -331,7 +372,8 @@ __global__ void __launch_bounds__(CL_THREADS, 1) k_solve_cl(const ClArgs<T> p) {
                 for (int u = 0; u < 8; ++u) {
                     const int d = d0 + u, j = i + off[d & 15];
                     const bool in = d < M.ndiag && j >= 0 && j < n;
-                    v[u] = in ? __ldg(&M.val[(size_t)d * n + i]) : 0.0;
+                    const double* vp = &M.val[(size_t)d * n + i];
+                    v[u] = in ? (GRID && p.cs ? __ldcs(vp) : __ldg(vp)) : 0.0;
                     xv[u] = in ? x[j] : 0.0;
                 }
 #pragma unroll
@@ -428,11 +470,61 @@ __global__ void __launch_bounds__(CL_THREADS, 1) k_solve_cl(const ClArgs<T> p) {
                     else a[q] = sh.wsum[q][v];
                 }
                 const unsigned long long bits = cl_bits(pair_tree(a, add_t));
-                for (int q = 0; q < C; ++q) cl_store8(&sh.x[buf][rank][v], q, bits);
+                if constexpr (GRID)
+                    reinterpret_cast<unsigned long long*>(p.part + (size_t)buf * CL_XV * C)[(size_t)rank * NV + v] = bits;
+                else
+                    for (int q = 0; q < C; ++q) cl_store8(&sh.x[buf][rank][v], q, bits);
             }
         }
-        cl_sync();
-        if (warp == 0) {
+        sync_all();
+        if constexpr (GRID) {
+            // as k_mrs: FP32 a warp every 16th block, a lane a value; FP64 a lane an addition
+            const P2* gp = reinterpret_cast<const P2*>(p.part + (size_t)buf * CL_XV * C);
+            P2* bs = reinterpret_cast<P2*>(&sh.bsum[0][0]);
+            constexpr int NG = sizeof(T) == 4 ? NW : NT / NV;
+            for (int t = tid; t < (sizeof(T) == 4 ? NT : NG * NV); t += NT) {
+                const int g = sizeof(T) == 4 ? warp : t / NV;
+                for (int v = sizeof(T) == 4 ? lane : t % NV; v < NV; v += sizeof(T) == 4 ? 32 : NV) {
+                    P2 acc{};
+                    for (int b0 = g; b0 < C; b0 += NG * 10) {
+                        P2 ld[10];
+#pragma unroll
+                        for (int u = 0; u < 10; ++u) {
+                            const int b = b0 + u * NG;
+                            ld[u] = b < C ? __ldcg(&gp[(size_t)b * NV + v]) : P2{};
+                        }
+#pragma unroll
+                        for (int u = 0; u < 10; ++u)
+                            if (b0 + u * NG < C) acc = add_t(acc, ld[u]);
+                    }
+                    bs[g * NV + v] = acc;
+                }
+            }
+            __syncthreads();
+            if constexpr (sizeof(T) == 4) {
+                if (warp == 0) {
+                    for (int v = lane; v < NV; v += 32) {
+                        P2 a[NW];
+#pragma unroll
+                        for (int q = 0; q < NW; ++q) a[q] = bs[q * NV + v];
+                        const P2 t = pair_tree(a, add_t);
+                        sh.red[v] = t.x + t.y;
+                    }
+                    __syncwarp();
+                }
+            } else {
+                for (int t0 = 0; t0 < 4 * NV; t0 += NT) {
+                    const int t = t0 + tid, v = t >> 2;
+                    double a = 0.0;
+                    if (v < NV)
+                        for (int g = t & 3; g < NG && g < C; g += 4) a += sh.bsum[g][v];
+                    a += __shfl_xor_sync(0xffffffffu, a, 1);
+                    a += __shfl_xor_sync(0xffffffffu, a, 2);
+                    if (v < NV && (t & 3) == 0) sh.red[v] = (T)a;
+                }
+                __syncthreads();
+            }
+        } else if (warp == 0) {
             for (int v = lane; v < NV; v += 32) {
                 P2 a[CL_MAX];
 #pragma unroll
@@ -498,11 +590,12 @@ __global__ void __launch_bounds__(CL_THREADS, 1) k_solve_cl(const ClArgs<T> p) {
             P[nn + i] = (T)0;
             tacc[0] += b * b;
             T q[KQ];
-            load_qrow<T, KP, q_blocked<T>(true)>(p.Q, i, q);
+            load_qrow<T, KP, q_blocked<T>(true)>(p.Q, i, q, GRID && p.cs);
 #pragma unroll
             for (int a = 0; a < KP; ++a) tacc[1 + a] += q[a] * b;
         }
         mrs_sums(tacc);
+        if (GRID && dead) return 0;
         if (warp == 0) {
             if (lane == 0) {
                 MrsScalars<T>& c = sh.sc;
@@ -569,7 +662,7 @@ __global__ void __launch_bounds__(CL_THREADS, 1) k_solve_cl(const ClArgs<T> p) {
                     }
                 }
                 T q[KQ];
-                load_qrow<T, KP, q_blocked<T>(true)>(p.Q, i, q);
+                load_qrow<T, KP, q_blocked<T>(true)>(p.Q, i, q, GRID && p.cs);
                 T dq = (T)0;
 #pragma unroll
                 for (int a = 0; a < KP; ++a) dq += q[a] * sh.u[a];
@@ -585,6 +678,7 @@ __global__ void __launch_bounds__(CL_THREADS, 1) k_solve_cl(const ClArgs<T> p) {
                 }
             }
             mrs_sums(tacc);
+            if (GRID && dead) break;
             if (warp == 0) {
                 MrsScalars<T>& c = sh.sc;
                 // beta and 1 / beta in lane 0, theta and 1 / theta in lane 1
@@ -693,7 +787,7 @@ __global__ void __launch_bounds__(CL_THREADS, 1) k_solve_cl(const ClArgs<T> p) {
         return wv[i] - s;
     };
 
-    for (int col = (int)cl_id(); col < p.ncol; col += (int)cl_count()) {
+    for (int col = GRID ? 0 : (int)cl_id(); col < p.ncol; col += GRID ? 1 : (int)cl_count()) {
         const double* b = p.b + (size_t)col * p.ldb;
         double* x = p.x + (size_t)col * p.ldx;
         unsigned long long ns_inner = 0, ns_op = 0, ns_orth = 0;
@@ -741,11 +835,11 @@ __global__ void __launch_bounds__(CL_THREADS, 1) k_solve_cl(const ClArgs<T> p) {
                 }
             } else {
                 for (int i = rb + tid; i < re; i += NT) t1[i] = p.dc[i] * r[i];
-                cl_sync();
+                sync_all();
                 for (int i = rb + tid; i < re; i += NT) rs[i] = p.w[i] * mat_row(p.Sm, sh.moff[2], t1, i);
             }
             if constexpr (FMT == 3) {
-                cl_sync();
+                sync_all();
                 apply_F(rs, rh);
             }
             const double eta = fmin(0.5, 0.5 * p.outer_tol * bn / rn);
@@ -765,7 +859,7 @@ __global__ void __launch_bounds__(CL_THREADS, 1) k_solve_cl(const ClArgs<T> p) {
                     ++solves;
                     // z_j = z - Y (U^T z)
                     if (p.r > 0 && p.m > 0) {
-                        cl_sync();   // z complete: U_r^T z gathers from every CTA's rows
+                        sync_all();   // z complete: U_r^T z gathers from every CTA's rows
                         for (int a = tid; a < p.r; a += NT) {
                             double v;
                             if (!p.neg2) {
@@ -786,7 +880,7 @@ __global__ void __launch_bounds__(CL_THREADS, 1) k_solve_cl(const ClArgs<T> p) {
                             const float4* y4 = reinterpret_cast<const float4*>(yr);
 #pragma unroll 5
                             for (int c = 0; c < (p.m >> 2); ++c) {
-                                const float4 v = __ldg(y4 + c);
+                                const float4 v = GRID && p.cs ? __ldcs(y4 + c) : __ldg(y4 + c);
                                 acc += (T)v.x * sh.wv[4 * c] + (T)v.y * sh.wv[4 * c + 1] + (T)v.z * sh.wv[4 * c + 2] +
                                        (T)v.w * sh.wv[4 * c + 3];
                             }
@@ -796,19 +890,19 @@ __global__ void __launch_bounds__(CL_THREADS, 1) k_solve_cl(const ClArgs<T> p) {
                         zj[i] = (double)(z[i] - acc);
                     }
                     // w = A_cal z_j
-                    cl_sync();
+                    sync_all();
                     const unsigned long long tm2 = now();
                     if constexpr (FMT == 3) {   // F A^ G z_j
                         apply_G(zj, t2);
-                        cl_sync();
+                        sync_all();
                     }
                     const double* zin = FMT == 3 ? t2 : zj;
                     for (int i = rb + tid; i < re; i += NT) t1[i] = mat_row(p.op1, sh.moff[0], zin, i);
-                    cl_sync();
+                    sync_all();
                     double* wout = FMT == 3 ? t2 : wv;
                     for (int i = rb + tid; i < re; i += NT) wout[i] = mat_row(p.op2, sh.moff[1], t1, i);
                     if constexpr (FMT == 3) {
-                        cl_sync();
+                        sync_all();
                         apply_F(t2, wv);
                     }
                     const unsigned long long tm3 = now();
@@ -919,7 +1013,7 @@ __global__ void __launch_bounds__(CL_THREADS, 1) k_solve_cl(const ClArgs<T> p) {
                     ns_orth += tm4 - tm3;
                     ++orths;
                     steps = j + 1;
-                    if (sh.stop) break;
+                    if (sh.stop || (GRID && dead)) break;
                 }
                 // y from the triangular system, column by column
                 if (warp == 0) {
@@ -955,7 +1049,7 @@ __global__ void __launch_bounds__(CL_THREADS, 1) k_solve_cl(const ClArgs<T> p) {
                     x[q] += p.dr[q] * p.w[i] * dy;
                 }
             }
-            cl_sync();
+            sync_all();
             if constexpr (FMT == 3) {   // G dy instead of W dy
                 apply_G(t2, t1);
                 if (p.tr)
@@ -963,16 +1057,17 @@ __global__ void __launch_bounds__(CL_THREADS, 1) k_solve_cl(const ClArgs<T> p) {
                         const int q = p.perm ? p.perm[i] : i;
                         x[q] += p.dr[q] * t1[i];
                     }
-                cl_sync();
+                sync_all();
             }
             if (!p.tr) {
                 for (int i = rb + tid; i < re; i += NT) x[i] += p.dc[i] * mat_row(p.Sm, sh.moff[2], t1, i);
-                cl_sync();
+                sync_all();
             }
             for (int i = rb + tid; i < re; i += NT) r[i] = b[i] - mat_row(p.Am, sh.moff[3], x, i);
             outer += steps;
             ++cycles;
             rn = sqrt(norm2(r));
+            if (GRID && dead) status = ASSS_ERR_TIMEOUT;
         }
         if (rank == 0 && tid == 0) {
             ClStat st;
@@ -990,7 +1085,8 @@ __global__ void __launch_bounds__(CL_THREADS, 1) k_solve_cl(const ClArgs<T> p) {
             st.relres = relres;
             p.stats[col] = st;
         }
-        cl_sync();   // the column is done before the cluster's buffers are reused
+        sync_all();   // the column is done before its buffers are reused
+        if (GRID && dead) return;
     }
 }
 
@@ -1000,7 +1096,7 @@ __global__ void __launch_bounds__(CL_THREADS, 1) k_solve_cl(const ClArgs<T> p) {
 // clusters of `size` CTAs that can be resident at once (0: none fits)
 template <class T, int KP, int FMT>
 static asss_status cl_clusters(int size, size_t smem, int* count) {
-    const void* fn = (const void*)k_solve_cl<T, KP, FMT>;
+    const void* fn = (const void*)k_solve_cl<T, KP, FMT, false>;
     ASSS_TRY(raise_dynamic_smem(fn, (int)smem));
     if (size > 8) ASSS_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
     cudaLaunchConfig_t cfg = {};
@@ -1026,7 +1122,7 @@ template <class T, int KP, int FMT>
 static asss_status cl_run(const Ctx& c, const ClArgs<T>& a, int size, int count, int* counts) {
     ClArgs<T> b = a;
     auto bytes = [&](int sz) -> size_t {
-        size_t smem = ((sizeof(ClShared<T, KP>) + 15) & ~(size_t)15) +
+        size_t smem = ((sizeof(ClShared<T, KP, false>) + 15) & ~(size_t)15) +
                       sizeof(double) * (size_t)(a.restart + 1) * (size_t)a.restart;
         if (FMT == 3) {
             b.fac.own_max = a.n / sz + a.fac.ncol + 1;
@@ -1054,7 +1150,23 @@ static asss_status cl_run(const Ctx& c, const ClArgs<T>& a, int size, int count,
     at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
     cfg.attrs = at;
     cfg.numAttrs = 1;
-    ASSS_CUDA(cudaLaunchKernelEx(&cfg, k_solve_cl<T, KP, FMT>, b));
+    ASSS_CUDA(cudaLaunchKernelEx(&cfg, k_solve_cl<T, KP, FMT, false>, b));
+    count_launch();
+    return ASSS_OK;
+}
+
+// grid scope: a cooperative launch of one block per SM (size < 0)
+template <class T, int KP>
+static asss_status cl_run_grid(const Ctx& c, const ClArgs<T>& a) {
+    const size_t smem = ((sizeof(ClShared<T, KP, true>) + 15) & ~(size_t)15) +
+                        sizeof(double) * (size_t)(a.restart + 1) * (size_t)a.restart;
+    const void* fn = (const void*)k_solve_cl<T, KP, 1, true>;
+    ASSS_TRY(raise_dynamic_smem(fn, (int)smem));
+    const int need = cdiv(a.n, 32);
+    ClArgs<T> b = a;
+    void* args[] = {&b};
+    ASSS_CUDA(cudaLaunchCooperativeKernel(fn, dim3(c.sms < need ? c.sms : need), dim3(CL_THREADS), args, smem,
+                                          c.stream));
     count_launch();
     return ASSS_OK;
 }
@@ -1064,6 +1176,7 @@ asss_status cl_dispatch(const Ctx& c, const ClArgs<T>& a, int kp, int size, int 
     switch (kp) {
 #define ASSS_CL_CASE(KPV) \
     case KPV:             \
+        if constexpr (FMT == 1) { if (size < 0) return cl_run_grid<T, KPV>(c, a); } \
         return cl_run<T, KPV, FMT>(c, a, size, count, counts);
         ASSS_CL_CASE(0)
         ASSS_CL_CASE(4)

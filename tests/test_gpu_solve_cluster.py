@@ -1,4 +1,4 @@
-"""Cluster-scope solves against the launch-by-launch path (which ASSS_TRACE asks for) on every
+"""Cluster- and grid-scope solves against the launch-by-launch path (which ASSS_TRACE asks for) on every
 form that takes them: both inner precisions, forward and adjoint, one to seventeen columns
 (chunks of sixteen), fewer rows than a cluster has CTAs, a row permutation, matrices without a
 diagonal copy, negative pivots, and right-hand sides and limits that end a solve early.  Same
@@ -40,7 +40,7 @@ def banded(n, offsets, seed):
 
 @pytest.mark.parametrize("precision", ["mixed", "fp64"])
 @pytest.mark.parametrize("side,nrhs,block", [(2, 1, False), (5, 2, False), (7, 17, False), (11, 3, True), (19, 1, False),
-                                             (19, 9, True)])
+                                             (19, 9, True), (24, 1, False), (31, 2, True)])
 def test_columns_match(pkg, monkeypatch, side, nrhs, block, precision):  # noqa: F811
     A = dissipative_hamiltonian_3d(side=side, seed=side, with_rhs=False)[0]
     n = A.shape[0]
@@ -55,8 +55,9 @@ def test_columns_match(pkg, monkeypatch, side, nrhs, block, precision):  # noqa:
 
 
 @pytest.mark.parametrize("precision", ["mixed", "fp64"])
-def test_adjoint_matches(pkg, monkeypatch, precision):  # noqa: F811
-    A = dissipative_hamiltonian_3d(side=13, seed=2, with_rhs=False)[0]
+@pytest.mark.parametrize("side", [13, 25])
+def test_adjoint_matches(pkg, monkeypatch, side, precision):  # noqa: F811
+    A = dissipative_hamiltonian_3d(side=side, seed=2, with_rhs=False)[0]
     rng = np.random.default_rng(1)
     g, x = rng.standard_normal(A.shape[0]), rng.standard_normal(A.shape[0])
     s = pkg.Solver(A, **OPTS[precision])
@@ -67,8 +68,8 @@ def test_adjoint_matches(pkg, monkeypatch, precision):  # noqa: F811
 
 
 @pytest.mark.parametrize("precision", ["mixed", "fp64"])
-def test_permutation_and_csr_operators_match(pkg, monkeypatch, precision):  # noqa: F811
-    n = 1500
+@pytest.mark.parametrize("n", [1500, 15001])
+def test_permutation_and_csr_operators_match(pkg, monkeypatch, n, precision):  # noqa: F811
     offs = [o for o in range(-11, 12) if o and o != 4]      # 22 diagonals: no diagonal copy of Abar
     Ab = banded(n, offs, 3)
     perm = np.random.default_rng(4).permutation(n)
@@ -86,10 +87,12 @@ def test_permutation_and_csr_operators_match(pkg, monkeypatch, precision):  # no
 
 
 @pytest.mark.parametrize("precision", ["mixed", "fp64"])
-def test_negative_pivots_match(pkg, monkeypatch, precision):  # noqa: F811
-    n = 700
+@pytest.mark.parametrize("n,loads", [(700, ""), (14001, ""), (14001, "1")])
+def test_negative_pivots_match(pkg, monkeypatch, n, loads, precision):  # noqa: F811
+    if loads:
+        monkeypatch.setenv("ASSS_FORCE_EVICT_FIRST", loads)
     A = banded(n, (-9, -2, 3), 6).tolil()
-    for i in (0, 5, 333, 699):
+    for i in (0, 5, 333, n - 1):
         A[i, i] = -A[i, i]
     A = A.tocsr()
     s = pkg.Solver(A, s_pattern=pattern_diagonal(n), s_values=np.ones(n), lls_maxit=0, **OPTS[precision])
@@ -103,11 +106,13 @@ def test_negative_pivots_match(pkg, monkeypatch, precision):  # noqa: F811
     close(la, lb)
 
 
+@pytest.mark.parametrize("side", [9, 24])
 @pytest.mark.parametrize("what", ["zero", "nan", "inf", "maxit", "restart", "tol_one", "in_place"])
-def test_early_ends_match(pkg, monkeypatch, what):  # noqa: F811
-    A = dissipative_hamiltonian_3d(side=9, seed=9, with_rhs=False)[0]
+def test_early_ends_match(pkg, monkeypatch, what, side):  # noqa: F811
+    A = dissipative_hamiltonian_3d(side=side, seed=9, with_rhs=False)[0]
     n = A.shape[0]
-    opts = dict(OPTS["mixed"], inner_maxit=2)
+    # an iterate that a limit cut off carries the FP32 roundings of its inner solves: FP64 there
+    opts = dict(OPTS["fp64" if what == "maxit" else "mixed"], inner_maxit=2)
     opts.update({"maxit": dict(outer_maxit=3), "restart": dict(restart=2), "tol_one": dict(outer_tol=1.0)}.get(what, {}))
     b = np.random.default_rng(9).standard_normal(n)
     b = {"zero": 0.0 * b, "nan": np.where(np.arange(n) == 5, np.nan, b), "inf": np.where(np.arange(n) == 5, np.inf, b)
