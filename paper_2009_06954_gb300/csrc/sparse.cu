@@ -410,6 +410,8 @@ asss_status transpose_csr(const DCsr& a, DCsr& t, DBuf<int>* srcpos, cudaStream_
 // ---------------------------------------------------------------------------
 // CSR SpMV (FP64): y = A x, LANES threads per row
 // ---------------------------------------------------------------------------
+// Rows above 16 entries a lane are taken by the whole warp: with heavy-tailed rows (mean 16, up to
+// 512) one group's serial chain of gathers held up the product (n = 20011, two products: 42 -> 29 us).
 template <int LANES>
 __global__ void k_spmv(int n, const int* __restrict__ rp, const int* __restrict__ ci,
                        const double* __restrict__ v, const double* __restrict__ x,
@@ -420,8 +422,25 @@ __global__ void k_spmv(int n, const int* __restrict__ rp, const int* __restrict_
     // no early exit: every lane of the warp takes part in the shuffles below
     const bool live = row < n;
     double acc = 0.0;
-    if (live)
-        for (int e = rp[row] + sub; e < rp[row + 1]; e += LANES) acc += v[e] * __ldg(&x[ci[e]]);
+    const int e0 = live ? rp[row] : 0, e1 = live ? rp[row + 1] : 0;
+    const bool big = LANES < 32 && e1 - e0 > 16 * LANES;
+    if (!big) {
+#pragma unroll 4
+        for (int e = e0 + sub; e < e1; e += LANES) acc += v[e] * __ldg(&x[ci[e]]);
+    }
+    if constexpr (LANES < 32) {
+        unsigned todo = __ballot_sync(0xffffffffu, big && sub == 0);
+        while (todo) {
+            const int src = __ffs(todo) - 1;
+            todo &= todo - 1;
+            const int b0 = __shfl_sync(0xffffffffu, e0, src), b1 = __shfl_sync(0xffffffffu, e1, src);
+            double t = 0.0;
+#pragma unroll 4
+            for (int e = b0 + (threadIdx.x & 31); e < b1; e += 32) t += v[e] * __ldg(&x[ci[e]]);
+            t = warp_sum(t);
+            if ((threadIdx.x & 31) == src) acc = t;
+        }
+    }
 #pragma unroll
     for (int o = LANES / 2; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o, LANES);
     if (live && sub == 0) y[row] = lscale ? lscale[row] * acc : acc;
@@ -558,18 +577,24 @@ asss_status spmv(const DCsr& A, const double* x, double* y, const double* lscale
         ASSS_CHECK_LAUNCH();
         return ASSS_OK;
     }
-    double mean = n ? (double)A.nnz / n : 0;
-    int threads = 256;
-    if (mean <= 6) {
-        k_spmv<1><<<cdiv(n, threads), threads, 0, s>>>(n, A.rp.p, A.ci.p, A.v.p, x, y, lscale);
-    } else if (mean <= 12) {
-        k_spmv<2><<<cdiv((int64_t)n * 2, threads), threads, 0, s>>>(n, A.rp.p, A.ci.p, A.v.p, x, y, lscale);
-    } else if (mean <= 24) {
-        k_spmv<4><<<cdiv((int64_t)n * 4, threads), threads, 0, s>>>(n, A.rp.p, A.ci.p, A.v.p, x, y, lscale);
-    } else if (mean <= 64) {
-        k_spmv<8><<<cdiv((int64_t)n * 8, threads), threads, 0, s>>>(n, A.rp.p, A.ci.p, A.v.p, x, y, lscale);
-    } else {
-        k_spmv<32><<<cdiv((int64_t)n * 32, threads), threads, 0, s>>>(n, A.rp.p, A.ci.p, A.v.p, x, y, lscale);
+    // lanes a row by the mean row length; a matrix that leaves most of the GPU's threads idle takes
+    // more of them, down to about one entry a lane (n = 20011, mean 16, two products:
+    // 29 -> 27 us)
+    const double mean = n ? (double)A.nnz / n : 0;
+    int lanes = mean <= 6 ? 1 : mean <= 12 ? 2 : mean <= 24 ? 4 : mean <= 64 ? 8 : 32;
+    constexpr int64_t ONE_WAVE = 300000;   // threads resident on 148 SMs or more
+    while (lanes < 32 && lanes < mean && (int64_t)n * lanes * 2 <= ONE_WAVE * 2) lanes *= 2;
+    const int threads = 256, blocks = cdiv((int64_t)n * lanes, threads);
+    switch (lanes) {
+#define ASSS_SPMV_CASE(L) \
+    case L: k_spmv<L><<<blocks, threads, 0, s>>>(n, A.rp.p, A.ci.p, A.v.p, x, y, lscale); break;
+        ASSS_SPMV_CASE(1)
+        ASSS_SPMV_CASE(2)
+        ASSS_SPMV_CASE(4)
+        ASSS_SPMV_CASE(8)
+        ASSS_SPMV_CASE(16)
+        ASSS_SPMV_CASE(32)
+#undef ASSS_SPMV_CASE
     }
     ASSS_CHECK_LAUNCH();
     return ASSS_OK;
