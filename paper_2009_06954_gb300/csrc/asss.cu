@@ -644,11 +644,14 @@ struct asss_handle {
     // the clusters, staging of the columns and statistics
     int cl_counts[CL_NSIZES] = {-1, -1, -1, -1};
     DBuf<double> cl_work, cl_b, cl_x;
-    DBuf<ClStat> cl_st;
+    static constexpr int CL_CHUNK = 16;   // columns of a launch
+    ClStat* cl_st = nullptr;   // pinned, CL_CHUNK entries
+    unsigned cl_phase = 0;     // barriers passed on cl_bar
     DBuf<double> cl_part;      // grid scope: block partials, barrier and status
     DBuf<unsigned> cl_bar;
     ~asss_handle() {
         if (mw) mrs_work_destroy(mw);
+        if (cl_st) cudaFreeHost(cl_st);
     }
 };
 
@@ -2189,10 +2192,11 @@ static asss_status cluster_plan(asss_handle* h, int nrhs, int* size) {
     return ASSS_OK;
 }
 
-// nc columns of a solve by clusters of `size` CTAs, x on the device; out: one entry per column
+// enqueues nc columns of a solve (size: see cluster_size), b and x on the device and apart; their
+// statistics are in h->cl_st once the stream is synchronised
 template <class T>
-static asss_status solve_cluster(asss_handle* h, int tr, int size, int nc, const double* b, int64_t ldb, double* x, int64_t ldx,
-                                 ClStat* out) {
+static asss_status solve_cluster(asss_handle* h, int tr, int size, int nc, const double* b, int64_t ldb, double* x,
+                                 int64_t ldx) {
     NvtxRange nv_(tr ? "asss:adjoint-solve" : "asss:solve");
     const Ctx& c = h->ctx;
     cudaStream_t s = c.stream;
@@ -2206,8 +2210,12 @@ static asss_status solve_cluster(asss_handle* h, int tr, int size, int nc, const
     if (size < 0) {   // grid scope
         const int64_t np = 2LL * CL_XV * c.sms;
         if (h->cl_part.n < np) ASSS_TRY(h->cl_part.alloc(np));
-        if (!h->cl_bar.p) ASSS_TRY(h->cl_bar.alloc(2));
-        ASSS_CUDA(cudaMemsetAsync(h->cl_bar.p, 0, 2 * sizeof(unsigned), s));   // arrivals and status
+        if (!h->cl_bar.p || h->cl_phase == 0 || h->cl_phase > 0x1000000u) {   // (152 arrivals a barrier in 32 bits)
+            if (!h->cl_bar.p) ASSS_TRY(h->cl_bar.alloc(2));
+            ASSS_CUDA(cudaMemsetAsync(h->cl_bar.p, 0, 2 * sizeof(unsigned), s));   // arrivals and status
+            h->cl_phase = 0;
+        }
+        a.phase0 = h->cl_phase;
         a.part = h->cl_part.p;
         a.gb.count = h->cl_bar.p;
         a.gb.err = reinterpret_cast<int*>(h->cl_bar.p + 1);
@@ -2222,19 +2230,11 @@ static asss_status solve_cluster(asss_handle* h, int tr, int size, int nc, const
     a.ldx = ldx;
     a.work_stride = cl_work_doubles(h->n, a.halo, o.restart, (int)sizeof(T));
     if (h->cl_work.n < a.work_stride * count) ASSS_TRY(h->cl_work.alloc(a.work_stride * count));
-    if (h->cl_st.n < nc) ASSS_TRY(h->cl_st.alloc(nc));
+    if (!h->cl_st) ASSS_CUDA(cudaMallocHost((void**)&h->cl_st, sizeof(ClStat) * asss_handle::CL_CHUNK));
     a.work = h->cl_work.p;
-    a.stats = h->cl_st.p;
+    a.stats = h->cl_st;
     if (h->factored) ASSS_TRY((cl_dispatch<T, 3>(c, a, h->kp, size, count, nullptr)));
     else ASSS_TRY((cl_dispatch<T, 1>(c, a, h->kp, size, count, nullptr)));
-    int herr = 0;
-    if (size < 0) ASSS_CUDA(cudaMemcpyAsync(&herr, a.gb.err, sizeof(int), cudaMemcpyDeviceToHost, s));
-    ASSS_CUDA(cudaMemcpyAsync(out, h->cl_st.p, sizeof(ClStat) * nc, cudaMemcpyDeviceToHost, s));
-    ASSS_CUDA(cudaStreamSynchronize(s));
-    if (herr) {
-        set_error("solve: a grid barrier wait exceeded its budget");
-        return (asss_status)herr;
-    }
     return ASSS_OK;
 }
 
@@ -2385,33 +2385,46 @@ static asss_status solve_common(asss_handle* h, int tr, int nrhs, const double* 
     ASSS_TRY(cluster_plan(h, nrhs, &cl));
     // whole solves in one launch: a cluster per column, or the whole grid column by column
     for (int j0 = 0; cl != 0 && j0 < nrhs;) {
-        constexpr int CHUNK = 16;   // columns staged at a time
-        const int nc = nrhs - j0 < CHUNK ? nrhs - j0 : CHUNK;
-        // b is copied (x may be the same memory), x staged when it is the host's
-        if (h->cl_b.n < (int64_t)nc * n) ASSS_TRY(h->cl_b.alloc((int64_t)nc * n));
+        const int nc = nrhs - j0 < asss_handle::CL_CHUNK ? nrhs - j0 : asss_handle::CL_CHUNK;
+        const double* b0 = b + (size_t)j0 * ldb;
+        double* x0 = x + (size_t)j0 * ldx;
+        // the kernel reads b to the end, so it is staged where x overlaps it, and what is the host's
+        const bool apart = b0 + (size_t)(nc - 1) * ldb + n <= x0 || x0 + (size_t)(nc - 1) * ldx + n <= b0;
+        const double* bt = b0;
+        int64_t ldbt = ldb;
+        if (!bdev || !apart) {
+            if (h->cl_b.n < (int64_t)nc * n) ASSS_TRY(h->cl_b.alloc((int64_t)nc * n));
+            const cudaMemcpyKind kind = bdev ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice;
+            if (nc == 1) ASSS_CUDA(cudaMemcpyAsync(h->cl_b.p, b0, sizeof(double) * n, kind, s));
+            else
+                ASSS_CUDA(cudaMemcpy2DAsync(h->cl_b.p, sizeof(double) * n, b0, sizeof(double) * ldb, sizeof(double) * n,
+                                            nc, kind, s));
+            bt = h->cl_b.p;
+            ldbt = n;
+        }
         if (!xdev && h->cl_x.n < (int64_t)nc * n) ASSS_TRY(h->cl_x.alloc((int64_t)nc * n));
-        if (nc == 1)
-            ASSS_CUDA(cudaMemcpyAsync(h->cl_b.p, b + (size_t)j0 * ldb, sizeof(double) * n,
-                                      bdev ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice, s));
-        else
-            ASSS_CUDA(cudaMemcpy2DAsync(h->cl_b.p, sizeof(double) * n, b + (size_t)j0 * ldb, sizeof(double) * ldb,
-                                        sizeof(double) * n, nc,
-                                        bdev ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice, s));
-        double* xt = xdev ? x + (size_t)j0 * ldx : h->cl_x.p;
+        double* xt = xdev ? x0 : h->cl_x.p;
         const int64_t ldt = xdev ? ldx : n;
-        ClStat cs[CHUNK];
-        if (h->opt.precision == ASSS_PREC_MIXED)
-            ASSS_TRY(solve_cluster<float>(h, tr, cl, nc, h->cl_b.p, n, xt, ldt, cs));
-        else
-            ASSS_TRY(solve_cluster<double>(h, tr, cl, nc, h->cl_b.p, n, xt, ldt, cs));
+        if (h->opt.precision == ASSS_PREC_MIXED) ASSS_TRY(solve_cluster<float>(h, tr, cl, nc, bt, ldbt, xt, ldt));
+        else ASSS_TRY(solve_cluster<double>(h, tr, cl, nc, bt, ldbt, xt, ldt));
         if (!xdev && nc == 1)
-            ASSS_CUDA(cudaMemcpyAsync(x + (size_t)j0 * ldx, xt, sizeof(double) * n, cudaMemcpyDeviceToHost, s));
+            ASSS_CUDA(cudaMemcpyAsync(x0, xt, sizeof(double) * n, cudaMemcpyDeviceToHost, s));
         else if (!xdev)
-            ASSS_CUDA(cudaMemcpy2DAsync(x + (size_t)j0 * ldx, sizeof(double) * ldx, xt, sizeof(double) * n,
-                                        sizeof(double) * n, nc, cudaMemcpyDeviceToHost, s));
+            ASSS_CUDA(cudaMemcpy2DAsync(x0, sizeof(double) * ldx, xt, sizeof(double) * n, sizeof(double) * n, nc,
+                                        cudaMemcpyDeviceToHost, s));
         if (tr && xfwd && dA)
             for (int t = 0; t < nc; ++t) ASSS_TRY(grad_A(h, j0 + t, xt + (size_t)t * ldt, xfwd, ldxf, dA));
         ASSS_CUDA(cudaStreamSynchronize(s));
+        const ClStat* cs = h->cl_st;
+        if (cl < 0) {
+            h->cl_phase = cs[nc - 1].phase;
+            for (int t = 0; t < nc; ++t)
+                if (cs[t].status == ASSS_ERR_TIMEOUT) {
+                    h->cl_phase = 0;   // the barrier starts anew
+                    set_error("solve: a grid barrier wait exceeded its budget");
+                    return ASSS_ERR_TIMEOUT;
+                }
+        }
         for (int t = 0; t < nc; ++t) {
             const asss_stats prev = lst;
             cluster_stats(h, tr, cs[t], &lst);

@@ -64,6 +64,7 @@ struct ClStat {
     long long inner_its, orth_vecs;
     unsigned long long ns_inner, ns_op, ns_orth;
     double relres;
+    unsigned phase;   // grid scope: barriers passed on the counter
 };
 
 template <class T>
@@ -94,7 +95,8 @@ struct ClArgs {
     long long work_stride;
     double outer_tol, inner_tol;
     int outer_maxit, inner_maxit;
-    ClStat* stats;
+    ClStat* stats;            // pinned host memory, read after the stream is synchronised
+    unsigned phase0;          // grid scope: barriers passed before this launch
     // grid scope: block partials (2 x [blocks][CL_XV]), barrier and its budget, evict-first loads of
     // what is read once (the data of a step exceed L2)
     double* part;
@@ -234,7 +236,7 @@ __global__ void __launch_bounds__(CL_THREADS, 1) k_solve_cl(const ClArgs<T> p) {
     T* z = P + 2 * nn;
 
     bool dead = false;      // grid scope: a barrier gave up
-    unsigned gphase = 0;
+    unsigned gphase = p.phase0;
     auto sync_all = [&]() {
         if constexpr (GRID) {
             if (!dead) dead = !grid_sync_phase(p.gb, C, gphase++, p.budget);
@@ -804,6 +806,7 @@ __global__ void __launch_bounds__(CL_THREADS, 1) k_solve_cl(const ClArgs<T> p) {
             status = ASSS_ERR_BREAKDOWN;
             relres = 1.0;
         }
+        if (GRID && dead) status = ASSS_ERR_TIMEOUT;
         // a right-hand side of norm 0, infinity or NaN counts the one inner solve of zero steps
         // that the launch-by-launch path has enqueued by the time it knows
         if (!(bn > 0.0 && bn < INFINITY) && p.outer_tol < 1.0 && p.outer_maxit > 0) solves = 1;
@@ -1083,6 +1086,7 @@ __global__ void __launch_bounds__(CL_THREADS, 1) k_solve_cl(const ClArgs<T> p) {
             st.ns_op = ns_op;
             st.ns_orth = ns_orth;
             st.relres = relres;
+            st.phase = gphase + 1;   // with the column's last barrier, below
             p.stats[col] = st;
         }
         sync_all();   // the column is done before its buffers are reused
