@@ -8,6 +8,12 @@
 // changes is the scope: block reductions and __syncthreads instead of grid
 // barriers and kernel launches, so small systems do not pay a launch or a grid
 // synchronisation per step.
+// 32 systems of sides 10..32 with 32 columns each take 10.2 ms (512 threads, 2 CTAs per SM):
+// 6.0 in mrs (loads of Q and y from L2, and the step's block reduction), 1.6 in Gram-Schmidt
+// and 1.2 in the operator (FP64 pipe).  With a shuffle tree per sum, five Gram-Schmidt sweeps
+// and a division per row it took 11.0; 24 systems of sides 10..14 1.31 -> 1.14, 8 systems of
+// sides 12..20 with 4 columns 1.04 -> 0.95.  Two columns a CTA, sharing the reads of Q, were
+// slower (12.4 ms): half the warps to hide the latency.
 #pragma once
 
 #include <cuda_bf16.h>
@@ -21,6 +27,7 @@ namespace asss {
 constexpr int BMAX_WARPS = 32;
 constexpr int BKPMAX = 32;   // largest padded Lanczos width handled by the batched kernel
 constexpr int BMMAX = 320;   // largest SMW rank k + r
+constexpr int BGV = 6;       // Krylov vectors whose dot products and updates share one sweep
 
 
 // scalar state of the FP32 inner recurrence (kept in FP32 like its vectors: the
@@ -37,8 +44,7 @@ struct BatchShared {
     BatchMat M;
     float red[BKPMAX + 1];
     float wsum[BMAX_WARPS][BKPMAX + 1];
-    double tmp[BMAX_WARPS + 1];
-    double wd[BMAX_WARPS][4];
+    double wd[BMAX_WARPS][BGV + 2], gs[BGV + 2];   // warps' and block's FP64 sums (bsums)
     float u[BKPMAX];
     float cf[12];
     float alpha[BKPMAX];
@@ -51,60 +57,59 @@ struct BatchShared {
     // Q^T p of the last two directions, Q^T z, and step j's nu, delta, 1/theta, xcoef
     float qty[BKPMAX], qtp[2][BKPMAX], qtx[BKPMAX], pq[4];
     BScalars sc;
+    double nrm[2];   // |w|^2 after the first projection, 1 / |w| after the second
     unsigned long long prof[BATCH_NPROF + 1];  // phase times of this CTA (thread 0), last stamp
     int item;
     int steps;
     int brk;
 };
 
-// sum over the block of one double per thread; every thread gets the result
-__device__ __forceinline__ double bsum(double v, BatchShared& sh) {
+// Block sums of N <= 8 doubles a thread into sh.gs.  The FP64 pipe takes a warp instruction
+// every 16 cycles, so the adds count: the folded warp sums take 9 of them for 7 values (a
+// tree a value: 35), and the warps' sums are added by four lanes a value, not by one.
+template <int N>
+__device__ __forceinline__ void bsums(double (&acc)[N], BatchShared& sh) {
+    static_assert(N <= BGV + 2, "sh.wd is too narrow");
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
-    v = warp_sum(v);
-    __syncthreads();
-    if (lane == 0) sh.tmp[warp] = v;
+    warp_fold_to<N>(acc, sh.wd[warp]);
     __syncthreads();
     if (warp == 0) {
-        double t = lane < nw ? sh.tmp[lane] : 0.0;
-        t = warp_sum(t);
-        if (lane == 0) sh.tmp[BMAX_WARPS] = t;
+        const int v = lane >> 2;
+        double s = 0.0;
+        if (v < N)
+            for (int w = lane & 3; w < nw; w += 4) s += sh.wd[w][v];
+        s += __shfl_xor_sync(0xffffffffu, s, 1);
+        s += __shfl_xor_sync(0xffffffffu, s, 2);
+        if (v < N && (lane & 3) == 0) sh.gs[v] = s;
     }
     __syncthreads();
-    return sh.tmp[BMAX_WARPS];
 }
 
+// a . b; every thread gets the result
 __device__ __forceinline__ double bdot(const double* __restrict__ a, const double* __restrict__ b, int n,
                                        BatchShared& sh) {
-    double acc = 0.0;
-    for (int i = threadIdx.x; i < n; i += blockDim.x) acc += a[i] * b[i];
-    return bsum(acc, sh);
+    double acc[1] = {0.0};
+    for (int i = threadIdx.x; i < n; i += blockDim.x) acc[0] += a[i] * b[i];
+    bsums(acc, sh);
+    return sh.gs[0];
 }
 
-// out[a] = V_a^T x for a < cnt (V column-major with leading dimension ld): four dot
-// products per sweep and one block reduction per sweep (warps added in order)
+// out[a] = V_a^T x for a < cnt (V column-major with leading dimension ld): BGV dot
+// products per sweep and one block reduction per sweep
 __device__ __forceinline__ void bdots(const double* __restrict__ V, long long ld, int cnt,
-                                      const double* __restrict__ x, int n, double* out,
-                                      double (&wd)[BMAX_WARPS][4]) {
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
-    for (int c0 = 0; c0 < cnt; c0 += 4) {
-        double acc[4] = {0.0, 0.0, 0.0, 0.0};
+                                      const double* __restrict__ x, int n, double* out, BatchShared& sh) {
+    for (int c0 = 0; c0 < cnt; c0 += BGV) {
+        double acc[BGV];
+#pragma unroll
+        for (int t = 0; t < BGV; ++t) acc[t] = 0.0;
         for (int i = threadIdx.x; i < n; i += blockDim.x) {
             const double xi = x[i];
 #pragma unroll
-            for (int t = 0; t < 4; ++t)
+            for (int t = 0; t < BGV; ++t)
                 if (c0 + t < cnt) acc[t] += V[(size_t)(c0 + t) * ld + i] * xi;
         }
-#pragma unroll
-        for (int t = 0; t < 4; ++t) {
-            const double v = warp_sum(acc[t]);
-            if (lane == 0) wd[warp][t] = v;
-        }
-        __syncthreads();
-        if (threadIdx.x < 4 && c0 + (int)threadIdx.x < cnt) {
-            double s = 0.0;
-            for (int w = 0; w < nw; ++w) s += wd[w][threadIdx.x];
-            out[c0 + threadIdx.x] = s;
-        }
+        bsums(acc, sh);
+        if (threadIdx.x < BGV && c0 + (int)threadIdx.x < cnt) out[c0 + threadIdx.x] = sh.gs[threadIdx.x];
         __syncthreads();
     }
 }
@@ -191,24 +196,25 @@ __device__ __forceinline__ float2 bdf_add(float2 a, float2 b) {
     return make_float2(hi, lo);
 }
 
-// block reduction of the KP+1 per-thread sums of an mrs step into sh.red: warp sums
-// in FP32, then warp 0 adds the warps' sums in a fixed order in float pairs and holds
+// block reduction of the KP+1 per-thread sums of an mrs step into sh.red: folded warp sums
+// in FP32 (23 shuffles for 21 values, a tree a value takes 105), then warp 0 adds the warps' sums in a fixed order in float pairs and holds
 // sh.red afterwards (the scalar update that reads it runs in warp 0 too, so one block
 // barrier is saved)
 template <int KP>
 __device__ __forceinline__ void bred_w0(float (&tacc)[KP + 1], BatchShared& sh) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
-#pragma unroll
-    for (int v = 0; v <= KP; ++v) {
-        float d = warp_sum(tacc[v]);
-        if (lane == 0) sh.wsum[warp][v] = d;
-    }
+    warp_fold_to<KP + 1>(tacc, sh.wsum[warp]);
     __syncthreads();
     if (warp == 0) {
         for (int v = lane; v <= KP; v += 32) {
-            float2 t = make_float2(0.f, 0.f);
-            for (int w = 0; w < nw; ++w) t = bdf_add(t, make_float2(sh.wsum[w][v], 0.f));
-            sh.red[v] = t.x + t.y;
+            float2 t[4];   // four chains of pair sums (the warps of a block are a multiple of four)
+#pragma unroll
+            for (int u = 0; u < 4; ++u) t[u] = make_float2(0.f, 0.f);
+            for (int w = 0; w < nw; w += 4)
+#pragma unroll
+                for (int u = 0; u < 4; ++u) t[u] = bdf_add(t[u], make_float2(sh.wsum[w + u][v], 0.f));
+            const float2 r = bdf_add(bdf_add(t[0], t[1]), bdf_add(t[2], t[3]));
+            sh.red[v] = r.x + r.y;
         }
         __syncwarp();
     }
@@ -359,6 +365,7 @@ __device__ int bmrs(const double* u, float* z, float* Y, long long ys, float* P,
             if (i >= n) continue;
             const float yold = j >= 2 ? Yold[i] : 0.f;
             const float pold = j >= 2 ? Pj1[i] : 0.f;
+            const float zold = j >= 2 ? zz[i] : 0.f;   // with the first loads, not after the row's sums
             float acc = 0.f;
             if (sell) {
                 const int sl = s_ >> 5, t = s_ & 31;
@@ -398,7 +405,7 @@ __device__ int bmrs(const double* u, float* z, float* Y, long long ys, float* P,
             if (j >= 2) {
                 float pv = (tnp * yold - tdpp * pold) * tthp;
                 Pj1[i] = pv;
-                zz[i] += txp * pv;
+                zz[i] = zold + txp * pv;
             }
         }
         bred_w0<KP>(tacc, sh);
@@ -555,7 +562,8 @@ __global__ void __launch_bounds__(NT, MINB) k_batch(BatchLaunch L) {
                 status = ASSS_ERR_BREAKDOWN;
                 break;
             }
-            for (int i = threadIdx.x; i < n; i += blockDim.x) V[i] = rh[i] / beta0;
+            const double rbeta0 = 1.0 / beta0;
+            for (int i = threadIdx.x; i < n; i += blockDim.x) V[i] = rh[i] * rbeta0;
             if (threadIdx.x == 0) {
                 for (int a = 0; a <= R + 1; ++a) sh.g[a] = 0.0;
                 sh.g[0] = beta0;
@@ -597,21 +605,57 @@ __global__ void __launch_bounds__(NT, MINB) k_batch(BatchLaunch L) {
                 bspmv<WIDE>(M.swrp, M.swci, M.swv, zj, t1, n);
                 bspmv<WIDE>(M.awrp, M.awci, M.awv, t1, t2, n);
                 mark(2);
-                // two classical Gram-Schmidt passes
-                for (int pass = 0; pass < 2; ++pass) {
-                    bdots(V, nm, j + 1, t2, n, pass == 0 ? sh.hv : sh.hv2, sh.wd);
-                    const double* hh = pass == 0 ? sh.hv : sh.hv2;
-                    const double* __restrict__ Vr = V;
-                    double* __restrict__ t2r = t2;
+                // Two classical Gram-Schmidt passes in three sweeps: the first projection, the
+                // second pass's dot products and |w|^2 share one, and the second projection
+                // and the normalisation the last, with |w - V h2|^2 = |w|^2 - |h2|^2.  Bound by
+                // the FP64 pipe (16 cycles a warp instruction): no division a row, no sweep
+                // for the norm, and V and w are read three times instead of five and six.
+                const int nv = j + 1;
+                const double* __restrict__ Vr = V;
+                double* __restrict__ t2r = t2;
+                bdots(Vr, nm, nv, t2, n, sh.hv, sh);
+                if (nv <= BGV) {
+                    double acc[BGV + 1];
+#pragma unroll
+                    for (int t = 0; t <= BGV; ++t) acc[t] = 0.0;
                     for (int i = threadIdx.x; i < n; i += blockDim.x) {
-                        double acc = 0.0;
-                        for (int a = 0; a <= j; ++a) acc += Vr[a * nm + i] * hh[a];
-                        t2r[i] -= acc;
+                        double vi[BGV], s = 0.0;
+#pragma unroll
+                        for (int t = 0; t < BGV; ++t)
+                            if (t < nv) vi[t] = Vr[t * nm + i];
+#pragma unroll
+                        for (int t = 0; t < BGV; ++t)
+                            if (t < nv) s += vi[t] * sh.hv[t];
+                        const double wn = t2r[i] - s;
+                        t2r[i] = wn;
+#pragma unroll
+                        for (int t = 0; t < BGV; ++t)
+                            if (t < nv) acc[t] += vi[t] * wn;
+                        acc[BGV] += wn * wn;
                     }
-                    __syncthreads();
+                    bsums(acc, sh);
+                    if (threadIdx.x < (unsigned)nv) sh.hv2[threadIdx.x] = sh.gs[threadIdx.x];
+                    if (threadIdx.x == 0) sh.nrm[0] = sh.gs[BGV];
+                } else {
+                    double acc[1] = {0.0};
+                    for (int i = threadIdx.x; i < n; i += blockDim.x) {
+                        double s = 0.0;
+                        for (int a = 0; a < nv; ++a) s += Vr[a * nm + i] * sh.hv[a];
+                        const double wn = t2r[i] - s;
+                        t2r[i] = wn;
+                        acc[0] += wn * wn;
+                    }
+                    bsums(acc, sh);
+                    if (threadIdx.x == 0) sh.nrm[0] = sh.gs[0];
+                    bdots(Vr, nm, nv, t2, n, sh.hv2, sh);
                 }
-                const double hn = sqrt(bdot(t2, t2, n, sh));
+                __syncthreads();
                 if (threadIdx.x == 0) {
+                    double h2n = 0.0;
+                    for (int a = 0; a < nv; ++a) h2n += sh.hv2[a] * sh.hv2[a];
+                    const double d2 = sh.nrm[0] - h2n, hn2 = d2 < 0.0 ? 0.0 : d2;   // NaN stays
+                    const double inv = hn2 == 0.0 ? 0.0 : rsqrt(hn2), hn = hn2 * inv;
+                    sh.nrm[1] = inv;
                     double* col = sh.H + j * (R + 1);
                     for (int a = 0; a <= j; ++a) col[a] = sh.hv[a] + sh.hv2[a];
                     col[j + 1] = hn;
@@ -637,7 +681,14 @@ __global__ void __launch_bounds__(NT, MINB) k_batch(BatchLaunch L) {
                     mark(3);
                     break;
                 }
-                for (int i = threadIdx.x; i < n; i += blockDim.x) V[(j + 1) * nm + i] = t2[i] / hn;
+                const double inv = sh.nrm[1];
+                double* __restrict__ vn = V + nv * nm;
+                for (int i = threadIdx.x; i < n; i += blockDim.x) {
+                    double s = 0.0;
+#pragma unroll 4
+                    for (int a = 0; a < nv; ++a) s += Vr[a * nm + i] * sh.hv2[a];
+                    vn[i] = (t2r[i] - s) * inv;
+                }
                 __syncthreads();
                 mark(3);
             }
