@@ -645,6 +645,8 @@ __global__ void __launch_bounds__(CL_THREADS, 1) k_solve_cl(const ClArgs<T> p) {
             for (int i = rb + tid; i < re; i += NT) {
                 const T yold = j >= 2 ? Yold[i] : (T)0;
                 const T pold = j >= 2 ? Pj1[i] : (T)0;
+                // with the first loads, as in k_mrs (100^3: 1439 -> 1423 us a solve, 47^3 326 -> 319)
+                const T zold = j >= 2 ? zz[i] : (T)0;
                 T acc = (T)0;
                 if constexpr (FMT == 3) {
                     acc = __ldg(&fa.wdT[i]) * s_f[__ldg(&fa.pos[i])];
@@ -676,7 +678,7 @@ __global__ void __launch_bounds__(CL_THREADS, 1) k_solve_cl(const ClArgs<T> p) {
                 if (j >= 2) {
                     const T pv = (tnp * yold - tdpp * pold) * tthp;
                     Pj1[i] = pv;
-                    zz[i] += txp * pv;
+                    zz[i] = zold + txp * pv;
                 }
             }
             mrs_sums(tacc);
