@@ -2048,24 +2048,24 @@ static asss_status do_setup(asss_handle* h, const asss_csr* Ain, asss_stats* st)
 // company; grid scope has the whole GPU and pays two to three microseconds a synchronisation.
 // Both grow linearly with n; in microseconds for 4 outer and 20 inner steps, measured at n = 8^3 ..
 // 100^3 (dissipative Hamiltonian, k = 20; all scale with the steps alike):
-//   FP32 inner: cluster 100 + 0.0082 n x 16 / size a wave of columns, grid 215 + 0.00124 n a column
-//   FP64 inner: cluster 200 + 0.034 n x 16 / size,                    grid 330 + 0.00365 n
-// (one column, cluster / grid / launch by launch: 10^3 144 / 184 / 394, 24^3 257 / 254 / 504, 47^3
-// 924 / 346 / 604, 64^3 - / 540 / 765, 100^3 - / 1459 / 1687; FP64 10^3 219 / 272 / 431, 24^3 665 /
-// 381 / 604, 64^3 - / 1286 / 1450; eight columns at 16^3 199 against 3193 in lockstep blocks, at
-// 48^3 1266 against 4963).
+//   FP32 inner: cluster 125 + 0.0083 n x 16 / size a wave of columns, grid 215 + 0.00105 n a column
+//   FP64 inner: cluster 200 + 0.034 n x 16 / size,                     grid 330 + 0.00365 n
+// (one column, cluster / grid / launch by launch: 10^3 127 / 166 / 394, 16^3 176 / 233 / -, 22^3 235 /
+// 234 / -, 24^3 247 / 236 / 504, 28^3 302 / 236 / -, 47^3 - / 317 / 604, 64^3 - / 487 / 765, 100^3
+// - / 1413 / 1687; FP64 10^3 219 / 272 / 431, 16^3 342 / 376 / -, 24^3 665 / 381 / 604, 64^3 - / 1263 /
+// 1450; eight columns at 16^3 188 against 3193 in lockstep blocks, at 48^3 1259 against 4963).
 static int cluster_size(const asss_handle* h, int nrhs) {
     constexpr int CL_MOST = 300000;   // above it the columns' vectors leave L2 (not measured)
     const bool fp32 = h->opt.precision == ASSS_PREC_MIXED;
     const double n = h->n;
-    double best = nrhs * (fp32 ? 215.0 + 0.00124 * n : 330.0 + 0.00365 * n);
+    double best = nrhs * (fp32 ? 215.0 + 0.00105 * n : 330.0 + 0.00365 * n);
     if (h->factored) best = nrhs * 3000.0;   // a grid barrier or a launch per colour: 24^3 4295 us against 1133
     int size = h->factored ? 0 : -1;
     if (h->n > CL_MOST) return size;
     for (int t = 0; t < CL_NSIZES; ++t) {
         if (h->cl_counts[t] < 1) continue;
         const int waves = cdiv(nrhs, h->cl_counts[t]);
-        const double us = waves * (fp32 ? 100.0 + 0.0082 * n * 16 / CL_SIZES[t] : 200.0 + 0.034 * n * 16 / CL_SIZES[t]);
+        const double us = waves * (fp32 ? 125.0 + 0.0083 * n * 16 / CL_SIZES[t] : 200.0 + 0.034 * n * 16 / CL_SIZES[t]);
         if (us < best) {
             best = us;
             size = CL_SIZES[t];

@@ -230,6 +230,13 @@ __device__ __forceinline__ void warp_fold_to(T (&v)[NV], T* out) {
     }
 }
 
+// 16 bytes from global into shared memory without a register, and the wait for all of a thread's
+__device__ __forceinline__ void cp_async16(void* dst, const void* src) {
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((unsigned)__cvta_generic_to_shared(dst)), "l"(src)
+                 : "memory");
+}
+__device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;" ::: "memory"); }
+
 // Grid-wide barrier for a cooperative (co-resident) launch, on a counter that only grows
 // during a launch: barrier number `phase` (0-based) is complete once the counter reaches
 // (phase + 1) * nblocks.  One atomic per block between acquire-release fences (the

@@ -139,6 +139,32 @@ inline long long cl_factor_smem(int n, int own_max, int ncol) {
            4LL * (2 * ncol + 2);
 }
 
+constexpr size_t CL_SMEM_MAX = 227 * 1024;
+// shared memory behind the `used` bytes for the rows of Q_k of a block; 0: they do not fit
+inline size_t cl_q_bytes(int n, int kp, int blocks, size_t used) {
+    const size_t need = 16 + 32 * 4 * (size_t)kp * cdiv(cdiv(n, 32), blocks);
+    return used + need <= CL_SMEM_MAX ? need : 0;
+}
+
+// row i of Q_k, from a CTA's slices in shared memory (its first row rb) or from global memory
+template <class T, int KP, bool QS>
+__device__ __forceinline__ void cl_qrow(const T* __restrict__ Q, const float4* s_q, int rb, int i,
+                                        T (&q)[KP > 0 ? KP : 1], bool cs) {
+    if constexpr (QS) {
+        const float4* a = s_q + (size_t)((i - rb) >> 5) * 8 * KP + (i & 31);
+#pragma unroll
+        for (int m = 0; m < KP; m += 4, a += 32) {
+            const float4 v = *a;
+            q[m] = v.x;
+            q[m + 1] = v.y;
+            q[m + 2] = v.z;
+            q[m + 3] = v.w;
+        }
+    } else {
+        load_qrow<T, KP, q_blocked<T>(true)>(Q, i, q, cs);
+    }
+}
+
 // One triangular solve, colour by colour (back: from the last colour down): vec[e] =
 // own[row of e] - sum_q v_q vec[col_q], vec replicated in every CTA; own: this CTA's right-hand
 // side, in the order of its rows.  Four lanes share a row (an FP64 operation of a warp takes 64
@@ -209,7 +235,12 @@ __device__ __noinline__ void cl_tri_sweep(E* vec, const E* own, const int2* rows
 // share of the GPU would slow down: a synchronisation is the grid barrier, block sums go through L2
 // and every block adds them; what it saves against the launch-by-launch path is the launches and
 // the host's part.  A barrier that gives up ends the solve (dead).
-template <class T, int KP, int FMT, bool GRID>
+// QS (grid scope, FP32): every block keeps its rows of Q_k, more than half of what a row of an mrs
+// pass reads, in shared memory for the whole solve, where they fit (at k = 20 up to about 2600
+// rows a block, 395 000 in all): 64^3 513 -> 487 us, 70^3 650 -> 596, adjoint at 64^3 543 -> 505,
+// 47^3 323 -> 317.  Not in clusters (24^3 249 -> 246, 48^3 with eight columns does not fit), and not
+// a part of the rows: the L1 that shared memory takes costs as much (100^3 1423 -> 1425 .. 1481).
+template <class T, int KP, int FMT, bool GRID, bool QS = false>
 __global__ void __launch_bounds__(CL_THREADS, 1) k_solve_cl(const ClArgs<T> p) {
     constexpr int NT = CL_THREADS, NW = CL_WARPS, NV = KP + 1, KQ = KP > 0 ? KP : 1;
     using Sh = ClShared<T, KP, GRID>;
@@ -295,6 +326,13 @@ __global__ void __launch_bounds__(CL_THREADS, 1) k_solve_cl(const ClArgs<T> p) {
                 s_uq[o] = make_int2(fa.U.rp[e], fa.U.rp[e + 1] - fa.U.rp[e]);
                 s_jq[o] = make_int2(fa.J.rp[e], fa.J.rp[e + 1] - fa.J.rp[e]);
             }
+    }
+    // own rows of Q_k in shared memory, in the slices of the global copy; on their way until mrs
+    float4* s_q = reinterpret_cast<float4*>((reinterpret_cast<size_t>(H + (size_t)(R + 1) * R) + 15) & ~(size_t)15);
+    if constexpr (QS) {
+        const float4* src = reinterpret_cast<const float4*>(p.Q + (size_t)rb * KP);
+        for (int e = tid; e < ((re - rb + 31) >> 5) * 8 * KP; e += NT)
+            if (rb + e / (8 * KP) * 32 + (e & 31) < re) cp_async16(s_q + e, src + e);
     }
     sync_all();   // every CTA of the cluster runs: its shared memory may be written
 
@@ -581,6 +619,10 @@ __global__ void __launch_bounds__(CL_THREADS, 1) k_solve_cl(const ClArgs<T> p) {
             sh.qtp[1][a] = (T)0;
             sh.qtx[a] = (T)0;
         }
+        if constexpr (QS) {
+            cp_async_wait_all();
+            __syncthreads();
+        }
         T tacc[NV];
 #pragma unroll
         for (int v = 0; v < NV; ++v) tacc[v] = (T)0;
@@ -592,7 +634,7 @@ __global__ void __launch_bounds__(CL_THREADS, 1) k_solve_cl(const ClArgs<T> p) {
             P[nn + i] = (T)0;
             tacc[0] += b * b;
             T q[KQ];
-            load_qrow<T, KP, q_blocked<T>(true)>(p.Q, i, q, GRID && p.cs);
+            cl_qrow<T, KP, QS>(p.Q, s_q, rb, i, q, GRID && p.cs);
 #pragma unroll
             for (int a = 0; a < KP; ++a) tacc[1 + a] += q[a] * b;
         }
@@ -666,7 +708,7 @@ __global__ void __launch_bounds__(CL_THREADS, 1) k_solve_cl(const ClArgs<T> p) {
                     }
                 }
                 T q[KQ];
-                load_qrow<T, KP, q_blocked<T>(true)>(p.Q, i, q, GRID && p.cs);
+                cl_qrow<T, KP, QS>(p.Q, s_q, rb, i, q, GRID && p.cs);
                 T dq = (T)0;
 #pragma unroll
                 for (int a = 0; a < KP; ++a) dq += q[a] * sh.u[a];
@@ -1140,7 +1182,7 @@ static asss_status cl_run(const Ctx& c, const ClArgs<T>& a, int size, int count,
         for (int t = 0; t < CL_NSIZES; ++t) {
             const size_t need = bytes(CL_SIZES[t]);
             counts[t] = 0;
-            if (need <= 227 * 1024) ASSS_TRY((cl_clusters<T, KP, FMT>(CL_SIZES[t], need, &counts[t])));
+            if (need <= CL_SMEM_MAX) ASSS_TRY((cl_clusters<T, KP, FMT>(CL_SIZES[t], need, &counts[t])));
         }
         return ASSS_OK;
     }
@@ -1164,15 +1206,20 @@ static asss_status cl_run(const Ctx& c, const ClArgs<T>& a, int size, int count,
 // grid scope: a cooperative launch of one block per SM (size < 0)
 template <class T, int KP>
 static asss_status cl_run_grid(const Ctx& c, const ClArgs<T>& a) {
-    const size_t smem = ((sizeof(ClShared<T, KP, true>) + 15) & ~(size_t)15) +
-                        sizeof(double) * (size_t)(a.restart + 1) * (size_t)a.restart;
+    size_t smem = ((sizeof(ClShared<T, KP, true>) + 15) & ~(size_t)15) +
+                  sizeof(double) * (size_t)(a.restart + 1) * (size_t)a.restart;
     const void* fn = (const void*)k_solve_cl<T, KP, 1, true>;
-    ASSS_TRY(raise_dynamic_smem(fn, (int)smem));
-    const int need = cdiv(a.n, 32);
+    const int need = cdiv(a.n, 32), blocks = c.sms < need ? c.sms : need;
+    if constexpr (sizeof(T) == 4 && KP > 0) {
+        if (const size_t q = cl_q_bytes(a.n, KP, blocks, smem)) {
+            fn = (const void*)k_solve_cl<T, KP, 1, true, true>;
+            smem += q;
+        }
+    }
     ClArgs<T> b = a;
+    ASSS_TRY(raise_dynamic_smem(fn, (int)smem));
     void* args[] = {&b};
-    ASSS_CUDA(cudaLaunchCooperativeKernel(fn, dim3(c.sms < need ? c.sms : need), dim3(CL_THREADS), args, smem,
-                                          c.stream));
+    ASSS_CUDA(cudaLaunchCooperativeKernel(fn, dim3(blocks), dim3(CL_THREADS), args, smem, c.stream));
     count_launch();
     return ASSS_OK;
 }
