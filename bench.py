@@ -397,13 +397,13 @@ class ClockSampler:
 
 
 def _traffic_record():
-    """ncu DRAM bytes per mrs launch, valid only for the current kernel source."""
-    path = os.path.join(ROOT, "profiles", "mrs_traffic.json")
-    src = os.path.join(ROOT, "paper_2009_06954_gb300", "csrc", "mrs.cu")
+    """ncu DRAM bytes of a whole-solve launch, valid only for the current kernel source."""
+    path = os.path.join(ROOT, "profiles", "solve_traffic.json")
+    src = os.path.join(ROOT, "paper_2009_06954_gb300", "csrc", "solve_cluster.cuh")
     try:
         rec = json.load(open(path))
         h = hashlib.sha256(open(src, "rb").read()).hexdigest()
-        if rec.get("mrs_cu_sha256") == h:
+        if rec.get("solve_cluster_cuh_sha256") == h:
             return rec
     except Exception:
         pass
@@ -727,11 +727,11 @@ def main_adjoint(args, world, rank, local):
         "gpu_launches": int(launches),
         "e2e": {"value": e2e_val, "unit": "gradients/s", "h2d_bytes_per_step": 16 * n,
                 "d2h_bytes_per_step": 8 * n + 8 * A.nnz},
-        "roofline": {"bound": "hbm", "kernel": "k_mrs<float,20> (persistent mrs, transposed operator)",
+        "roofline": {"bound": "hbm", "kernel": "k_solve_cl<float,20> (mrs of the whole-solve launch, transposed operator)",
                      "achieved": achieved, "peak": peak, "unit": "GB/s", "frac": achieved / peak if peak else None,
                      "peak_source": f"{peak_kind} hbm_gbs", "traffic": None,
-                     "algorithmic_bytes_per_launch": inner_bytes / max(inner_launches, 1),
-                     "avg_launch_ms": inner_ms / max(inner_launches, 1), "launches": inner_launches,
+                     "algorithmic_bytes_per_inner_solve": inner_bytes / max(inner_launches, 1),
+                     "avg_inner_solve_ms": inner_ms / max(inner_launches, 1), "inner_solves": inner_launches,
                      "others": phase_rooflines(stats, peak)},
         "clocks": clk.summary(),
         "cpu_baseline": cpu,
@@ -743,8 +743,8 @@ def main_adjoint(args, world, rank, local):
 
 
 # ----------------------------------------------------------------------------
-# many right-hand sides of the 100^3 system in one call (lockstep FGMRES blocks,
-# multi-column mrs): the SpMM form of the inner solve
+# many right-hand sides of the 100^3 system in one call (a whole-solve launch in grid scope,
+# its columns one after another)
 # ----------------------------------------------------------------------------
 MULTI_NRHS = 8
 
@@ -846,7 +846,7 @@ def main_multi_rhs(args, world, rank, local):
         "warmup": args.warmup, "ms_per_step": tmax / args.steps, "higher_is_better": True, "scaling": "weak",
         "vs_baseline": None, "dtype": "f32-inner/f64-outer", "data": "synthetic",
         "config": {"workload": (f"dh3d_100_rhs{R}: the dh3d_100 system with {R} right-hand sides per call "
-                                f"(lockstep FGMRES, one multi-column FP32 mrs launch per Arnoldi step)"),
+                                f"(one whole-solve launch, a column after another)"),
                    "parallelism": f"replicas x{world}" if world > 1 else "single GPU",
                    "l2": "256 MB buffer written between steps (not timed); working set > L2",
                    "setup_s": round(t_setup, 3), "rhs_per_call": R, "outer_its_max": stats[-1]["outer_its"],
@@ -854,12 +854,11 @@ def main_multi_rhs(args, world, rank, local):
                    "one_after_another_solves_per_s": seq_val},
         "gpu_launches": int(launches),
         "e2e": {"value": e2e_val, "unit": UNIT, "h2d_bytes_per_step": 8 * n * R, "d2h_bytes_per_step": 8 * n * R},
-        "roofline": {"bound": "hbm", "kernel": "k_mrs_multi<float,20> (8 right-hand sides per launch)",
+        "roofline": {"bound": "hbm", "kernel": "k_solve_cl<float,20> (mrs of the whole-solve launch)",
                      "achieved": achieved, "peak": peak, "unit": "GB/s", "frac": achieved / peak if peak else None,
                      "peak_source": f"{peak_kind} hbm_gbs", "traffic": None,
-                     "algorithmic_bytes_per_launch": inner_bytes / max(inner_launches, 1),
-                     "bytes_model": "matrix and Q rows once per step for all columns, 28 B per live column",
-                     "avg_launch_ms": inner_ms / max(inner_launches, 1), "launches": inner_launches,
+                     "algorithmic_bytes_per_inner_solve": inner_bytes / max(inner_launches, 1),
+                     "avg_inner_solve_ms": inner_ms / max(inner_launches, 1), "inner_solves": inner_launches,
                      "share_of_step": inner_ms / total_ms if total_ms else None},
         "clocks": clk.summary(),
         "cpu_baseline": None,
@@ -1031,8 +1030,9 @@ FP64_PEAK_TFLOPS = 152 * 2.07e9 * 4 / 1e12   # SMs x max SM clock x FP64 flops p
 
 
 def phase_rooflines(stats, peak):
-    """Roofline entries of the outer operator and the fused Arnoldi step, from the CUDA
-    events the library records around them inside the timed solves."""
+    """Roofline entries of the outer operator and the fused Arnoldi step, from the times the
+    library takes inside the timed solves (the whole-solve kernel's own timer; CUDA events
+    around the launches where a solve is many launches)."""
     out = []
     t_op = sum(s_["t_op_ms"] for s_ in stats)
     if t_op > 0:
@@ -1041,12 +1041,12 @@ def phase_rooflines(stats, peak):
         calls = sum(s_["op_calls"] for s_ in stats)
         ach = b / (t_op / 1000.0) / 1e9
         tf = f / (t_op / 1000.0) / 1e12
-        out.append({"kernel": "k_dia_spmv x2 (outer operator W Abar S W v)" if DH["factor"] == "diag" else
+        out.append({"kernel": "outer operator W Abar S W v (two products by diagonals)" if DH["factor"] == "diag" else
                     "outer operator with triangular solves per colour", "bound": "hbm", "achieved": ach,
                     "peak": peak, "unit": "GB/s", "frac": ach / peak if peak else None, "calls": calls,
                     "bytes_per_call": b / max(calls, 1), "ms_per_call": t_op / max(calls, 1),
                     "fp64_tflops": tf, "fp64_frac": tf / FP64_PEAK_TFLOPS,
-                    "note": "CUDA events around each application inside the timed solves; one FP64 FMA per "
+                    "note": "timed around each application inside the timed solves; one FP64 FMA per "
                             "stored value, so the FP64 pipe (fp64_frac) bounds it about as much as HBM"})
     t_or = sum(s_["t_orth_ms"] for s_ in stats)
     if t_or > 0:
@@ -1055,7 +1055,7 @@ def phase_rooflines(stats, peak):
         calls = sum(s_["orth_calls"] for s_ in stats)
         tf = f / (t_or / 1000.0) / 1e12
         gb = b / (t_or / 1000.0) / 1e9
-        out.append({"kernel": "k_arnoldi_orth (fused CGS2 Arnoldi step, FP64)", "bound": "alu", "achieved": tf,
+        out.append({"kernel": "fused CGS2 Arnoldi step, FP64", "bound": "alu", "achieved": tf,
                     "peak": FP64_PEAK_TFLOPS, "unit": "TFLOP/s", "frac": tf / FP64_PEAK_TFLOPS, "calls": calls,
                     "ms_per_call": t_or / max(calls, 1), "hbm_achieved_gbs": gb,
                     "hbm_frac": gb / peak if peak else None,
@@ -1255,7 +1255,7 @@ def main():
                 "max_relres": max(s_["relres"] for s_ in st64),
                 "converged": all(s_["status"] == 0 for s_ in st64) and max(s_["relres"] for s_ in st64) <= 1e-8,
                 "setup_s": round(t_setup64, 3),
-                "mrs_avg_launch_ms": sum(s_["t_inner_ms"] for s_ in st64) / max(sum(s_["inner_launches"] for s_ in st64), 1)}
+                "mrs_avg_ms": sum(s_["t_inner_ms"] for s_ in st64) / max(sum(s_["inner_launches"] for s_ in st64), 1)}
         s64.close()
 
     inner_ms = sum(s_["t_inner_ms"] for s_ in stats)
@@ -1301,12 +1301,15 @@ def main():
                    "fp64_gpu": fp64, "rel_error_vs_oracle": rel_err},
         "gpu_launches": int(launches),
         "e2e": {"value": e2e_val, "unit": UNIT, "h2d_bytes_per_step": 8 * n, "d2h_bytes_per_step": 8 * n},
-        "roofline": {"bound": "hbm", "kernel": "k_mrs<float,20> (persistent mrs)" if DH["factor"] == "diag" else
+        "roofline": {"bound": "hbm", "kernel": "k_solve_cl<float,20> (mrs of the whole-solve launch)" if DH["factor"] == "diag" else
                      "k_mrs<float,20,factored> (persistent mrs, J~ by triangular solves per colour)", "achieved": achieved,
                      "peak": peak, "unit": "GB/s", "frac": achieved / peak if peak else None,
                      "peak_source": f"{peak_kind} hbm_gbs", "traffic": traffic,
-                     "algorithmic_bytes_per_launch": inner_bytes / max(inner_launches, 1),
-                     "avg_launch_ms": inner_ms / max(inner_launches, 1), "launches": inner_launches,
+                     "traffic_scope": "DRAM bytes of a whole solve launch, all phases",
+                     "algorithmic_bytes_per_solve": sum(s_["inner_bytes"] + s_["op_bytes"] + s_["orth_bytes"]
+                                                        for s_ in stats) / len(stats),
+                     "algorithmic_bytes_per_inner_solve": inner_bytes / max(inner_launches, 1),
+                     "avg_inner_solve_ms": inner_ms / max(inner_launches, 1), "inner_solves": inner_launches,
                      "share_of_step": inner_ms / total_ms if total_ms else None, "others": others},
         "clocks": clk.summary(),
         "cpu_baseline": cpu,

@@ -109,10 +109,13 @@ typedef struct {
                                  or ASSS_SCALING_MATCHING (maximum-product matching and its dual
                                  scalings, the role of MC64 in §2: |diag| = 1, other entries
                                  <= 1 up to a relative 1e-12 * max(1, max cost))                */
-    int    rhs_block;         /* 1: asss_solve with several right-hand sides (FGMRES, k <= 32, FP32 Q)
-                                 runs them in lockstep blocks of up to 8 whose preconditioner
+    int    rhs_block;         /* several right-hand sides in asss_solve (FGMRES, k <= 32, FP32 Q) whose
+                                 solves do not run as one launch each (J~ in SELL-C, or restart
+                                 > 60): 1: lockstep blocks of up to 8 columns whose preconditioner
                                  applications are one multi-column mrs launch per Arnoldi step
-                                 (App. B's simultaneous iterations); 0: one column after another */
+                                 (App. B's simultaneous iterations); 0: one column after another.
+                                 Elsewhere a column is one launch, and on small systems several
+                                 columns run side by side in it, whatever this says             */
     int    sell_sigma;        /* J~ in SELL-C (general patterns): rows are sorted by length within
                                  windows of sell_sigma rows when natural-order slices would pad the
                                  storage by more than a fifth; a power of two in [1024, 16384], or
@@ -162,18 +165,20 @@ typedef struct {
     long long nnz_pattern;    /* entries of pat(Abar S) + pat(Abar S)^T (LLS rows + mirror)      */
     double t_setup_ms;
     double t_solve_ms;
-    double t_inner_ms;        /* device time of the mrs kernel launches (CUDA events on the stream) */
-    long long inner_bytes;    /* algorithmic bytes those launches move (matrix entries, Q_k rows, vectors) */
-    int    inner_launches;    /* mrs kernel launches counted in t_inner_ms / inner_bytes */
+    double t_inner_ms;        /* device time of the inner solves: CUDA events around the mrs launches,
+                                 or the kernel's own timer where a whole solve is one launch    */
+    long long inner_bytes;    /* algorithmic bytes they move (matrix entries, Q_k rows, vectors) */
+    int    inner_launches;    /* mrs launches, or inner solves inside whole-solve launches, counted
+                                 in t_inner_ms / inner_bytes                                     */
     int    sell_sigma;        /* set-up, J~ in SELL-C: sorting window in rows (0: natural order) */
     int    sell_split;        /* set-up, J~ in SELL-C: entries per lane of one work unit; both picked
                                  by timing mrs steps for systems of 10^5 rows and more (FP32 path) */
     int    factor_colours;    /* set-up, ASSS_FACTOR_ILDL0: colours of the factorization order  */
-    double t_op_ms;           /* solve: CUDA-event time of the outer operator applications      */
+    double t_op_ms;           /* solve: time of the outer operator applications, as t_inner_ms  */
     int    op_calls;
     long long op_bytes;       /* their algorithmic bytes (stored values, x and y per product)   */
     long long op_flops;       /* and FP64 flops (one FMA per stored value)                      */
-    double t_orth_ms;         /* solve: CUDA-event time of the fused Arnoldi steps (FGMRES)     */
+    double t_orth_ms;         /* solve: time of the fused Arnoldi steps (FGMRES), as t_inner_ms */
     int    orth_calls;
     long long orth_bytes;     /* their algorithmic bytes (basis read twice, w r/w, v_{j+1} out) */
     long long orth_flops;     /* and FP64 flops (4(j+1) FMAs a row)                             */

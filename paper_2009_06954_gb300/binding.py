@@ -265,7 +265,8 @@ class Solver:
     inner_tol, setup_tol, outer_tol, inner_maxit, outer_maxit, restart, r_max,
     seed, lls_tol, lls_maxit, zero_tol, wait_timeout_ms, row_perm, dr, dc, stream, s_values,
     scaling ('maxes' | 'matching': how Eq. mc64's P, D_r, D_c are found when none is given),
-    rhs_block (several right-hand sides in lockstep blocks sharing multi-column mrs launches),
+    rhs_block (several right-hand sides in lockstep blocks sharing multi-column mrs launches, where
+    a solve is not one launch),
     factor ('diag' | 'ildl0': the no-fill incomplete L D L^T of M^, §3 / §4.1 ~ildl(0)),
     sell_sigma, sell_split (SELL-C storage of J~: sorting window and work-unit width; 0 = tuned)
     (saved S values to resume the set-up from, e.g. ``export(nnz)["s_val"]`` of an
