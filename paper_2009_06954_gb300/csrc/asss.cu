@@ -2046,26 +2046,35 @@ static asss_status do_setup(asss_handle* h, const asss_csr* Ain, asss_stats* st)
 // grid scope (-1), or launch by launch (0: the incomplete factor where no cluster fits).
 // One cluster has its SMs' share of the bandwidth and the FP64 pipe, but cheap synchronisations and
 // company; grid scope has the whole GPU and pays two to three microseconds a synchronisation.
-// Both grow linearly with n; in microseconds for 4 outer and 20 inner steps, measured at n = 8^3 ..
-// 100^3 (dissipative Hamiltonian, k = 20; all scale with the steps alike):
-//   FP32 inner: cluster 125 + 0.0083 n x 16 / size a wave of columns, grid 215 + 0.00105 n a column
-//   FP64 inner: cluster 200 + 0.034 n x 16 / size,                     grid 330 + 0.00365 n
-// (one column, cluster / grid / launch by launch: 10^3 127 / 166 / 394, 16^3 176 / 233 / -, 22^3 235 /
-// 234 / -, 24^3 247 / 236 / 504, 28^3 302 / 236 / -, 47^3 - / 317 / 604, 64^3 - / 487 / 765, 100^3
-// - / 1413 / 1687; FP64 10^3 219 / 272 / 431, 16^3 342 / 376 / -, 24^3 665 / 381 / 604, 64^3 - / 1263 /
-// 1450; eight columns at 16^3 188 against 3193 in lockstep blocks, at 48^3 1259 against 4963).
+// Both grow linearly with the rows of a CTA; in microseconds for 4 outer and 20 inner steps, measured
+// at n = 8^3 .. 100^3 (dissipative Hamiltonian, k = 20; all scale with the steps alike), m = n / size:
+//   FP32 inner: cluster 105 + 0.176 m (m <= CL_FEW_ROWS) or 125 + 0.133 m a wave of columns,
+//               grid 200 + 0.00105 n a column
+//   FP64 inner: cluster 185 + 0.51 m, grid 285 + 0.0037 n
+// (one column, cluster / grid / launch by launch: 10^3 111 / 166 / 394, 20^3 191 / 233 / -, 22^3 224 /
+// 234 / -, 24^3 247 / 215 / 504, 47^3 - / 304 / 604, 64^3 - / 487 / 765, 100^3 - / 1413 / 1687; FP64
+// 8^3 214 / - / -, 16^3 318 / 376 / -, 24^3 665 / 325 / 604, 64^3 - / 1252 / 1450; eight columns at
+// 16^3 188 against 3193 in lockstep blocks, at 48^3 1259 against 4963).
+// CL_FEW_ROWS: up to that many rows a CTA, 256 threads with up to 255 registers each (half the warps to
+// synchronise and to fold sums over), above it 512, whose loads hide more latency.  256 / 512 threads:
+// 10^3 (63 rows) 111 / 130, 16^3 (256) 157 / 179, 24^3 (91, grid) 215 / 236, 36^3 (307) 254 / 251, 47^3 (683)
+// 304 / 318, 56^3 (1155) 436 / 430, 64^3 (1725) 538 / 494; eight columns at 24^3 (864) 299 / 300, at 32^3 (2048)
+// 523 / 471.  FP64 always 256 (8^3 215 / 255, 24^3 325 / 374, 36^3 466 / 461, 64^3 1252 / 1270): at 512 its
+// registers spill.
+constexpr int CL_FEW_ROWS = 768;
 static int cluster_size(const asss_handle* h, int nrhs) {
     constexpr int CL_MOST = 300000;   // above it the columns' vectors leave L2 (not measured)
     const bool fp32 = h->opt.precision == ASSS_PREC_MIXED;
     const double n = h->n;
-    double best = nrhs * (fp32 ? 215.0 + 0.00105 * n : 330.0 + 0.00365 * n);
+    double best = nrhs * (fp32 ? 200.0 + 0.00105 * n : 285.0 + 0.0037 * n);
     if (h->factored) best = nrhs * 3000.0;   // a grid barrier or a launch per colour: 24^3 4295 us against 1133
     int size = h->factored ? 0 : -1;
     if (h->n > CL_MOST) return size;
     for (int t = 0; t < CL_NSIZES; ++t) {
         if (h->cl_counts[t] < 1) continue;
         const int waves = cdiv(nrhs, h->cl_counts[t]);
-        const double us = waves * (fp32 ? 125.0 + 0.0083 * n * 16 / CL_SIZES[t] : 200.0 + 0.034 * n * 16 / CL_SIZES[t]);
+        const double m = n / CL_SIZES[t];
+        const double us = waves * (!fp32 ? 185.0 + 0.51 * m : m <= CL_FEW_ROWS ? 105.0 + 0.176 * m : 125.0 + 0.133 * m);
         if (us < best) {
             best = us;
             size = CL_SIZES[t];
@@ -2179,13 +2188,17 @@ static asss_status cluster_plan(asss_handle* h, int nrhs, int* size) {
         if (o.precision == ASSS_PREC_MIXED) {
             ClArgs<float> a = {};
             ASSS_TRY(cluster_args<float>(h, 0, a));
-            if (h->factored) ASSS_TRY((cl_dispatch<float, 3>(h->ctx, a, h->kp, 0, 0, h->cl_counts)));
-            else ASSS_TRY((cl_dispatch<float, 1>(h->ctx, a, h->kp, 0, 0, h->cl_counts)));
+            if (h->factored) ASSS_TRY((cl_dispatch<float, 3, 512>(h->ctx, a, h->kp, 0, 0, h->cl_counts)));
+            else {
+                int few[CL_NSIZES];   // (256 threads: not fewer clusters)
+                if (h->kp > 0) ASSS_TRY((cl_dispatch<float, 1, 256>(h->ctx, a, h->kp, 0, 0, few)));
+                ASSS_TRY((cl_dispatch<float, 1, 512>(h->ctx, a, h->kp, 0, 0, h->cl_counts)));
+            }
         } else {
             ClArgs<double> a = {};
             ASSS_TRY(cluster_args<double>(h, 0, a));
-            if (h->factored) ASSS_TRY((cl_dispatch<double, 3>(h->ctx, a, h->kp, 0, 0, h->cl_counts)));
-            else ASSS_TRY((cl_dispatch<double, 1>(h->ctx, a, h->kp, 0, 0, h->cl_counts)));
+            if (h->factored) ASSS_TRY((cl_dispatch<double, 3, 512>(h->ctx, a, h->kp, 0, 0, h->cl_counts)));
+            else ASSS_TRY((cl_dispatch<double, 1, 256>(h->ctx, a, h->kp, 0, 0, h->cl_counts)));
         }
     }
     *size = cluster_size(h, nrhs);
@@ -2233,9 +2246,12 @@ static asss_status solve_cluster(asss_handle* h, int tr, int size, int nc, const
     if (!h->cl_st) ASSS_CUDA(cudaMallocHost((void**)&h->cl_st, sizeof(ClStat) * asss_handle::CL_CHUNK));
     a.work = h->cl_work.p;
     a.stats = h->cl_st;
-    if (h->factored) ASSS_TRY((cl_dispatch<T, 3>(c, a, h->kp, size, count, nullptr)));
-    else ASSS_TRY((cl_dispatch<T, 1>(c, a, h->kp, size, count, nullptr)));
-    return ASSS_OK;
+    if (h->factored) return cl_dispatch<T, 3, 512>(c, a, h->kp, size, count, nullptr);
+    if constexpr (sizeof(T) == 4) {
+        const int rows = cdiv(h->n, size < 0 ? c.sms : size);   // of a CTA
+        if (h->kp == 0 || rows > CL_FEW_ROWS) return cl_dispatch<T, 1, 512>(c, a, h->kp, size, count, nullptr);
+    }
+    return cl_dispatch<T, 1, 256>(c, a, h->kp, size, count, nullptr);
 }
 
 // statistics of one column, as refine fills them

@@ -8,8 +8,6 @@
 
 namespace asss {
 
-constexpr int CL_THREADS = 512;
-constexpr int CL_WARPS = CL_THREADS / 32;
 constexpr int CL_MAX = 16;   // CTAs of a cluster (the non-portable maximum)
 
 __device__ __forceinline__ unsigned cl_rank() {

@@ -112,13 +112,14 @@ inline long long cl_work_doubles(int n, int halo, int restart, int tbytes) {
     return nd + (nt * tbytes + 7) / 8 + 64;
 }
 
-template <class T, int KP, bool GRID>
+template <class T, int KP, bool GRID, int NT>
 struct ClShared {
+    static constexpr int NW = NT / 32;
     using P2 = typename std::conditional<sizeof(T) == 4, float2, double>::type;
     unsigned long long x[2][GRID ? 1 : CL_MAX][CL_XV];   // exchanged block sums, written by the other CTAs
-    double bsum[GRID ? CL_THREADS / (KP + 1) + 1 : 1][KP + 1];   // grid scope: parts of the cross-block sums
-    T wsum[CL_WARPS][KP + 1];
-    double wd[CL_WARPS][CL_REGV + 2];
+    double bsum[GRID ? NT / (KP + 1) + 1 : 1][KP + 1];   // grid scope: parts of the cross-block sums
+    T wsum[NW][KP + 1];
+    double wd[NW][CL_REGV + 2];
     double bp[CL_XV], tot[CL_XV];
     T red[KP + 1], u[KP > 0 ? KP : 1], alpha[KP > 0 ? KP : 1], cf[12];
     T qty[KP > 0 ? KP : 1], qtp[2][KP > 0 ? KP : 1], qtx[KP > 0 ? KP : 1], pq[4];
@@ -171,7 +172,7 @@ __device__ __forceinline__ void cl_qrow(const T* __restrict__ Q, const float4* s
 // cycles, however many of its lanes work) and its stores to the other CTAs; the entries
 // of the next two colours are on their way while a colour is solved.  Not inlined: its
 // registers would add to the solve's, at five places.
-template <class E>
+template <class E, int NT>
 __device__ __noinline__ void cl_tri_sweep(E* vec, const E* own, const int2* rows, const int* __restrict__ ci,
                                           const E* __restrict__ v, bool back, int ncol, const int* s_off,
                                           const int* s_beg) {
@@ -199,7 +200,7 @@ __device__ __noinline__ void cl_tri_sweep(E* vec, const E* own, const int2* rows
     };
     auto phase = [&](int k, Slot& S) {
         const int c = back ? ncol - 1 - k : k, o0 = s_off[c], o1 = s_off[c + 1];
-        for (int b0 = o0; b0 < o1; b0 += CL_THREADS / 4) {
+        for (int b0 = o0; b0 < o1; b0 += NT / 4) {
             const int o = b0 + (tid >> 2);
             if (b0 > o0) fetch(o, o1, S);
             E a = (E)0;
@@ -240,10 +241,11 @@ __device__ __noinline__ void cl_tri_sweep(E* vec, const E* own, const int2* rows
 // rows a block, 395 000 in all): 64^3 513 -> 487 us, 70^3 650 -> 596, adjoint at 64^3 543 -> 505,
 // 47^3 323 -> 317.  Not in clusters (24^3 249 -> 246, 48^3 with eight columns does not fit), and not
 // a part of the rows: the L1 that shared memory takes costs as much (100^3 1423 -> 1425 .. 1481).
-template <class T, int KP, int FMT, bool GRID, bool QS = false>
-__global__ void __launch_bounds__(CL_THREADS, 1) k_solve_cl(const ClArgs<T> p) {
-    constexpr int NT = CL_THREADS, NW = CL_WARPS, NV = KP + 1, KQ = KP > 0 ? KP : 1;
-    using Sh = ClShared<T, KP, GRID>;
+// NT: 256 threads where a CTA has few rows and in FP64, else 512 (see cluster_size).
+template <class T, int KP, int FMT, bool GRID, int NT, bool QS = false>
+__global__ void __launch_bounds__(NT, 1) k_solve_cl(const ClArgs<T> p) {
+    constexpr int NW = NT / 32, NV = KP + 1, KQ = KP > 0 ? KP : 1;
+    using Sh = ClShared<T, KP, GRID, NT>;
     using P2 = typename Sh::P2;
     extern __shared__ __align__(16) unsigned char s_dyn[];
     Sh& sh = *reinterpret_cast<Sh*>(s_dyn);
@@ -443,7 +445,7 @@ __global__ void __launch_bounds__(CL_THREADS, 1) k_solve_cl(const ClArgs<T> p) {
     auto apply_F = [&](const double* a, double* out) {
         for (int o = tid; o < s_off[fa.ncol]; o += NT) s_own[o] = a[s_lvl[o]];
         __syncthreads();
-        cl_tri_sweep<double>(s_vecd, s_own, s_lq, fa.L.ci, fa.L.d, false, fa.ncol, s_off, s_beg);
+        cl_tri_sweep<double, NT>(s_vecd, s_own, s_lq, fa.L.ci, fa.L.d, false, fa.ncol, s_off, s_beg);
         for (int i = rb + tid; i < re; i += NT) {
             double v = fa.wd[i] * s_vecd[fa.pos[i]];
             if (fa.part && fa.part[i] >= 0) v += fa.wo[i] * s_vecd[fa.pos[fa.part[i]]];
@@ -459,7 +461,7 @@ __global__ void __launch_bounds__(CL_THREADS, 1) k_solve_cl(const ClArgs<T> p) {
             s_own[o] = v;
         }
         __syncthreads();
-        cl_tri_sweep<double>(s_vecd, s_own, s_uq, fa.U.ci, fa.U.d, true, fa.ncol, s_off, s_beg);
+        cl_tri_sweep<double, NT>(s_vecd, s_own, s_uq, fa.U.ci, fa.U.d, true, fa.ncol, s_off, s_beg);
         for (int i = rb + tid; i < re; i += NT) out[i] = s_vecd[fa.pos[i]];
     };
     // s_f = (I + L)^-1 J^ (I + L)^-T (wd .* y) by position, y complete in L2
@@ -472,7 +474,7 @@ __global__ void __launch_bounds__(CL_THREADS, 1) k_solve_cl(const ClArgs<T> p) {
             own[o] = v;
         }
         __syncthreads();
-        cl_tri_sweep<T>(s_t, own, s_uq, fa.U.ci, fa.U.v, true, fa.ncol, s_off, s_beg);
+        cl_tri_sweep<T, NT>(s_t, own, s_uq, fa.U.ci, fa.U.v, true, fa.ncol, s_off, s_beg);
         for (int o = tid; o < s_off[fa.ncol]; o += NT) {
             const int2 rw = s_jq[o];
             T a = (T)0;
@@ -491,7 +493,7 @@ __global__ void __launch_bounds__(CL_THREADS, 1) k_solve_cl(const ClArgs<T> p) {
             own[o] = a;
         }
         __syncthreads();
-        cl_tri_sweep<T>(s_f, own, s_lq, fa.L.ci, fa.L.v, false, fa.ncol, s_off, s_beg);
+        cl_tri_sweep<T, NT>(s_f, own, s_lq, fa.L.ci, fa.L.v, false, fa.ncol, s_off, s_beg);
     };
 
     // ---------------------------------------------------------------------------
@@ -521,20 +523,20 @@ __global__ void __launch_bounds__(CL_THREADS, 1) k_solve_cl(const ClArgs<T> p) {
             // as k_mrs: FP32 a warp every 16th block, a lane a value; FP64 a lane an addition
             const P2* gp = reinterpret_cast<const P2*>(p.part + (size_t)buf * CL_XV * C);
             P2* bs = reinterpret_cast<P2*>(&sh.bsum[0][0]);
-            constexpr int NG = sizeof(T) == 4 ? NW : NT / NV;
+            constexpr int NG = sizeof(T) == 4 ? NW : NT / NV, UB = NT == 256 ? 20 : 10;   // UB: parts in flight
             for (int t = tid; t < (sizeof(T) == 4 ? NT : NG * NV); t += NT) {
                 const int g = sizeof(T) == 4 ? warp : t / NV;
                 for (int v = sizeof(T) == 4 ? lane : t % NV; v < NV; v += sizeof(T) == 4 ? 32 : NV) {
                     P2 acc{};
-                    for (int b0 = g; b0 < C; b0 += NG * 10) {
-                        P2 ld[10];
+                    for (int b0 = g; b0 < C; b0 += NG * UB) {
+                        P2 ld[UB];
 #pragma unroll
-                        for (int u = 0; u < 10; ++u) {
+                        for (int u = 0; u < UB; ++u) {
                             const int b = b0 + u * NG;
                             ld[u] = b < C ? __ldcg(&gp[(size_t)b * NV + v]) : P2{};
                         }
 #pragma unroll
-                        for (int u = 0; u < 10; ++u)
+                        for (int u = 0; u < UB; ++u)
                             if (b0 + u * NG < C) acc = add_t(acc, ld[u]);
                     }
                     bs[g * NV + v] = acc;
@@ -1142,14 +1144,14 @@ __global__ void __launch_bounds__(CL_THREADS, 1) k_solve_cl(const ClArgs<T> p) {
 // host side
 // ---------------------------------------------------------------------------
 // clusters of `size` CTAs that can be resident at once (0: none fits)
-template <class T, int KP, int FMT>
+template <class T, int KP, int FMT, int NT>
 static asss_status cl_clusters(int size, size_t smem, int* count) {
-    const void* fn = (const void*)k_solve_cl<T, KP, FMT, false>;
+    const void* fn = (const void*)k_solve_cl<T, KP, FMT, false, NT>;
     ASSS_TRY(raise_dynamic_smem(fn, (int)smem));
     if (size > 8) ASSS_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(size);
-    cfg.blockDim = dim3(CL_THREADS);
+    cfg.blockDim = dim3(NT);
     cfg.dynamicSmemBytes = smem;
     cudaLaunchAttribute at[1];
     at[0].id = cudaLaunchAttributeClusterDimension;
@@ -1166,11 +1168,11 @@ static asss_status cl_clusters(int size, size_t smem, int* count) {
 
 // launches `count` clusters of `size` CTAs, or (size == 0) asks how many clusters of each of
 // CL_SIZES can be resident, into counts
-template <class T, int KP, int FMT>
+template <class T, int KP, int FMT, int NT>
 static asss_status cl_run(const Ctx& c, const ClArgs<T>& a, int size, int count, int* counts) {
     ClArgs<T> b = a;
     auto bytes = [&](int sz) -> size_t {
-        size_t smem = ((sizeof(ClShared<T, KP, false>) + 15) & ~(size_t)15) +
+        size_t smem = ((sizeof(ClShared<T, KP, false, NT>) + 15) & ~(size_t)15) +
                       sizeof(double) * (size_t)(a.restart + 1) * (size_t)a.restart;
         if (FMT == 3) {
             b.fac.own_max = a.n / sz + a.fac.ncol + 1;
@@ -1182,14 +1184,14 @@ static asss_status cl_run(const Ctx& c, const ClArgs<T>& a, int size, int count,
         for (int t = 0; t < CL_NSIZES; ++t) {
             const size_t need = bytes(CL_SIZES[t]);
             counts[t] = 0;
-            if (need <= CL_SMEM_MAX) ASSS_TRY((cl_clusters<T, KP, FMT>(CL_SIZES[t], need, &counts[t])));
+            if (need <= CL_SMEM_MAX) ASSS_TRY((cl_clusters<T, KP, FMT, NT>(CL_SIZES[t], need, &counts[t])));
         }
         return ASSS_OK;
     }
     const size_t smem = bytes(size);
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(size * count);
-    cfg.blockDim = dim3(CL_THREADS);
+    cfg.blockDim = dim3(NT);
     cfg.dynamicSmemBytes = smem;
     cfg.stream = c.stream;
     cudaLaunchAttribute at[1];
@@ -1198,40 +1200,45 @@ static asss_status cl_run(const Ctx& c, const ClArgs<T>& a, int size, int count,
     at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
     cfg.attrs = at;
     cfg.numAttrs = 1;
-    ASSS_CUDA(cudaLaunchKernelEx(&cfg, k_solve_cl<T, KP, FMT, false>, b));
+    ASSS_CUDA(cudaLaunchKernelEx(&cfg, k_solve_cl<T, KP, FMT, false, NT>, b));
     count_launch();
     return ASSS_OK;
 }
 
 // grid scope: a cooperative launch of one block per SM (size < 0)
-template <class T, int KP>
+template <class T, int KP, int NT>
 static asss_status cl_run_grid(const Ctx& c, const ClArgs<T>& a) {
-    size_t smem = ((sizeof(ClShared<T, KP, true>) + 15) & ~(size_t)15) +
+    size_t smem = ((sizeof(ClShared<T, KP, true, NT>) + 15) & ~(size_t)15) +
                   sizeof(double) * (size_t)(a.restart + 1) * (size_t)a.restart;
-    const void* fn = (const void*)k_solve_cl<T, KP, 1, true>;
     const int need = cdiv(a.n, 32), blocks = c.sms < need ? c.sms : need;
+    const size_t q = sizeof(T) == 4 && KP > 0 ? cl_q_bytes(a.n, KP, blocks, smem) : 0;
+    const void* fn = nullptr;
     if constexpr (sizeof(T) == 4 && KP > 0) {
-        if (const size_t q = cl_q_bytes(a.n, KP, blocks, smem)) {
-            fn = (const void*)k_solve_cl<T, KP, 1, true, true>;
-            smem += q;
-        }
+        if (q) fn = (const void*)k_solve_cl<T, KP, 1, true, NT, true>;
     }
+    if constexpr (sizeof(T) == 8 || NT == 512) {
+        if (!q) fn = (const void*)k_solve_cl<T, KP, 1, true, NT>;
+    }
+    if (!fn) {   // (few rows a block: they fit)
+        set_error("solve: Q_k does not fit shared memory");
+        return ASSS_ERR_UNSUPPORTED;
+    }
+    smem += q;
     ClArgs<T> b = a;
     ASSS_TRY(raise_dynamic_smem(fn, (int)smem));
     void* args[] = {&b};
-    ASSS_CUDA(cudaLaunchCooperativeKernel(fn, dim3(blocks), dim3(CL_THREADS), args, smem, c.stream));
+    ASSS_CUDA(cudaLaunchCooperativeKernel(fn, dim3(blocks), dim3(NT), args, smem, c.stream));
     count_launch();
     return ASSS_OK;
 }
 
-template <class T, int FMT>
+template <class T, int FMT, int NT>
 asss_status cl_dispatch(const Ctx& c, const ClArgs<T>& a, int kp, int size, int count, int* counts) {
     switch (kp) {
 #define ASSS_CL_CASE(KPV) \
     case KPV:             \
-        if constexpr (FMT == 1) { if (size < 0) return cl_run_grid<T, KPV>(c, a); } \
-        return cl_run<T, KPV, FMT>(c, a, size, count, counts);
-        ASSS_CL_CASE(0)
+        if constexpr (FMT == 1) { if (size < 0) return cl_run_grid<T, KPV, NT>(c, a); } \
+        return cl_run<T, KPV, FMT, NT>(c, a, size, count, counts);
         ASSS_CL_CASE(4)
         ASSS_CL_CASE(8)
         ASSS_CL_CASE(12)
@@ -1239,6 +1246,11 @@ asss_status cl_dispatch(const Ctx& c, const ClArgs<T>& a, int kp, int size, int 
         ASSS_CL_CASE(20)
         ASSS_CL_CASE(24)
         ASSS_CL_CASE(32)
+        case 0:
+            if constexpr (sizeof(T) == 8 || NT == 512) {
+                if constexpr (FMT == 1) { if (size < 0) return cl_run_grid<T, 0, NT>(c, a); }
+                return cl_run<T, 0, FMT, NT>(c, a, size, count, counts);
+            }
 #undef ASSS_CL_CASE
         default:
             set_error("cluster solve: unsupported padded Lanczos width %d", kp);
@@ -1246,10 +1258,11 @@ asss_status cl_dispatch(const Ctx& c, const ClArgs<T>& a, int kp, int size, int 
     }
 }
 
-// (solve_cluster32.cu, solve_cluster64.cu, solve_cluster_fac32.cu, solve_cluster_fac64.cu)
-extern template asss_status cl_dispatch<float, 1>(const Ctx&, const ClArgs<float>&, int, int, int, int*);
-extern template asss_status cl_dispatch<double, 1>(const Ctx&, const ClArgs<double>&, int, int, int, int*);
-extern template asss_status cl_dispatch<float, 3>(const Ctx&, const ClArgs<float>&, int, int, int, int*);
-extern template asss_status cl_dispatch<double, 3>(const Ctx&, const ClArgs<double>&, int, int, int, int*);
+// (solve_cluster32.cu, solve_cluster32s.cu, solve_cluster64.cu, solve_cluster_fac32.cu, solve_cluster_fac64.cu)
+extern template asss_status cl_dispatch<float, 1, 512>(const Ctx&, const ClArgs<float>&, int, int, int, int*);
+extern template asss_status cl_dispatch<float, 1, 256>(const Ctx&, const ClArgs<float>&, int, int, int, int*);
+extern template asss_status cl_dispatch<double, 1, 256>(const Ctx&, const ClArgs<double>&, int, int, int, int*);
+extern template asss_status cl_dispatch<float, 3, 512>(const Ctx&, const ClArgs<float>&, int, int, int, int*);
+extern template asss_status cl_dispatch<double, 3, 512>(const Ctx&, const ClArgs<double>&, int, int, int, int*);
 
 }  // namespace asss

@@ -3,6 +3,6 @@
 
 namespace asss {
 
-template asss_status cl_dispatch<float, 1>(const Ctx&, const ClArgs<float>&, int, int, int, int*);
+template asss_status cl_dispatch<float, 1, 512>(const Ctx&, const ClArgs<float>&, int, int, int, int*);
 
 }  // namespace asss

@@ -3,6 +3,6 @@
 
 namespace asss {
 
-template asss_status cl_dispatch<double, 1>(const Ctx&, const ClArgs<double>&, int, int, int, int*);
+template asss_status cl_dispatch<double, 1, 256>(const Ctx&, const ClArgs<double>&, int, int, int, int*);
 
 }  // namespace asss

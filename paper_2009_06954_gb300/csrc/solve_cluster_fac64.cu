@@ -3,6 +3,6 @@
 
 namespace asss {
 
-template asss_status cl_dispatch<double, 3>(const Ctx&, const ClArgs<double>&, int, int, int, int*);
+template asss_status cl_dispatch<double, 3, 512>(const Ctx&, const ClArgs<double>&, int, int, int, int*);
 
 }  // namespace asss

@@ -1,6 +1,7 @@
 """Grid-scope solves that keep Q_k in shared memory, against the launch-by-launch path: the
-smallest systems of that path, ragged last slices, every width class, and the last sizes that
-fit and the first that do not (32 columns: about 250 000 rows on 152 SMs)."""
+smallest systems of that path, ragged last slices, every width class, both block sizes (up to
+768 rows a block and above), and the last sizes that fit and the first that do not (32 columns: about
+250 000 rows on 152 SMs)."""
 import numpy as np
 import pytest
 
@@ -11,8 +12,8 @@ from workloads import pattern_diagonal
 pytestmark = pytest.mark.gpu
 
 
-@pytest.mark.parametrize("n,k", [(14001, 1), (14016, 8), (15999, 11), (20033, 16), (31337, 20), (40000, 23), (240001, 32),
-                                 (262145, 32)])
+@pytest.mark.parametrize("n,k", [(14001, 1), (14016, 8), (15999, 11), (20033, 16), (31337, 20), (40000, 23), (116736, 4),
+                                 (116737, 4), (240001, 32), (262145, 32)])
 def test_matches(pkg, monkeypatch, n, k):  # noqa: F811
     A = banded(n, (-77, -9, -2, 3, 40), 6).tolil()
     A[3, 3] = -A[3, 3]
