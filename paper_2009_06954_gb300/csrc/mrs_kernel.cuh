@@ -519,11 +519,14 @@ __global__ void __launch_bounds__((mrs_threads<T, FMT>()), 1) k_mrs(MrsParams<T>
     // warp 1: fold direction p_jj into Q^T x (s_pq holds step jj's scalars, s_qty Q^T y_jj)
     auto qtx_fold = [&](int jj) {
         if constexpr (KP > 0) {
-            if (lane < p.k) {
-                T* pp = s_qtp[jj & 1];
-                const T v = (s_pq[0] * s_qty[lane] - s_pq[1] * pp[lane]) * s_pq[2];
-                pp[lane] = v;
-                s_qtx[lane] += s_pq[3] * v;
+#pragma unroll
+            for (int m = lane; m < lane + KP; m += 32) {   // two values a lane above k = 32
+                if (m < p.k) {
+                    T* pp = s_qtp[jj & 1];
+                    const T v = (s_pq[0] * s_qty[m] - s_pq[1] * pp[m]) * s_pq[2];
+                    pp[m] = v;
+                    s_qtx[m] += s_pq[3] * v;
+                }
             }
         }
     };
@@ -647,7 +650,9 @@ __global__ void __launch_bounds__((mrs_threads<T, FMT>()), 1) k_mrs(MrsParams<T>
             // off the synchronisation chain: step j-1's direction, then Q^T y_j from the
             // last reduction (s_red is next written after this pass's block barrier)
             if (j >= 2) qtx_fold(j - 1);
-            if (lane < p.k) s_qty[lane] = s_red[1 + lane];
+#pragma unroll
+            for (int m = lane; m < lane + KP; m += 32)
+                if (m < p.k) s_qty[m] = s_red[1 + m];
         }
         // the step's vectors do not overlap: restrict lets later rows' loads be scheduled
         // ahead of this row's stores
@@ -1002,7 +1007,11 @@ __global__ void __launch_bounds__((mrs_threads<T, FMT>()), 1) k_mrs(MrsParams<T>
             }
             if (want_qtx && warp == 1) {
                 qtx_fold(j);
-                if (blockIdx.x == 0 && lane < p.k) p.qtz[lane] = (double)s_qtx[lane];
+                if (blockIdx.x == 0) {
+#pragma unroll
+                    for (int m = lane; m < lane + KP; m += 32)
+                        if (m < p.k) p.qtz[m] = (double)s_qtx[m];
+                }
             }
             break;
         }
