@@ -113,6 +113,7 @@ struct DCsr {
 // last row map to row n (no row).
 constexpr int SELL_SIGMA = 4096;          // default sorting window
 constexpr int SELL_SIGMA_MAX = 16384;     // largest window the sort kernel takes
+constexpr double SELL_PAD = 1.2;          // rows are sorted when their natural order pads the entries by more
 template <class T>
 struct DSell {
     int n = 0;

@@ -19,9 +19,11 @@ asss_status build_pattern(const DCsr& Abar, const DCsr& AbarT, const DCsr& S, co
                           DBuf<int>& mirror, DBuf<int>& diagpos, cudaStream_t s);
 template <class T>
 asss_status build_sell(const DCsr& A, bool skip_diag, DSell<T>& out, cudaStream_t s, int sigma = 0, int split = 0);
-// the slices of rows of the given lengths (SELL-C, sorted in windows when they differ much)
+// the slices of rows of the given lengths (SELL-C, sorted in windows when they differ much); sptr
+// stays empty when the padded total exceeds 32-bit offsets
 asss_status sell_layout(const int* len, int n, int sigma, DBuf<int>& rowmap, DBuf<int>& rowpos, DBuf<int>& sptr,
                         int64_t* nnz, int64_t* total, cudaStream_t s);
+asss_status sort_windows(const int* len, int n, int sigma, DBuf<int>& rowmap, DBuf<int>& rowpos, cudaStream_t s);
 // Row-stream storage of A without its diagonal (see DStream); stream_fits: whether the
 // vector fits shared memory (in T) and the rows are long enough for a warp each
 template <class T>

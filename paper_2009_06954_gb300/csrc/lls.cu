@@ -213,14 +213,22 @@ __global__ void k_pair_flags(int nS, const int* partner, int* lead, int* single)
     lead[u] = p > u ? 1 : 0;
     single[u] = p < 0 ? 1 : 0;
 }
-__global__ void k_pair_slots(int nS, const int* partner, const int* lpos, const int* spos, int npairs, int* upos,
-                             int* uslot) {
+// (pmap, smap: places of the pairs and of the single unknowns, null for their own order)
+__global__ void k_pair_slots(int nS, const int* partner, const int* lpos, const int* spos, const int* pmap,
+                             const int* smap, int npairs, int* upos, int* uslot) {
     int u = blockIdx.x * blockDim.x + threadIdx.x;
     if (u >= nS) return;
     const int p = partner[u];
-    const int slot = p < 0 ? 2 * npairs + spos[u] : p > u ? 2 * lpos[u] : 2 * lpos[p] + 1;
+    const int t = p < 0 ? spos[u] : lpos[p > u ? u : p];   // number of the single unknown or of the pair
+    const int slot = p < 0 ? 2 * npairs + (smap ? smap[t] : t) : 2 * (pmap ? pmap[t] : t) + (p > u ? 0 : 1);
     upos[u] = slot;
     uslot[slot] = u;
+}
+// lengths by pair (the longer of its two rows) and by single unknown, from the lengths by slot
+__global__ void k_pair_len(int npairs, int nsingle, const int* tlen, int* plen, int* slen) {
+    const int t = blockIdx.x * blockDim.x + threadIdx.x;
+    if (t < npairs) plen[t] = max(tlen[2 * t], tlen[2 * t + 1]);
+    else if (t - npairs < nsingle) slen[t - npairs] = tlen[npairs + t];
 }
 // walk of row u of B^T (as k_lls_BT): count, or fill with columns in constraint slots
 __device__ __forceinline__ int btx_row(int u, const int* __restrict__ srow, const int* __restrict__ sci,
@@ -560,7 +568,7 @@ asss_status lls_product_on_pattern(const Ctx& c, const DCsr& Abar, const DCsr& S
     return ASSS_OK;
 }
 
-// slice offsets of rows in the given order (no sorting)
+// slice offsets of rows in the given order; sptr stays empty when the total exceeds 32 bits
 __global__ void k_slice_width(const int* len, int ns, int* w) {
     const int sl = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
     if (sl >= ns) return;
@@ -574,18 +582,16 @@ static asss_status pair_layout(const int* len, int nslots, DBuf<int>& sptr, int6
     DBuf<long long> off64;
     ASSS_TRY(w.alloc(ns > 0 ? ns : 1));
     ASSS_TRY(off64.alloc(ns + 1));
-    ASSS_TRY(sptr.alloc(ns + 1));
+    sptr.free();
     k_slice_width<<<cdiv(32LL * ns, 256), 256, 0, s>>>(len, ns, w.p);
     ASSS_CHECK_LAUNCH();
     long long tot = 0;
     ASSS_TRY(exclusive_scan64(w.p, off64.p, ns, &tot, s));
-    if (tot >= (1LL << 31) - 1) {
-        set_error("least-squares storage of %lld entries exceeds 32-bit slice offsets", tot);
-        return ASSS_ERR_UNSUPPORTED;
-    }
+    *total = tot;
+    if (tot >= (1LL << 31) - 1) return ASSS_OK;
+    ASSS_TRY(sptr.alloc(ns + 1));
     ASSS_TRY(exclusive_scan(w.p, sptr.p, ns, nullptr, s));
     ASSS_CUDA(cudaStreamSynchronize(s));   // w is freed here
-    *total = tot;
     return ASSS_OK;
 }
 
@@ -624,8 +630,9 @@ asss_status lls_fit(const Ctx& c, const DCsr& Abar, const DCsr& AbarT, const DCs
 
     const double sg = sqrt(gamma);
     // B and B^T stored explicitly when they fit min(8 GiB, a quarter of the free device
-    // memory), and the whole iteration in one launch; otherwise the merge kernels apply them
-    // matrix-free
+    // memory) with their slices' padding and the iteration's vectors, and the whole iteration in
+    // one launch; otherwise the merge kernels apply them matrix-free (ASSS_LLS_STORE_BYTES: another
+    // bound)
     {
         DBuf<int> bcnt, cflag, cidx, uslot, upos, lead, single, lpos, spos, tlen;
         ASSS_TRY(bcnt.alloc(nP > 0 ? nP : 1));
@@ -634,7 +641,7 @@ asss_status lls_fit(const Ctx& c, const DCsr& Abar, const DCsr& AbarT, const DCs
         k_bx_count<<<cdiv(nP, 256), 256, 0, s>>>(nP, prow.p, P.ci.p, Abar.rp.p, Abar.ci.p, Abar.v.p, ST.rp.p, ST.ci.p,
                                                   st_src.p, bcnt.p, cflag.p);
         ASSS_CHECK_LAUNCH();
-        int64_t nC = 0, npairs = 0, nsingle = 0, nb = 0, nt = 0;
+        int64_t nC = 0, npairs = 0, nsingle = 0, nb = 0, nt = 0, bt = 0, tt = 0;
         ASSS_TRY(exclusive_scan(cflag.p, cidx.p, nP, &nC, s));
         ASSS_TRY(lead.alloc(nS));
         ASSS_TRY(single.alloc(nS));
@@ -645,35 +652,57 @@ asss_status lls_fit(const Ctx& c, const DCsr& Abar, const DCsr& AbarT, const DCs
         ASSS_TRY(exclusive_scan(lead.p, lpos.p, nS, &npairs, s));
         ASSS_TRY(exclusive_scan(single.p, spos.p, nS, &nsingle, s));
         const int nuslots = cdiv(2 * npairs + nsingle, 32) * 32;
+        const int nbs = cdiv(nC, 32), nts = nuslots / 32;
         ASSS_TRY(upos.alloc(nS));
         ASSS_TRY(uslot.alloc(nuslots));
         ASSS_TRY(tlen.alloc(nuslots));
-        ASSS_CUDA(cudaMemsetAsync(uslot.p, 0xff, sizeof(int) * (size_t)nuslots, s));
-        k_pair_slots<<<cdiv(nS, 256), 256, 0, s>>>(nS, partner.p, lpos.p, spos.p, (int)npairs, upos.p, uslot.p);
-        ASSS_CHECK_LAUNCH();
-        k_btx_count<<<cdiv(nuslots, 256), 256, 0, s>>>(nuslots, uslot.p, srow.p, Spat.ci.p, AbarT.rp.p, AbarT.ci.p,
-                                                        AbarT.v.p, P.rp.p, P.ci.p, mirror.p, tlen.p);
-        ASSS_CHECK_LAUNCH();
+        // slots of the unknowns (pmap, smap: see k_pair_slots) and the lengths of their rows of B^T
+        auto place = [&](const int* pmap, const int* smap) -> asss_status {
+            ASSS_CUDA(cudaMemsetAsync(uslot.p, 0xff, sizeof(int) * (size_t)nuslots, s));
+            k_pair_slots<<<cdiv(nS, 256), 256, 0, s>>>(nS, partner.p, lpos.p, spos.p, pmap, smap, (int)npairs, upos.p,
+                                                        uslot.p);
+            ASSS_CHECK_LAUNCH();
+            k_btx_count<<<cdiv(nuslots, 256), 256, 0, s>>>(nuslots, uslot.p, srow.p, Spat.ci.p, AbarT.rp.p, AbarT.ci.p,
+                                                            AbarT.v.p, P.rp.p, P.ci.p, mirror.p, tlen.p);
+            ASSS_CHECK_LAUNCH();
+            return ASSS_OK;
+        };
+        ASSS_TRY(place(nullptr, nullptr));
         ASSS_TRY(sum_counts(bcnt.p, nP, &nb, s));
         ASSS_TRY(sum_counts(tlen.p, nuslots, &nt, s));
         size_t fr = 0, tot = 0;
         ASSS_CUDA(cudaMemGetInfo(&fr, &tot));
-        const double need = 12.0 * (double)(nb + nt) + 8.0 * (double)(nP + nS);
-        const double budget = fmin(8.0 * 1024 * 1024 * 1024, 0.25 * (double)fr);
-        if (nb < 0x3fffffffLL && nt < 0x3fffffffLL && need <= budget) {
-            DBuf<int> klist, blen, bmap, bpos, bsp, tmap, tpos, tsp, bcol, tcol, its_d;
-            DBuf<double> bval, tval, m1, m2, sv, zz, pp, qq, rr, part, rel_d;
-            DBuf<unsigned> bar;
-            DBuf<int> err;
+        const char* bound = getenv("ASSS_LLS_STORE_BYTES");
+        const double budget = bound ? atof(bound) : fmin(8.0 * 1024 * 1024 * 1024, 0.25 * (double)fr);
+        const double vectors = 8.0 * (5.0 * nuslots + 2.0 * 32 * nbs);
+        DBuf<int> klist, blen, bmap, bpos, bsp, tsp;
+        if (12.0 * (double)(nb + nt) + vectors <= budget) {   // else the padded form is above it too
             ASSS_TRY(klist.alloc(nC));
             ASSS_TRY(blen.alloc(nC));
             k_bx_list<<<cdiv(nP, 256), 256, 0, s>>>(nP, cflag.p, cidx.p, bcnt.p, klist.p, blen.p);
             ASSS_CHECK_LAUNCH();
-            int64_t bn = 0, bt = 0, tt = 0;
-            ASSS_TRY(sell_layout(blen.p, (int)nC, SELL_SIGMA, bmap, bpos, bsp, &bn, &bt, s));
-            // pairs stay together: the unknowns keep their slots whatever the padding
+            ASSS_TRY(sell_layout(blen.p, (int)nC, SELL_SIGMA, bmap, bpos, bsp, &nb, &bt, s));
+            // B^T: the pairs, and behind them the single unknowns, are sorted by length within
+            // windows where their own order pads much (a pair then takes the longer of its rows
+            // twice, so what stays is at most about twice the entries)
             ASSS_TRY(pair_layout(tlen.p, nuslots, tsp, &tt, s));
-            const int nbs = cdiv(nC, 32), nts = nuslots / 32;
+            if ((double)tt > SELL_PAD * (double)nt) {
+                DBuf<int> plen, slen, back, pmap, smap;
+                ASSS_TRY(plen.alloc(npairs));
+                ASSS_TRY(slen.alloc(nsingle));
+                k_pair_len<<<cdiv(npairs + nsingle, 256), 256, 0, s>>>((int)npairs, (int)nsingle, tlen.p, plen.p, slen.p);
+                ASSS_CHECK_LAUNCH();
+                ASSS_TRY(sort_windows(plen.p, (int)npairs, SELL_SIGMA, back, pmap, s));
+                ASSS_TRY(sort_windows(slen.p, (int)nsingle, SELL_SIGMA, back, smap, s));
+                ASSS_TRY(place(pmap.p, smap.p));
+                ASSS_TRY(pair_layout(tlen.p, nuslots, tsp, &tt, s));   // (synchronises: the maps are freed here)
+            }
+        }
+        if (bsp.p && tsp.p && 12.0 * (double)(bt + tt) + vectors <= budget) {
+            DBuf<int> bcol, tcol, its_d;
+            DBuf<double> bval, tval, m1, m2, sv, zz, pp, qq, rr, part, rel_d;
+            DBuf<unsigned> bar;
+            DBuf<int> err;
             ASSS_TRY(bcol.alloc(bt > 0 ? bt : 1));
             ASSS_TRY(bval.alloc(bt > 0 ? bt : 1));
             ASSS_TRY(tcol.alloc(tt > 0 ? tt : 1));

@@ -990,9 +990,23 @@ __global__ void k_sell_fill(int n, int nslices, const int* rp, const int* ci, co
     }
 }
 
+// rowmap (slot -> row, n for padding) and rowpos (row -> slot) with each window of sigma rows sorted
+// by length
+asss_status sort_windows(const int* len, int n, int sigma, DBuf<int>& rowmap, DBuf<int>& rowpos, cudaStream_t s) {
+    const int nslots = cdiv(n, 32) * 32;
+    ASSS_TRY(rowmap.alloc(nslots));
+    ASSS_TRY(rowpos.alloc(n));
+    if (n < 1) return ASSS_OK;
+    const size_t smem = sizeof(long long) * (size_t)sigma;
+    ASSS_TRY(raise_dynamic_smem((const void*)k_sell_sort_window, (int)smem));
+    k_sell_sort_window<<<cdiv(nslots, sigma), SELL_SORT_THREADS, smem, s>>>(n, nslots, sigma, len, rowmap.p, rowpos.p);
+    ASSS_CHECK_LAUNCH();
+    return ASSS_OK;
+}
+
 // The slices of rows of the given lengths: natural order, or (sorted windows of sigma rows) when
 // that pads the stored entries by more than a fifth.  rowmap / rowpos stay empty in natural
-// order; *total counts the padding.
+// order; *total counts the padding.  sptr stays empty when the total exceeds its 32-bit offsets.
 asss_status sell_layout(const int* len, int n, int sigma, DBuf<int>& rowmap, DBuf<int>& rowpos, DBuf<int>& sptr,
                         int64_t* nnz, int64_t* total, cudaStream_t s) {
     const int ns = cdiv(n, 32);
@@ -1004,6 +1018,7 @@ asss_status sell_layout(const int* len, int n, int sigma, DBuf<int>& rowmap, DBu
     ASSS_TRY(off64.alloc(ns + 1));
     rowmap.free();
     rowpos.free();
+    sptr.free();
     long long tot = 0;
     unsigned long long hn = 0;
     for (int pass = 0; pass < 2; ++pass) {
@@ -1013,23 +1028,12 @@ asss_status sell_layout(const int* len, int n, int sigma, DBuf<int>& rowmap, DBu
         ASSS_CHECK_LAUNCH();
         ASSS_CUDA(cudaMemcpyAsync(&hn, cnt.p, sizeof(hn), cudaMemcpyDeviceToHost, s));
         ASSS_TRY(exclusive_scan64(w.p, off64.p, ns, &tot, s));   // 64-bit total (synchronises)
-        if (pass == 1 || (double)tot <= 1.2 * (double)hn) break;
-        // heavy-tailed rows: sort each window of sigma rows by length
-        const int nslots = ns * 32;
-        ASSS_TRY(rowmap.alloc(nslots));
-        ASSS_TRY(rowpos.alloc(n));
-        const size_t smem = sizeof(long long) * (size_t)sigma;
-        ASSS_TRY(raise_dynamic_smem((const void*)k_sell_sort_window, (int)smem));
-        k_sell_sort_window<<<cdiv(nslots, sigma), SELL_SORT_THREADS, smem, s>>>(n, nslots, sigma, len, rowmap.p,
-                                                                                rowpos.p);
-        ASSS_CHECK_LAUNCH();
+        if (pass == 1 || (double)tot <= SELL_PAD * (double)hn) break;
+        ASSS_TRY(sort_windows(len, n, sigma, rowmap, rowpos, s));   // heavy-tailed rows
     }
     *nnz = (int64_t)hn;
     *total = tot;
-    if (tot >= (1LL << 31) - 1) {
-        set_error("SELL-C storage of %lld entries exceeds 32-bit slice offsets", tot);
-        return ASSS_ERR_UNSUPPORTED;
-    }
+    if (tot >= (1LL << 31) - 1) return ASSS_OK;
     ASSS_TRY(sptr.alloc(ns + 1));
     ASSS_TRY(exclusive_scan(w.p, sptr.p, ns, nullptr, s));
     ASSS_CUDA(cudaStreamSynchronize(s));   // w is freed here
@@ -1064,6 +1068,10 @@ asss_status build_sell(const DCsr& A, bool skip_diag, DSell<T>& out, cudaStream_
     ASSS_CHECK_LAUNCH();
     int64_t tot = 0;
     ASSS_TRY(sell_layout(len.p, n, sigma, out.rowmap, out.rowpos, out.sptr, &out.nnz, &tot, s));
+    if (!out.sptr.p) {
+        set_error("SELL-C storage of %lld entries exceeds 32-bit slice offsets", (long long)tot);
+        return ASSS_ERR_UNSUPPORTED;
+    }
     if (out.rowmap.p) out.sigma = sigma;
     out.nstored = tot;
     ASSS_TRY(out.col.alloc(tot > 0 ? tot : 1));
