@@ -644,14 +644,13 @@ struct asss_handle {
     // the clusters, staging of the columns and statistics
     int cl_counts[CL_NSIZES] = {-1, -1, -1, -1};
     DBuf<double> cl_work, cl_b, cl_x;
-    static constexpr int CL_CHUNK = 16;   // columns of a launch
-    ClStat* cl_st = nullptr;   // pinned, CL_CHUNK entries
-    unsigned cl_phase = 0;     // barriers passed on cl_bar
-    DBuf<double> cl_part;      // grid scope: block partials, barrier and status
+    ClReport* cl_rep = nullptr;   // pinned
+    unsigned cl_phase = 0;     // barriers passed on cl_bar (0: it is cleared before the next launch)
+    DBuf<double> cl_part;      // grid scope: block partials and barrier
     DBuf<unsigned> cl_bar;
     ~asss_handle() {
         if (mw) mrs_work_destroy(mw);
-        if (cl_st) cudaFreeHost(cl_st);
+        if (cl_rep) cudaFreeHost(cl_rep);
     }
 };
 
@@ -2206,7 +2205,7 @@ static asss_status cluster_plan(asss_handle* h, int nrhs, int* size) {
 }
 
 // enqueues nc columns of a solve (size: see cluster_size), b and x on the device and apart; their
-// statistics are in h->cl_st once the stream is synchronised
+// statistics are in h->cl_rep once the stream is synchronised
 template <class T>
 static asss_status solve_cluster(asss_handle* h, int tr, int size, int nc, const double* b, int64_t ldb, double* x,
                                  int64_t ldx) {
@@ -2220,18 +2219,21 @@ static asss_status solve_cluster(asss_handle* h, int tr, int size, int nc, const
     int count = 1;
     for (int t = 0; t < CL_NSIZES; ++t)
         if (CL_SIZES[t] == size) count = nc < h->cl_counts[t] ? nc : h->cl_counts[t];
+    if (!h->cl_rep) ASSS_CUDA(cudaMallocHost((void**)&h->cl_rep, sizeof(ClReport)));
+    cl_expect(*h->cl_rep, nc);
     if (size < 0) {   // grid scope
         const int64_t np = 2LL * CL_XV * c.sms;
         if (h->cl_part.n < np) ASSS_TRY(h->cl_part.alloc(np));
         if (!h->cl_bar.p || h->cl_phase == 0 || h->cl_phase > 0x1000000u) {   // (152 arrivals a barrier in 32 bits)
-            if (!h->cl_bar.p) ASSS_TRY(h->cl_bar.alloc(2));
-            ASSS_CUDA(cudaMemsetAsync(h->cl_bar.p, 0, 2 * sizeof(unsigned), s));   // arrivals and status
+            if (!h->cl_bar.p) ASSS_TRY(h->cl_bar.alloc(1));
+            ASSS_CUDA(cudaMemsetAsync(h->cl_bar.p, 0, sizeof(unsigned), s));   // arrivals
             h->cl_phase = 0;
         }
         a.phase0 = h->cl_phase;
+        h->cl_phase = 0;   // until the launch is known to have passed its barriers
         a.part = h->cl_part.p;
         a.gb.count = h->cl_bar.p;
-        a.gb.err = reinterpret_cast<int*>(h->cl_bar.p + 1);
+        a.gb.err = &h->cl_rep->wait;
         a.budget = c.wait_cycles;
         const long long tb = (long long)sizeof(T), nnz = tb == 4 ? h->D32.nnz : h->D64.nnz;
         a.cs = stream_evict_first(c, nnz * tb + (long long)h->n * (7 * tb + tb * h->kp)) ? 1 : 0;
@@ -2243,9 +2245,8 @@ static asss_status solve_cluster(asss_handle* h, int tr, int size, int nc, const
     a.ldx = ldx;
     a.work_stride = cl_work_doubles(h->n, a.halo, o.restart, (int)sizeof(T));
     if (h->cl_work.n < a.work_stride * count) ASSS_TRY(h->cl_work.alloc(a.work_stride * count));
-    if (!h->cl_st) ASSS_CUDA(cudaMallocHost((void**)&h->cl_st, sizeof(ClStat) * asss_handle::CL_CHUNK));
     a.work = h->cl_work.p;
-    a.stats = h->cl_st;
+    a.stats = h->cl_rep->st;
     if (h->factored) return cl_dispatch<T, 3, 512>(c, a, h->kp, size, count, nullptr);
     if constexpr (sizeof(T) == 4) {
         const int rows = cdiv(h->n, size < 0 ? c.sms : size);   // of a CTA
@@ -2401,7 +2402,7 @@ static asss_status solve_common(asss_handle* h, int tr, int nrhs, const double* 
     ASSS_TRY(cluster_plan(h, nrhs, &cl));
     // whole solves in one launch: a cluster per column, or the whole grid column by column
     for (int j0 = 0; cl != 0 && j0 < nrhs;) {
-        const int nc = nrhs - j0 < asss_handle::CL_CHUNK ? nrhs - j0 : asss_handle::CL_CHUNK;
+        const int nc = nrhs - j0 < CL_CHUNK ? nrhs - j0 : CL_CHUNK;
         const double* b0 = b + (size_t)j0 * ldb;
         double* x0 = x + (size_t)j0 * ldx;
         // the kernel reads b to the end, so it is staged where x overlaps it, and what is the host's
@@ -2431,16 +2432,14 @@ static asss_status solve_common(asss_handle* h, int tr, int nrhs, const double* 
         if (tr && xfwd && dA)
             for (int t = 0; t < nc; ++t) ASSS_TRY(grad_A(h, j0 + t, xt + (size_t)t * ldt, xfwd, ldxf, dA));
         ASSS_CUDA(cudaStreamSynchronize(s));
-        const ClStat* cs = h->cl_st;
-        if (cl < 0) {
-            h->cl_phase = cs[nc - 1].phase;
-            for (int t = 0; t < nc; ++t)
-                if (cs[t].status == ASSS_ERR_TIMEOUT) {
-                    h->cl_phase = 0;   // the barrier starts anew
-                    set_error("solve: a grid barrier wait exceeded its budget");
-                    return ASSS_ERR_TIMEOUT;
-                }
+        unsigned phase = 0;
+        const asss_status waits = cl_outcome(*h->cl_rep, nc, &phase);
+        if (cl < 0) h->cl_phase = phase;
+        if (waits != ASSS_OK) {
+            set_error("solve: a grid barrier wait exceeded its budget");
+            return waits;
         }
+        const ClStat* cs = h->cl_rep->st;
         for (int t = 0; t < nc; ++t) {
             const asss_stats prev = lst;
             cluster_stats(h, tr, cs[t], &lst);

@@ -19,6 +19,7 @@
 #include "cluster_dev.cuh"
 #include "internal.h"
 #include "mrs_dev.cuh"
+#include "solve_rules.h"
 
 namespace asss {
 
@@ -59,14 +60,6 @@ struct ClFactor {
     const int* part;
 };
 
-struct ClStat {
-    int outer_its, cycles, status, solves, op_calls, orth_calls;
-    long long inner_its, orth_vecs;
-    unsigned long long ns_inner, ns_op, ns_orth;
-    double relres;
-    unsigned phase;   // grid scope: barriers passed on the counter
-};
-
 template <class T>
 struct ClArgs {
     int n, ncol, restart;
@@ -95,10 +88,11 @@ struct ClArgs {
     long long work_stride;
     double outer_tol, inner_tol;
     int outer_maxit, inner_maxit;
-    ClStat* stats;            // pinned host memory, read after the stream is synchronised
+    ClStat* stats;            // pinned host memory (ClReport), read after the stream is synchronised
     unsigned phase0;          // grid scope: barriers passed before this launch
     // grid scope: block partials (2 x [blocks][CL_XV]), barrier and its budget, evict-first loads of
-    // what is read once (the data of a step exceed L2)
+    // what is read once (the data of a step exceed L2); the barrier's status word stands in the
+    // pinned report too, so the host has it without a copy (a wait reads it every 64th poll only)
     double* part;
     GridBarrier gb;
     long long budget;

@@ -1,0 +1,41 @@
+// Rules of the solve path that need no CUDA, so that any host can check them.
+#pragma once
+
+#include "asss.h"
+
+namespace asss {
+
+// what a whole-solve launch reports of a column; block 0 writes it before the column's last barrier
+struct ClStat {
+    int outer_its, cycles, status, solves, op_calls, orth_calls;
+    long long inner_its, orth_vecs;
+    unsigned long long ns_inner, ns_op, ns_orth;
+    double relres;
+    unsigned phase;   // grid scope: barriers passed on the counter
+};
+constexpr int CL_CHUNK = 16;   // columns of a launch
+struct ClReport {
+    int wait;   // grid scope: the barrier's status word, ASSS_ERR_TIMEOUT from any block that gave up
+    ClStat st[CL_CHUNK];
+};
+
+// before a launch of nc columns: nothing is reported yet, so that what the kernel does not get to
+// write (the columns after a wait that ran out) does not pass for an earlier launch's result
+inline void cl_expect(ClReport& r, int nc) {
+    r.wait = ASSS_OK;
+    for (int t = 0; t < nc; ++t) r.st[t].status = ASSS_ERR_TIMEOUT;
+}
+
+// after it: ASSS_ERR_TIMEOUT when any wait ran out, also one at a column's last barrier, where
+// that column's own status says nothing; *phase: barriers passed on the counter, 0 when the
+// counter has to be cleared before the next launch
+inline asss_status cl_outcome(const ClReport& r, int nc, unsigned* phase) {
+    *phase = 0;
+    if (r.wait != ASSS_OK) return ASSS_ERR_TIMEOUT;
+    for (int t = 0; t < nc; ++t)
+        if (r.st[t].status == ASSS_ERR_TIMEOUT) return ASSS_ERR_TIMEOUT;
+    *phase = r.st[nc - 1].phase;
+    return ASSS_OK;
+}
+
+}  // namespace asss
