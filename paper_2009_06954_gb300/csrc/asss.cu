@@ -2402,14 +2402,18 @@ static asss_status solve_common(asss_handle* h, int tr, int nrhs, const double* 
     ASSS_TRY(cluster_plan(h, nrhs, &cl));
     // whole solves in one launch: a cluster per column, or the whole grid column by column
     for (int j0 = 0; cl != 0 && j0 < nrhs;) {
-        const int nc = nrhs - j0 < CL_CHUNK ? nrhs - j0 : CL_CHUNK;
+        int nc = nrhs - j0 < CL_CHUNK ? nrhs - j0 : CL_CHUNK;
         const double* b0 = b + (size_t)j0 * ldb;
         double* x0 = x + (size_t)j0 * ldx;
-        // the kernel reads b to the end, so it is staged where x overlaps it, and what is the host's
+        // the kernel reads b to the end and in place: it is staged where x overlaps it, where it is
+        // the host's or another device's, and where it is not aligned to its entries
         const bool apart = b0 + (size_t)(nc - 1) * ldb + n <= x0 || x0 + (size_t)(nc - 1) * ldx + n <= b0;
+        const bool stage = !apart || !is_on_device(b0, h->ctx.device) || (uintptr_t)b0 % sizeof(double) != 0;
+        // in grid scope the columns run one after another, so fewer of large ones are staged at once
+        if (cl < 0 && (stage || !xdev)) nc = std::max(1, std::min(nc, (int)((1 << 25) / (int64_t)n)));
         const double* bt = b0;
         int64_t ldbt = ldb;
-        if (!bdev || !apart) {
+        if (stage) {
             if (h->cl_b.n < (int64_t)nc * n) ASSS_TRY(h->cl_b.alloc((int64_t)nc * n));
             const cudaMemcpyKind kind = bdev ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice;
             if (nc == 1) ASSS_CUDA(cudaMemcpyAsync(h->cl_b.p, b0, sizeof(double) * n, kind, s));

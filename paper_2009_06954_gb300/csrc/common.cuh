@@ -322,6 +322,8 @@ asss_status make_ctx(Ctx& c, void* stream, double wait_timeout_ms);
 
 // pointer classification
 bool is_device_ptr(const void* p);
+// device (or managed) memory that belongs to device dev, which its kernels read in place
+bool is_on_device(const void* p, int dev);
 
 // copy n elements from a host-or-device pointer into a device buffer
 template <class T>

@@ -285,17 +285,6 @@ constexpr long long NOALLOC_DOUBLES = NOALLOC_CTRL + NOALLOC_PART + NOALLOC_BLK 
 // [ctrl | partials | block table | Y: 3 slots of n | P: 2 slots of n]
 static __device__ __align__(256) double g_noalloc_scratch[NOALLOC_DOUBLES];
 
-// device (or managed) memory that belongs to device dev
-static bool noalloc_on_device(const void* p, int dev) {
-    cudaPointerAttributes a;
-    if (cudaPointerGetAttributes(&a, p) != cudaSuccess) {
-        cudaGetLastError();
-        return false;
-    }
-    if (a.type == cudaMemoryTypeManaged) return true;
-    return a.type == cudaMemoryTypeDevice && a.device == dev;
-}
-
 static double* noalloc_base(int* status) {
     static std::mutex mu;
     static double* base[256] = {};
@@ -402,7 +391,7 @@ extern "C" asss_status asss_mrs_noalloc(int64_t n, int64_t nnz, const int64_t* r
                         {k > 1 ? alpha : nullptr, 8, "alpha"}};
     for (const Arr& a : arrs) {
         if (!a.p) continue;
-        if (!noalloc_on_device(a.p, cur_dev)) {
+        if (!is_on_device(a.p, cur_dev)) {
             set_error("asss_mrs_noalloc: %s must be device memory of the current device %d", a.name, cur_dev);
             return ASSS_ERR_ARG;
         }
