@@ -1969,9 +1969,9 @@ static asss_status do_setup(asss_handle* h, const asss_csr* Ain, asss_stats* st)
         // long rows, no layout asked for: the single-column solve of this precision takes the row
         // stream (the SELL copies stay for the multi-column and batched kernels and the set-up)
         const bool rows = o.inner_format == ASSS_FORMAT_AUTO && o.sell_sigma == 0 && o.sell_split == 0;
-        if (rows && o.precision == ASSS_PREC_MIXED && stream_fits<float>(n, h->J32.nnz))
+        if (rows && o.precision == ASSS_PREC_MIXED && stream_fits(n, h->J32.nnz, sizeof(float)))
             ASSS_TRY(build_stream<float>(h->Jt, h->R32, s));
-        if (rows && o.precision == ASSS_PREC_FP64 && stream_fits<double>(n, h->J64.nnz))
+        if (rows && o.precision == ASSS_PREC_FP64 && stream_fits(n, h->J64.nnz, sizeof(double)))
             ASSS_TRY(build_stream<double>(h->Jt, h->R64, s));
         st->sell_sigma = h->J64.sigma;
         st->sell_split = h->J64.split;

@@ -24,10 +24,7 @@ asss_status build_sell(const DCsr& A, bool skip_diag, DSell<T>& out, cudaStream_
 asss_status sell_layout(const int* len, int n, int sigma, DBuf<int>& rowmap, DBuf<int>& rowpos, DBuf<int>& sptr,
                         int64_t* nnz, int64_t* total, cudaStream_t s);
 asss_status sort_windows(const int* len, int n, int sigma, DBuf<int>& rowmap, DBuf<int>& rowpos, cudaStream_t s);
-// Row-stream storage of A without its diagonal (see DStream); stream_fits: whether the
-// vector fits shared memory (in T) and the rows are long enough for a warp each
-template <class T>
-bool stream_fits(int n, int64_t nnz);
+// Row-stream storage of A without its diagonal (see DStream; where: stream_fits in solve_rules.h)
 template <class T>
 asss_status build_stream(const DCsr& A, DStream<T>& out, cudaStream_t s);
 // Skew half-diagonal storage of J when J is exactly skew, has at most max_diag

@@ -1,9 +1,20 @@
 // Rules of the solve path that need no CUDA, so that any host can check them.
 #pragma once
 
+#include <cstdint>
+
 #include "asss.h"
 
 namespace asss {
+
+// Whether the single-column solve takes the row stream (DStream) for n rows with nnz entries off the
+// diagonal, vectors of tbytes a value.  The vector stays below 192 KB, which leaves the block its partial
+// sums and row sums, and its indices below 16 bits.  From 64 entries a row on, half of a warp's lanes
+// or more have an entry in the row's first load; below that SELL's lane per row wastes less.
+// Offsets are 32-bit: a matrix whose rows, padded by up to 3 entries each, may pass them stays in SELL.
+inline bool stream_fits(int n, int64_t nnz, int tbytes) {
+    return (int64_t)n * tbytes <= 192000 && nnz >= (int64_t)64 * n && nnz + 3LL * n < (1LL << 31) - 1024;
+}
 
 // what a whole-solve launch reports of a column; block 0 writes it before the column's last barrier
 struct ClStat {

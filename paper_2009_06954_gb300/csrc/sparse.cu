@@ -1127,16 +1127,6 @@ template asss_status build_sell<float>(const DCsr&, bool, DSell<float>&, cudaStr
 // ---------------------------------------------------------------------------
 // row-stream storage (DStream) of A without its diagonal
 // ---------------------------------------------------------------------------
-// The vector stays below 192 KB, which leaves the block its partial sums and row sums, and
-// its indices below 16 bits.  From 64 entries a row on, half of a warp's lanes or more
-// have an entry in the row's first load; below that SELL's lane per row wastes less.
-template <class T>
-bool stream_fits(int n, int64_t nnz) {
-    return (int64_t)n * (int64_t)sizeof(T) <= 192000 && nnz >= (int64_t)64 * n;
-}
-template bool stream_fits<double>(int, int64_t);
-template bool stream_fits<float>(int, int64_t);
-
 __global__ void k_stream_len(int n, const int* len, int* padded) {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i < n) padded[i] = (len[i] + 3) & ~3;
@@ -1174,16 +1164,8 @@ asss_status build_stream(const DCsr& A, DStream<T>& out, cudaStream_t s) {
     k_stream_len<<<cdiv(n, 256), 256, 0, s>>>(n, len.p, padded.p);
     ASSS_CHECK_LAUNCH();
     ASSS_TRY(out.rp.alloc(n + 1));
-    // every offset is below n^2 <= 48000^2 < 2^32; one that reaches 2^31 is refused here
-    long long tot = 0;
-    DBuf<long long> off64;
-    ASSS_TRY(off64.alloc(n + 1));
-    ASSS_TRY(exclusive_scan64(padded.p, off64.p, n, &tot, s));
-    if (tot >= (1LL << 31) - 1024) {
-        set_error("row-stream storage of %lld entries exceeds 32-bit offsets", tot);
-        return ASSS_ERR_UNSUPPORTED;
-    }
-    ASSS_TRY(exclusive_scan(padded.p, out.rp.p, n, nullptr, s));
+    int64_t tot = 0;
+    ASSS_TRY(exclusive_scan(padded.p, out.rp.p, n, &tot, s));   // (below 2^31: see stream_fits)
     ASSS_TRY(out.col.alloc(tot > 0 ? tot : 1));
     ASSS_TRY(out.val.alloc(tot > 0 ? tot : 1));
     k_stream_fill<T><<<cdiv((int64_t)n * 32, 256), 256, 0, s>>>(n, A.rp.p, A.ci.p, A.v.p, len.p, out.rp.p, out.col.p,

@@ -1,8 +1,9 @@
-"""What the host makes of a whole-solve launch's report, for a wait that runs out at any barrier of
-any block (csrc/solve_rules.h, compiled here with the host's compiler).  The model follows the
-kernel's protocol: a block that gave up arrives at no later barrier, block 0 writes a column's
-status before the column's last barrier and leaves behind it if it gave up, and whoever gives up sets
-the barrier's status word."""
+"""The host's rules of the solve path (csrc/solve_rules.h, compiled here with the host's compiler).
+
+What the host makes of a whole-solve launch's report, for a wait that runs out at any barrier of
+any block: the model follows the kernel's protocol (a block that gave up arrives at no later barrier,
+block 0 writes a column's status before the column's last barrier and leaves behind it if it gave
+up, and whoever gives up sets the barrier's status word)."""
 import os
 import shutil
 import subprocess
@@ -76,13 +77,40 @@ int main() {
 """
 
 
-def test_a_wait_that_runs_out_is_never_a_success(tmp_path):
+STREAM = r"""
+#include "solve_rules.h"
+using namespace asss;
+
+int main() {
+    int bad = 0;
+    for (int tb = 4; tb <= 8; tb += 4) {
+        const int most = 192000 / tb;
+        bad += !stream_fits(1000, 64000, tb) + stream_fits(1000, 63999, tb);
+        bad += !stream_fits(most, 64LL * most, tb) + stream_fits(most + 1, 64LL * (most + 1), tb);
+        // padded by up to 3 entries a row the offsets stay below 2^31; SELL takes what may not
+        const long long full = (1LL << 31) - 1024 - 3LL * most;
+        if ((long long)most * (most - 1) >= full) bad += !stream_fits(most, full - 1, tb) + stream_fits(most, full, tb);
+    }
+    return bad;
+}
+"""
+
+
+def _run(tmp_path, source):
     cxx = shutil.which("g++") or shutil.which("c++")
     if not cxx:
         pytest.skip("no host C++ compiler")
     src, exe = tmp_path / "model.cpp", tmp_path / "model"
-    src.write_text(MODEL)
+    src.write_text(source)
     inc = [f"-I{os.path.join(ROOT, 'include')}", f"-I{os.path.join(ROOT, 'paper_2009_06954_gb300', 'csrc')}"]
     subprocess.run([cxx, "-std=c++17", "-O1", "-Wall", "-Werror", *inc, str(src), "-o", str(exe)], check=True)
     p = subprocess.run([str(exe)], capture_output=True, text=True, timeout=60)
     assert p.returncode == 0, p.stdout
+
+
+def test_a_wait_that_runs_out_is_never_a_success(tmp_path):
+    _run(tmp_path, MODEL)
+
+
+def test_row_stream_leaves_to_sell_what_its_offsets_cannot_hold(tmp_path):
+    _run(tmp_path, STREAM)
