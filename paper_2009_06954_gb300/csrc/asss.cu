@@ -2071,7 +2071,7 @@ static int cluster_size(const asss_handle* h, int nrhs) {
     if (h->n > CL_MOST) return size;
     for (int t = 0; t < CL_NSIZES; ++t) {
         if (h->cl_counts[t] < 1) continue;
-        const int waves = cdiv(nrhs, h->cl_counts[t]);
+        const int waves = cl_waves(nrhs, h->cl_counts[t]);
         const double m = n / CL_SIZES[t];
         const double us = waves * (!fp32 ? 185.0 + 0.51 * m : m <= CL_FEW_ROWS ? 105.0 + 0.176 * m : 125.0 + 0.133 * m);
         if (us < best) {

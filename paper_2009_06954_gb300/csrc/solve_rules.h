@@ -30,6 +30,12 @@ struct ClReport {
     ClStat st[CL_CHUNK];
 };
 
+// rounds that nrhs columns take when `side` of them are solved side by side, in launches of CL_CHUNK
+inline int cl_waves(int nrhs, int side) {
+    const int rest = nrhs % CL_CHUNK;
+    return nrhs / CL_CHUNK * ((CL_CHUNK + side - 1) / side) + (rest + side - 1) / side;
+}
+
 // before a launch of nc columns: nothing is reported yet, so that what the kernel does not get to
 // write (the columns after a wait that ran out) does not pass for an earlier launch's result
 inline void cl_expect(ClReport& r, int nc) {

@@ -96,6 +96,24 @@ int main() {
 """
 
 
+WAVES = r"""
+#include "solve_rules.h"
+using namespace asss;
+
+int main() {
+    int bad = 0;
+    for (int side = 1; side <= 20; ++side)
+        for (int nrhs = 1; nrhs <= 70; ++nrhs) {
+            int rounds = 0;
+            for (int left = nrhs; left > 0; left -= CL_CHUNK)   // a launch each
+                for (int c = left < CL_CHUNK ? left : CL_CHUNK; c > 0; c -= side) ++rounds;
+            bad += cl_waves(nrhs, side) != rounds;
+        }
+    return bad != 0;
+}
+"""
+
+
 def _run(tmp_path, source):
     cxx = shutil.which("g++") or shutil.which("c++")
     if not cxx:
@@ -114,3 +132,7 @@ def test_a_wait_that_runs_out_is_never_a_success(tmp_path):
 
 def test_row_stream_leaves_to_sell_what_its_offsets_cannot_hold(tmp_path):
     _run(tmp_path, STREAM)
+
+
+def test_waves_are_counted_by_launch(tmp_path):
+    _run(tmp_path, WAVES)
