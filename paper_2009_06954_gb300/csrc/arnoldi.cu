@@ -143,8 +143,10 @@ __device__ __forceinline__ void ao_close(const AoParams& p, const double* s_h1, 
 // in registers through the three passes, which are read once and all at the start (up to
 // R (NVC + 1) loads in flight).  8 warps a block: the FP64 pipe needs no more, and each warp
 // costs its share of FP64 adds in the block's sums.  Bound: the chain of two grid barriers
-// with their sums.  Mean over the steps of a solve, against the sweeping kernel this replaced
-// at these sizes: n = 10^3 22 -> 12 us, 47^3 29 -> 17 us, 64^3 36 -> 22 us.
+// with their sums.  It serves the Lanczos set-up and FGMRES launch by launch (restarts above 60,
+// general patterns; the whole-solve kernel has its own step).  Mean over the steps of a
+// launch-by-launch solve, against the sweeping kernel this replaced at these sizes: n = 10^3
+// 22 -> 12 us, 47^3 29 -> 17 us, 64^3 36 -> 22 us.
 template <int NVC, int R>
 __global__ void __launch_bounds__(AO_TIGHT, 1) k_arnoldi_tight(AoParams p) {
     __shared__ double s_w[AO_TIGHT / 32][NVC + 1];
@@ -244,7 +246,7 @@ __global__ void __launch_bounds__(AO_TIGHT, 1) k_arnoldi_tight(AoParams p) {
 // AO_REGV vectors a row's dot products run together, U rows at a time, so that U (nv + 1) loads
 // are in flight; above that the dot products are spread over the warps (a warp takes a vector,
 // or a share of its rows) and need no sums across warps in registers: 41 -> 19 us a step at
-// n = 20011 over 15 steps; 56 -> 47 us at 100^3, where FP64 FMAs and bytes need about 20.
+// n = 20011 over 15 steps; 56 -> 47 us at 100^3 launch by launch, where FP64 FMAs and bytes need about 20.
 __global__ void __launch_bounds__(AO_WIDE, 1) k_arnoldi_orth(AoParams p) {
     constexpr int NW = AO_WIDE / 32;
     __shared__ double s_w[NW][AO_REGV + 1];

@@ -1,4 +1,4 @@
-// Device helpers of the cluster-scope kernels: one thread-block cluster (16 or 8 CTAs) works
+// Device helpers of the cluster-scope kernels: one thread-block cluster (8 to 16 CTAs) works
 // on a system of its own, so a synchronisation is the hardware's cluster barrier and a sum over
 // the system goes through distributed shared memory (a few hundred ns together), where a
 // grid-wide step pays two to three microseconds for its counter and its partials in L2.

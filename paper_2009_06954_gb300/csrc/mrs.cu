@@ -425,7 +425,7 @@ extern "C" asss_status asss_mrs_noalloc(int64_t n, int64_t nnz, const int64_t* r
     int nslices = (int)((n + 31) / 32);
     int nblk = mrs_blocks<double, 2>(c.sms, occ, nslices);
     if (nblk > NOALLOC_MAX_BLOCKS) nblk = NOALLOC_MAX_BLOCKS;
-    unsigned* ctrl = reinterpret_cast<unsigned*>(base);  // [0] count [1] gen [2] err [3] its; ratio at base[3]
+    unsigned* ctrl = reinterpret_cast<unsigned*>(base);  // [0] count [2] err [3] its; ratio at base[3]
     double* part = base + NOALLOC_CTRL;
     int* blk = reinterpret_cast<int*>(base + NOALLOC_CTRL + NOALLOC_PART);
     double* Y = base + NOALLOC_CTRL + NOALLOC_PART + NOALLOC_BLK;

@@ -5,11 +5,11 @@
 //
 // What bounds a solve of a small or middling system in the launch-by-launch path is not its
 // data but its 30 to 100 launches, the host's decisions between them and the grid-wide
-// barriers inside them.  Here the 16 CTAs of a cluster own contiguous rows; sums over the system
+// barriers inside them.  Here the CTAs of a cluster own contiguous rows; sums over the system
 // are exchanged through distributed shared memory, every CTA adds them in the same order and
 // takes the same decisions, and vectors that other CTAs read go through L2 around a cluster
-// barrier.  Several right-hand sides are as many clusters side by side (nine fit on the GPU).
-// Bound: the latency of a row's loads and of a synchronisation; for larger systems 16 SMs' share
+// barrier.  Several right-hand sides are as many clusters side by side (see CL_SIZES).
+// Bound: the latency of a row's loads and of a synchronisation; for larger systems a cluster's share
 // of the bandwidth and of the FP64 pipe, so those run the same code in grid scope (cluster_size
 // in asss.cu has both sides measured).
 #pragma once
