@@ -2058,9 +2058,10 @@ static asss_status do_setup(asss_handle* h, const asss_csr* Ain, asss_stats* st)
 // synchronise and to fold sums over), above it 512, whose loads hide more latency.  256 / 512 threads:
 // 10^3 (63 rows) 111 / 130, 16^3 (256) 157 / 179, 24^3 (91, grid) 215 / 236, 36^3 (307) 254 / 251, 47^3 (683)
 // 304 / 318, 56^3 (1155) 436 / 430, 64^3 (1725) 538 / 494; eight columns at 24^3 (864) 299 / 300, at 32^3 (2048)
-// 523 / 471.  FP64 always 256 (8^3 215 / 255, 24^3 325 / 374, 36^3 466 / 461, 64^3 1252 / 1270): at 512 its
-// registers spill.
-constexpr int CL_FEW_ROWS = 768;
+// 523 / 471.  FP64, whose registers spill at 512: 24^3 313 / 360, 36^3 500 / 490, 47^3 663 / 735, 56^3 (1155 rows
+// a block) 991 / 1044, 64^3 (1725) 1192 / 1207, 72^3 (2456) 1894 / 1778, 80^3 2250 / 2060, 100^3 4548 / 4100,
+// 120^3 7357 / 6507: 256 up to CL_FEW_ROWS64 rows, and in clusters (8^3 215 / 255).
+constexpr int CL_FEW_ROWS = 768, CL_FEW_ROWS64 = 2048;
 static int cluster_size(const asss_handle* h, int nrhs) {
     constexpr int CL_MOST = 300000;   // above it the columns' vectors leave L2 (not measured)
     const bool fp32 = h->opt.precision == ASSS_PREC_MIXED;
@@ -2251,6 +2252,8 @@ static asss_status solve_cluster(asss_handle* h, int tr, int size, int nc, const
     if constexpr (sizeof(T) == 4) {
         const int rows = cdiv(h->n, size < 0 ? c.sms : size);   // of a CTA
         if (h->kp == 0 || rows > CL_FEW_ROWS) return cl_dispatch<T, 1, 512>(c, a, h->kp, size, count, nullptr);
+    } else if (size < 0 && cdiv(h->n, c.sms) > CL_FEW_ROWS64) {
+        return cl_dispatch<T, 1, 512>(c, a, h->kp, size, count, nullptr);
     }
     return cl_dispatch<T, 1, 256>(c, a, h->kp, size, count, nullptr);
 }

@@ -235,7 +235,7 @@ __device__ __noinline__ void cl_tri_sweep(E* vec, const E* own, const int2* rows
 // rows a block, 395 000 in all): 64^3 513 -> 487 us, 70^3 650 -> 596, adjoint at 64^3 543 -> 505,
 // 47^3 323 -> 317.  Not in clusters (24^3 249 -> 246, 48^3 with eight columns does not fit), and not
 // a part of the rows: the L1 that shared memory takes costs as much (100^3 1423 -> 1425 .. 1481).
-// NT: 256 threads where a CTA has few rows and in FP64, else 512 (see cluster_size).
+// NT: 256 threads where a CTA has few rows, else 512 (see cluster_size).
 template <class T, int KP, int FMT, bool GRID, int NT, bool QS = false>
 __global__ void __launch_bounds__(NT, 1) k_solve_cl(const ClArgs<T> p) {
     constexpr int NW = NT / 32, NV = KP + 1, KQ = KP > 0 ? KP : 1;
@@ -1226,13 +1226,16 @@ static asss_status cl_run_grid(const Ctx& c, const ClArgs<T>& a) {
     return ASSS_OK;
 }
 
+// (FP64 on diagonals takes 512 threads in grid scope only)
 template <class T, int FMT, int NT>
 asss_status cl_dispatch(const Ctx& c, const ClArgs<T>& a, int kp, int size, int count, int* counts) {
+    constexpr bool CLUSTERS = !(sizeof(T) == 8 && FMT == 1 && NT == 512);
     switch (kp) {
 #define ASSS_CL_CASE(KPV) \
     case KPV:             \
         if constexpr (FMT == 1) { if (size < 0) return cl_run_grid<T, KPV, NT>(c, a); } \
-        return cl_run<T, KPV, FMT, NT>(c, a, size, count, counts);
+        if constexpr (CLUSTERS) return cl_run<T, KPV, FMT, NT>(c, a, size, count, counts); \
+        break;
         ASSS_CL_CASE(4)
         ASSS_CL_CASE(8)
         ASSS_CL_CASE(12)
@@ -1243,18 +1246,20 @@ asss_status cl_dispatch(const Ctx& c, const ClArgs<T>& a, int kp, int size, int 
         case 0:
             if constexpr (sizeof(T) == 8 || NT == 512) {
                 if constexpr (FMT == 1) { if (size < 0) return cl_run_grid<T, 0, NT>(c, a); }
-                return cl_run<T, 0, FMT, NT>(c, a, size, count, counts);
+                if constexpr (CLUSTERS) return cl_run<T, 0, FMT, NT>(c, a, size, count, counts);
             }
+            break;
 #undef ASSS_CL_CASE
-        default:
-            set_error("cluster solve: unsupported padded Lanczos width %d", kp);
-            return ASSS_ERR_UNSUPPORTED;
     }
+    set_error("cluster solve: unsupported padded Lanczos width %d", kp);
+    return ASSS_ERR_UNSUPPORTED;
 }
 
-// (solve_cluster32.cu, solve_cluster32s.cu, solve_cluster64.cu, solve_cluster_fac32.cu, solve_cluster_fac64.cu)
+// (solve_cluster32.cu, solve_cluster32s.cu, solve_cluster64.cu, solve_cluster64w.cu, solve_cluster_fac32.cu,
+// solve_cluster_fac64.cu)
 extern template asss_status cl_dispatch<float, 1, 512>(const Ctx&, const ClArgs<float>&, int, int, int, int*);
 extern template asss_status cl_dispatch<float, 1, 256>(const Ctx&, const ClArgs<float>&, int, int, int, int*);
+extern template asss_status cl_dispatch<double, 1, 512>(const Ctx&, const ClArgs<double>&, int, int, int, int*);
 extern template asss_status cl_dispatch<double, 1, 256>(const Ctx&, const ClArgs<double>&, int, int, int, int*);
 extern template asss_status cl_dispatch<float, 3, 512>(const Ctx&, const ClArgs<float>&, int, int, int, int*);
 extern template asss_status cl_dispatch<double, 3, 512>(const Ctx&, const ClArgs<double>&, int, int, int, int*);
