@@ -281,6 +281,10 @@ __global__ void __launch_bounds__((mrs_threads<T, FMT>()), 1) k_mrs(MrsParams<T>
     constexpr int NV = KP + 1;
     constexpr bool QBLK = q_blocked<T>(FMT == 1 || FMT == 3);
     constexpr int NT = mrs_threads<T, FMT>(), NW = NT / 32;
+    // x is read with a row's first loads; not in the FP64 SELL pass, where 16 entries in flight and
+    // 2 (k + 1) values fill the registers and one more row value cuts the batch (n = 30 000, k = 20:
+    // 286 us a step against 236; at k = 8 190 against 198)
+    constexpr bool XEARLY = !(FMT == 0 && sizeof(T) == 8 && KP > 12);
     if (p.skip && *p.skip) {  // enqueued ahead of a decision that went the other way
         if (blockIdx.x == 0 && threadIdx.x == 0) {
             *p.out_its = -1;
@@ -709,7 +713,7 @@ __global__ void __launch_bounds__((mrs_threads<T, FMT>()), 1) k_mrs(MrsParams<T>
             if (j >= 2) {
                 T pv = (tnp * yold - tdpp * pold) * tthp;
                 Pj1[i] = pv;
-                xv[i] = xold + txp * pv;
+                xv[i] = (XEARLY ? xold : xv[i]) + txp * pv;
             }
         };
         if constexpr (FMT == 4) {
@@ -817,7 +821,7 @@ __global__ void __launch_bounds__((mrs_threads<T, FMT>()), 1) k_mrs(MrsParams<T>
             const T pold = (live && j >= 2) ? Pj1[i] : (T)0;
             // x with the other loads ahead of the products: read at its use, its latency stood
             // at the end of every row (FP32 pass at 100^3: 26.4 -> 24.5 us, at 47^3 3.55 -> 3.33)
-            const T xold = (live && j >= 2) ? xv[i] : (T)0;
+            const T xold = (XEARLY && live && j >= 2) ? xv[i] : (T)0;
             uint4 qraw[(QB && KP > 0) ? KP / 8 : 1];
             if constexpr (QB && KP > 0) {
                 if (live) {
