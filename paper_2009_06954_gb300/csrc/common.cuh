@@ -139,6 +139,8 @@ struct DSell {
     DBuf<unsigned> hcnt;
 };
 constexpr int SELL_SPLIT = 1024;
+// rows rounded up to whole slices: vectors that stand one behind the other start on 128 bytes
+__host__ __device__ constexpr long long pad32(long long n) { return (n + 31) / 32 * 32; }
 
 // Row-stream storage for long rows whose vector fits shared memory: the rows one after
 // the other, each padded to a multiple of 4 entries (value 0 on its own column), columns in

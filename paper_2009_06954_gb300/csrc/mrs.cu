@@ -46,7 +46,8 @@ void mrs_work_destroy(MrsWork* w) { delete w; }
 // the layout changes; the kernel never writes the halos)
 template <class T>
 static asss_status y_layout(MrsWork* w, DBuf<T>& Ybuf, int& cur, int H, cudaStream_t s, T** Y, long long* ystride) {
-    long long st = ((long long)w->n + 2LL * H + 31) / 32 * 32;   // every slot starts on 128 bytes (H = 0)
+    H = (int)pad32(H);   // every slot's row 0 starts on 128 bytes
+    const long long st = pad32(w->n) + 2LL * H;
     if (cur != H || Ybuf.n < 3 * st) {
         if (Ybuf.n < 3 * st) ASSS_TRY(Ybuf.alloc(3 * st));
         ASSS_CUDA(cudaMemsetAsync(Ybuf.p, 0, sizeof(T) * (size_t)Ybuf.n, s));
@@ -169,7 +170,7 @@ asss_status mrs_solve(const Ctx& c, MrsWork* w, const MrsOperator& op, bool fp32
             set_error("FP32 mrs needs the FP32 operator and an FP32 output");
             return ASSS_ERR_ARG;
         }
-        if (!w->P32.p) ASSS_TRY(w->P32.alloc((int64_t)2 * n));
+        if (!w->P32.p) ASSS_TRY(w->P32.alloc(2 * pad32(n)));
         ASSS_TRY(dispatch_mrs<float>(c, w, op.J32, op.D32, op.Q32, op.alpha, op.k, op.kp, shift, sign, rhs, x32,
                                      w->Y32, w->halo32, w->P32.p, tol, maxit, &nnz_read, lo,
                                      (const __nv_bfloat16*)op.Q16, op.kp16, op.F, op.R32));
@@ -178,7 +179,7 @@ asss_status mrs_solve(const Ctx& c, MrsWork* w, const MrsOperator& op, bool fp32
             set_error("FP64 mrs needs the FP64 operator and an FP64 output");
             return ASSS_ERR_ARG;
         }
-        if (!w->P64.p) ASSS_TRY(w->P64.alloc((int64_t)2 * n));
+        if (!w->P64.p) ASSS_TRY(w->P64.alloc(2 * pad32(n)));
         ASSS_TRY(dispatch_mrs<double>(c, w, op.J64, op.D64, op.Q64, op.alpha, op.k, op.kp, shift, sign, rhs, x64,
                                       w->Y64, w->halo64, w->P64.p, tol, maxit, &nnz_read, lo, nullptr, 0, op.F,
                                       op.R64));
@@ -469,6 +470,7 @@ extern "C" asss_status asss_mrs_noalloc(int64_t n, int64_t nnz, const int64_t* r
     prm.cci = col_idx;
     prm.cval = val;
     prm.ystride = n;
+    prm.pstride = n;
     prm.Q = q_rowmajor;
     prm.alpha = alpha;
     prm.k = k;

@@ -89,6 +89,34 @@ __device__ __forceinline__ float2 df_add(float2 a, float2 b) {
     return make_float2(hi, lo);
 }
 
+// Row i of J~ y over skew half-diagonals, G at a time, the 4 G loads of a group ahead of its products
+// (Ud: U_0 at the row, yi: y at the row).  The order in which ptxas issues the loads of the
+// plain loop changes with everything around it; where that costs, the kernels take this one.
+// k_mrs, FP32, G = 12 against the plain loop, solves launch by launch at 115^3: k = 8 2205 -> 2127 us,
+// 12 2273 -> 2141, 20 2384 -> 2308, 32 2514 -> 2360, BF16 Q_k 20 2344 -> 2070; at 150^3 k = 20 5131 -> 4928,
+// BF16 5126 -> 4281; at 100^3 equal (k = 20 1621 / 1628, BF16 1602 -> 1530).  G = 6 and 8 lose in places.
+template <class T, int G>
+__device__ __forceinline__ T dia_row(const T* __restrict__ Ud, long long ustride, const T* yi, const int* off,
+                                     int ndiag) {
+    T acc = (T)0;
+    for (int d0 = 0; d0 < ndiag; d0 += G) {
+        T ua[G], ub[G], ya[G], yb[G];
+#pragma unroll
+        for (int u = 0; u < G; ++u) {
+            const bool in = d0 + u < ndiag;
+            const int m = in ? off[d0 + u] : 0;
+            const T* Um = Ud + (in ? d0 + u : 0) * ustride;
+            ua[u] = in ? __ldg(Um) : (T)0;
+            ub[u] = in ? __ldg(Um - m) : (T)0;
+            ya[u] = yi[m];
+            yb[u] = yi[-m];
+        }
+#pragma unroll
+        for (int u = 0; u < G; ++u) acc += ua[u] * ya[u] - ub[u] * yb[u];
+    }
+    return acc;
+}
+
 // sum of N values by a balanced tree in a fixed order (log2 N dependent additions)
 template <class P, int N, class Add>
 __device__ __forceinline__ P pair_tree(P (&a)[N], Add add) {

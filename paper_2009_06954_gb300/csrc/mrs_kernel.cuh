@@ -136,6 +136,7 @@ struct MrsParams {
     T* ft;               // (I + L)^-T (wd .* y)
     T* fw;               // (I + L)^-1 J^ ft
     long long ystride;  // distance between the three Y slots (n + 2 halo)
+    long long pstride;  // distance between the two P slots
     const T* Q;
     const __nv_bfloat16* Q16;  // BF16 copy of Q (row stride KP) when the kernel reads Q in BF16
     const double* alpha;
@@ -144,7 +145,7 @@ struct MrsParams {
     const double* rhs;
     T* x;
     T* Y;  // 3 slots of unnormalised Lanczos vectors, each with a zero halo on both ends
-    T* P;  // 2n ring of update directions
+    T* P;  // ring of two update directions
     double* part;  // [2][NV][nblk]
     GridBarrier gb;
     const int* blk_slice;
@@ -592,7 +593,7 @@ __global__ void __launch_bounds__((mrs_threads<T, FMT>()), 1) k_mrs(MrsParams<T>
             p.Y[i] = b;
             p.x[i] = (T)0;
             p.P[i] = (T)0;
-            p.P[p.n + i] = (T)0;
+            p.P[p.pstride + i] = (T)0;
             tacc[0] += b * b;
             T q[KP > 0 ? KP : 1];
             if constexpr (QB) load_qrow16<T, KP>(p.Q16, i, q);
@@ -663,7 +664,7 @@ __global__ void __launch_bounds__((mrs_threads<T, FMT>()), 1) k_mrs(MrsParams<T>
         const T* __restrict__ Ycur = p.Y + (size_t)((j - 1) % 3) * ys;
         const T* __restrict__ Yold = p.Y + (size_t)((j + 1) % 3) * ys;
         T* __restrict__ Ynew = p.Y + (size_t)(j % 3) * ys;
-        T* __restrict__ Pj1 = p.P + (size_t)((j - 1) & 1) * p.n;
+        T* __restrict__ Pj1 = p.P + (size_t)((j - 1) & 1) * p.pstride;
         T* __restrict__ xv = p.x;
         const T* __restrict__ Ub = p.U;
         const T* __restrict__ Qr = p.Q;
@@ -909,14 +910,14 @@ __global__ void __launch_bounds__((mrs_threads<T, FMT>()), 1) k_mrs(MrsParams<T>
                 if (i < n) {
                     const T* Ud = Ub + i;
                     const T* yi = Ycur + i;
+                    if constexpr (sizeof(T) == 4) {
+                        acc = dia_row<T, 12>(Ud, p.ustride, yi, s_off, p.ndiag);
+                    } else {
 #pragma unroll 12
-                    for (int d = 0; d < p.ndiag; ++d, Ud += p.ustride) {
-                        const int m = s_off[d];
-                        if constexpr (sizeof(T) == 8) {   // two FMAs a diagonal, no separate product and sum
+                        for (int d = 0; d < p.ndiag; ++d, Ud += p.ustride) {
+                            const int m = s_off[d];   // two FMAs a diagonal, no separate product and sum
                             acc = fma(__ldg(Ud), yi[m], acc);
                             acc = fma(-__ldg(Ud - m), yi[-m], acc);
-                        } else {
-                            acc += __ldg(Ud) * yi[m] - __ldg(Ud - m) * yi[-m];
                         }
                     }
                 }
@@ -998,7 +999,7 @@ __global__ void __launch_bounds__((mrs_threads<T, FMT>()), 1) k_mrs(MrsParams<T>
         }
         __syncthreads();
         if (sc.stop) {
-            T* Pj = p.P + (size_t)(j & 1) * p.n;
+            T* Pj = p.P + (size_t)(j & 1) * p.pstride;
             const T tn = s_cf[7], td = s_cf[8], tth = s_cf[9], tx = s_cf[10];
 #pragma unroll
             for (int v = 0; v < NV; ++v) tacc[v] = (T)0;
@@ -1162,6 +1163,7 @@ static asss_status launch_mrs(const Ctx& c, MrsWork* w, const OpView<T>& J, cons
         }
     }
     prm.ystride = ystride;
+    prm.pstride = pad32(J.n);
     prm.Q = Q;
     prm.Q16 = Q16;
     prm.alpha = alpha;
