@@ -2042,7 +2042,8 @@ static asss_status do_setup(asss_handle* h, const asss_csr* Ain, asss_stats* st)
 // cluster-scope solves (solve_cluster.cuh)
 // ---------------------------------------------------------------------------
 // How nrhs columns are solved: by clusters of that many CTAs side by side, one after another in
-// grid scope (-1), or launch by launch (0: the incomplete factor where no cluster fits).
+// grid scope (-1), or launch by launch (0: the incomplete factor where no cluster fits, and the
+// systems too large for grid_scope_pays).
 // One cluster has its SMs' share of the bandwidth and the FP64 pipe, but cheap synchronisations and
 // company; grid scope has the whole GPU and pays two to three microseconds a synchronisation.
 // Both grow linearly with the rows of a CTA; in microseconds for 4 outer and 20 inner steps, measured
@@ -2065,6 +2066,7 @@ constexpr int CL_FEW_ROWS = 768, CL_FEW_ROWS64 = 2048;
 static int cluster_size(const asss_handle* h, int nrhs) {
     constexpr int CL_MOST = 300000;   // above it the columns' vectors leave L2 (not measured)
     const bool fp32 = h->opt.precision == ASSS_PREC_MIXED;
+    if (fp32 && !h->factored && !grid_scope_pays(h->n, h->kp)) return 0;
     const double n = h->n;
     double best = nrhs * (fp32 ? 200.0 + 0.00105 * n : 285.0 + 0.0037 * n);
     if (h->factored) best = nrhs * 3000.0;   // a grid barrier or a launch per colour: 24^3 4295 us against 1133

@@ -101,8 +101,8 @@ struct ClArgs {
 
 // doubles of workspace per cluster
 inline long long cl_work_doubles(int n, int halo, int restart, int tbytes) {
-    const long long nd = (long long)(5 + 2 * restart + 1) * n;
-    const long long nt = 3LL * ((long long)n + 2LL * halo + 32) + 3LL * n;
+    const long long nd = (5 + 2 * restart + 1) * pad32(n);
+    const long long nt = 3 * (pad32(n) + 2LL * halo + 32) + 3 * pad32(n);
     return nd + (nt * tbytes + 7) / 8 + 64;
 }
 
@@ -236,11 +236,20 @@ __device__ __noinline__ void cl_tri_sweep(E* vec, const E* own, const int2* rows
 // 47^3 323 -> 317.  Not in clusters (24^3 249 -> 246, 48^3 with eight columns does not fit), and not
 // a part of the rows: the L1 that shared memory takes costs as much (100^3 1423 -> 1425 .. 1481).
 // NT: 256 threads where a CTA has few rows, else 512 (see cluster_size).
+// WIDE: the FP32 form whose Q_k comes from global memory, for large systems.  Its time hangs on the
+// order in which ptxas issues a row's loads, which differs between widths that read the same source: with
+// the plain loop over the diagonals a mrs step at 100^3 took 45 us at k = 8 against 35 at k = 20, and at
+// 130^3 solves at k = 4, 8 and 12 were slower than launch by launch.  Up to k = 12 the loads of all
+// diagonals are issued together (dia_row), and the vectors start on 128 bytes.  Solves at 130^3, k = 4 / 8 /
+// 12 / 16 / 20 / 24 / 32, before: 4053 / 5060 / 4015 / 3275 / 3295 / 3631 / 4168 us, now 3117 / 2917 / 3349 / 3295 /
+// 3282 / 3340 / 3930; at 100^3 from k = 8 on 1609 / 1454 / 1351 / 1403 / 1519 / 1775, now 1334 / 1449 / 1380 / 1404 /
+// 1467 / 1697.  (dia_row at k = 16 / 20 / 24 / 32: 1423 / 1461 / 1532 / 1651.)
 template <class T, int KP, int FMT, bool GRID, int NT, bool QS = false>
 __global__ void __launch_bounds__(NT, 1) k_solve_cl(const ClArgs<T> p) {
     constexpr int NW = NT / 32, NV = KP + 1, KQ = KP > 0 ? KP : 1;
     using Sh = ClShared<T, KP, GRID, NT>;
     using P2 = typename Sh::P2;
+    constexpr bool WIDE = sizeof(T) == 4 && FMT == 1 && GRID && NT == 512 && !QS && KP > 0;
     extern __shared__ __align__(16) unsigned char s_dyn[];
     Sh& sh = *reinterpret_cast<Sh*>(s_dyn);
     double* H = reinterpret_cast<double*>(s_dyn + ((sizeof(Sh) + 15) & ~15));   // (restart + 1) x restart, column-major
@@ -252,7 +261,7 @@ __global__ void __launch_bounds__(NT, 1) k_solve_cl(const ClArgs<T> p) {
     const int re = min(n, (int)((long long)nsl * (rank + 1) / C) * 32);
     const int nact = min(NW, max(re - rb + 31, 0) >> 5);   // warps that hold rows; the others' sums stay zero
     double* base = p.work + (GRID ? (size_t)0 : (size_t)cl_id() * (size_t)p.work_stride);
-    const long long nn = n;
+    const long long nn = WIDE ? pad32(n) : n;
     double *r = base, *rh = r + nn, *t1 = rh + nn, *t2 = t1 + nn, *wv = t2 + nn;
     double* V = wv + nn;
     double* Z = V + (R + 1) * nn;
@@ -283,7 +292,7 @@ __global__ void __launch_bounds__(NT, 1) k_solve_cl(const ClArgs<T> p) {
     // the halos of the three Lanczos slots (nothing else writes them)
     for (int t = rank * NT + tid; t < 6 * p.halo; t += C * NT) {
         const int slot = t / (2 * p.halo), e = t % (2 * p.halo);
-        Y[slot * ys + (e < p.halo ? e - p.halo : nn + (e - p.halo))] = (T)0;
+        Y[slot * ys + (e < p.halo ? e - p.halo : n + (e - p.halo))] = (T)0;
     }
     // FMT 3: replicated vectors, own rows
     const ClFactor<T>& fa = p.fac;
@@ -693,14 +702,18 @@ __global__ void __launch_bounds__(NT, 1) k_solve_cl(const ClArgs<T> p) {
                 }
                 const T* Ud = p.U + i;
                 const T* yi = Ycur + i;
+                if constexpr (WIDE && KP <= 12) {
+                    acc = dia_row<T, 12>(Ud, p.ustride, yi, sh.off, p.ndiag);
+                } else {
 #pragma unroll 12
-                for (int d = 0; d < (FMT == 1 ? p.ndiag : 0); ++d, Ud += p.ustride) {
-                    const int mo = sh.off[d];
-                    if constexpr (sizeof(T) == 8) {
-                        acc = fma(__ldg(Ud), yi[mo], acc);
-                        acc = fma(-__ldg(Ud - mo), yi[-mo], acc);
-                    } else {
-                        acc += __ldg(Ud) * yi[mo] - __ldg(Ud - mo) * yi[-mo];
+                    for (int d = 0; d < (FMT == 1 ? p.ndiag : 0); ++d, Ud += p.ustride) {
+                        const int mo = sh.off[d];
+                        if constexpr (sizeof(T) == 8) {
+                            acc = fma(__ldg(Ud), yi[mo], acc);
+                            acc = fma(-__ldg(Ud - mo), yi[-mo], acc);
+                        } else {
+                            acc += __ldg(Ud) * yi[mo] - __ldg(Ud - mo) * yi[-mo];
+                        }
                     }
                 }
                 T q[KQ];

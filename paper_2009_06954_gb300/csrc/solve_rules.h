@@ -30,6 +30,13 @@ struct ClReport {
     ClStat st[CL_CHUNK];
 };
 
+// Whether an FP32 solve on skew diagonals is faster in grid scope than launch by launch.  A large
+// solve's launches cost little beside its steps, and k_mrs has more registers for them: at 130^3
+// (2.2 * 10^6 rows), k = 12 / 16 / 20 / 24, grid 3366 / 3308 / 3289 / 3341 us, launches 3210 / 3399 / 3439 / 3294;
+// at 150^3 (3.4 * 10^6) 4829 / 4767 / 4858 / 5055 and 4447 / 4705 / 4867 / 4753.  Without deflation, whose
+// rows have the fewest loads: 100^3 1125 / 1300, 115^3 1673 / 1700, 130^3 2937 / 2548, 150^3 4128 / 3387.
+inline bool grid_scope_pays(int n, int kp) { return n <= (kp > 0 ? 2500000 : 1600000); }
+
 // rounds that nrhs columns take when `side` of them are solved side by side, in launches of CL_CHUNK
 inline int cl_waves(int nrhs, int side) {
     const int rest = nrhs % CL_CHUNK;

@@ -102,6 +102,9 @@ using namespace asss;
 
 int main() {
     int bad = 0;
+    // the benchmark's 100^3 is in grid scope at every width, the largest systems go launch by launch
+    bad += !grid_scope_pays(1000000, 0) + !grid_scope_pays(2500000, 4) + grid_scope_pays(2500001, 32) +
+           grid_scope_pays(1600001, 0);
     for (int side = 1; side <= 20; ++side)
         for (int nrhs = 1; nrhs <= 70; ++nrhs) {
             int rounds = 0;
@@ -134,5 +137,5 @@ def test_row_stream_leaves_to_sell_what_its_offsets_cannot_hold(tmp_path):
     _run(tmp_path, STREAM)
 
 
-def test_waves_are_counted_by_launch(tmp_path):
+def test_waves_are_counted_by_launch_and_scopes_by_rows(tmp_path):
     _run(tmp_path, WAVES)
