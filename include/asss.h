@@ -110,8 +110,8 @@ typedef struct {
                                  scalings, the role of MC64 in §2: |diag| = 1, other entries
                                  <= 1 up to a relative 1e-12 * max(1, max cost))                */
     int    rhs_block;         /* several right-hand sides in asss_solve (FGMRES, k <= 32, FP32 Q) whose
-                                 solves do not run as one launch each (J~ in SELL-C, or restart
-                                 > 60): 1: lockstep blocks of up to 8 columns whose preconditioner
+                                 solves do not run as one launch each (J~ in SELL-C, restart > 60,
+                                 or FP32 above 2.5 * 10^6 rows): 1: lockstep blocks of up to 8 columns whose preconditioner
                                  applications are one multi-column mrs launch per Arnoldi step
                                  (App. B's simultaneous iterations); 0: one column after another.
                                  Elsewhere a column is one launch, and on small systems several
