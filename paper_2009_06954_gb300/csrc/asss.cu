@@ -2396,7 +2396,8 @@ static asss_status solve_common(asss_handle* h, int tr, int nrhs, const double* 
     cudaStream_t s = h->ctx.stream;
     int n = h->n;
     auto t0 = std::chrono::steady_clock::now();
-    bool bdev = is_device_ptr(b), xdev = is_device_ptr(x);
+    const PtrPlace bplace = ptr_place(b, h->ctx.device);
+    bool bdev = bplace != PtrPlace::HOST, xdev = is_device_ptr(x);
     asss_stats lst = h->setup_stats;
     asss_status worst = ASSS_OK;
     // several right-hand sides of a forward FGMRES solve: lockstep blocks of up to 8
@@ -2413,7 +2414,7 @@ static asss_status solve_common(asss_handle* h, int tr, int nrhs, const double* 
         // the kernel reads b to the end and in place: it is staged where x overlaps it, where it is
         // the host's or another device's, and where it is not aligned to its entries
         const bool apart = b0 + (size_t)(nc - 1) * ldb + n <= x0 || x0 + (size_t)(nc - 1) * ldx + n <= b0;
-        const bool stage = !apart || !is_on_device(b0, h->ctx.device) || (uintptr_t)b0 % sizeof(double) != 0;
+        const bool stage = !apart || bplace != PtrPlace::HERE || (uintptr_t)b0 % sizeof(double) != 0;
         // in grid scope the columns run one after another, so fewer of large ones are staged at once
         if (cl < 0 && (stage || !xdev)) nc = std::max(1, std::min(nc, (int)((1 << 25) / (int64_t)n)));
         const double* bt = b0;

@@ -322,10 +322,11 @@ inline bool stream_evict_first(const Ctx& c, long long pass_bytes) {
 }
 asss_status make_ctx(Ctx& c, void* stream, double wait_timeout_ms);
 
-// pointer classification
+// pointer classification: the host's, managed or device dev's (its kernels read it in place), another
+// device's
+enum class PtrPlace { HOST, HERE, ELSEWHERE };
+PtrPlace ptr_place(const void* p, int dev);
 bool is_device_ptr(const void* p);
-// device (or managed) memory that belongs to device dev, which its kernels read in place
-bool is_on_device(const void* p, int dev);
 
 // copy n elements from a host-or-device pointer into a device buffer
 template <class T>

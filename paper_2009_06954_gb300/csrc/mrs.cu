@@ -392,7 +392,7 @@ extern "C" asss_status asss_mrs_noalloc(int64_t n, int64_t nnz, const int64_t* r
                         {k > 1 ? alpha : nullptr, 8, "alpha"}};
     for (const Arr& a : arrs) {
         if (!a.p) continue;
-        if (!is_on_device(a.p, cur_dev)) {
+        if (ptr_place(a.p, cur_dev) != PtrPlace::HERE) {
             set_error("asss_mrs_noalloc: %s must be device memory of the current device %d", a.name, cur_dev);
             return ASSS_ERR_ARG;
         }

@@ -103,26 +103,19 @@ asss_status make_ctx(Ctx& c, void* stream, double wait_timeout_ms) {
     return ASSS_OK;
 }
 
-bool is_device_ptr(const void* p) {
-    if (!p) return false;
+PtrPlace ptr_place(const void* p, int dev) {
+    if (!p) return PtrPlace::HOST;
     cudaPointerAttributes a;
     cudaError_t e = cudaPointerGetAttributes(&a, p);
     if (e != cudaSuccess) {
         cudaGetLastError();
-        return false;
+        return PtrPlace::HOST;
     }
-    return a.type == cudaMemoryTypeDevice || a.type == cudaMemoryTypeManaged;
+    if (a.type == cudaMemoryTypeManaged) return PtrPlace::HERE;
+    if (a.type != cudaMemoryTypeDevice) return PtrPlace::HOST;
+    return a.device == dev ? PtrPlace::HERE : PtrPlace::ELSEWHERE;
 }
-
-bool is_on_device(const void* p, int dev) {
-    cudaPointerAttributes a;
-    if (cudaPointerGetAttributes(&a, p) != cudaSuccess) {
-        cudaGetLastError();
-        return false;
-    }
-    if (a.type == cudaMemoryTypeManaged) return true;
-    return a.type == cudaMemoryTypeDevice && a.device == dev;
-}
+bool is_device_ptr(const void* p) { return ptr_place(p, -1) != PtrPlace::HOST; }
 
 // ---------------------------------------------------------------------------
 // scans
